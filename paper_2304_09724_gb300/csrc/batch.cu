@@ -65,7 +65,7 @@ struct BatchCtl {
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 constexpr size_t kBatchSmem1D = sizeof(double) * 2 * 3 * (1024 + 1);  // F-hat and W(t+dt) of a tile
 // the largest item: a face segment, a first-pass tile (16 fields with halo) or a 1D tile
-constexpr size_t kBatchSmem = cmax(cmax(kFaceSmem, sizeof(double) * 16 * (TYB + 2) * (TX + 2)), kBatchSmem1D);
+constexpr size_t kBatchSmem = cmax(cmax(face_smem<4>(), sizeof(double) * 16 * (TYB + 2) * (TX + 2)), kBatchSmem1D);
 
 __device__ __forceinline__ long long enc(int p, int ph, long long idx) {
   return ((long long)p << 40) | ((long long)ph << 36) | idx;
@@ -251,7 +251,7 @@ template <bool HAS2D>
 __global__ void __launch_bounds__(BT, HAS2D ? 1 : 4) batch_kernel(const BatchProblem* __restrict__ probs, int* pstate,
                                                    BatchCtl* bc, long long* items, unsigned long long* seq,
                                                    unsigned long long mask, long long spin_limit) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
   __shared__ long long s_item;
   __shared__ int s_state;
   for (;;) {
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(BT, HAS2D ? 1 : 4) batch_kernel(const BatchPro
     const int p = (int)(item >> 40), ph = (int)((item >> 36) & 15);
     const long long idx = item & ((1ll << 36) - 1);
     const BatchProblem& B = probs[p];
-    do_item<HAS2D>(B, B.phase_kind[ph], idx, smem);
+    do_item<HAS2D>(B, B.phase_kind[ph], idx, dyn_smem);
     __threadfence();  // this thread's results visible device-wide before the item counts as done
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -378,7 +378,7 @@ constexpr int kNumLockKinds = 6;
 template <int KIND>
 __global__ void __launch_bounds__(BT) lockstep_kernel(const BatchProblem* __restrict__ probs,
                                                       const int* __restrict__ start, int n) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
   int lo = 0, hi = n;  // the last problem whose first block is at or before this one
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(BT) lockstep_kernel(const BatchProblem* __rest
   }
   const BatchProblem& B = probs[lo];
   if (!((const volatile Ctl*)B.ctl)->active) return;  // done, or stopped: its blocks idle
-  item_body<true>(B, KIND, (long long)blockIdx.x - __ldg(start + lo), smem);
+  item_body<true>(B, KIND, (long long)blockIdx.x - __ldg(start + lo), dyn_smem);
 }
 
 // One thread per problem: commits the round's step of every running problem and counts the
@@ -569,7 +569,7 @@ shweno_status shweno_batch_create(shweno_handle* const* hs, int n, void* cuda_st
   if (cudaMemcpy(b->chunk0, ch.data(), n * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaFuncSetAttribute(batch_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem) != cudaSuccess ||
       cudaFuncSetAttribute(batch_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem1D) != cudaSuccess ||
-      cudaFuncSetAttribute(lockstep_kernel<PH_FACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFaceSmem) != cudaSuccess ||
+      cudaFuncSetAttribute(lockstep_kernel<PH_FACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)face_smem<4>()) != cudaSuccess ||
       cudaFuncSetAttribute(lockstep_kernel<PH_TILE1D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem1D) != cudaSuccess) {
     cudaGetLastError();
     shweno_batch_destroy(b);
@@ -676,7 +676,7 @@ size_t lock_smem(const shweno_batch* b, int kind) {
   switch (kind) {
     case PH_INFER: return sizeof(float) * NPARAM;
     case PH_COEF: return sizeof(double) * 16 * (TYB + 2) * (TX + 2);
-    case PH_FACE: return kFaceSmem;
+    case PH_FACE: return face_smem<4>();
     case PH_TILE1D: return sizeof(double) * 2 * 3 * (b->tile1d + 1);
     default: return 0;
   }

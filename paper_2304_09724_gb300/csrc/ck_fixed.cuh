@@ -1,0 +1,165 @@
+// Cauchy-Kovalevskaya procedure of one point in block fixed point: scales and conversions around the
+// generated recursions (ck_fixed_generated.cuh).
+//
+// Units.  Length: L = min(dx, dy) divided by 2^g; velocity: 2^eu; density: 2^e0; so a coefficient
+// of total degree s of rho, (m, n), E is held times 2^-(e0 + g s), 2^-(e0 + eu + g s) and
+// 2^-(e0 + 2 eu + g s), and the equations keep their form.  e0 and eu come from the leading
+// state (rho0, |u0|, |v0|, sqrt(H0) <= 1 in these units); g >= 0 is the smallest growth for which
+// every coefficient of degree s >= 1 is below 1 (the recursion then checks that everything stays
+// below 1/4 and is repeated with a larger g where it does not), so that a steep point, whose
+// coefficients grow with the degree, fits as a smooth one does.  What is rounded is 2^-62 of the
+// field's scale times (2^g)^s, the size its coefficients of that degree have themselves; FP64
+// rounds the leading coefficients at 2^-54.
+#pragma once
+#include <cmath>
+
+#include "ck_fixed_generated.cuh"
+
+namespace shweno {
+
+// Constants for one mesh.
+struct CkFixed {
+  CkFixedConst K;
+  double iL;      // 1 / L: the time coefficients come in units of L
+  double rx, ry;  // L / dx, L / dy: coordinates in units of L
+};
+
+FX_FN Fx fx_const(double x) {
+  FxRange r{0};
+  return fx_split(fx_from_double<FX_C>(x, 0) + FX_HALF, r);
+}
+
+inline void finalize_ck_fixed(CkFixed& C, int dim, double dx, double dy, double gamma) {
+  const double L = dim == 2 && dy < dx ? dy : dx;
+  C.rx = L / dx;
+  C.ry = dim == 2 ? L / dy : 1.0;
+  C.iL = 1.0 / L;
+  C.K.third = fx_const(1.0 / 3.0);
+  C.K.gshift = 0;
+  for (double h = gamma - 1.0; h >= 4.0 && C.K.gshift < 60; h *= 0.5) ++C.K.gshift;
+  C.K.gm1 = fx_const(std::ldexp(gamma - 1.0, -C.K.gshift));
+}
+
+FX_FN int fx_max(int a, int b) { return a > b ? a : b; }
+
+// Leading state of a point as the scales need it (Euler): 1/rho0 and the high words (magnitude
+// bits) of max(|u0|, |v0|) and of H0 = (E0 + p0)/rho0.
+struct CkLead {
+  double ir;
+  int32_t hu, hH;
+};
+
+// Scales of one point: the exponents of its fields and the growth.
+template <int NC>
+struct CkScale {
+  static constexpr int NG = NC == 1 ? 1 : 3;  // groups: {u} or {rho}, {m, n}, {E}
+  int base[NG], eu, g;
+  bool finite;
+  static FX_FN int group(int q) { return NC == 1 || q == 0 ? 0 : (q == NC - 1 ? 2 : 1); }
+  FX_FN int of(int q, int s) const { return base[group(q)] + g * s; }
+};
+
+// a(q, m*5+n) (m + n <= 4; n = 0 only when DIM == 1): spatial Taylor coefficients in cell units.
+template <int NC, int DIM, typename Coef>
+FX_FN CkScale<NC> ck_scale(const Coef& a, const CkLead& lead) {
+  using Scale = CkScale<NC>;
+  constexpr int NG = Scale::NG;
+  Scale S;
+  int top[NG][5];  // largest high word (magnitude bits) by group and degree
+#pragma unroll
+  for (int i = 0; i < NG; ++i)
+#pragma unroll
+    for (int s = 0; s < 5; ++s) top[i][s] = 0;
+#pragma unroll
+  for (int q = 0; q < NC; ++q)
+#pragma unroll
+    for (int m = 0; m < 5; ++m)
+#pragma unroll
+      for (int n = 0; n + m < 5; ++n)
+        if (DIM == 2 || n == 0) {
+          int& t = top[Scale::group(q)][m + n];
+          t = fx_max(t, fx_hi(a(q, m * 5 + n)) & 0x7fffffff);
+        }
+  int all = 0;
+#pragma unroll
+  for (int i = 0; i < NG; ++i)
+#pragma unroll
+    for (int s = 0; s < 5; ++s) all = fx_max(all, top[i][s]);
+  S.finite = all < 0x7ff00000;
+  if constexpr (NC == 1) {
+    // u0 may vanish; 2^-40 of the steepest coefficient is as good a scale then
+    int e = fx_exp(top[0][0]);
+#pragma unroll
+    for (int s = 1; s < 5; ++s) e = fx_max(e, fx_exp(top[0][s]) - 40);
+    S.base[0] = S.eu = fx_max(e, -900);  // an exact 0 then converts to 0
+  } else {
+    const int e0 = fx_max(fx_exp(top[0][0]), -300);  // an exact 0 then converts to 0 in every field
+    int eh = fx_exp(lead.hH);
+    // a negative density or pressure (E0 + p0 then no longer bounds E0 and the kinetic energy)
+    const int ee = fx_exp(top[2][0]) - e0 + 3;
+    if (ee > eh + 3) eh = ee;
+    S.eu = fx_max(fx_max(fx_exp(lead.hu), (eh + 1) >> 1), -300);
+    S.base[0] = e0;
+    S.base[1] = e0 + S.eu;
+    S.base[2] = e0 + 2 * S.eu;
+    S.finite = S.finite && lead.hH < 0x7ff00000 && lead.hu < 0x7ff00000 && (fx_hi(lead.ir) & 0x7fffffff) < 0x7ff00000;
+  }
+  S.g = 0;
+#pragma unroll
+  for (int s = 1; s < 5; ++s) {
+    int d = fx_exp(top[0][s]) - S.base[0];
+#pragma unroll
+    for (int i = 1; i < NG; ++i) d = fx_max(d, fx_exp(top[i][s]) - S.base[i]);
+    d = fx_max(d, 0);
+    S.g = fx_max(S.g, (d + s - 1) / s);
+  }
+  return S;
+}
+
+// The same coefficient in a growth larger by one: X of total degree s divided by 2^s.
+FX_FN Fx fx_regrow(Fx v, int s, FxRange& r) { return fx_split(((fx_join(v) + (int64_t(1) << (s - 1))) >> s) + FX_HALF, r); }
+
+// Coefficient a of component q and degree s in the point's scale.
+template <int NC>
+FX_FN Fx ck_convert(const CkScale<NC>& S, double a, int q, int s, FxRange& r) {
+  return fx_split(fx_from_double(a, S.of(q, s)) + FX_HALF, r);
+}
+template <int NC>
+FX_FN Fx ck_ninv(const CkScale<NC>& S, const CkLead& lead) {
+  FxRange r{0};
+  return fx_split(fx_from_double<FX_C>(-lead.ir, -S.base[0]) + FX_HALF, r);
+}
+
+constexpr int kCkTries = 8;  // growths tried at most; inputs below 2^-5s cannot leave the range
+
+// Burgers: the whole recursion in one thread's registers.  Writes tc[q][k],
+// k = 1..4, per L^k (tc[q][0] is left to the caller); NaN where the input is not finite.
+template <int NC, int DIM>
+FX_FN void ck_fixed(const double (&a)[NC][25], const CkLead& lead, const CkFixedConst& K, double (&tc)[NC][5]) {
+  auto coef = [&a](int q, int mn) { return a[q][mn]; };
+  CkScale<NC> S = ck_scale<NC, DIM>(coef, lead);
+  Fx w[NC][25], ninv{0, 0};
+  int64_t t[NC][5];
+  if constexpr (NC > 1) ninv = ck_ninv<NC>(S, lead);
+#pragma unroll 1
+  for (int tries = 0; tries < kCkTries; ++tries, ++S.g) {
+    FxRange r{0}, r0{0};
+#pragma unroll
+    for (int q = 0; q < NC; ++q)
+#pragma unroll
+      for (int m = 0; m < 5; ++m)
+#pragma unroll
+        for (int n = 0; n + m < 5; ++n)
+          if (DIM == 2 || n == 0) w[q][m * 5 + n] = ck_convert<NC>(S, a[q][m * 5 + n], q, m + n, m + n ? r : r0);
+    static_assert(NC == 1 && DIM == 2, "2D Euler runs on two lanes");
+    ck_burgers2d_fx(w, ninv, K, t, r);
+    if (!r.bad()) break;
+  }
+#pragma unroll
+  for (int q = 0; q < NC; ++q)
+#pragma unroll
+    for (int k = 1; k < 5; ++k)
+      tc[q][k] = S.finite ? fx_to_double(t[q][k], S.of(q, 0) + k * (S.eu + S.g)) : fx_from_bits(0x7ff8000000000000ull);
+}
+
+}  // namespace shweno

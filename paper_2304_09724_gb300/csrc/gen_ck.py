@@ -1,5 +1,6 @@
-"""Writes ck_generated.cuh: straight-line CUDA for the Cauchy-Kovalevskaya (Lax-Wendroff)
-procedure of Eq. (2.6) and Section 3.1, for 1D/2D Burgers and 1D/2D Euler.
+"""Writes the Cauchy-Kovalevskaya (Lax-Wendroff) procedure of Eq. (2.6) and Section 3.1 as
+straight-line CUDA: ck_generated.cuh in FP64 (1D Burgers and Euler) and ck_fixed_generated.cuh in
+block fixed point (2D Burgers and Euler, see fixed.cuh).
 
 Method.  At an interface quadrature point the solution is a truncated power series in
 (X, Y, t), X = (x - x_p)/dx and Y = (y - y_p)/dy, with normalised coefficients
@@ -205,13 +206,267 @@ class Gen:
         return "\n".join(head + self.lines + outs + ["}"])
 
 
+class GenFixed(Gen):
+    """The same recursion in block fixed point (fixed.cuh): every coefficient an Fx (two 32-bit
+    limbs), sums of products in two 64-bit accumulators, the constants (time update factors,
+    1/rho0, (gamma - 1)/2) as Fx operands."""
+
+    def fx(self, name, m, n, k):
+        """C name of coefficient (m,n,k) of series `name` as an Fx; emits code on first use."""
+        if not self.idx_ok(m, n, k):
+            return None
+        key = ("fx", name, m, n, k)
+        if key in self.done:
+            return self.done[key]
+        v = f"{name}_{m}{n}{k}"
+        W = self.state_names()
+        if name in W and k == 0:
+            v = f"w[{W.index(name)}][{m * 5 + n}]"
+        elif name in W:
+            q = W.index(name)
+            z = f"{m + 1} * {self.zf(f'F{q}', m + 1, n, k - 1)}"
+            if self.dim == 2:
+                z += f" + {n + 1} * {self.zf(f'G{q}', m, n + 1, k - 1)}"
+            self.lines.append(f"  const Fx {v} = fx_split(fx_time<{k}>({z}, K.third) + FX_HALF, r);")
+        elif name in ("u", "v"):
+            num, den = W[1 if name == "u" else 2], W[0]
+            acc = [f"fx_mac_int(s, {self.fx(num, m, n, k)}, -(1 << 29));"]
+            for p, q, t in self.sub_indices(m, n, k):
+                if (p, q, t) != (0, 0, 0):
+                    acc.append(f"fx_mac(s, {self.fx(den, p, q, t)}, {self.fx(name, m - p, n - q, k - t)});")
+            self.block(v + "n", acc, lead=(m, n, k) == (0, 0, 0))  # rho0 times minus the coefficient
+            self.block(v, [f"fx_mac(s, {v}n, ninv);"], const=True, lead=(m, n, k) == (0, 0, 0))
+        elif name == "H":
+            self.lines.append(f"  const Fx {v} = fx_split({self.z(W[-1], m, n, k)} + {self.z('p', m, n, k)} + FX_HALF, {self.rng(m, n, k)});")
+        else:
+            raise KeyError(name)
+        self.done[key] = v
+        return v
+
+    def block(self, v, acc, const=False, lead=False):
+        q, r = ("<FX_C>", "r0" if lead else "r") if const else ("", "r0" if lead else "r")
+        self.lines.append(f"  Fx {v}; {{ FxAcc s = fx_zero{q}(true); " + " ".join(acc)
+                          + f" {v} = fx_split(fx_sum{q}(s), {r}); }}")
+
+    @staticmethod
+    def rng(m, n, k):
+        return "r0" if m + n + k == 0 else "r"
+
+    def products(self, A, B, m, n, k):
+        return [f"fx_mac(s, {self.fx(A, p, q, t)}, {self.fx(B, m - p, n - q, k - t)});"
+                for p, q, t in self.sub_indices(m, n, k)]
+
+    def zf(self, name, m, n, k):
+        """A flux coefficient as a 64-bit integer expression."""
+        W = self.state_names()
+        if self.eq == "burgers":  # u^2 / 2
+            return self.half_square(m, n, k)
+        one = {"F0": (W[1],), "F1": ("mu", "p"), "F2": ("uH",)} if self.dim == 1 else \
+            {"F0": (W[1],), "F1": ("mu", "p"), "F2": ("mv",), "F3": ("uH",), "G0": (W[2],), "G1": ("mv",), "G2": ("nv", "p"), "G3": ("vH",)}
+        return "(" + " + ".join(self.z(t, m, n, k) for t in one[name]) + ")"
+
+    def half_square(self, m, n, k):
+        """Coefficient of u^2 / 2: each unordered pair once, half of the middle square."""
+        key = ("hs", m, n, k)
+        if key not in self.done:
+            ps = sorted({tuple(sorted(((p, q, t), (m - p, n - q, k - t)))) for p, q, t in self.sub_indices(m, n, k)})
+            acc = [f"fx_mac(s, {self.fx('w0', *a)}, {self.fx('w0', *b)});" for a, b in ps if a != b]
+            mid = [f"{{ FxAcc s = fx_zero(); fx_mac(s, {self.fx('w0', *a)}, {self.fx('w0', *a)}); f += fx_sum(s) >> 1; }}" for a, b in ps if a == b]
+            v = f"f_{m}{n}{k}"
+            self.lines.append(f"  int64_t {v}; {{ FxAcc s = fx_zero(); " + " ".join(acc) + f" {v} = fx_sum(s); }}" + " ".join(x.replace("f +=", v + " +=") for x in mid))
+            self.done[key] = v
+        return self.done[key]
+
+    def z(self, name, m, n, k):
+        """C name of a coefficient as a 64-bit integer."""
+        key = ("z", name, m, n, k)
+        if key in self.done:
+            return self.done[key]
+        v = f"z_{name}_{m}{n}{k}"
+        W = self.state_names()
+        if name in W:
+            self.lines.append(f"  const int64_t {v} = fx_join({self.fx(name, m, n, k)});")
+        elif name == "p":
+            kin = self.z("mu", m, n, k) + (f" + {self.z('nv', m, n, k)}" if self.dim == 2 else "")
+            self.lines.append(f"  const Fx e_{m}{n}{k} = fx_split((({self.z(W[-1], m, n, k)} - (({kin}) >> 1)) << K.gshift) + FX_HALF, {self.rng(m, n, k)});")
+            self.lines.append(f"  int64_t {v}; {{ FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_{m}{n}{k}, K.gm1); {v} = fx_sum<FX_C>(s); }}")
+        else:
+            A, B = {"mu": (W[1], "u"), "mv": (W[1], "v"), "nv": (W[-2], "v"), "uH": ("u", "H"), "vH": ("v", "H")}[name]
+            acc = self.products(A, B, m, n, k)
+            self.lines.append(f"  int64_t {v}; {{ FxAcc s = fx_zero(); " + " ".join(acc) + f" {v} = fx_sum(s); }}")
+        self.done[key] = v
+        return v
+
+    def emit(self, fname):
+        W = self.state_names()
+        outs = []
+        for q in range(self.ncomp):
+            for k in range(1, 5):
+                outs.append(f"  t[{q}][{k}] = fx_join({self.fx(W[q], 0, 0, k)});")
+        nc = self.ncomp
+        head = [
+            f"// {fname}: {self.dim}D {self.eq} in block fixed point; inputs w[q][m*5+n], outputs t[q][k], k = 1..4, in",
+            "// the fields' units (fixed.cuh, ck_fixed.cuh); ninv = -1/rho0 in fixed point (Euler).",
+            f"FX_FN void {fname}(const Fx (&w)[{nc}][25], Fx ninv, const CkFixedConst& K, int64_t (&t)[{nc}][5], FxRange& r) {{",
+            "  (void)ninv; FxRange r0{0}; (void)r0;  // leading coefficients are in range by their scales",
+        ]
+        return "\n".join(head + self.lines + outs + ["}"])
+
+
+class GenLane:
+    """2D Euler in block fixed point with two lanes per point: lane "x" carries u and the x-fluxes,
+    lane "y" (16 lanes up) v and the y-fluxes.  Both run the same code in their own coordinates:
+    (i, j) = (m, n) for x and (n, m) for y, vel = u / v, mom = m / n, oth = n / m; what they share (rho,
+    both momenta, H) lies in shared memory, what they exchange (the two kinetic terms of p, the flux
+    derivatives) goes through shuffles."""
+
+    def __init__(self):
+        self.lines = []
+
+    def out(self, s):
+        self.lines.append("  " + s)
+
+    def run(self):
+        for c in range(4):
+            self.level(c)
+        return "\n".join(self.lines)
+
+    @staticmethod
+    def pairs(d):
+        return [(s - j, j) for s in range(d + 1) for j in range(s + 1)]
+
+    @staticmethod
+    def subs(i, j, c):
+        return [(p, q, t) for p in range(i + 1) for q in range(j + 1) for t in range(c + 1)]
+
+    def use(self, name, i, j, t):
+        """A shared series' coefficient as a local of the current block, loaded on first use."""
+        v = f"{name}{i}{j}{t}"
+        if v not in self.loaded:
+            self.loaded.add(v)
+            self.out(f"const Fx {v} = S.ld{name}({t}, {i}, {j});")
+        return v
+
+    def uses(self, series, i, j, c):
+        for p, q, t in self.subs(i, j, c):
+            self.use(series, p, q, t)
+
+    def level(self, c):
+        D = 4 - c
+        rng = lambda i, j: "r0" if i + j + c == 0 else "r"
+        self.out(f"// ---- slice {c}")
+        # the velocity: rho vel = mom
+        for i, j in self.pairs(D):
+            self.out(f"Fx vel{i}{j}{c};")
+        self.out("{")
+        self.loaded = set()
+        ps = self.pairs(D)
+        for x, (i, j) in enumerate(ps):
+            for i2, j2 in ps[x:x + 2]:  # loads run one target ahead of the sums
+                for p, q, t in self.subs(i2, j2, c):
+                    if p + q + t:
+                        self.use("rho", p, q, t)
+            self.out(f"{{ FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom({c}, {i}, {j}), -(1 << 30));")
+            for p, q, t in self.subs(i, j, c):
+                if p + q + t:
+                    self.out(f"  fx_mac(s, rho{p}{q}{t}, vel{i - p}{j - q}{c - t});")
+            self.out(f"  const Fx n = fx_split(fx_sum(s), {rng(i, j)});")
+            self.out(f"  FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel{i}{j}{c} = fx_split(fx_sum<FX_C>(z), {rng(i, j)}); }}")
+        self.out("}")
+        # mom vel, then the pressure and H
+        for i, j in self.pairs(D):
+            self.out(f"int64_t k{i}{j}{c};")
+        self.out("{")
+        self.loaded = set()
+        for x, (i, j) in enumerate(ps):
+            for i2, j2 in ps[x:x + 2]:
+                self.uses("mom", i2, j2, c)
+            self.product("mom", f"k{i}{j}{c}", i, j, c)
+        self.out("}")
+        for i, j in self.pairs(D):
+            if i >= 1:
+                self.out(f"int64_t f{i}{j}{c};")
+        for i, j in self.pairs(D):
+            E = f"S.ldE(0, {i}, {j})" if c == 0 else f"E{i}{j}{c}"
+            self.out(f"{{ const int64_t E = {E};")
+            self.out(f"  const Fx e = fx_split(((E - ((k{i}{j}{c} + S.swap(k{j}{i}{c})) >> 1)) << gshift) + FX_HALF, {rng(i, j)});")
+            self.out(f"  FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);")
+            self.out(f"  S.stH({c}, {i}, {j}, fx_split(E + p + FX_HALF, {rng(i, j)}));")
+            if i >= 1:
+                self.out(f"  f{i}{j}{c} = k{i}{j}{c} + p;")
+            self.out("}")
+        # the time update: (i + 1) times the lane's fluxes, added to the other lane's
+        nxt = self.pairs(D - 1)
+        for q in ("rho", "mom", "oth", "E"):
+            for i, j in nxt:
+                self.out(f"int64_t d{q}{i}{j}{c};")
+        for i, j in nxt:
+            self.out(f"drho{i}{j}{c} = {i + 1} * fx_join(S.ldmom({c}, {i + 1}, {j}));")
+            self.out(f"dmom{i}{j}{c} = {i + 1} * f{i + 1}{j}{c};")
+        for q, series in (("oth", "oth"), ("E", "H")):
+            self.out("{")
+            self.loaded = set()
+            for x, (i, j) in enumerate(nxt):
+                for i2, j2 in nxt[x:x + 2]:
+                    self.uses(series, i2 + 1, j2, c)
+                z = f"z{i}{j}"
+                self.out(f"int64_t {z};")
+                self.product(series, z, i + 1, j, c)
+                self.out(f"d{q}{i}{j}{c} = {i + 1} * {z};")
+            self.out("}")
+        # each lane finishes its own momentum, lane x the density, lane y the energy
+        n = c + 1
+        for i, j in nxt:
+            self.out(f"{{ const int64_t own = dmom{i}{j}{c} + S.swap(doth{j}{i}{c});")
+            self.out(f"  const int64_t both = S.pick(drho{i}{j}{c}, dE{i}{j}{c}) + S.swap(S.pick(dE{j}{i}{c}, drho{j}{i}{c}));")
+            self.out(f"  S.next({n}, {i}, {j}, fx_time<{n}>(own, third), fx_time<{n}>(both, third), {'r' if n < 4 else 'r0'}); }}")
+        if n < 4:
+            self.out("S.sync();")
+            for i, j in nxt:
+                self.out(f"const int64_t E{i}{j}{n} = S.ldE({n}, {i}, {j});")
+
+    def product(self, series, z, i, j, c):
+        self.out("{ FxAcc s = fx_zero();")
+        for p, q, t in self.subs(i, j, c):
+            self.out(f"  fx_mac(s, {series}{p}{q}{t}, vel{i - p}{j - q}{c - t});")
+        self.out(f"  {z} = fx_sum(s); }}")
+
+
+def main_fixed():
+    parts = ["// Generated by gen_ck.py -- do not edit.  The Cauchy-Kovalevskaya recursions in two dimensions",
+             "// in block fixed point (see fixed.cuh, ck_fixed.cuh and gen_ck.py for the method).",
+             "#pragma once", '#include "fixed.cuh"', "", "namespace shweno {", "",
+             "// Constants of the recursion: 1/3 and (gamma - 1) 2^-gshift.",
+             "struct CkFixedConst {", "  Fx third, gm1;", "  int32_t gshift;", "};", "",
+             "// Minus z / k: from the flux derivatives of slice k - 1 to slice k.",
+             "template <int K>",
+             "FX_FN int64_t fx_time(int64_t z, Fx third) {",
+             "  if (K == 1) return -z;",
+             "  if (K == 2) return -((z + 1) >> 1);",
+             "  if (K == 4) return -((z + 2) >> 2);",
+             "  FxRange r0{0};",
+             "  FxAcc s = fx_zero<FX_C>();",
+             "  fx_mac(s, fx_split(FX_HALF - z, r0), third);",
+             "  return fx_sum<FX_C>(s);", "}", ""]
+    parts += [GenFixed(2, "burgers").emit("ck_burgers2d_fx"), ""]
+    parts += ["// 2D Euler, two lanes per point: S gives the shared series and constants, ninv = -1/rho0;",
+              "// S.next() takes the coefficients of the next slice.",
+              "template <typename Store>",
+              "FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxRange& r) {",
+              "  FxRange r0{0};  // leading coefficients are in range by their scales",
+              GenLane().run(), "}", ""]
+    parts.append("}  // namespace shweno")
+    out = os.path.join(os.path.dirname(os.path.abspath(__file__)), "ck_fixed_generated.cuh")
+    with open(out, "w") as f:
+        f.write("\n".join(parts) + "\n")
+
+
 def main():
     parts = ["// Generated by gen_ck.py -- do not edit.  Cauchy-Kovalevskaya procedure, Eq. (2.6) and",
              "// Section 3.1, as truncated power-series recursions (see gen_ck.py for the method).",
              "#pragma once", ""]
     stats = []
-    for dim, eq, fname in ((1, "burgers", "ck_burgers1d"), (2, "burgers", "ck_burgers2d"),
-                           (1, "euler", "ck_euler1d"), (2, "euler", "ck_euler2d")):
+    for dim, eq, fname in ((1, "burgers", "ck_burgers1d"), (1, "euler", "ck_euler1d")):
         g = Gen(dim, eq)
         parts.append(g.emit(fname))
         parts.append("")
@@ -225,3 +480,4 @@ def main():
 
 if __name__ == "__main__":
     main()
+    main_fixed()

@@ -6,6 +6,7 @@
 #pragma once
 #include <cstdint>
 
+#include "ck_fixed.cuh"
 #include "recon_tables.cuh"
 
 namespace shweno {
@@ -29,23 +30,18 @@ struct Params {
   int32_t flag_mode;      // FLAG_*
   int32_t charwise;       // 1: Euler reconstructions across a face in characteristic fields
   int32_t quintic;        // 1: reading R1' (quintic p1 that also matches the cell's own V)
-  // Cauchy-Kovalevskaya scale factors (m+1)/((k+1) dx) and (n+1)/((k+1) dy), set by the host
-  double ckx[5][4], cky[5][4];
   double igam[3];  // 1 / gam, set by the host
   double idx, idy, idxy;  // 1 / dx, 1 / dy, 1 / (dx dy), set by the host
+  CkFixed ck;             // constants of the fixed-point Cauchy-Kovalevskaya recursion, set by the host
 };
 
-// Fills the derived members of Params (ckx, cky, igam, idx, idy, idxy) from dx, dy and gam.
+// Fills the derived members of Params (igam, idx, idy, idxy, ck) from dx, dy, gam and gamma.
 inline void finalize_params(Params& P) {
-  for (int m = 0; m < 5; ++m)
-    for (int k = 0; k < 4; ++k) {
-      P.ckx[m][k] = (m + 1) / ((k + 1) * P.dx);
-      P.cky[m][k] = (m + 1) / ((k + 1) * P.dy);
-    }
   for (int l = 0; l < 3; ++l) P.igam[l] = 1.0 / P.gam[l];
   P.idx = 1.0 / P.dx;
   P.idy = 1.0 / P.dy;
   P.idxy = 1.0 / (P.dx * P.dy);
+  finalize_ck_fixed(P.ck, P.dim, P.dx, P.dy, P.eq == EQ_EULER ? P.gamma : 1.4);
 }
 
 // Device-resident time-stepping control block.  One step = begin_step, the step kernels,
@@ -494,6 +490,7 @@ struct Upwinder {
   double l[NC][NC];  // l[k] = k-th left eigenvector
   double s[NC];      // wave coefficients (0 for a wave that does not contribute)
   int base_left;
+  CkLead lead;       // scales of the leading state (Euler)
 
   __device__ __forceinline__ void setup(const double* Ws, double g, int dir, double burgers_scale = 0.0) {
     double lam[NC];
@@ -505,6 +502,10 @@ struct Upwinder {
       const Prim P = euler_prim(Ws, NC, g);
       tol = 1e-12 * P.c;
       euler_eigvecs<NC>(P, g, dir, r, l, lam);
+      lead.ir = P.ir;
+      lead.hu = fx_hi(P.u) & 0x7fffffff;
+      if (NC == 4) lead.hu = fx_max(lead.hu, fx_hi(P.v) & 0x7fffffff);
+      lead.hH = fx_hi(P.H) & 0x7fffffff;
     }
     int npos = 0, nneg = 0;
     for (int k = 0; k < NC; ++k) {

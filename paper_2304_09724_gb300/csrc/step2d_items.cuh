@@ -1,7 +1,6 @@
 // Per-item device functions of the 2D step, shared by the one-mesh kernels (step2d.cu) and the
 // batched persistent kernel (batch.cu).  See step2d.cu for the structure of the step.
 #pragma once
-#include "ck_generated.cuh"
 #include "shweno_device.cuh"
 
 namespace shweno {
@@ -193,15 +192,213 @@ __device__ __forceinline__ void pass_order(const Params& P, const double (*ev)[5
   if (has_face) face_order<NC, K>(P, et, eR, threadIdx.x, dir, Ws, U, a);
 }
 
+// ------------------------------------------------------------------ Cauchy-Kovalevskaya of the points
+// The points of a CTA go through the recursion in fixed point (ck_fixed.cuh) on the integer pipe.
+// Euler: the owner of a point converts its 60 coefficients into shared memory (in the place of the
+// first- and second-pass tables, which no thread reads any more), then each warp takes 16 points
+// at a time, two lanes a point (ck_euler2d_lane: one lane per direction, 16 lanes apart, so that a
+// half-warp reads 128 consecutive bytes), and the owner converts the results back.  One thread
+// cannot hold the recursion's series in registers beside its accumulators (10 KB of spills);
+// split over two lanes and shared memory it needs about 5500 instructions a lane and no spills.
+constexpr int CKP = 64;               // points in work at a time
+constexpr int kCkRow = CKP * 8;       // bytes of one coefficient of them
+constexpr int kCkIn = 0;              // [2 halves][4 comps][15] level 0 (in the end: the results)
+constexpr int kCkLev = kCkIn + 2 * 60 * kCkRow;  // [rho, m, n, H][10 + 6 + 3] levels 1..3
+constexpr int kCkH0 = kCkLev + 4 * 19 * kCkRow;  // [15] H, level 0
+constexpr int kCkE = kCkH0 + 15 * kCkRow;        // [10] E of the level in work, 64-bit
+constexpr int kCkNinv = kCkE + 10 * kCkRow;      // [SEG] -1/rho0
+constexpr int kCkGrow = kCkNinv + SEG * 8;       // [SEG] growth added on the way
+constexpr size_t kCkBytes = kCkGrow + SEG * 4;
+
+template <int NC>
+constexpr size_t face_smem() {
+  return NC == 4 && kCkBytes > kFaceSmem ? kCkBytes : kFaceSmem;
+}
+
+__host__ __device__ constexpr int ck_pair(int i, int j) { return (i + j) * (i + j + 1) / 2 + j; }
+__host__ __device__ constexpr int ck_level_row(int t) { return t == 1 ? 0 : t == 2 ? 10 : 16; }
+
+__device__ __forceinline__ Fx ck_ld(int at) {
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  const int2 v = *reinterpret_cast<const int2*>(dyn_smem + at);
+  return Fx{v.x, v.y};
+}
+__device__ __forceinline__ int64_t ck_ld64(int at) {
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  return *reinterpret_cast<const long long*>(dyn_smem + at);
+}
+__device__ __forceinline__ void ck_st64(int at, int64_t v) {
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  *reinterpret_cast<long long*>(dyn_smem + at) = v;
+}
+__device__ __forceinline__ void ck_st(int at, Fx v) {
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  *reinterpret_cast<int2*>(dyn_smem + at) = make_int2(v.h, v.l);
+}
+
+// A lane's view of its point's series in shared memory, in the lane's own coordinates.
+struct CkLane {
+  int off[15];                    // row offset of the coefficient (i, j) of the lane's directions
+  int in, lev, h0, e0;            // the point's column in the four areas
+  int mom0, oth0, momL, othL;     // the lane's momentum and the other one, level 0 and above
+  int dir;
+  int64_t mom_out[4], both_out[4];  // results: the lane's momentum; density (x) or energy (y)
+  __device__ __forceinline__ CkLane(int half, int pt, int d) : dir(d) {
+#pragma unroll
+    for (int s = 0; s < 5; ++s)
+#pragma unroll
+      for (int j = 0; j <= s; ++j) off[ck_pair(s - j, j)] = (dir ? ck_pair(j, s - j) : ck_pair(s - j, j)) * kCkRow;
+    in = kCkIn + half * 60 * kCkRow + pt * 8;
+    lev = kCkLev + pt * 8;
+    h0 = kCkH0 + pt * 8;
+    e0 = kCkE + pt * 8;
+    mom0 = in + (1 + dir) * 15 * kCkRow;
+    oth0 = in + (2 - dir) * 15 * kCkRow;
+    momL = lev + (1 + dir) * 19 * kCkRow;
+    othL = lev + (2 - dir) * 19 * kCkRow;
+  }
+  __device__ __forceinline__ int at(int base0, int baseL, int t, int i, int j) const {
+    return (t == 0 ? base0 : baseL + ck_level_row(t) * kCkRow) + off[ck_pair(i, j)];
+  }
+  __device__ __forceinline__ Fx ldrho(int t, int i, int j) const { return ck_ld(at(in, lev, t, i, j)); }
+  __device__ __forceinline__ Fx ldmom(int t, int i, int j) const { return ck_ld(at(mom0, momL, t, i, j)); }
+  __device__ __forceinline__ Fx ldoth(int t, int i, int j) const { return ck_ld(at(oth0, othL, t, i, j)); }
+  __device__ __forceinline__ Fx ldH(int t, int i, int j) const { return ck_ld(at(h0, lev + 57 * kCkRow, t, i, j)); }
+  // both lanes of a point compute and write the same H
+  __device__ __forceinline__ void stH(int t, int i, int j, Fx v) const { ck_st(at(h0, lev + 57 * kCkRow, t, i, j), v); }
+  __device__ __forceinline__ int64_t ldE(int t, int i, int j) const {
+    if (t == 0) return fx_join(ck_ld(in + 45 * kCkRow + off[ck_pair(i, j)]));
+    return ck_ld64(e0 + off[ck_pair(i, j)]);
+  }
+  __device__ __forceinline__ int64_t pick(int64_t x, int64_t y) const { return dir ? y : x; }
+  // the other lane's value
+  __device__ __forceinline__ int64_t swap(int64_t z) const { return __shfl_xor_sync(0xffffffffu, (long long)z, 16); }
+  __device__ __forceinline__ void sync() const { __syncwarp(); }
+  // coefficient (i, j) of slice n: the lane's momentum, and density (lane x) or energy (lane y)
+  __device__ __forceinline__ void next(int n, int i, int j, int64_t own, int64_t both, FxRange& r) {
+    if (i + j == 0) {
+      mom_out[n - 1] = own;
+      both_out[n - 1] = both;
+    }
+    if (n == 4) return;
+    ck_st(momL + ck_level_row(n) * kCkRow + off[ck_pair(i, j)], fx_split(own + FX_HALF, r));
+    FxRange rb{0};
+    const Fx v = fx_split(both + FX_HALF, rb);
+    r.h |= dir ? 0u : rb.h;
+    const Fx e = Fx{(int32_t)((uint64_t)both & 0xffffffffu), (int32_t)(both >> 32)};  // low word first
+    ck_st((dir ? e0 : lev + ck_level_row(n) * kCkRow) + off[ck_pair(i, j)], dir ? e : v);
+  }
+};
+
+// The recursion of the 16 points p0.. of a half (valid: points that exist), by one whole warp.
+// Results: t[q][k] (64-bit, k = 1..4) in row q * 4 + k - 1 of the point's column of the half's input.
+// Out of line: one copy of the recursion for all kernels of a translation unit.
+static __device__ __noinline__ void ck_warp_euler2d(int half, int p0, int valid, Fx third, Fx gm1, int gshift) {
+  const int lane = threadIdx.x & 31, dir = lane >> 4, pt = p0 + (lane & 15);
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  CkLane S(half, pt, dir);
+  const Fx ninv = ck_ld(kCkNinv + (half * CKP + pt) * 8);
+#pragma unroll 1
+  for (int tries = 1;; ++tries) {
+    FxRange r{0};
+    ck_euler2d_lane(S, ninv, gm1, third, gshift, r);
+    int bad = (lane & 15) < valid && r.bad() ? 1 : 0;
+    bad |= __shfl_xor_sync(0xffffffffu, bad, 16);
+    if (!__any_sync(0xffffffffu, bad) || tries == kCkTries) break;
+    __syncwarp();
+    if (bad) {  // divide the coefficients of degree s by 2^s: each lane half of the components
+      FxRange none{0};
+#pragma unroll 1
+      for (int q = 2 * dir; q < 2 * dir + 2; ++q)
+#pragma unroll
+        for (int s = 1; s < 5; ++s)
+#pragma unroll
+          for (int j = 0; j <= s; ++j) {
+            const int at = S.in + (q * 15 + ck_pair(s - j, j)) * kCkRow;
+            ck_st(at, fx_regrow(ck_ld(at), s, none));
+          }
+      if (dir == 0) *reinterpret_cast<int*>(dyn_smem + kCkGrow + (half * CKP + pt) * 4) += 1;
+    }
+    __syncwarp();
+  }
+  __syncwarp();  // the inputs are read no more
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    ck_st64(S.in + ((1 + dir) * 4 + k) * kCkRow, S.mom_out[k]);
+    ck_st64(S.in + (dir * 12 + k) * kCkRow, S.both_out[k]);
+  }
+}
+
+// Time-Taylor coefficients per unit L^k (P.ck.iL = 1 / L) of the CTA's nf points from their spatial
+// ones; called by every thread after the barrier that ends the use of the tables.
+template <int NC>
+__device__ __forceinline__ void ck_points(const Params& P, int nf, bool has_face, double (&a)[NC][25],
+                                          const CkLead& lead, double (&tc)[NC][5]) {
+  if (P.ck.rx != P.ck.ry) {  // dx != dy: both coordinates in units of L
+    double fx = 1.0;
+#pragma unroll
+    for (int m = 0; m < 5; ++m, fx *= P.ck.rx) {
+      double f = fx;
+#pragma unroll
+      for (int n = 0; n + m < 5; ++n, f *= P.ck.ry)
+#pragma unroll
+        for (int q = 0; q < NC; ++q) a[q][m * 5 + n] *= f;
+    }
+  }
+  if constexpr (NC == 1) {
+    if (!has_face) return;
+    ck_fixed<1, 2>(a, lead, P.ck.K, tc);
+    tc[0][0] = a[0][0];
+  } else {
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    const int tid = threadIdx.x;
+    const int col = kCkIn + (tid / CKP) * 60 * kCkRow + (tid % CKP) * 8;
+    CkScale<NC> S{};
+    if (has_face) {
+      S = ck_scale<NC, 2>([&a](int q, int mn) { return a[q][mn]; }, lead);
+      FxRange none{0};  // the recursion checks its operands
+#pragma unroll
+      for (int q = 0; q < NC; ++q)
+#pragma unroll
+        for (int s = 0; s < 5; ++s)
+#pragma unroll
+          for (int n = 0; n <= s; ++n)
+            ck_st(col + (q * 15 + ck_pair(s - n, n)) * kCkRow, ck_convert<NC>(S, a[q][(s - n) * 5 + n], q, s, none));
+      ck_st(kCkNinv + tid * 8, ck_ninv<NC>(S, lead));
+      *reinterpret_cast<int*>(dyn_smem + kCkGrow + tid * 4) = 0;
+#pragma unroll
+      for (int q = 0; q < NC; ++q) tc[q][0] = a[q][0];
+    }
+    __syncthreads();
+    const int p0 = (tid >> 5) * 16;
+#pragma unroll 1
+    for (int half = 0; half * CKP < nf; ++half) {
+      const int valid = nf - half * CKP - p0;
+      if (valid > 0) ck_warp_euler2d(half, p0, valid, P.ck.K.third, P.ck.K.gm1, P.ck.K.gshift);
+      __syncwarp();
+    }
+    __syncthreads();
+    if (!has_face) return;
+    S.g += *reinterpret_cast<const int*>(dyn_smem + kCkGrow + tid * 4);
+#pragma unroll
+    for (int q = 0; q < NC; ++q)
+#pragma unroll
+      for (int k = 1; k < 5; ++k) {
+        const int64_t t = ck_ld64(col + (q * 4 + k - 1) * kCkRow);
+        tc[q][k] = S.finite ? fx_to_double(t, S.of(q, 0) + k * (S.eu + S.g)) : fx_from_bits(0x7ff8000000000000ull);
+      }
+  }
+}
+
 // Second pass, leading term, upwinding and CK of the nf faces of a CTA (nf <= NFACE): thread t
 // owns the cell in column t + 1 (t <= nf) and the face between columns t + 1 and t + 2 (t < nf).
 // Returns true for a face thread, whose tc[q][0..4] are then the time-Taylor coefficients of its
-// face point.  nl(c): whether the cell in column c uses the nonlinear weights.
+// face point per L^k.  nl(c): whether the cell in column c uses the nonlinear weights.
 template <int NC, bool FLAGS, bool Q, typename FlagOf>
-__device__ __forceinline__ bool second_pass_cells(const Params& P, const double (*ev)[5][SPAN],
-                                                  unsigned char* tbl, int nf, int dir, FlagOf nl,
-                                                  double tc[NC][5]) {
-  EndTable& et = *reinterpret_cast<EndTable*>(tbl);
+__device__ __forceinline__ bool second_pass_cells(const Params& P, unsigned char* smem_raw, int nf, int dir,
+                                                  FlagOf nl, double (&tc)[NC][5]) {
+  const double(*ev)[5][SPAN] = reinterpret_cast<const double(*)[5][SPAN]>(smem_raw);
+  EndTable& et = *reinterpret_cast<EndTable*>(smem_raw + kEvBytes);
   const bool has_cell = (int)threadIdx.x <= nf, has_face = (int)threadIdx.x < nf;
   CellMix<NC> m;
   if (has_cell) cell_mix<NC, Q>(P, ev, threadIdx.x + 1, FLAGS && !nl(threadIdx.x + 1), m);
@@ -212,19 +409,12 @@ __device__ __forceinline__ bool second_pass_cells(const Params& P, const double 
   pass_order<NC, FLAGS, Q, 2>(P, ev, et, has_cell, m, has_face, dir, Ws, U, a);
   pass_order<NC, FLAGS, Q, 3>(P, ev, et, has_cell, m, has_face, dir, Ws, U, a);
   pass_order<NC, FLAGS, Q, 4>(P, ev, et, has_cell, m, has_face, dir, Ws, U, a);
-  if (!has_face) return false;
+  __syncthreads();  // the tables are read no more
+  if (has_face)
 #pragma unroll
-  for (int q = 0; q < NC; ++q) a[q][0] = Ws[q];
-  double t4[NC][5];
-  if constexpr (NC == 1) ck_burgers2d(a, t4, P.ckx, P.cky, P.gamma - 1.0);
-  else ck_euler2d(a, t4, P.ckx, P.cky, P.gamma - 1.0);
-#pragma unroll
-  for (int q = 0; q < NC; ++q) {
-    tc[q][0] = Ws[q];
-#pragma unroll
-    for (int k = 1; k < 5; ++k) tc[q][k] = t4[q][k];
-  }
-  return true;
+    for (int q = 0; q < NC; ++q) a[q][0] = Ws[q];
+  ck_points<NC>(P, nf, has_face, a, U.lead, tc);
+  return has_face;
 }
 
 // ------------------------------------------------------------------ characteristic-wise face point
@@ -306,15 +496,15 @@ __device__ __forceinline__ void char_sides(const CharBasis<NC>& Bs, const double
 // Face point of the characteristic-wise option (Euler): the second pass across the face runs in
 // the characteristic fields of the Jacobian along the face normal at Wref (the mean of the cell
 // averages next to the point), with its own weights per field and side; then the leading term
-// (HLLC), the upwinding and CK.  Left cell in column c0 + 1, right cell in c0 + 2; dir = 0:
-// x-face (first pass along y), 1: y-face.  Returns the time-Taylor coefficients tc[q][0..4].
+// (HLLC) and the upwinding.  Left cell in column c0 + 1, right cell in c0 + 2; dir = 0:
+// x-face (first pass along y), 1: y-face.  Returns the spatial Taylor coefficients a[q][m*5+n] and
+// the scales of the leading state.
 template <int NC, bool FLAGS, bool Q>
 __device__ __forceinline__ void char_face_point(const Params& P, const double (*ev)[5][SPAN],
-                                                const FlagTable& ft, int c0, int dir, double tc[NC][5],
-                                                const double* Wref) {
+                                                const FlagTable& ft, int c0, int dir, double (&a)[NC][25],
+                                                CkLead& lead, const double* Wref) {
   static_assert(NC == 4, "characteristic fields are for the Euler system");
   const double g = P.gamma;
-  double a[NC][25];
   double dl[NC][5], dr[NC][5];
   double AL[NC], BL[NC], CL[NC], AR[NC], BR[NC], CR[NC];
   // FLAGS = false: every cell uses the nonlinear weights (compile-time, no branch)
@@ -371,14 +561,7 @@ __device__ __forceinline__ void char_face_point(const Params& P, const double (*
   }
 #pragma unroll
   for (int q = 0; q < NC; ++q) a[q][0] = Ws[q];
-  double t4[NC][5];
-  ck_euler2d(a, t4, P.ckx, P.cky, g - 1.0);
-#pragma unroll
-  for (int q = 0; q < NC; ++q) {
-    tc[q][0] = Ws[q];
-#pragma unroll
-    for (int k = 1; k < 5; ++k) tc[q][k] = t4[q][k];
-  }
+  lead = U.lead;
 }
 
 // Lobatto time average of the flux along dir and the state at tau = dt.  Euler: the nodes tau > 0
@@ -599,8 +782,10 @@ __device__ __forceinline__ void xface_item(const Params& P, const StepView& sv, 
     FlagTable& ft = *reinterpret_cast<FlagTable*>(smem_raw + kEvBytes);
     for (int c = 1 + threadIdx.x; c <= nf + 1; c += SEG) ft.lin[c] = !nl(c);
     __syncthreads();
-    if ((int)threadIdx.x >= nf) return;  // no barrier follows
-    double Wref[NC];  // cells next to the face point (the four around a corner)
+    double a[NC][25], Wref[NC];  // Wref: cells next to the face point (the four around a corner)
+    CkLead lead;
+    const bool has_face = (int)threadIdx.x < nf;
+    if (has_face) {
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
       if (slice < 3)
@@ -609,11 +794,15 @@ __device__ __forceinline__ void xface_item(const Params& P, const StepView& sv, 
         Wref[q] = 0.25 * (fetch(P, st, 0, q, fi - 1, row - 1, sv.t) + fetch(P, st, 0, q, fi, row - 1, sv.t) +
                           fetch(P, st, 0, q, fi - 1, row, sv.t) + fetch(P, st, 0, q, fi, row, sv.t));
     }
-    char_face_point<NC, FLAGS, Q>(P, ev, ft, threadIdx.x, 0, tc, Wref);
+    char_face_point<NC, FLAGS, Q>(P, ev, ft, threadIdx.x, 0, a, lead, Wref);
+    }
+    __syncthreads();  // the tables are read no more
+    ck_points<NC>(P, nf, has_face, a, lead, tc);
+    if (!has_face) return;
   } else {
-    if (!second_pass_cells<NC, FLAGS, Q>(P, ev, smem_raw + kEvBytes, nf, 0, nl, tc)) return;
+    if (!second_pass_cells<NC, FLAGS, Q>(P, smem_raw, nf, 0, nl, tc)) return;
   }
-  const double dt = sv.dt;
+  const double dt = sv.dt * P.ck.iL;  // in the coefficients' unit of time
   if (slice < 3) {
     double Fh[NC], We[NC];
     lobatto<NC>(tc, dt, P.gamma, 0, Fh, We);
@@ -667,17 +856,23 @@ __device__ __forceinline__ void yface_item(const Params& P, const StepView& sv, 
     FlagTable& ft = *reinterpret_cast<FlagTable*>(smem_raw + kEvBytes);
     for (int c = 1 + threadIdx.x; c <= nf + 1; c += SEG) ft.lin[c] = !nl(c);
     __syncthreads();
-    if ((int)threadIdx.x >= nf) return;
-    double Wref[NC];
+    double a[NC][25], Wref[NC];
+    CkLead lead;
+    const bool has_face = (int)threadIdx.x < nf;
+    if (has_face) {
 #pragma unroll
-    for (int q = 0; q < NC; ++q)
-      Wref[q] = 0.5 * (fetch(P, st, 0, q, col, fj - 1, sv.t) + fetch(P, st, 0, q, col, fj, sv.t));
-    char_face_point<NC, FLAGS, Q>(P, ev, ft, threadIdx.x, 1, tc, Wref);
+      for (int q = 0; q < NC; ++q)
+        Wref[q] = 0.5 * (fetch(P, st, 0, q, col, fj - 1, sv.t) + fetch(P, st, 0, q, col, fj, sv.t));
+      char_face_point<NC, FLAGS, Q>(P, ev, ft, threadIdx.x, 1, a, lead, Wref);
+    }
+    __syncthreads();  // the tables are read no more
+    ck_points<NC>(P, nf, has_face, a, lead, tc);
+    if (!has_face) return;
   } else {
-    if (!second_pass_cells<NC, FLAGS, Q>(P, ev, smem_raw + kEvBytes, nf, 1, nl, tc)) return;
+    if (!second_pass_cells<NC, FLAGS, Q>(P, smem_raw, nf, 1, nl, tc)) return;
   }
   double Gh[NC], We[NC];
-  lobatto<NC>(tc, sv.dt, P.gamma, 1, Gh, We);
+  lobatto<NC>(tc, sv.dt * P.ck.iL, P.gamma, 1, Gh, We);
 #pragma unroll
   for (int q = 0; q < NC; ++q) {
     const size_t o = ((size_t)(slice * NC + q) * (P.ny + 1) + fj) * P.nx + col;

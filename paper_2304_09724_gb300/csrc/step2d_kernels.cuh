@@ -50,14 +50,14 @@ __global__ void __launch_bounds__(SEG) xface2d_kernel(Params P, const Ctl* __res
                                                       double* __restrict__ FX,
                                                       double* __restrict__ WX,
                                                       double* __restrict__ WC) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
   if (!ctl->active) return;
   const int slice = blockIdx.z;  // 0..2: Gauss point of the rows; 3: corner rows
   const int row = blockIdx.y;    // Gauss: cell row j; corner: corner row jc (y_{jc-1/2})
   if (slice < 3 && row >= P.ny) return;
   const StepView sv = step_view(ctl);
   xface_item<NC, FLAGS, CHAR, Q>(P, sv, sv.odd ? s1 : s0, ycoef, flag, FX, WX, WC, blockIdx.x * NFACE, row, slice,
-                              smem_raw);
+                              dyn_smem);
 }
 
 template <int NC, bool FLAGS, bool CHAR, bool Q>
@@ -67,11 +67,11 @@ __global__ void __launch_bounds__(SEG) yface2d_kernel(Params P, const Ctl* __res
                                                       const uint8_t* __restrict__ flag,
                                                       double* __restrict__ FY,
                                                       double* __restrict__ WY) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
   if (!ctl->active) return;
   const StepView sv = step_view(ctl);
   yface_item<NC, FLAGS, CHAR, Q>(P, sv, sv.odd ? s1 : s0, xcoef, flag, FY, WY, blockIdx.x * NFACE, blockIdx.y,
-                              blockIdx.z, smem_raw);
+                              blockIdx.z, dyn_smem);
 }
 
 template <int NC>
@@ -101,10 +101,10 @@ static cudaError_t init_kernels2d_nc() {
     const cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) e = r;
   };
-  set((const void*)xface2d_kernel<NC, false, CHAR, Q>, kFaceSmem);
-  set((const void*)yface2d_kernel<NC, false, CHAR, Q>, kFaceSmem);
-  set((const void*)xface2d_kernel<NC, true, CHAR, Q>, kFaceSmem);
-  set((const void*)yface2d_kernel<NC, true, CHAR, Q>, kFaceSmem);
+  set((const void*)xface2d_kernel<NC, false, CHAR, Q>, face_smem<NC>());
+  set((const void*)yface2d_kernel<NC, false, CHAR, Q>, face_smem<NC>());
+  set((const void*)xface2d_kernel<NC, true, CHAR, Q>, face_smem<NC>());
+  set((const void*)yface2d_kernel<NC, true, CHAR, Q>, face_smem<NC>());
   return e;
 }
 
@@ -124,15 +124,15 @@ static void launch_faces2d(const Params& P, Ctl* ctl, const double* s0, const do
                            const uint8_t* flag, const Scratch2D& S, cudaStream_t st, cudaEvent_t* ev) {
   dim3 xg((P.nx + 1 + NFACE - 1) / NFACE, P.ny + 1, 4);
   if (P.flag_mode == FLAG_ALL_NONLINEAR)
-    xface2d_kernel<NC, false, CHAR, Q><<<xg, SEG, kFaceSmem, st>>>(P, ctl, s0, s1, S.ycoef, flag, S.FX, S.WX, S.WC);
+    xface2d_kernel<NC, false, CHAR, Q><<<xg, SEG, face_smem<NC>(), st>>>(P, ctl, s0, s1, S.ycoef, flag, S.FX, S.WX, S.WC);
   else
-    xface2d_kernel<NC, true, CHAR, Q><<<xg, SEG, kFaceSmem, st>>>(P, ctl, s0, s1, S.ycoef, flag, S.FX, S.WX, S.WC);
+    xface2d_kernel<NC, true, CHAR, Q><<<xg, SEG, face_smem<NC>(), st>>>(P, ctl, s0, s1, S.ycoef, flag, S.FX, S.WX, S.WC);
   if (ev) cudaEventRecord(ev[2], st);
   dim3 yg((P.ny + 1 + NFACE - 1) / NFACE, P.nx, 3);
   if (P.flag_mode == FLAG_ALL_NONLINEAR)
-    yface2d_kernel<NC, false, CHAR, Q><<<yg, SEG, kFaceSmem, st>>>(P, ctl, s0, s1, S.xcoef, flag, S.FY, S.WY);
+    yface2d_kernel<NC, false, CHAR, Q><<<yg, SEG, face_smem<NC>(), st>>>(P, ctl, s0, s1, S.xcoef, flag, S.FY, S.WY);
   else
-    yface2d_kernel<NC, true, CHAR, Q><<<yg, SEG, kFaceSmem, st>>>(P, ctl, s0, s1, S.xcoef, flag, S.FY, S.WY);
+    yface2d_kernel<NC, true, CHAR, Q><<<yg, SEG, face_smem<NC>(), st>>>(P, ctl, s0, s1, S.xcoef, flag, S.FY, S.WY);
 }
 
 template <int NC, bool Q>
