@@ -2,10 +2,12 @@
 //
 // Time stepping protocol.  A device control block (Ctl) holds the committed time, step count,
 // the CFL rate of the committed state and a sticky error word.  One step is
-//   begin_step (1 thread): dt from the fixed value or from cfl / rate, clipped to t_final;
+//   begin: dt from the fixed value or from cfl / rate, clipped to t_final;
 //   the step kernels (read Ctl, never write it except the error word and the next rate);
-//   end_step (1 thread): commit t += dt, nsteps += 1, rate_cur = rate_next, unless an error
-//   was raised, in which case nothing is committed.
+//   end: commit t += dt, nsteps += 1, rate_cur = rate_next, unless an error was raised, in which
+//   case nothing is committed.
+// The first step of a call is begun by a one-thread kernel; after that the last CTA of a step's
+// last kernel ends it and begins the next (ctl_commit_last), so a step is its kernels and no more.
 // The committed state always lives in buffer nsteps % 2, so a failed step leaves the previous
 // state in place and no copy is needed.  All launches of a step have fixed arguments, so a run
 // of several steps is captured once as a CUDA graph and replayed; the host only polls Ctl.
@@ -64,30 +66,9 @@ __global__ void reset_kernel(Ctl* c, double t) {
   c->rate_cur = 0ull;
   c->rate_next = 0ull;
   c->mode = 0;
+  c->done = 0;
 }
-__global__ void begin_step_kernel(Ctl* c) {
-  if (c->err != shweno::ERR_NONE) { c->active = 0; return; }
-  double dt;
-  if (c->mode == 0) {
-    dt = c->dt_fixed;
-  } else {
-    if (!(c->t < c->t_final)) { c->active = 0; return; }
-    const double rate = __longlong_as_double((long long)c->rate_cur);
-    dt = c->cfl / rate;
-    if (!(dt <= c->t_final - c->t)) dt = c->t_final - c->t;
-  }
-  c->dt = dt;
-  c->rate_next = 0ull;
-  c->active = 1;
-}
-__global__ void end_step_kernel(Ctl* c) {
-  if (!c->active) return;
-  c->active = 0;
-  if (c->err != shweno::ERR_NONE) { c->err_step = c->nsteps; return; }
-  c->t = c->t + c->dt;
-  c->nsteps += 1;
-  c->rate_cur = c->rate_next;
-}
+__global__ void begin_step_kernel(Ctl* c) { shweno::ctl_begin(c); }
 __global__ void rate_kernel(Params P, Ctl* ctl, const double* s0, const double* s1) {
   __shared__ double red[32];
   const size_t cells = (size_t)P.nx * (P.dim == 2 ? P.ny : 1);
@@ -108,7 +89,6 @@ __global__ void zero_rate_kernel(Ctl* c) { c->rate_cur = 0ull; }
 
 namespace shweno {
 void launch_begin_step(Ctl* ctl, cudaStream_t st) { begin_step_kernel<<<1, 1, 0, st>>>(ctl); }
-void launch_end_step(Ctl* ctl, cudaStream_t st) { end_step_kernel<<<1, 1, 0, st>>>(ctl); }
 void launch_rate(const Params& P, Ctl* ctl, const double* s0, const double* s1, cudaStream_t st) {
   const size_t cells = (size_t)P.nx * (P.dim == 2 ? P.ny : 1);
   zero_rate_kernel<<<1, 1, 0, st>>>(ctl);
@@ -124,8 +104,6 @@ struct shweno_handle {
   double* buf[2] = {nullptr, nullptr};
   double* scratch = nullptr;
   shweno::Scratch2D S{};
-  double* FH = nullptr;
-  double* WE = nullptr;
   uint8_t* flags = nullptr;
   Ctl* ctl = nullptr;
   Ctl* ctl_host = nullptr;  // pinned, two slots
@@ -180,10 +158,9 @@ cudaError_t enqueue_step(shweno_handle* h) {
     h->tev_used = need;
     ++h->timed_steps;
   }
-  shweno::launch_begin_step(h->ctl, h->stream);
   if (h->P.dim == 1) {
     shweno::launch_step1d(h->P, h->ctl, h->buf[0], h->buf[1], h->buf[0], h->buf[1], h->flags,
-                          h->FH, h->WE, h->stream, ev);
+                          h->stream, ev);
   } else {
     if (h->learned) {
       if (ev) cudaEventRecord(ev[0], h->stream);
@@ -194,7 +171,6 @@ cudaError_t enqueue_step(shweno_handle* h) {
     shweno::launch_step2d(h->P, h->ctl, h->buf[0], h->buf[1], h->buf[0], h->buf[1], h->flags,
                           h->S, h->stream, ev);
   }
-  shweno::launch_end_step(h->ctl, h->stream);
   return cudaGetLastError();
 }
 
@@ -339,10 +315,9 @@ shweno_status shweno_create(const shweno_grid* grid, double gamma, const shweno_
     h->buf[b] = (double*)dev_alloc(h->state_doubles * sizeof(double));
     if (!h->buf[b]) return bail(SHWENO_E_NOMEM, "device allocation of the state failed");
   }
-  const size_t scr = dim == 2 ? shweno::scratch2d_doubles(P) : 2 * (size_t)P.ncomp * (P.nx + 1);
-  h->scratch = (double*)dev_alloc(scr * sizeof(double));
-  if (!h->scratch) return bail(SHWENO_E_NOMEM, "device allocation of the step scratch failed");
-  if (dim == 2) {
+  if (dim == 2) {  // the 1D step needs no scratch
+    h->scratch = (double*)dev_alloc(shweno::scratch2d_doubles(P) * sizeof(double));
+    if (!h->scratch) return bail(SHWENO_E_NOMEM, "device allocation of the step scratch failed");
     h->S = shweno::carve_scratch2d(P, h->scratch);
     const cudaError_t ea = shweno::init_kernels2d();
     if (ea != cudaSuccess) {
@@ -351,7 +326,6 @@ shweno_status shweno_create(const shweno_grid* grid, double gamma, const shweno_
                                      cudaGetErrorString(ea));
     }
   }
-  else { h->FH = h->scratch; h->WE = h->scratch + (size_t)P.ncomp * (P.nx + 1); }
   h->ctl = (Ctl*)dev_alloc(sizeof(Ctl));
   if (!h->ctl) return bail(SHWENO_E_NOMEM, "device allocation of the control block failed");
   if (cudaMallocHost(&h->ctl_host, 2 * sizeof(Ctl)) != cudaSuccess) return bail(SHWENO_E_CUDA, "cudaMallocHost failed");
@@ -447,6 +421,7 @@ shweno_status shweno_step(shweno_handle* h, double dt) {
   if (h->P.flag_mode == shweno::FLAG_PER_CELL && !h->flags)
     return fail(h, SHWENO_E_STATE, "flag_mode 2 needs flags (shweno_set_flags)");
   config_kernel<<<1, 1, 0, h->stream>>>(h->ctl, 0, 0.0, 0.0, dt);
+  shweno::launch_begin_step(h->ctl, h->stream);
   CK(h, enqueue_step(h));
   Ctl c;
   shweno_status s = read_ctl(h, &c);
@@ -480,6 +455,7 @@ shweno_status shweno_run(shweno_handle* h, double t_final, double cfl, double* t
     return fail(h, SHWENO_E_STATE, "flag_mode 2 needs flags (shweno_set_flags)");
   config_kernel<<<1, 1, 0, h->stream>>>(h->ctl, 1, t_final, cfl, 0.0);
   shweno::launch_rate(h->P, h->ctl, h->buf[0], h->buf[1], h->stream);
+  shweno::launch_begin_step(h->ctl, h->stream);
   CK(h, cudaGetLastError());
   Ctl c;
   shweno_status s = read_ctl(h, &c);
@@ -542,6 +518,7 @@ shweno_status shweno_advance(shweno_handle* h, int64_t nsteps, double cfl) {
     return fail(h, SHWENO_E_STATE, "flag_mode 2 needs flags (shweno_set_flags)");
   config_kernel<<<1, 1, 0, h->stream>>>(h->ctl, 1, INFINITY, cfl, 0.0);
   shweno::launch_rate(h->P, h->ctl, h->buf[0], h->buf[1], h->stream);
+  shweno::launch_begin_step(h->ctl, h->stream);
   CK(h, cudaGetLastError());
   if (h->timing) {
     for (int64_t k = 0; k < nsteps; ++k) CK(h, enqueue_step(h));
@@ -594,7 +571,7 @@ shweno_status shweno_get_timing(shweno_handle* h, double* ms, int max_kernels, i
 }
 
 const char* shweno_kernel_name(const shweno_handle* h, int k) {
-  static const char* n1[] = {"face1d", "update1d"};
+  static const char* n1[] = {"step1d"};
   static const char* n2[] = {"coef2d", "xface2d", "yface2d", "update2d"};
   if (!h || k < 0 || k >= kernel_count(h)) return "";
   if (h->P.dim == 1) return n1[k];

@@ -2,7 +2,7 @@
 // each with its own time step and end time, advanced by one persistent kernel.
 //
 // Work is cut into items (problem, phase, index).  The phases of one step of a problem are
-//   1D: tiles of `tile1d` cells (faces of the tile into shared memory, then the tile's update);
+//   1D: tiles of `tile1d` cells, W1D cells per warp at a time (step1d_items.cuh);
 //   2D: [flag inference, flag dilation,] first-pass tiles, face segments (x-face Gauss points,
 //       corner points and y-face Gauss points), update segments.
 // A device queue holds the items that are ready: a ring of slots with published sequence
@@ -63,9 +63,8 @@ struct BatchCtl {
 };
 
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
-constexpr size_t kBatchSmem1D = sizeof(double) * 2 * 3 * (1024 + 1);  // F-hat and W(t+dt) of a tile
-// the largest item: a face segment, a first-pass tile (16 fields with halo) or a 1D tile
-constexpr size_t kBatchSmem = cmax(cmax(face_smem<4>(), sizeof(double) * 16 * (TYB + 2) * (TX + 2)), kBatchSmem1D);
+// the largest item: a face segment or a first-pass tile (16 fields with halo); 1D tiles need none
+constexpr size_t kBatchSmem = cmax(face_smem<4>(), sizeof(double) * 16 * (TYB + 2) * (TX + 2));
 
 __device__ __forceinline__ long long enc(int p, int ph, long long idx) {
   return ((long long)p << 40) | ((long long)ph << 36) | idx;
@@ -127,34 +126,18 @@ __device__ __forceinline__ void item_body(const BatchProblem& B, int kind, long 
   __shared__ double red[BT / 32];
   if (!HAS2D) kind = PH_TILE1D;
   switch (kind) {
-    case PH_TILE1D: {  // 1D: faces of the tile into shared memory, then the cells' update
+    case PH_TILE1D: {  // 1D: the warps take the tile's cells in turn, W1D at a time
       const int c0 = (int)idx * B.tile1d;
       const int nc = min(B.tile1d, P.nx - c0);
-      double* FH = reinterpret_cast<double*>(smem);
-      double* WE = FH + 3 * (B.tile1d + 1);
       const double* st = sv.odd ? B.s1 : B.s0;
       double* out = sv.odd ? B.s0 : B.s1;
-      for (int k = threadIdx.x; k <= nc; k += BT) {
-        double Fh[3], We[3];
-        if (P.ncomp == 1) face1d_point<1, false>(P, st, B.flag, c0 + k, sv.t, sv.dt, Fh, We);
-        else face1d_point<3, false>(P, st, B.flag, c0 + k, sv.t, sv.dt, Fh, We);
-        for (int q = 0; q < P.ncomp; ++q) { FH[q * (B.tile1d + 1) + k] = Fh[q]; WE[q * (B.tile1d + 1) + k] = We[q]; }
+      double speed = 0.0;
+      for (int k = (threadIdx.x >> 5) * W1D; k < nc; k += (BT / 32) * W1D) {
+        const int n = min(W1D, nc - k);
+        speed = fmax(speed, P.ncomp == 1 ? step1d_warp<1, false>(P, ctl, st, out, B.flag, c0 + k, n, sv.t, sv.dt)
+                                         : step1d_warp<3, false>(P, ctl, st, out, B.flag, c0 + k, n, sv.t, sv.dt));
       }
-      __syncthreads();
-      double rate = 0.0;
-      for (int k = threadIdx.x; k < nc; k += BT) {
-        const int j = c0 + k;
-        double Wn[4];
-        for (int q = 0; q < P.ncomp; ++q) {
-          const int fo = q * (B.tile1d + 1) + k;
-          Wn[q] = __ldcg(st + (size_t)q * P.nx + j) - sv.dt / P.dx * (FH[fo + 1] - FH[fo]);
-          out[(size_t)q * P.nx + j] = Wn[q];
-          out[(size_t)(P.ncomp + q) * P.nx + j] = (WE[fo + 1] - WE[fo]) * P.idx;
-        }
-        if (!cell_physical(P, Wn)) atomicCAS(&ctl->err, ERR_NONE, ERR_NONPHYSICAL);
-        else rate = fmax(rate, cell_rate(P, Wn));
-      }
-      block_max_rate(rate, &ctl->rate_next, red);
+      report_speed1d(P, ctl, speed);
       break;
     }
   }
@@ -248,7 +231,7 @@ __device__ void do_item(const BatchProblem& B, int kind, long long idx, unsigned
 
 // ------------------------------------------------------------------ persistent kernel
 template <bool HAS2D>
-__global__ void __launch_bounds__(BT, HAS2D ? 1 : 4) batch_kernel(const BatchProblem* __restrict__ probs, int* pstate,
+__global__ void __launch_bounds__(BT, HAS2D ? 1 : 3) batch_kernel(const BatchProblem* __restrict__ probs, int* pstate,
                                                    BatchCtl* bc, long long* items, unsigned long long* seq,
                                                    unsigned long long mask, long long spin_limit) {
   extern __shared__ __align__(16) unsigned char dyn_smem[];
@@ -431,7 +414,7 @@ struct shweno_batch {
   bool own_stream = false;
   int tile1d = 512;
   int ctas_per_sm = 2;
-  bool has2d = true;  // false: every problem is 1D (the lighter kernel, up to 4 CTAs per SM)
+  bool has2d = true;  // false: every problem is 1D (the lighter kernel)
   int grid = 0;
   long long spin_limit = 4000000;  // x ~256 ns sleeps: about a second
   std::string err;
@@ -450,6 +433,10 @@ shweno_status bfail(shweno_batch* b, shweno_status s, const std::string& m) {
   return s;
 }
 
+// Cells of a 1D item: the nominal tile (a power of 2) rounded down to whole rounds of the CTA's four
+// warps (W1D = 30 cells each), 15/16 of it; 512 cells as such would take 5 rounds for 4.27.
+int tile1d_cells(int tile1d) { return tile1d / 128 * (shweno::BT / 32 * shweno::W1D); }
+
 void fill_problem(shweno_batch* b, int p) {
   using namespace shweno;
   const HandleView& v = b->views[p];
@@ -467,10 +454,10 @@ void fill_problem(shweno_batch* b, int p) {
   B.logit_thr = v.logit_thr;
   B.max_steps = INT64_MAX;
   if (v.P.dim == 1) {
-    B.tile1d = b->tile1d;
+    B.tile1d = tile1d_cells(b->tile1d);
     B.nphase = 1;
     B.phase_kind[0] = PH_TILE1D;
-    B.nitems[0] = (v.P.nx + b->tile1d - 1) / b->tile1d;
+    B.nitems[0] = (v.P.nx + B.tile1d - 1) / B.tile1d;
   } else {
     const int nx = v.P.nx, ny = v.P.ny;
     const int cells_items = (int)(((size_t)nx * ny + BT - 1) / BT);
@@ -518,7 +505,7 @@ shweno_status shweno_batch_create(shweno_handle* const* hs, int n, void* cuda_st
   }
   b->has2d = false;
   for (int p = 0; p < n; ++p) b->has2d |= b->views[p].P.dim == 2;
-  if (!b->has2d) b->ctas_per_sm = 4;
+  if (!b->has2d) b->ctas_per_sm = 3;  // what its registers leave room for
   if (cuda_stream) b->stream = (cudaStream_t)cuda_stream;
   else {
     if (cudaStreamCreate(&b->stream) != cudaSuccess) {
@@ -547,7 +534,10 @@ shweno_status shweno_batch_create(shweno_handle* const* hs, int n, void* cuda_st
     int mx = 0;
     for (int k = 0; k < b->host_probs[p].nphase; ++k) mx = std::max(mx, b->host_probs[p].nitems[k]);
     // 1D problems may be re-tiled by the autotuner down to 128 cells per item
-    if (b->views[p].P.dim == 1) mx = std::max(mx, (b->views[p].P.nx + 127) / 128);
+    if (b->views[p].P.dim == 1) {
+      const int t = tile1d_cells(128);
+      mx = std::max(mx, (b->views[p].P.nx + t - 1) / t);
+    }
     cap_need += mx;
   }
   cap_need += 4 * (size_t)sms * 8 + 1;
@@ -568,9 +558,7 @@ shweno_status shweno_batch_create(shweno_handle* const* hs, int n, void* cuda_st
   }
   if (cudaMemcpy(b->chunk0, ch.data(), n * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaFuncSetAttribute(batch_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem) != cudaSuccess ||
-      cudaFuncSetAttribute(batch_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem1D) != cudaSuccess ||
-      cudaFuncSetAttribute(lockstep_kernel<PH_FACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)face_smem<4>()) != cudaSuccess ||
-      cudaFuncSetAttribute(lockstep_kernel<PH_TILE1D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem1D) != cudaSuccess) {
+      cudaFuncSetAttribute(lockstep_kernel<PH_FACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)face_smem<4>()) != cudaSuccess) {
     cudaGetLastError();
     shweno_batch_destroy(b);
     return SHWENO_E_CUDA;
@@ -616,7 +604,7 @@ void enqueue_batch(shweno_batch* b, double cfl) {
     batch_kernel<true><<<b->grid, BT, kBatchSmem, b->stream>>>(b->probs, b->pstate, b->bc, b->items, b->seq,
                                                                cap - 1, b->spin_limit);
   else
-    batch_kernel<false><<<b->grid, BT, kBatchSmem1D, b->stream>>>(b->probs, b->pstate, b->bc, b->items, b->seq,
+    batch_kernel<false><<<b->grid, BT, 0, b->stream>>>(b->probs, b->pstate, b->bc, b->items, b->seq,
                                                                   cap - 1, b->spin_limit);
 }
 
@@ -677,7 +665,6 @@ size_t lock_smem(const shweno_batch* b, int kind) {
     case PH_INFER: return sizeof(float) * NPARAM;
     case PH_COEF: return sizeof(double) * 16 * (TYB + 2) * (TX + 2);
     case PH_FACE: return face_smem<4>();
-    case PH_TILE1D: return sizeof(double) * 2 * 3 * (b->tile1d + 1);
     default: return 0;
   }
 }

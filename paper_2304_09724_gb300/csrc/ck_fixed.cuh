@@ -132,7 +132,7 @@ FX_FN Fx ck_ninv(const CkScale<NC>& S, const CkLead& lead) {
 
 constexpr int kCkTries = 8;  // growths tried at most; inputs below 2^-5s cannot leave the range
 
-// Burgers: the whole recursion in one thread's registers.  Writes tc[q][k],
+// Burgers and 1D Euler: the whole recursion in one thread's registers (2D Euler: step2d_items.cuh).  Writes tc[q][k],
 // k = 1..4, per L^k (tc[q][0] is left to the caller); NaN where the input is not finite.
 template <int NC, int DIM>
 FX_FN void ck_fixed(const double (&a)[NC][25], const CkLead& lead, const CkFixedConst& K, double (&tc)[NC][5]) {
@@ -151,8 +151,9 @@ FX_FN void ck_fixed(const double (&a)[NC][25], const CkLead& lead, const CkFixed
 #pragma unroll
         for (int n = 0; n + m < 5; ++n)
           if (DIM == 2 || n == 0) w[q][m * 5 + n] = ck_convert<NC>(S, a[q][m * 5 + n], q, m + n, m + n ? r : r0);
-    static_assert(NC == 1 && DIM == 2, "2D Euler runs on two lanes");
-    ck_burgers2d_fx(w, ninv, K, t, r);
+    if constexpr (NC == 1 && DIM == 1) ck_burgers1d_fx(w, ninv, K, t, r);
+    else if constexpr (NC == 1) ck_burgers2d_fx(w, ninv, K, t, r);
+    else ck_euler1d_fx(w, ninv, K, t, r);
     if (!r.bad()) break;
   }
 #pragma unroll

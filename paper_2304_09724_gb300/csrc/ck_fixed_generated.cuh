@@ -1,4 +1,4 @@
-// Generated by gen_ck.py -- do not edit.  The Cauchy-Kovalevskaya recursions in two dimensions
+// Generated by gen_ck.py -- do not edit.  The Cauchy-Kovalevskaya recursions
 // in block fixed point (see fixed.cuh, ck_fixed.cuh and gen_ck.py for the method).
 #pragma once
 #include "fixed.cuh"
@@ -23,10 +23,40 @@ FX_FN int64_t fx_time(int64_t z, Fx third) {
   return fx_sum<FX_C>(s);
 }
 
+// ck_burgers1d_fx: 1D burgers in block fixed point; inputs w[q][m*5+n], outputs t[q][k], k = 1..4, in
+// the fields' units (fixed.cuh, ck_fixed.cuh); ninv = -1/rho0 in fixed point (Euler).
+FX_FN void ck_burgers1d_fx(const Fx (&w)[1][25], Fx ninv, const CkFixedConst& K, int64_t (&t)[1][5], FxRange& r) {
+  (void)ninv;
+  int64_t f_100; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][5]); f_100 = fx_sum(s); }
+  const Fx w0_001 = fx_split(fx_time<1>(1 * f_100, K.third) + FX_HALF, r);
+  int64_t f_200; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][10]); f_200 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w[0][5], w[0][5]); f_200 += fx_sum(s) >> 1; }
+  const Fx w0_101 = fx_split(fx_time<1>(2 * f_200, K.third) + FX_HALF, r);
+  int64_t f_101; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_101); fx_mac(s, w0_001, w[0][5]); f_101 = fx_sum(s); }
+  const Fx w0_002 = fx_split(fx_time<2>(1 * f_101, K.third) + FX_HALF, r);
+  int64_t f_300; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][15]); fx_mac(s, w[0][5], w[0][10]); f_300 = fx_sum(s); }
+  const Fx w0_201 = fx_split(fx_time<1>(3 * f_300, K.third) + FX_HALF, r);
+  int64_t f_201; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_201); fx_mac(s, w0_001, w[0][10]); fx_mac(s, w[0][5], w0_101); f_201 = fx_sum(s); }
+  const Fx w0_102 = fx_split(fx_time<2>(2 * f_201, K.third) + FX_HALF, r);
+  int64_t f_102; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_102); fx_mac(s, w0_001, w0_101); fx_mac(s, w0_002, w[0][5]); f_102 = fx_sum(s); }
+  const Fx w0_003 = fx_split(fx_time<3>(1 * f_102, K.third) + FX_HALF, r);
+  int64_t f_400; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][20]); fx_mac(s, w[0][5], w[0][15]); f_400 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w[0][10], w[0][10]); f_400 += fx_sum(s) >> 1; }
+  const Fx w0_301 = fx_split(fx_time<1>(4 * f_400, K.third) + FX_HALF, r);
+  int64_t f_301; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_301); fx_mac(s, w0_001, w[0][15]); fx_mac(s, w[0][5], w0_201); fx_mac(s, w0_101, w[0][10]); f_301 = fx_sum(s); }
+  const Fx w0_202 = fx_split(fx_time<2>(3 * f_301, K.third) + FX_HALF, r);
+  int64_t f_202; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_202); fx_mac(s, w0_001, w0_201); fx_mac(s, w0_002, w[0][10]); fx_mac(s, w[0][5], w0_102); f_202 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w0_101, w0_101); f_202 += fx_sum(s) >> 1; }
+  const Fx w0_103 = fx_split(fx_time<3>(2 * f_202, K.third) + FX_HALF, r);
+  int64_t f_103; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_103); fx_mac(s, w0_001, w0_102); fx_mac(s, w0_002, w0_101); fx_mac(s, w0_003, w[0][5]); f_103 = fx_sum(s); }
+  const Fx w0_004 = fx_split(fx_time<4>(1 * f_103, K.third) + FX_HALF, r);
+  t[0][1] = fx_join(w0_001);
+  t[0][2] = fx_join(w0_002);
+  t[0][3] = fx_join(w0_003);
+  t[0][4] = fx_join(w0_004);
+}
+
 // ck_burgers2d_fx: 2D burgers in block fixed point; inputs w[q][m*5+n], outputs t[q][k], k = 1..4, in
 // the fields' units (fixed.cuh, ck_fixed.cuh); ninv = -1/rho0 in fixed point (Euler).
 FX_FN void ck_burgers2d_fx(const Fx (&w)[1][25], Fx ninv, const CkFixedConst& K, int64_t (&t)[1][5], FxRange& r) {
-  (void)ninv; FxRange r0{0}; (void)r0;  // leading coefficients are in range by their scales
+  (void)ninv;
   int64_t f_100; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][5]); f_100 = fx_sum(s); }
   int64_t f_010; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][1]); f_010 = fx_sum(s); }
   const Fx w0_001 = fx_split(fx_time<1>(1 * f_100 + 1 * f_010, K.third) + FX_HALF, r);
@@ -81,6 +111,173 @@ FX_FN void ck_burgers2d_fx(const Fx (&w)[1][25], Fx ninv, const CkFixedConst& K,
   t[0][2] = fx_join(w0_002);
   t[0][3] = fx_join(w0_003);
   t[0][4] = fx_join(w0_004);
+}
+
+// ck_euler1d_fx: 1D euler in block fixed point; inputs w[q][m*5+n], outputs t[q][k], k = 1..4, in
+// the fields' units (fixed.cuh, ck_fixed.cuh); ninv = -1/rho0 in fixed point (Euler).
+FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, int64_t (&t)[3][5], FxRange& r) {
+  (void)ninv;
+  FxRange r0{0};  // leading coefficients are in range by their scales
+  const int64_t z_w1_100 = fx_join(w[1][5]);
+  const Fx w0_001 = fx_split(fx_time<1>(1 * (z_w1_100), K.third) + FX_HALF, r);
+  Fx u_000n; { FxAcc s = fx_zero(true); fx_mac_int(s, w[1][0], -(1 << 30)); u_000n = fx_split(fx_sum(s), r0); }
+  Fx u_000; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_000n, ninv); u_000 = fx_split(fx_sum<FX_C>(s), r0); }
+  Fx u_100n; { FxAcc s = fx_zero(true); fx_mac_int(s, w[1][5], -(1 << 30)); fx_mac(s, w[0][5], u_000); u_100n = fx_split(fx_sum(s), r); }
+  Fx u_100; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_100n, ninv); u_100 = fx_split(fx_sum<FX_C>(s), r); }
+  Fx u_200n; { FxAcc s = fx_zero(true); fx_mac_int(s, w[1][10], -(1 << 30)); fx_mac(s, w[0][5], u_100); fx_mac(s, w[0][10], u_000); u_200n = fx_split(fx_sum(s), r); }
+  Fx u_200; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_200n, ninv); u_200 = fx_split(fx_sum<FX_C>(s), r); }
+  int64_t z_mu_200; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_200); fx_mac(s, w[1][5], u_100); fx_mac(s, w[1][10], u_000); z_mu_200 = fx_sum(s); }
+  const int64_t z_w2_200 = fx_join(w[2][10]);
+  const Fx e_200 = fx_split(((z_w2_200 - ((z_mu_200) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_200; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_200, K.gm1); z_p_200 = fx_sum<FX_C>(s); }
+  const Fx w1_101 = fx_split(fx_time<1>(2 * (z_mu_200 + z_p_200), K.third) + FX_HALF, r);
+  const int64_t z_w1_101 = fx_join(w1_101);
+  const Fx w0_002 = fx_split(fx_time<2>(1 * (z_w1_101), K.third) + FX_HALF, r);
+  Fx u_300n; { FxAcc s = fx_zero(true); fx_mac_int(s, w[1][15], -(1 << 30)); fx_mac(s, w[0][5], u_200); fx_mac(s, w[0][10], u_100); fx_mac(s, w[0][15], u_000); u_300n = fx_split(fx_sum(s), r); }
+  Fx u_300; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_300n, ninv); u_300 = fx_split(fx_sum<FX_C>(s), r); }
+  int64_t z_mu_300; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_300); fx_mac(s, w[1][5], u_200); fx_mac(s, w[1][10], u_100); fx_mac(s, w[1][15], u_000); z_mu_300 = fx_sum(s); }
+  const int64_t z_w2_300 = fx_join(w[2][15]);
+  const Fx e_300 = fx_split(((z_w2_300 - ((z_mu_300) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_300; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_300, K.gm1); z_p_300 = fx_sum<FX_C>(s); }
+  const Fx w1_201 = fx_split(fx_time<1>(3 * (z_mu_300 + z_p_300), K.third) + FX_HALF, r);
+  int64_t z_mu_100; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_100); fx_mac(s, w[1][5], u_000); z_mu_100 = fx_sum(s); }
+  const int64_t z_w2_100 = fx_join(w[2][5]);
+  const Fx e_100 = fx_split(((z_w2_100 - ((z_mu_100) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_100; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_100, K.gm1); z_p_100 = fx_sum<FX_C>(s); }
+  const Fx w1_001 = fx_split(fx_time<1>(1 * (z_mu_100 + z_p_100), K.third) + FX_HALF, r);
+  Fx u_001n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_001, -(1 << 30)); fx_mac(s, w0_001, u_000); u_001n = fx_split(fx_sum(s), r); }
+  Fx u_001; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_001n, ninv); u_001 = fx_split(fx_sum<FX_C>(s), r); }
+  const int64_t z_w1_200 = fx_join(w[1][10]);
+  const Fx w0_101 = fx_split(fx_time<1>(2 * (z_w1_200), K.third) + FX_HALF, r);
+  Fx u_101n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_101, -(1 << 30)); fx_mac(s, w0_001, u_100); fx_mac(s, w[0][5], u_001); fx_mac(s, w0_101, u_000); u_101n = fx_split(fx_sum(s), r); }
+  Fx u_101; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_101n, ninv); u_101 = fx_split(fx_sum<FX_C>(s), r); }
+  const int64_t z_w1_300 = fx_join(w[1][15]);
+  const Fx w0_201 = fx_split(fx_time<1>(3 * (z_w1_300), K.third) + FX_HALF, r);
+  Fx u_201n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_201, -(1 << 30)); fx_mac(s, w0_001, u_200); fx_mac(s, w[0][5], u_101); fx_mac(s, w0_101, u_100); fx_mac(s, w[0][10], u_001); fx_mac(s, w0_201, u_000); u_201n = fx_split(fx_sum(s), r); }
+  Fx u_201; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_201n, ninv); u_201 = fx_split(fx_sum<FX_C>(s), r); }
+  int64_t z_mu_201; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_201); fx_mac(s, w1_001, u_200); fx_mac(s, w[1][5], u_101); fx_mac(s, w1_101, u_100); fx_mac(s, w[1][10], u_001); fx_mac(s, w1_201, u_000); z_mu_201 = fx_sum(s); }
+  const Fx H_300 = fx_split(z_w2_300 + z_p_300 + FX_HALF, r);
+  const Fx H_200 = fx_split(z_w2_200 + z_p_200 + FX_HALF, r);
+  const Fx H_100 = fx_split(z_w2_100 + z_p_100 + FX_HALF, r);
+  const int64_t z_w2_000 = fx_join(w[2][0]);
+  int64_t z_mu_000; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_000); z_mu_000 = fx_sum(s); }
+  const Fx e_000 = fx_split(((z_w2_000 - ((z_mu_000) >> 1)) << K.gshift) + FX_HALF, r0);
+  int64_t z_p_000; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_000, K.gm1); z_p_000 = fx_sum<FX_C>(s); }
+  const Fx H_000 = fx_split(z_w2_000 + z_p_000 + FX_HALF, r0);
+  int64_t z_uH_300; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_300); fx_mac(s, u_100, H_200); fx_mac(s, u_200, H_100); fx_mac(s, u_300, H_000); z_uH_300 = fx_sum(s); }
+  const Fx w2_201 = fx_split(fx_time<1>(3 * (z_uH_300), K.third) + FX_HALF, r);
+  const int64_t z_w2_201 = fx_join(w2_201);
+  const Fx e_201 = fx_split(((z_w2_201 - ((z_mu_201) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_201; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_201, K.gm1); z_p_201 = fx_sum<FX_C>(s); }
+  const Fx w1_102 = fx_split(fx_time<2>(2 * (z_mu_201 + z_p_201), K.third) + FX_HALF, r);
+  const int64_t z_w1_102 = fx_join(w1_102);
+  const Fx w0_003 = fx_split(fx_time<3>(1 * (z_w1_102), K.third) + FX_HALF, r);
+  Fx u_400n; { FxAcc s = fx_zero(true); fx_mac_int(s, w[1][20], -(1 << 30)); fx_mac(s, w[0][5], u_300); fx_mac(s, w[0][10], u_200); fx_mac(s, w[0][15], u_100); fx_mac(s, w[0][20], u_000); u_400n = fx_split(fx_sum(s), r); }
+  Fx u_400; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_400n, ninv); u_400 = fx_split(fx_sum<FX_C>(s), r); }
+  int64_t z_mu_400; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_400); fx_mac(s, w[1][5], u_300); fx_mac(s, w[1][10], u_200); fx_mac(s, w[1][15], u_100); fx_mac(s, w[1][20], u_000); z_mu_400 = fx_sum(s); }
+  const int64_t z_w2_400 = fx_join(w[2][20]);
+  const Fx e_400 = fx_split(((z_w2_400 - ((z_mu_400) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_400; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_400, K.gm1); z_p_400 = fx_sum<FX_C>(s); }
+  const Fx w1_301 = fx_split(fx_time<1>(4 * (z_mu_400 + z_p_400), K.third) + FX_HALF, r);
+  const int64_t z_w1_400 = fx_join(w[1][20]);
+  const Fx w0_301 = fx_split(fx_time<1>(4 * (z_w1_400), K.third) + FX_HALF, r);
+  Fx u_301n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_301, -(1 << 30)); fx_mac(s, w0_001, u_300); fx_mac(s, w[0][5], u_201); fx_mac(s, w0_101, u_200); fx_mac(s, w[0][10], u_101); fx_mac(s, w0_201, u_100); fx_mac(s, w[0][15], u_001); fx_mac(s, w0_301, u_000); u_301n = fx_split(fx_sum(s), r); }
+  Fx u_301; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_301n, ninv); u_301 = fx_split(fx_sum<FX_C>(s), r); }
+  int64_t z_mu_301; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_301); fx_mac(s, w1_001, u_300); fx_mac(s, w[1][5], u_201); fx_mac(s, w1_101, u_200); fx_mac(s, w[1][10], u_101); fx_mac(s, w1_201, u_100); fx_mac(s, w[1][15], u_001); fx_mac(s, w1_301, u_000); z_mu_301 = fx_sum(s); }
+  const Fx H_400 = fx_split(z_w2_400 + z_p_400 + FX_HALF, r);
+  int64_t z_uH_400; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_400); fx_mac(s, u_100, H_300); fx_mac(s, u_200, H_200); fx_mac(s, u_300, H_100); fx_mac(s, u_400, H_000); z_uH_400 = fx_sum(s); }
+  const Fx w2_301 = fx_split(fx_time<1>(4 * (z_uH_400), K.third) + FX_HALF, r);
+  const int64_t z_w2_301 = fx_join(w2_301);
+  const Fx e_301 = fx_split(((z_w2_301 - ((z_mu_301) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_301; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_301, K.gm1); z_p_301 = fx_sum<FX_C>(s); }
+  const Fx w1_202 = fx_split(fx_time<2>(3 * (z_mu_301 + z_p_301), K.third) + FX_HALF, r);
+  int64_t z_mu_101; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_101); fx_mac(s, w1_001, u_100); fx_mac(s, w[1][5], u_001); fx_mac(s, w1_101, u_000); z_mu_101 = fx_sum(s); }
+  int64_t z_uH_200; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_200); fx_mac(s, u_100, H_100); fx_mac(s, u_200, H_000); z_uH_200 = fx_sum(s); }
+  const Fx w2_101 = fx_split(fx_time<1>(2 * (z_uH_200), K.third) + FX_HALF, r);
+  const int64_t z_w2_101 = fx_join(w2_101);
+  const Fx e_101 = fx_split(((z_w2_101 - ((z_mu_101) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_101; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_101, K.gm1); z_p_101 = fx_sum<FX_C>(s); }
+  const Fx w1_002 = fx_split(fx_time<2>(1 * (z_mu_101 + z_p_101), K.third) + FX_HALF, r);
+  Fx u_002n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_002, -(1 << 30)); fx_mac(s, w0_001, u_001); fx_mac(s, w0_002, u_000); u_002n = fx_split(fx_sum(s), r); }
+  Fx u_002; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_002n, ninv); u_002 = fx_split(fx_sum<FX_C>(s), r); }
+  const int64_t z_w1_201 = fx_join(w1_201);
+  const Fx w0_102 = fx_split(fx_time<2>(2 * (z_w1_201), K.third) + FX_HALF, r);
+  Fx u_102n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_102, -(1 << 30)); fx_mac(s, w0_001, u_101); fx_mac(s, w0_002, u_100); fx_mac(s, w[0][5], u_002); fx_mac(s, w0_101, u_001); fx_mac(s, w0_102, u_000); u_102n = fx_split(fx_sum(s), r); }
+  Fx u_102; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_102n, ninv); u_102 = fx_split(fx_sum<FX_C>(s), r); }
+  const int64_t z_w1_301 = fx_join(w1_301);
+  const Fx w0_202 = fx_split(fx_time<2>(3 * (z_w1_301), K.third) + FX_HALF, r);
+  Fx u_202n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_202, -(1 << 30)); fx_mac(s, w0_001, u_201); fx_mac(s, w0_002, u_200); fx_mac(s, w[0][5], u_102); fx_mac(s, w0_101, u_101); fx_mac(s, w0_102, u_100); fx_mac(s, w[0][10], u_002); fx_mac(s, w0_201, u_001); fx_mac(s, w0_202, u_000); u_202n = fx_split(fx_sum(s), r); }
+  Fx u_202; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_202n, ninv); u_202 = fx_split(fx_sum<FX_C>(s), r); }
+  int64_t z_mu_202; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_202); fx_mac(s, w1_001, u_201); fx_mac(s, w1_002, u_200); fx_mac(s, w[1][5], u_102); fx_mac(s, w1_101, u_101); fx_mac(s, w1_102, u_100); fx_mac(s, w[1][10], u_002); fx_mac(s, w1_201, u_001); fx_mac(s, w1_202, u_000); z_mu_202 = fx_sum(s); }
+  const Fx H_301 = fx_split(z_w2_301 + z_p_301 + FX_HALF, r);
+  const Fx H_201 = fx_split(z_w2_201 + z_p_201 + FX_HALF, r);
+  const Fx H_101 = fx_split(z_w2_101 + z_p_101 + FX_HALF, r);
+  int64_t z_uH_100; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_100); fx_mac(s, u_100, H_000); z_uH_100 = fx_sum(s); }
+  const Fx w2_001 = fx_split(fx_time<1>(1 * (z_uH_100), K.third) + FX_HALF, r);
+  const int64_t z_w2_001 = fx_join(w2_001);
+  int64_t z_mu_001; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_001); fx_mac(s, w1_001, u_000); z_mu_001 = fx_sum(s); }
+  const Fx e_001 = fx_split(((z_w2_001 - ((z_mu_001) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_001; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_001, K.gm1); z_p_001 = fx_sum<FX_C>(s); }
+  const Fx H_001 = fx_split(z_w2_001 + z_p_001 + FX_HALF, r);
+  int64_t z_uH_301; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_301); fx_mac(s, u_001, H_300); fx_mac(s, u_100, H_201); fx_mac(s, u_101, H_200); fx_mac(s, u_200, H_101); fx_mac(s, u_201, H_100); fx_mac(s, u_300, H_001); fx_mac(s, u_301, H_000); z_uH_301 = fx_sum(s); }
+  const Fx w2_202 = fx_split(fx_time<2>(3 * (z_uH_301), K.third) + FX_HALF, r);
+  const int64_t z_w2_202 = fx_join(w2_202);
+  const Fx e_202 = fx_split(((z_w2_202 - ((z_mu_202) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_202; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_202, K.gm1); z_p_202 = fx_sum<FX_C>(s); }
+  const Fx w1_103 = fx_split(fx_time<3>(2 * (z_mu_202 + z_p_202), K.third) + FX_HALF, r);
+  const int64_t z_w1_103 = fx_join(w1_103);
+  const Fx w0_004 = fx_split(fx_time<4>(1 * (z_w1_103), K.third) + FX_HALF, r);
+  int64_t z_mu_102; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_102); fx_mac(s, w1_001, u_101); fx_mac(s, w1_002, u_100); fx_mac(s, w[1][5], u_002); fx_mac(s, w1_101, u_001); fx_mac(s, w1_102, u_000); z_mu_102 = fx_sum(s); }
+  int64_t z_uH_201; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_201); fx_mac(s, u_001, H_200); fx_mac(s, u_100, H_101); fx_mac(s, u_101, H_100); fx_mac(s, u_200, H_001); fx_mac(s, u_201, H_000); z_uH_201 = fx_sum(s); }
+  const Fx w2_102 = fx_split(fx_time<2>(2 * (z_uH_201), K.third) + FX_HALF, r);
+  const int64_t z_w2_102 = fx_join(w2_102);
+  const Fx e_102 = fx_split(((z_w2_102 - ((z_mu_102) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_102; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_102, K.gm1); z_p_102 = fx_sum<FX_C>(s); }
+  const Fx w1_003 = fx_split(fx_time<3>(1 * (z_mu_102 + z_p_102), K.third) + FX_HALF, r);
+  Fx u_003n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_003, -(1 << 30)); fx_mac(s, w0_001, u_002); fx_mac(s, w0_002, u_001); fx_mac(s, w0_003, u_000); u_003n = fx_split(fx_sum(s), r); }
+  Fx u_003; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_003n, ninv); u_003 = fx_split(fx_sum<FX_C>(s), r); }
+  const int64_t z_w1_202 = fx_join(w1_202);
+  const Fx w0_103 = fx_split(fx_time<3>(2 * (z_w1_202), K.third) + FX_HALF, r);
+  Fx u_103n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_103, -(1 << 30)); fx_mac(s, w0_001, u_102); fx_mac(s, w0_002, u_101); fx_mac(s, w0_003, u_100); fx_mac(s, w[0][5], u_003); fx_mac(s, w0_101, u_002); fx_mac(s, w0_102, u_001); fx_mac(s, w0_103, u_000); u_103n = fx_split(fx_sum(s), r); }
+  Fx u_103; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_103n, ninv); u_103 = fx_split(fx_sum<FX_C>(s), r); }
+  int64_t z_mu_103; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_103); fx_mac(s, w1_001, u_102); fx_mac(s, w1_002, u_101); fx_mac(s, w1_003, u_100); fx_mac(s, w[1][5], u_003); fx_mac(s, w1_101, u_002); fx_mac(s, w1_102, u_001); fx_mac(s, w1_103, u_000); z_mu_103 = fx_sum(s); }
+  const Fx H_202 = fx_split(z_w2_202 + z_p_202 + FX_HALF, r);
+  const Fx H_102 = fx_split(z_w2_102 + z_p_102 + FX_HALF, r);
+  int64_t z_uH_101; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_101); fx_mac(s, u_001, H_100); fx_mac(s, u_100, H_001); fx_mac(s, u_101, H_000); z_uH_101 = fx_sum(s); }
+  const Fx w2_002 = fx_split(fx_time<2>(1 * (z_uH_101), K.third) + FX_HALF, r);
+  const int64_t z_w2_002 = fx_join(w2_002);
+  int64_t z_mu_002; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_002); fx_mac(s, w1_001, u_001); fx_mac(s, w1_002, u_000); z_mu_002 = fx_sum(s); }
+  const Fx e_002 = fx_split(((z_w2_002 - ((z_mu_002) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_002; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_002, K.gm1); z_p_002 = fx_sum<FX_C>(s); }
+  const Fx H_002 = fx_split(z_w2_002 + z_p_002 + FX_HALF, r);
+  int64_t z_uH_202; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_202); fx_mac(s, u_001, H_201); fx_mac(s, u_002, H_200); fx_mac(s, u_100, H_102); fx_mac(s, u_101, H_101); fx_mac(s, u_102, H_100); fx_mac(s, u_200, H_002); fx_mac(s, u_201, H_001); fx_mac(s, u_202, H_000); z_uH_202 = fx_sum(s); }
+  const Fx w2_103 = fx_split(fx_time<3>(2 * (z_uH_202), K.third) + FX_HALF, r);
+  const int64_t z_w2_103 = fx_join(w2_103);
+  const Fx e_103 = fx_split(((z_w2_103 - ((z_mu_103) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_103; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_103, K.gm1); z_p_103 = fx_sum<FX_C>(s); }
+  const Fx w1_004 = fx_split(fx_time<4>(1 * (z_mu_103 + z_p_103), K.third) + FX_HALF, r);
+  int64_t z_uH_102; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_102); fx_mac(s, u_001, H_101); fx_mac(s, u_002, H_100); fx_mac(s, u_100, H_002); fx_mac(s, u_101, H_001); fx_mac(s, u_102, H_000); z_uH_102 = fx_sum(s); }
+  const Fx w2_003 = fx_split(fx_time<3>(1 * (z_uH_102), K.third) + FX_HALF, r);
+  const Fx H_103 = fx_split(z_w2_103 + z_p_103 + FX_HALF, r);
+  const int64_t z_w2_003 = fx_join(w2_003);
+  int64_t z_mu_003; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_003); fx_mac(s, w1_001, u_002); fx_mac(s, w1_002, u_001); fx_mac(s, w1_003, u_000); z_mu_003 = fx_sum(s); }
+  const Fx e_003 = fx_split(((z_w2_003 - ((z_mu_003) >> 1)) << K.gshift) + FX_HALF, r);
+  int64_t z_p_003; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_003, K.gm1); z_p_003 = fx_sum<FX_C>(s); }
+  const Fx H_003 = fx_split(z_w2_003 + z_p_003 + FX_HALF, r);
+  int64_t z_uH_103; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_103); fx_mac(s, u_001, H_102); fx_mac(s, u_002, H_101); fx_mac(s, u_003, H_100); fx_mac(s, u_100, H_003); fx_mac(s, u_101, H_002); fx_mac(s, u_102, H_001); fx_mac(s, u_103, H_000); z_uH_103 = fx_sum(s); }
+  const Fx w2_004 = fx_split(fx_time<4>(1 * (z_uH_103), K.third) + FX_HALF, r);
+  t[0][1] = fx_join(w0_001);
+  t[0][2] = fx_join(w0_002);
+  t[0][3] = fx_join(w0_003);
+  t[0][4] = fx_join(w0_004);
+  t[1][1] = fx_join(w1_001);
+  t[1][2] = fx_join(w1_002);
+  t[1][3] = fx_join(w1_003);
+  t[1][4] = fx_join(w1_004);
+  t[2][1] = fx_join(w2_001);
+  t[2][2] = fx_join(w2_002);
+  t[2][3] = fx_join(w2_003);
+  t[2][4] = fx_join(w2_004);
 }
 
 // 2D Euler, two lanes per point: S gives the shared series and constants, ninv = -1/rho0;

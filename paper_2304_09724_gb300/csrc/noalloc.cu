@@ -51,6 +51,7 @@ __global__ void noalloc_begin_kernel(Ctl* c, double t, double dt) {
   c->rate_next = 0ull;
   c->mode = 0;
   c->err = shweno::ERR_NONE;
+  c->done = 0;
   c->active = 1;
 }
 
@@ -96,8 +97,6 @@ extern "C" shweno_status shweno_step1d_noalloc(int32_t eq, int64_t nx, double x0
     base = g_scratch_ptr[dev];
   }
   Ctl* ctl = (Ctl*)base;
-  double* FH = base + kCtlDoubles;
-  double* WE = FH + (size_t)ncomp * (nx + 1);
 
   Params P{};
   P.dim = 1;
@@ -123,7 +122,7 @@ extern "C" shweno_status shweno_step1d_noalloc(int32_t eq, int64_t nx, double x0
 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   noalloc_begin_kernel<<<1, 1, 0, st>>>(ctl, t, dt);
-  shweno::launch_step1d(P, ctl, state_in, state_in, state_out, state_out, nullptr, FH, WE, st, nullptr);
+  shweno::launch_step1d(P, ctl, state_in, state_in, state_out, state_out, nullptr, st, nullptr);
   if (cudaGetLastError() != cudaSuccess) return SHWENO_E_CUDA;
   Ctl h;
   if (cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

@@ -44,8 +44,9 @@ inline void finalize_params(Params& P) {
   finalize_ck_fixed(P.ck, P.dim, P.dx, P.dy, P.eq == EQ_EULER ? P.gamma : 1.4);
 }
 
-// Device-resident time-stepping control block.  One step = begin_step, the step kernels,
-// end_step; only begin_step/end_step (one thread each) write it, the step kernels only read.
+// Device-resident time-stepping control block.  A step is begun by ctl_begin, its kernels only
+// read the block (but for the error word and the next rate), and the CTA of its last kernel that
+// finishes last ends it and begins the next one (ctl_commit_last).
 struct Ctl {
   double t;                    // time of the committed state
   double dt;                   // step being taken (valid while active)
@@ -57,8 +58,43 @@ struct Ctl {
   int32_t mode;                // 0: fixed dt, 1: CFL with t_final
   int32_t active;              // 1 while a step is in flight
   int32_t err;                 // first error code seen (ERR_*), sticky
-  int32_t pad;
+  uint32_t done;               // CTAs of the step's last kernel that have finished (0 between steps)
 };
+
+// Begins a step: dt from the fixed value or from cfl / rate, clipped to t_final.
+__device__ inline void ctl_begin(volatile Ctl* c) {
+  c->active = 0;
+  if (c->err != ERR_NONE) return;
+  double dt;
+  if (c->mode == 0) {
+    dt = c->dt_fixed;
+  } else {
+    if (!(c->t < c->t_final)) return;
+    const double rate = __longlong_as_double((long long)c->rate_cur);
+    dt = c->cfl / rate;
+    if (!(dt <= c->t_final - c->t)) dt = c->t_final - c->t;
+  }
+  c->dt = dt;
+  c->rate_next = 0ull;
+  c->active = 1;
+}
+// Ends the step in flight: commits t, the step count and the rate, unless an error was raised.
+__device__ inline void ctl_end(volatile Ctl* c) {
+  if (c->err != ERR_NONE) { c->err_step = c->nsteps; return; }
+  c->t = c->t + c->dt;
+  c->nsteps += 1;
+  c->rate_cur = c->rate_next;
+}
+// Thread 0 of every CTA of a step's last kernel, after the CTA's errors and rate have been
+// reported: the last one ends the step and begins the next, which spares the two one-thread
+// launches (1.5 to 2 us each) that did it.  Every CTA has read the step's data by then.
+__device__ inline void ctl_commit_last(Ctl* c, unsigned nblocks) {
+  __threadfence();
+  if (atomicInc(&c->done, nblocks - 1) != nblocks - 1) return;
+  __threadfence();
+  ctl_end(c);
+  ctl_begin(c);
+}
 
 // Snapshot of the step in flight, read with volatile loads: inside the batched persistent
 // kernel the control block is rewritten by other CTAs between steps, so an L1-cached copy
@@ -429,6 +465,51 @@ __device__ __forceinline__ void phys_flux(const double* W, double g, int dir, do
   F[3] = un * (W[3] + p);
 }
 
+// Lobatto time average of the flux along dir and the state at tau = dt.  Euler: the nodes tau > 0
+// share one division (1/rho1 = rho2 rho3 / (rho1 rho2 rho3) and so on).
+template <int NC>
+__device__ __forceinline__ void lobatto(const double tc[NC][5], double dt, double g, int dir,
+                                        double Fh[NC], double We[NC]) {
+  using namespace shweno_tables;
+  const double taus[4] = {0.0, LOB_L1 * dt, LOB_L2 * dt, dt};
+  const double wts[4] = {LOB_W0, LOB_W1, LOB_W1, LOB_W0};
+  double W[4][NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) W[0][q] = tc[q][0];  // tau = 0: the leading term itself
+#pragma unroll
+  for (int al = 1; al < 4; ++al)
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const double tau = taus[al];
+      W[al][q] = (((tc[q][4] * tau + tc[q][3]) * tau + tc[q][2]) * tau + tc[q][1]) * tau + tc[q][0];
+    }
+  double ir[4] = {0.0, 0.0, 0.0, 0.0};
+  if constexpr (NC > 1) {
+    ir[0] = 1.0 / W[0][0];
+    const double r23 = W[2][0] * W[3][0];
+    const double inv = 1.0 / (W[1][0] * r23);
+    ir[1] = inv * r23;
+    const double i23 = inv * W[1][0];  // 1 / (rho2 rho3)
+    ir[2] = i23 * W[3][0];
+    ir[3] = i23 * W[2][0];
+  }
+#pragma unroll
+  for (int q = 0; q < NC; ++q) Fh[q] = 0.0;
+#pragma unroll
+  for (int al = 0; al < 4; ++al) {
+    double F[NC];
+    phys_flux_ir<NC>(W[al], ir[al], g, dir, F);
+#pragma unroll
+    for (int q = 0; q < NC; ++q) Fh[q] += wts[al] * F[q];
+  }
+#pragma unroll
+  for (int q = 0; q < NC; ++q) We[q] = W[3][q];
+}
+
+__device__ __forceinline__ double state_at(const double tc[5], double tau) {
+  return (((tc[4] * tau + tc[3]) * tau + tc[2]) * tau + tc[1]) * tau + tc[0];
+}
+
 // ------------------------------------------------------------------ linearised Riemann problem
 // Eq. (2.8) / (3.7): with A = F'(W*) = R diag(lambda) L, the derivative state is
 //   d* = R (H o L dL + (1-H) o L dR),  H = 1 / 0 / 1/2 for a right-moving / left-moving /
@@ -614,6 +695,15 @@ __device__ __forceinline__ bool cell_physical(const Params& P, const double* W) 
   const double ke = P.ncomp == 4 ? 0.5 * (W[1] * W[1] + W[2] * W[2]) / rho : 0.5 * W[1] * W[1] / rho;
   const double p = (P.gamma - 1.0) * (W[P.ncomp - 1] - ke);
   return rho > 0.0 && p > 0.0 && isfinite(rho) && isfinite(p);
+}
+
+// Both of a new state: its signal speed along x, |u| + c (Burgers: |u|), or -1 if it is not physical.
+template <int NC>
+__device__ __forceinline__ double signal_speed1d(const Params& P, const double* W) {
+  if constexpr (NC == 1) return isfinite(W[0]) ? fabs(W[0]) : -1.0;
+  const Prim s = euler_prim(W, NC, P.gamma);
+  const bool ok = s.rho > 0.0 && s.p > 0.0 && isfinite(s.rho) && isfinite(s.p);
+  return ok ? fabs(s.u) + s.c : -1.0;
 }
 
 // Block-wide max of a non-negative double, then one atomicMax on its bit pattern (the order of

@@ -20,11 +20,10 @@ struct Scratch2D {
 };
 
 // ev: NULL, or events recorded before each kernel and after the last (kernels + 1 events).
-constexpr int kKernels1D = 2;
+constexpr int kKernels1D = 1;
 constexpr int kKernels2D = 4;
 void launch_step1d(const Params& P, Ctl* ctl, const double* s0, const double* s1, double* o0,
-                   double* o1, const uint8_t* flag, double* FH, double* WE, cudaStream_t st,
-                   cudaEvent_t* ev);
+                   double* o1, const uint8_t* flag, cudaStream_t st, cudaEvent_t* ev);
 void launch_step2d(const Params& P, Ctl* ctl, const double* s0, const double* s1, double* o0,
                    double* o1, const uint8_t* flag, const Scratch2D& S, cudaStream_t st,
                    cudaEvent_t* ev);
@@ -66,7 +65,6 @@ struct HandleView {
   cudaStream_t stream;
 };
 void launch_begin_step(Ctl* ctl, cudaStream_t st);
-void launch_end_step(Ctl* ctl, cudaStream_t st);
 void launch_rate(const Params& P, Ctl* ctl, const double* s0, const double* s1, cudaStream_t st);
 
 }  // namespace shweno

@@ -1,13 +1,8 @@
-// One ADER-SHWENO time step in one space dimension (Section 2; Section 4 Steps 1-5).
-//   face1d:   one thread per interface x_{f-1/2}: SHWENO reconstruction of both neighbours
-//             (Section 2.4 reading), leading term (exact Burgers / HLLC, Eq. 2.5), linearised
-//             derivative Riemann problems (Eq. 2.8), Cauchy-Kovalevskaya (Eq. 2.6), Lobatto
-//             time quadrature of the flux (Eq. 2.9, Remark 2) and the state at t_{n+1}
-//             (Eq. 2.12, Remark 1).  Writes F-hat and W(t_{n+1}) per face.  Instantiated for
-//             reading R1 (quartic p1) and the R1' option (quintic p1).
-//   update1d: one thread per cell: Eq. (2.2) for the averages, Eq. (2.11) for the derivative
-//             averages; fused max characteristic rate of the new state (next CFL step) and the
-//             physical-state check.
+// One ADER-SHWENO time step in one space dimension (Section 2; Section 4 Steps 1-5), one kernel:
+// each warp advances W1D cells (step1d_items.cuh: SHWENO reconstruction of Section 2.4, leading
+// term of Eq. 2.5, derivative problems of Eq. 2.8, Cauchy-Kovalevskaya of Eq. 2.6, Lobatto flux of
+// Eq. 2.9 and Remark 2, the state at t_{n+1} of Eq. 2.12, updates of Eq. 2.2 and 2.11, physical
+// check and CFL rate); the last CTA ends the step and begins the next.
 #include <cuda_runtime.h>
 
 #include "shweno_kernels.h"
@@ -16,69 +11,61 @@
 namespace shweno {
 
 template <int NC, bool Q>
-__global__ void __launch_bounds__(128) face1d_kernel(Params P, const Ctl* __restrict__ ctl,
-                                                     const double* s0, const double* s1,
-                                                     const uint8_t* __restrict__ flag,
-                                                     double* __restrict__ FH,
-                                                     double* __restrict__ WE) {
+__global__ void __launch_bounds__(128, 3) step1d_kernel(Params P, Ctl* __restrict__ ctl, const double* s0,
+                                                     const double* s1, double* o0, double* o1,
+                                                     const uint8_t* __restrict__ flag) {
   if (!ctl->active) return;
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;  // face between cells f-1 and f
-  if (f > P.nx) return;
   const StepView sv = step_view(ctl);
-  double Fh[NC], We[NC];
-  face1d_point<NC, Q>(P, sv.odd ? s1 : s0, flag, f, sv.t, sv.dt, Fh, We);
-#pragma unroll
-  for (int q = 0; q < NC; ++q) {
-    FH[(size_t)q * (P.nx + 1) + f] = Fh[q];
-    WE[(size_t)q * (P.nx + 1) + f] = We[q];
+  const int c0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * W1D;
+  if (c0 < P.nx) {
+    const double speed = step1d_warp<NC, Q>(P, ctl, sv.odd ? s1 : s0, sv.odd ? o0 : o1, flag, c0,
+                                            min(W1D, P.nx - c0), sv.t, sv.dt);
+    report_speed1d(P, ctl, speed);
   }
+  __threadfence();  // each warp's report before the CTA counts as done
+  __syncthreads();
+  if (threadIdx.x == 0) ctl_commit_last(ctl, gridDim.x);
 }
 
-__global__ void __launch_bounds__(256) update1d_kernel(Params P, Ctl* __restrict__ ctl,
-                                                       const double* s0, const double* s1,
-                                                       double* o0, double* o1,
-                                                       const double* __restrict__ FH,
-                                                       const double* __restrict__ WE) {
-  __shared__ double red[32];
+template <bool Q>
+__global__ void __launch_bounds__(128) step1d_small_kernel(Params P, Ctl* __restrict__ ctl, const double* s0,
+                                                           const double* s1, double* o0, double* o1,
+                                                           const uint8_t* __restrict__ flag) {
+  __shared__ Small1D S;
   if (!ctl->active) return;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool odd = ctl->nsteps & 1;
-  const double* st = odd ? s1 : s0;
-  double* out = odd ? o0 : o1;
-  const double dt = ctl->dt;
-  const int nc = P.ncomp, N = P.nx;
-  double rate = 0.0;
-  if (j < N) {
-    double Wn[4];
-    for (int q = 0; q < nc; ++q) {
-      const size_t fo = (size_t)q * (N + 1) + j;
-      Wn[q] = st[(size_t)q * N + j] - dt / P.dx * (FH[fo + 1] - FH[fo]);
-      out[(size_t)q * N + j] = Wn[q];
-      out[(size_t)(nc + q) * N + j] = (WE[fo + 1] - WE[fo]) * P.idx;  // 1 / dx from the host
-    }
-    if (!cell_physical(P, Wn)) atomicCAS(&ctl->err, ERR_NONE, ERR_NONPHYSICAL);
-    else rate = cell_rate(P, Wn);
-  }
-  block_max_rate(rate, &ctl->rate_next, red);
+  const StepView sv = step_view(ctl);
+  const int c0 = blockIdx.x * W1D;
+  const double speed = step1d_cta<Q>(P, ctl, sv.odd ? s1 : s0, sv.odd ? o0 : o1, flag, c0, min(W1D, P.nx - c0),
+                                     sv.t, sv.dt, S);
+  if (threadIdx.x >= 32) return;  // the first warp updated the cells
+  report_speed1d(P, ctl, speed);
+  __syncwarp();
+  if (threadIdx.x == 0) ctl_commit_last(ctl, gridDim.x);
 }
 
 void launch_step1d(const Params& P, Ctl* ctl, const double* s0, const double* s1, double* o0,
-                   double* o1, const uint8_t* flag, double* FH, double* WE, cudaStream_t st,
-                   cudaEvent_t* ev) {
-  const int nf = P.nx + 1;
-  const int b = 128;
+                   double* o1, const uint8_t* flag, cudaStream_t st, cudaEvent_t* ev) {
+  const int warps = (P.nx + W1D - 1) / W1D;
   if (ev) cudaEventRecord(ev[0], st);
-  const dim3 g((nf + b - 1) / b);
-  if (P.ncomp == 1) {
-    if (P.quintic) face1d_kernel<1, true><<<g, b, 0, st>>>(P, ctl, s0, s1, flag, FH, WE);
-    else face1d_kernel<1, false><<<g, b, 0, st>>>(P, ctl, s0, s1, flag, FH, WE);
+  if (P.ncomp == 3 && !P.charwise && warps <= 152) {
+    // one CTA of four warps per SM and W1D cells: the latency of one chain of FP64 instructions is
+    // all there is, so it is shortened
+    if (P.quintic) step1d_small_kernel<true><<<warps, 128, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);
+    else step1d_small_kernel<false><<<warps, 128, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);
   } else {
-    if (P.quintic) face1d_kernel<3, true><<<g, b, 0, st>>>(P, ctl, s0, s1, flag, FH, WE);
-    else face1d_kernel<3, false><<<g, b, 0, st>>>(P, ctl, s0, s1, flag, FH, WE);
+    // One warp per CTA while the mesh does not fill the GPU: the CTAs then go to different SMs, each
+    // warp has a scheduler's FP64 unit to itself.  From 152 SMs x 4 schedulers x 2 warps on, four.
+    const int per = warps < 1216 ? 1 : 4;
+    const dim3 g((warps + per - 1) / per), b(32 * per);
+    if (P.ncomp == 1) {
+      if (P.quintic) step1d_kernel<1, true><<<g, b, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);
+      else step1d_kernel<1, false><<<g, b, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);
+    } else {
+      if (P.quintic) step1d_kernel<3, true><<<g, b, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);
+      else step1d_kernel<3, false><<<g, b, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);
+    }
   }
   if (ev) cudaEventRecord(ev[1], st);
-  update1d_kernel<<<(P.nx + 255) / 256, 256, 0, st>>>(P, ctl, s0, s1, o0, o1, FH, WE);
-  if (ev) cudaEventRecord(ev[2], st);
 }
 
 }  // namespace shweno

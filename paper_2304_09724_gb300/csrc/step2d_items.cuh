@@ -564,51 +564,6 @@ __device__ __forceinline__ void char_face_point(const Params& P, const double (*
   lead = U.lead;
 }
 
-// Lobatto time average of the flux along dir and the state at tau = dt.  Euler: the nodes tau > 0
-// share one division (1/rho1 = rho2 rho3 / (rho1 rho2 rho3) and so on).
-template <int NC>
-__device__ __forceinline__ void lobatto(const double tc[NC][5], double dt, double g, int dir,
-                                        double Fh[NC], double We[NC]) {
-  using namespace shweno_tables;
-  const double taus[4] = {0.0, LOB_L1 * dt, LOB_L2 * dt, dt};
-  const double wts[4] = {LOB_W0, LOB_W1, LOB_W1, LOB_W0};
-  double W[4][NC];
-#pragma unroll
-  for (int q = 0; q < NC; ++q) W[0][q] = tc[q][0];  // tau = 0: the leading term itself
-#pragma unroll
-  for (int al = 1; al < 4; ++al)
-#pragma unroll
-    for (int q = 0; q < NC; ++q) {
-      const double tau = taus[al];
-      W[al][q] = (((tc[q][4] * tau + tc[q][3]) * tau + tc[q][2]) * tau + tc[q][1]) * tau + tc[q][0];
-    }
-  double ir[4] = {0.0, 0.0, 0.0, 0.0};
-  if constexpr (NC > 1) {
-    ir[0] = 1.0 / W[0][0];
-    const double r23 = W[2][0] * W[3][0];
-    const double inv = 1.0 / (W[1][0] * r23);
-    ir[1] = inv * r23;
-    const double i23 = inv * W[1][0];  // 1 / (rho2 rho3)
-    ir[2] = i23 * W[3][0];
-    ir[3] = i23 * W[2][0];
-  }
-#pragma unroll
-  for (int q = 0; q < NC; ++q) Fh[q] = 0.0;
-#pragma unroll
-  for (int al = 0; al < 4; ++al) {
-    double F[NC];
-    phys_flux_ir<NC>(W[al], ir[al], g, dir, F);
-#pragma unroll
-    for (int q = 0; q < NC; ++q) Fh[q] += wts[al] * F[q];
-  }
-#pragma unroll
-  for (int q = 0; q < NC; ++q) We[q] = W[3][q];
-}
-
-__device__ __forceinline__ double state_at(const double tc[5], double tau) {
-  return (((tc[4] * tau + tc[3]) * tau + tc[2]) * tau + tc[1]) * tau + tc[0];
-}
-
 // Combined coefficients C[u] of NU = 1 or 2 components of one cell from their stencil averages
 // w[u] = (W-, W0, W+) and p1 coefficients c[u] (C = c for a cell with the linear weights).  PAIR
 // (Euler, reading R1): the two components' weights share one division, 1/S0 = S1 / (S0 S1) and
@@ -925,6 +880,7 @@ __device__ __forceinline__ double update2d_cell(const Params& P, Ctl* __restrict
   }
   if (!cell_physical(P, Wn)) {
     atomicCAS(&ctl->err, ERR_NONE, ERR_NONPHYSICAL);
+    __threadfence();  // before this CTA counts as done
     return 0.0;
   }
   return cell_rate(P, Wn);

@@ -89,7 +89,8 @@ __global__ void __launch_bounds__(256) update2d_kernel(Params P, Ctl* __restrict
   const StepView sv = step_view(ctl);
   double rate = 0.0;
   if (i < P.nx && j < P.ny) rate = update2d_cell<NC>(P, ctl, sv, sv.odd ? s1 : s0, sv.odd ? o0 : o1, FX, WX, FY, WY, WC, i, j);
-  block_max_rate(rate, &ctl->rate_next, red);
+  block_max_rate(rate, &ctl->rate_next, red);  // holds a barrier: every cell's error has been raised
+  if (threadIdx.x == 0 && threadIdx.y == 0) ctl_commit_last(ctl, gridDim.x * gridDim.y);
 }
 
 // ------------------------------------------------------------------ host side (templates)
