@@ -319,6 +319,10 @@ shweno_status shweno_create(const shweno_grid* grid, double gamma, const shweno_
     h->scratch = (double*)dev_alloc(shweno::scratch2d_doubles(P) * sizeof(double));
     if (!h->scratch) return bail(SHWENO_E_NOMEM, "device allocation of the step scratch failed");
     h->S = shweno::carve_scratch2d(P, h->scratch);
+    if (cudaStreamCreateWithFlags(&h->S.aux, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->S.fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->S.join, cudaEventDisableTiming) != cudaSuccess)
+      return bail(SHWENO_E_CUDA, "creating the handle's second stream failed");
     const cudaError_t ea = shweno::init_kernels2d();
     if (ea != cudaSuccess) {
       cudaGetLastError();
@@ -346,6 +350,9 @@ shweno_status shweno_destroy(shweno_handle* h) {
   if (!h) return SHWENO_OK;
   if (h->stream) cudaStreamSynchronize(h->stream);
   if (h->graph) cudaGraphExecDestroy(h->graph);
+  if (h->S.aux) cudaStreamDestroy(h->S.aux);  // its work is joined into the handle's stream
+  if (h->S.fork) cudaEventDestroy(h->S.fork);
+  if (h->S.join) cudaEventDestroy(h->S.join);
   for (int b = 0; b < 2; ++b) dev_free(h->buf[b]);
   dev_free(h->scratch);
   dev_free(h->flags);

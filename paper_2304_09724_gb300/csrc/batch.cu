@@ -50,7 +50,7 @@ struct BatchProblem {
   int32_t phase_kind[5];
   int32_t nitems[5];
   int32_t tile1d;
-  int32_t nsegx, nsegy, ncx, ncy, nsegu, nxitems;
+  int32_t nxs, nys, ncx, ncy, nsegu, nxitems;  // nxs, nys: face CTAs of a Gauss slice
   int64_t max_steps;  // stop after this many committed steps (in this run)
   int64_t step0;      // committed steps at the start of the run
 };
@@ -63,8 +63,8 @@ struct BatchCtl {
 };
 
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
-// the largest item: a face segment or a first-pass tile (16 fields with halo); 1D tiles need none
-constexpr size_t kBatchSmem = cmax(face_smem<4>(), sizeof(double) * 16 * (TYB + 2) * (TX + 2));
+// the largest item: a face segment or a first-pass tile (8 fields with halo); 1D tiles need none
+constexpr size_t kBatchSmem = cmax(face_smem<4>(), sizeof(double) * 8 * (TYB + 2) * (TX + 2));
 
 __device__ __forceinline__ long long enc(int p, int ph, long long idx) {
   return ((long long)p << 40) | ((long long)ph << 36) | idx;
@@ -166,41 +166,37 @@ __device__ __forceinline__ void item_body(const BatchProblem& B, int kind, long 
       break;
     }
     case PH_COEF: {
-      const int bxi = (int)(idx % B.ncx), byi = (int)(idx / B.ncx);
+      const int tile_idx = (int)(idx >> 2), unit = (int)(idx & 3);
+      const int bxi = tile_idx % B.ncx, byi = tile_idx / B.ncx;
       auto tile = reinterpret_cast<double(*)[TYB + 2][TX + 2]>(smem);
       if (P.ncomp == 1)
-        coef2d_item<1, TYB>(P, sv, B.s0, B.s1, B.flag, B.S.ycoef, B.S.xcoef, bxi * TX - 2, byi * TYB - 2,
+        coef2d_item<1, TYB>(P, sv, B.s0, B.s1, B.flag, B.S.ycoef, B.S.xcoef, unit, bxi * TX - 2, byi * TYB - 2,
                             tile, threadIdx.x % TX, threadIdx.x / TX);
       else
-        coef2d_item<4, TYB>(P, sv, B.s0, B.s1, B.flag, B.S.ycoef, B.S.xcoef, bxi * TX - 2, byi * TYB - 2,
+        coef2d_item<4, TYB>(P, sv, B.s0, B.s1, B.flag, B.S.ycoef, B.S.xcoef, unit, bxi * TX - 2, byi * TYB - 2,
                             tile, threadIdx.x % TX, threadIdx.x / TX);
       break;
     }
     case PH_FACE: {
       const bool flags = P.flag_mode != FLAG_ALL_NONLINEAR;
       if (idx < B.nxitems) {
-        const int seg = (int)(idx % B.nsegx), r = (int)(idx / B.nsegx);
-        const int slice = r < 3 * P.ny ? r / P.ny : 3;
-        const int row = r < 3 * P.ny ? r % P.ny : r - 3 * P.ny;
-        const int f0 = seg * NFACE;
+        const int slice = (int)(idx / B.nxs) < 3 ? (int)(idx / B.nxs) : 3;
+        const int c = (int)idx - slice * B.nxs;
         if (P.ncomp == 1) {
-          if (flags) xface_item<1, true>(P, sv, sv.odd ? B.s1 : B.s0, B.S.ycoef, B.flag, B.S.FX, B.S.WX, B.S.WC, f0, row, slice, smem);
-          else xface_item<1, false>(P, sv, sv.odd ? B.s1 : B.s0, B.S.ycoef, B.flag, B.S.FX, B.S.WX, B.S.WC, f0, row, slice, smem);
+          if (flags) xface_item<1, true>(P, sv, sv.odd ? B.s1 : B.s0, B.S.ycoef, B.flag, B.S.FX, B.S.WX, B.S.WC, c, slice, smem);
+          else xface_item<1, false>(P, sv, sv.odd ? B.s1 : B.s0, B.S.ycoef, B.flag, B.S.FX, B.S.WX, B.S.WC, c, slice, smem);
         } else {
-          if (flags) xface_item<4, true>(P, sv, sv.odd ? B.s1 : B.s0, B.S.ycoef, B.flag, B.S.FX, B.S.WX, B.S.WC, f0, row, slice, smem);
-          else xface_item<4, false>(P, sv, sv.odd ? B.s1 : B.s0, B.S.ycoef, B.flag, B.S.FX, B.S.WX, B.S.WC, f0, row, slice, smem);
+          if (flags) xface_item<4, true>(P, sv, sv.odd ? B.s1 : B.s0, B.S.ycoef, B.flag, B.S.FX, B.S.WX, B.S.WC, c, slice, smem);
+          else xface_item<4, false>(P, sv, sv.odd ? B.s1 : B.s0, B.S.ycoef, B.flag, B.S.FX, B.S.WX, B.S.WC, c, slice, smem);
         }
       } else {
-        const long long k = idx - B.nxitems;
-        const int seg = (int)(k % B.nsegy), r = (int)(k / B.nsegy);
-        const int slice = r / P.nx, col = r % P.nx;
-        const int f0 = seg * NFACE;
+        const int k = (int)idx - B.nxitems, slice = k / B.nys, c = k % B.nys;
         if (P.ncomp == 1) {
-          if (flags) yface_item<1, true>(P, sv, sv.odd ? B.s1 : B.s0, B.S.xcoef, B.flag, B.S.FY, B.S.WY, f0, col, slice, smem);
-          else yface_item<1, false>(P, sv, sv.odd ? B.s1 : B.s0, B.S.xcoef, B.flag, B.S.FY, B.S.WY, f0, col, slice, smem);
+          if (flags) yface_item<1, true>(P, sv, sv.odd ? B.s1 : B.s0, B.S.xcoef, B.flag, B.S.FY, B.S.WY, c, slice, smem);
+          else yface_item<1, false>(P, sv, sv.odd ? B.s1 : B.s0, B.S.xcoef, B.flag, B.S.FY, B.S.WY, c, slice, smem);
         } else {
-          if (flags) yface_item<4, true>(P, sv, sv.odd ? B.s1 : B.s0, B.S.xcoef, B.flag, B.S.FY, B.S.WY, f0, col, slice, smem);
-          else yface_item<4, false>(P, sv, sv.odd ? B.s1 : B.s0, B.S.xcoef, B.flag, B.S.FY, B.S.WY, f0, col, slice, smem);
+          if (flags) yface_item<4, true>(P, sv, sv.odd ? B.s1 : B.s0, B.S.xcoef, B.flag, B.S.FY, B.S.WY, c, slice, smem);
+          else yface_item<4, false>(P, sv, sv.odd ? B.s1 : B.s0, B.S.xcoef, B.flag, B.S.FY, B.S.WY, c, slice, smem);
         }
       }
       break;
@@ -463,17 +459,17 @@ void fill_problem(shweno_batch* b, int p) {
     const int cells_items = (int)(((size_t)nx * ny + BT - 1) / BT);
     B.ncx = (nx + 4 + TX - 1) / TX;
     B.ncy = (ny + 4 + TYB - 1) / TYB;
-    B.nsegx = (nx + 1 + NFACE - 1) / NFACE;
-    B.nsegy = (ny + 1 + NFACE - 1) / NFACE;
+    B.nxs = FaceSplit(nx + 1).ctas(ny);
+    B.nys = FaceSplit(ny + 1).ctas(nx);
     B.nsegu = (nx + BT - 1) / BT;
-    B.nxitems = B.nsegx * (3 * ny + ny + 1);
+    B.nxitems = 3 * B.nxs + FaceSplit(nx + 1).ctas(ny + 1);
     int k = 0;
     if (v.learned) {
       B.phase_kind[k] = PH_INFER; B.nitems[k++] = cells_items;
       B.phase_kind[k] = PH_DILATE; B.nitems[k++] = cells_items;
     }
-    B.phase_kind[k] = PH_COEF; B.nitems[k++] = B.ncx * B.ncy;
-    B.phase_kind[k] = PH_FACE; B.nitems[k++] = B.nxitems + B.nsegy * nx * 3;
+    B.phase_kind[k] = PH_COEF; B.nitems[k++] = 4 * B.ncx * B.ncy;
+    B.phase_kind[k] = PH_FACE; B.nitems[k++] = B.nxitems + 3 * B.nys;
     B.phase_kind[k] = PH_UPDATE; B.nitems[k++] = B.nsegu * ny;
     B.nphase = k;
   }
@@ -663,7 +659,7 @@ size_t lock_smem(const shweno_batch* b, int kind) {
   using namespace shweno;
   switch (kind) {
     case PH_INFER: return sizeof(float) * NPARAM;
-    case PH_COEF: return sizeof(double) * 16 * (TYB + 2) * (TX + 2);
+    case PH_COEF: return sizeof(double) * 8 * (TYB + 2) * (TX + 2);
     case PH_FACE: return face_smem<4>();
     default: return 0;
   }

@@ -17,6 +17,10 @@ struct Scratch2D {
   double* FY;     // [3 gauss][ncomp][ny+1][nx]
   double* WY;     // [3 gauss][ncomp][ny+1][nx]
   double* WC;     // [ncomp][ny+1][nx+1]          state at t_{n+1} at cell corners
+  // host side: a second stream of the handle for independent kernels of a small mesh, and the
+  // events that fork it off and join it (NULL: none)
+  cudaStream_t aux = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
 };
 
 // ev: NULL, or events recorded before each kernel and after the last (kernels + 1 events).

@@ -6,9 +6,42 @@
 namespace shweno {
 
 constexpr int SEG = 128;          // threads of a face CTA
-constexpr int NFACE = SEG - 1;    // faces of a face CTA: its threads own the SEG cells next to them
-constexpr int SPAN = NFACE + 3;   // first-pass evaluations a CTA needs
+constexpr int NFACE = SEG - 1;    // most faces of a face CTA: its threads own the SEG cells next to them
+constexpr int SPAN = 144;         // first-pass evaluations a CTA has room for
 constexpr int TX = 32;            // first-pass tile width
+
+// ------------------------------------------------------------------ the faces of a CTA
+// A line of n faces is cut into segments of NFACE faces, one CTA each; what remains of the lines
+// (rem faces each) goes together, per lines to a CTA, so that short lines and ragged ends fill
+// their warps too (an FP64 instruction costs a warp the same for one lane as for 32; 401 faces:
+// 3 segments and 20 faces that had a CTA and two CTA slots' worth of waiting to themselves).
+// A CTA's faces are runs of nf faces on nrun neighbouring lines; thread t owns the cell
+// t % (nf + 1) of run t / (nf + 1) and, but for the last cell of a run, the face right of it.
+struct FaceSplit {
+  int nfull, rem, per;
+  __host__ __device__ explicit FaceSplit(int n) : nfull(n / NFACE), rem(n % NFACE), per(1) {
+    if (rem > 0) per = SEG / (rem + 1) < SPAN / (rem + 3) ? SEG / (rem + 1) : SPAN / (rem + 3);
+  }
+  __host__ __device__ int ctas(int lines) const { return nfull * lines + (rem > 0 ? (lines + per - 1) / per : 0); }
+};
+struct FaceRuns {
+  int f0, nf, line, nrun;  // first face, faces per run, first line, runs
+  int run, ct, col;        // this thread's run, cell in it and stencil column (run * (nf + 3) + ct + 1)
+  bool has_cell, has_face;
+  __device__ __forceinline__ FaceRuns(int n, int lines, int b) {
+    const FaceSplit S(n);
+    if (b < S.nfull * lines) {
+      line = b / S.nfull; f0 = (b % S.nfull) * NFACE; nf = NFACE; nrun = 1;
+    } else {
+      line = (b - S.nfull * lines) * S.per; f0 = S.nfull * NFACE; nf = S.rem; nrun = min(S.per, lines - line);
+    }
+    run = threadIdx.x / (nf + 1);
+    ct = threadIdx.x % (nf + 1);
+    col = run * (nf + 3) + ct + 1;
+    has_cell = run < nrun;
+    has_face = has_cell && ct < nf;
+  }
+};
 
 // ------------------------------------------------------------------ second pass, cell by cell
 // Second pass across the face.  ev[set*NC+q][k][col] holds the first-pass Taylor coefficients
@@ -20,10 +53,11 @@ constexpr int TX = 32;            // first-pass tile width
 // end.  The two ends of a cell share their arithmetic: with s = W- + W+, a = W+ - W-,
 // dv = v+ - v-, sv = v- + v+, p1's coefficient p at xi = +-1/2 is U_p + V_p and (-1)^p (U_p - V_p)
 // (U_p from the even monomials, V_p from the odd ones; end_u / end_v of recon_tables.cuh).
+template <int NC>
 struct EndTable {
   // left ends (xi = -1/2) of the cells, two buffers (orders of even / odd K) so that one barrier
-  // per order suffices: [buffer][comp][p][slot], the cell in column c at slot c - 1
-  double L[2][4][5][SEG];
+  // per order suffices: [buffer][comp][p][slot], the cell of thread t at slot t
+  double L[2][NC][5][SEG];
 };
 // Flags of the cells next to the faces, for the characteristic-wise path (whose weights belong to
 // each face point): lin[c] = 1 when the cell in column c uses the linear weights.
@@ -31,8 +65,12 @@ struct FlagTable {
   int lin[SPAN];
 };
 
-constexpr size_t kEvBytes = sizeof(double) * 8 * 5 * SPAN;
-constexpr size_t kFaceSmem = kEvBytes + (sizeof(EndTable) > sizeof(FlagTable) ? sizeof(EndTable) : sizeof(FlagTable));
+template <int NC>
+constexpr size_t ev_bytes() { return sizeof(double) * 2 * NC * 5 * SPAN; }
+template <int NC>
+constexpr size_t table_bytes() {
+  return ev_bytes<NC>() + (sizeof(EndTable<NC>) > sizeof(FlagTable) ? sizeof(EndTable<NC>) : sizeof(FlagTable));
+}
 
 // Weights of one cell's reconstruction across the face: p = A p1 + B p2 + C p3 per component.
 template <int NC>
@@ -87,13 +125,13 @@ __device__ __forceinline__ void cell_mix(const Params& P, const double (*ev)[5][
 }
 
 // Taylor coefficients p = 0..4-K across the face of tangential order K at both ends of the cell in
-// column c, into slot c - 1 of the EndTable.  The small stencils p2 = W0 + (W0 - W-) xi and
+// column c, into the thread's slot of the EndTable.  The small stencils p2 = W0 + (W0 - W-) xi and
 // p3 = W0 + (W+ - W0) xi add h +- g/2 to the value and g to the slope at the ends, with
 // h = (B + C) W0 and g = B (W0 - W-) + C (W+ - W0).  LIN: a cell with the linear weights (p = p1,
 // A = 1, B = C = 0; the general form gives the same values bit for bit with more operations).
 template <int NC, bool LIN, bool Q, int K>
 __device__ __forceinline__ void cell_ends_t(const double (*ev)[5][SPAN], int c, const CellMix<NC>& m,
-                                            EndTable& et, double eRo[NC][5]) {
+                                            EndTable<NC>& et, double eRo[NC][5]) {
   using namespace shweno_tables;
 #pragma unroll
   for (int q = 0; q < NC; ++q) {
@@ -133,24 +171,24 @@ __device__ __forceinline__ void cell_ends_t(const double (*ev)[5][SPAN], int c, 
         }
       }
       eRo[q][p] = eR;
-      et.L[K & 1][q][p][c - 1] = eL;
+      et.L[K & 1][q][p][threadIdx.x] = eL;
     }
   }
 }
 // FLAGS = false: every cell is nonlinear (no branch on the flag); otherwise one branch per cell.
 template <int NC, bool FLAGS, bool Q, int K>
 __device__ __forceinline__ void cell_ends(const double (*ev)[5][SPAN], int c, const CellMix<NC>& m,
-                                          EndTable& et, double eR[NC][5]) {
+                                          EndTable<NC>& et, double eR[NC][5]) {
   if (FLAGS && m.lin) cell_ends_t<NC, true, Q, K>(ev, c, m, et, eR);
   else cell_ends_t<NC, false, Q, K>(ev, c, m, et, eR);
 }
 
-// Order K of the face point between cell columns f + 1 and f + 2: the two sides from the
+// Order K of the face point of thread f (its cell and thread f + 1's): the two sides from the
 // EndTable; at K = 0 the leading term (Burgers: exact Godunov state; Euler: HLLC) and the
 // eigen-decomposition of the upwinding; every derivative vector upwinded into a[q][m*5+n]
 // (m along x, n along y; dir = 0: x-face, p across = m; dir = 1: y-face, p across = n).
 template <int NC, int K>
-__device__ __forceinline__ void face_order(const Params& P, const EndTable& et, const double eR[NC][5], int f,
+__device__ __forceinline__ void face_order(const Params& P, const EndTable<NC>& et, const double eR[NC][5], int f,
                                            int dir, double Ws[NC], Upwinder<NC>& U, double a[NC][25]) {
   double dr[NC][5];
 #pragma unroll
@@ -183,13 +221,13 @@ __device__ __forceinline__ void face_order(const Params& P, const EndTable& et, 
 // against the next cell's left end.  The next order writes the other buffer, so a thread still
 // reading this one cannot be overtaken.  Called by all threads of the CTA (it holds the barrier).
 template <int NC, bool FLAGS, bool Q, int K>
-__device__ __forceinline__ void pass_order(const Params& P, const double (*ev)[5][SPAN], EndTable& et,
-                                           bool has_cell, const CellMix<NC>& m, bool has_face,
+__device__ __forceinline__ void pass_order(const Params& P, const double (*ev)[5][SPAN], EndTable<NC>& et,
+                                           const FaceRuns& fr, const CellMix<NC>& m,
                                            int dir, double Ws[NC], Upwinder<NC>& U, double a[NC][25]) {
   double eR[NC][5];
-  if (has_cell) cell_ends<NC, FLAGS, Q, K>(ev, threadIdx.x + 1, m, et, eR);
+  if (fr.has_cell) cell_ends<NC, FLAGS, Q, K>(ev, fr.col, m, et, eR);
   __syncthreads();
-  if (has_face) face_order<NC, K>(P, et, eR, threadIdx.x, dir, Ws, U, a);
+  if (fr.has_face) face_order<NC, K>(P, et, eR, threadIdx.x, dir, Ws, U, a);
 }
 
 // ------------------------------------------------------------------ Cauchy-Kovalevskaya of the points
@@ -212,7 +250,7 @@ constexpr size_t kCkBytes = kCkGrow + SEG * 4;
 
 template <int NC>
 constexpr size_t face_smem() {
-  return NC == 4 && kCkBytes > kFaceSmem ? kCkBytes : kFaceSmem;
+  return NC == 4 && kCkBytes > table_bytes<NC>() ? kCkBytes : table_bytes<NC>();
 }
 
 __host__ __device__ constexpr int ck_pair(int i, int j) { return (i + j) * (i + j + 1) / 2 + j; }
@@ -329,10 +367,11 @@ static __device__ __noinline__ void ck_warp_euler2d(int half, int p0, int valid,
   }
 }
 
-// Time-Taylor coefficients per unit L^k (P.ck.iL = 1 / L) of the CTA's nf points from their spatial
-// ones; called by every thread after the barrier that ends the use of the tables.
+// Time-Taylor coefficients per unit L^k (P.ck.iL = 1 / L) of the CTA's points (threads 0 .. npt - 1, those
+// with has_face) from their spatial ones; called by every thread after the barrier that ends the use
+// of the tables.
 template <int NC>
-__device__ __forceinline__ void ck_points(const Params& P, int nf, bool has_face, double (&a)[NC][25],
+__device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_face, double (&a)[NC][25],
                                           const CkLead& lead, double (&tc)[NC][5]) {
   if (P.ck.rx != P.ck.ry) {  // dx != dy: both coordinates in units of L
     double fx = 1.0;
@@ -368,12 +407,16 @@ __device__ __forceinline__ void ck_points(const Params& P, int nf, bool has_face
       *reinterpret_cast<int*>(dyn_smem + kCkGrow + tid * 4) = 0;
 #pragma unroll
       for (int q = 0; q < NC; ++q) tc[q][0] = a[q][0];
+    } else if (tid < npt) {  // the last cell of a run: zeros stay zeros
+#pragma unroll 1
+      for (int k = 0; k < 60; ++k) ck_st(col + k * kCkRow, Fx{0, 0});
+      ck_st(kCkNinv + tid * 8, Fx{0, 0});
     }
     __syncthreads();
     const int p0 = (tid >> 5) * 16;
 #pragma unroll 1
-    for (int half = 0; half * CKP < nf; ++half) {
-      const int valid = nf - half * CKP - p0;
+    for (int half = 0; half * CKP < npt; ++half) {
+      const int valid = npt - half * CKP - p0;
       if (valid > 0) ck_warp_euler2d(half, p0, valid, P.ck.K.third, P.ck.K.gm1, P.ck.K.gshift);
       __syncwarp();
     }
@@ -390,31 +433,28 @@ __device__ __forceinline__ void ck_points(const Params& P, int nf, bool has_face
   }
 }
 
-// Second pass, leading term, upwinding and CK of the nf faces of a CTA (nf <= NFACE): thread t
-// owns the cell in column t + 1 (t <= nf) and the face between columns t + 1 and t + 2 (t < nf).
-// Returns true for a face thread, whose tc[q][0..4] are then the time-Taylor coefficients of its
-// face point per L^k.  nl(c): whether the cell in column c uses the nonlinear weights.
-template <int NC, bool FLAGS, bool Q, typename FlagOf>
-__device__ __forceinline__ bool second_pass_cells(const Params& P, unsigned char* smem_raw, int nf, int dir,
-                                                  FlagOf nl, double (&tc)[NC][5]) {
+// Second pass, leading term, upwinding and CK of the CTA's faces.  A thread with a face gets in
+// tc[q][0..4] the time-Taylor coefficients of its face point per L^k.  nl: whether the thread's cell
+// uses the nonlinear weights.
+template <int NC, bool FLAGS, bool Q>
+__device__ __forceinline__ void second_pass_cells(const Params& P, unsigned char* smem_raw, const FaceRuns& fr, int dir,
+                                                  bool nl, double (&tc)[NC][5]) {
   const double(*ev)[5][SPAN] = reinterpret_cast<const double(*)[5][SPAN]>(smem_raw);
-  EndTable& et = *reinterpret_cast<EndTable*>(smem_raw + kEvBytes);
-  const bool has_cell = (int)threadIdx.x <= nf, has_face = (int)threadIdx.x < nf;
+  EndTable<NC>& et = *reinterpret_cast<EndTable<NC>*>(smem_raw + ev_bytes<NC>());
   CellMix<NC> m;
-  if (has_cell) cell_mix<NC, Q>(P, ev, threadIdx.x + 1, FLAGS && !nl(threadIdx.x + 1), m);
+  if (fr.has_cell) cell_mix<NC, Q>(P, ev, fr.col, FLAGS && !nl, m);
   double a[NC][25], Ws[NC];
   Upwinder<NC> U;
-  pass_order<NC, FLAGS, Q, 0>(P, ev, et, has_cell, m, has_face, dir, Ws, U, a);
-  pass_order<NC, FLAGS, Q, 1>(P, ev, et, has_cell, m, has_face, dir, Ws, U, a);
-  pass_order<NC, FLAGS, Q, 2>(P, ev, et, has_cell, m, has_face, dir, Ws, U, a);
-  pass_order<NC, FLAGS, Q, 3>(P, ev, et, has_cell, m, has_face, dir, Ws, U, a);
-  pass_order<NC, FLAGS, Q, 4>(P, ev, et, has_cell, m, has_face, dir, Ws, U, a);
+  pass_order<NC, FLAGS, Q, 0>(P, ev, et, fr, m, dir, Ws, U, a);
+  pass_order<NC, FLAGS, Q, 1>(P, ev, et, fr, m, dir, Ws, U, a);
+  pass_order<NC, FLAGS, Q, 2>(P, ev, et, fr, m, dir, Ws, U, a);
+  pass_order<NC, FLAGS, Q, 3>(P, ev, et, fr, m, dir, Ws, U, a);
+  pass_order<NC, FLAGS, Q, 4>(P, ev, et, fr, m, dir, Ws, U, a);
   __syncthreads();  // the tables are read no more
-  if (has_face)
+  if (fr.has_face)
 #pragma unroll
     for (int q = 0; q < NC; ++q) a[q][0] = Ws[q];
-  ck_points<NC>(P, nf, has_face, a, U.lead, tc);
-  return has_face;
+  ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, a, U.lead, tc);
 }
 
 // ------------------------------------------------------------------ characteristic-wise face point
@@ -590,105 +630,86 @@ __device__ __forceinline__ void first_pass_mix(const Params& P, int nl, const do
   }
 }
 
-// First-pass polynomials of the cells of one tile: thread (tx, ty) of a TX x TYB block owns the
-// extended cell (bx + tx, by + ty); the 4 * NC fields of the tile plus a one-cell halo are staged
-// in shared memory `tile` (room for 16) by all nthreads threads first.  Q: reading R1', whose
-// quintic p1 also uses the cell's own derivative average; it stores six coefficients per
-// polynomial instead of five (the scratch layout's KC).
+// First-pass polynomials of the cells of one tile, one of the four reconstructions (unit 0: y-pass
+// on {W, Y}, 1: y-pass on {V, Z}, 2: x-pass on {W, V}, 3: x-pass on {Y, Z}): thread (tx, ty) of a
+// TX x TYB block owns the extended cell (bx + tx, by + ty); the unit's 2 * NC fields of the tile plus a
+// one-cell halo are staged in shared memory `tile` (room for 8) by all threads first.  The units are
+// independent, so a small mesh spreads over four times as many CTAs (40^2 cells: 104 -> 30 us) and a
+// large one runs more warps per SM.  Q: reading R1', whose quintic p1 also uses the cell's own
+// derivative average; it stores six coefficients per polynomial instead of five (the scratch
+// layout's KC).
 template <int NC, int TYB, bool Q = false>
 __device__ __forceinline__ void coef2d_item(const Params& P, const StepView& sv, const double* s0,
                                             const double* s1, const uint8_t* __restrict__ flag,
-                                            double* __restrict__ ycoef, double* __restrict__ xcoef,
+                                            double* __restrict__ ycoef, double* __restrict__ xcoef, int unit,
                                             int bx, int by, double (*tile)[TYB + 2][TX + 2], int tx,
                                             int ty) {
   const double* st = sv.odd ? s1 : s0;
   const double t = sv.t;
+  const bool ypass = unit < 2;
+  const int s = unit & 1;
+  const int fa = s == 0 ? 0 : (ypass ? 1 : 2), fd = s == 1 ? 3 : (ypass ? 2 : 1);
   const int tid = ty * TX + tx;
-  for (int idx = tid; idx < 4 * NC * (TYB + 2) * (TX + 2); idx += TX * TYB) {
+  for (int idx = tid; idx < 2 * NC * (TYB + 2) * (TX + 2); idx += TX * TYB) {
     const int xx = idx % (TX + 2), rest = idx / (TX + 2);
     const int yy = rest % (TYB + 2), fq = rest / (TYB + 2);
     const int i = bx - 1 + xx, j = by - 1 + yy;
     double v = 0.0;
-    if (i >= -3 && i <= P.nx + 2 && j >= -3 && j <= P.ny + 2) v = fetch(P, st, fq / NC, fq % NC, i, j, t);
+    if (i >= -3 && i <= P.nx + 2 && j >= -3 && j <= P.ny + 2) v = fetch(P, st, fq < NC ? fa : fd, fq % NC, i, j, t);
     tile[fq][yy][xx] = v;
   }
   __syncthreads();
   const int ic = bx + tx, jr = by + ty;
+  if (ypass ? !(ic <= P.nx + 1 && jr >= -1 && jr <= P.ny) : !(ic >= 0 && ic < P.nx && jr <= P.ny + 1)) return;
   const int lx = tx + 1, ly = ty + 1;
-  const int NX4 = P.nx + 4, NY2 = P.ny + 2, NY4 = P.ny + 4;
+  const int dx = ypass ? 0 : 1, dy = ypass ? 1 : 0;
   constexpr int KC = Q ? 6 : 5;
   constexpr bool PAIR = NC == 4 && !Q;
   constexpr int NU = PAIR ? 2 : 1;
-  if (ic <= P.nx + 1 && jr >= -1 && jr <= P.ny) {  // y-pass: {W,Y} and {V,Z} along a column
-    const int nl = cell_flag(P, flag, ic, jr);
+  const int nl = cell_flag(P, flag, ic, jr);
+  const double h = ypass ? P.dy : P.dx;
+  const double sc = s == 0 ? 1.0 : (ypass ? P.dx : P.dy);  // derivative data of the pass across: h avg
+  const size_t NX4 = P.nx + 4, NY2 = P.ny + 2, NY4 = P.ny + 4;
+  double* out = ypass ? ycoef + (size_t)(jr + 1) * NX4 + (ic + 2) : xcoef + (size_t)ic * NY4 + (jr + 2);
+  const size_t plane = ypass ? NY2 * NX4 : (size_t)P.nx * NY4;
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
+  for (int q0 = 0; q0 < NC; q0 += NU) {
+    double w[NU][3], c[NU][6], C[NU][6];
 #pragma unroll
-      for (int q0 = 0; q0 < NC; q0 += NU) {
-        double w[NU][3], c[NU][6], C[NU][6];
+    for (int u = 0; u < NU; ++u) {
+      const int q = q0 + u;
+      w[u][0] = tile[q][ly - dy][lx - dx]; w[u][1] = tile[q][ly][lx]; w[u][2] = tile[q][ly + dy][lx + dx];
+      const double vm = h * tile[NC + q][ly - dy][lx - dx], vp = h * tile[NC + q][ly + dy][lx + dx];
+      const double v0 = Q ? h * tile[NC + q][ly][lx] : 0.0;
+      p1_coeffs_t<Q>(w[u][0], w[u][1], w[u][2], vm, v0, vp, c[u]);
+    }
+    first_pass_mix<Q, PAIR>(P, nl, w, c, C);
 #pragma unroll
-        for (int u = 0; u < NU; ++u) {
-          const int fa = (s == 0 ? 0 : 1) * NC + q0 + u, fd = (s == 0 ? 2 : 3) * NC + q0 + u;
-          w[u][0] = tile[fa][ly - 1][lx]; w[u][1] = tile[fa][ly][lx]; w[u][2] = tile[fa][ly + 1][lx];
-          const double vm = P.dy * tile[fd][ly - 1][lx], vp = P.dy * tile[fd][ly + 1][lx];
-          const double v0 = Q ? P.dy * tile[fd][ly][lx] : 0.0;
-          p1_coeffs_t<Q>(w[u][0], w[u][1], w[u][2], vm, v0, vp, c[u]);
-        }
-        first_pass_mix<Q, PAIR>(P, nl, w, c, C);
-        const double sc = s == 0 ? 1.0 : P.dx;  // x-pass derivative data: dx * avg(W_x)
+    for (int u = 0; u < NU; ++u)
 #pragma unroll
-        for (int u = 0; u < NU; ++u)
-#pragma unroll
-          for (int k = 0; k < KC; ++k)
-            ycoef[((size_t)((s * NC + q0 + u) * KC + k) * NY2 + (jr + 1)) * NX4 + (ic + 2)] = sc * C[u][k];
-      }
-  }
-  if (ic >= 0 && ic < P.nx && jr <= P.ny + 1) {  // x-pass: {W,V} and {Y,Z} along a row
-    const int nl = cell_flag(P, flag, ic, jr);
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-      for (int q0 = 0; q0 < NC; q0 += NU) {
-        double w[NU][3], c[NU][6], C[NU][6];
-#pragma unroll
-        for (int u = 0; u < NU; ++u) {
-          const int fa = (s == 0 ? 0 : 2) * NC + q0 + u, fd = (s == 0 ? 1 : 3) * NC + q0 + u;
-          w[u][0] = tile[fa][ly][lx - 1]; w[u][1] = tile[fa][ly][lx]; w[u][2] = tile[fa][ly][lx + 1];
-          const double vm = P.dx * tile[fd][ly][lx - 1], vp = P.dx * tile[fd][ly][lx + 1];
-          const double v0 = Q ? P.dx * tile[fd][ly][lx] : 0.0;
-          p1_coeffs_t<Q>(w[u][0], w[u][1], w[u][2], vm, v0, vp, c[u]);
-        }
-        first_pass_mix<Q, PAIR>(P, nl, w, c, C);
-        const double sc = s == 0 ? 1.0 : P.dy;  // y-pass derivative data: dy * avg(W_y)
-#pragma unroll
-        for (int u = 0; u < NU; ++u)
-#pragma unroll
-          for (int k = 0; k < KC; ++k)
-            xcoef[((size_t)((s * NC + q0 + u) * KC + k) * P.nx + ic) * NY4 + (jr + 2)] = sc * C[u][k];
-      }
+      for (int k = 0; k < KC; ++k) out[((size_t)(s * NC + q0 + u) * KC + k) * plane] = sc * C[u][k];
   }
 }
 
-// x-face Gauss points (slice 0..2, cell row `row`) or corner points (slice 3, corner row `row`
-// at y_{row-1/2}) of faces x_{f0-1/2} .. x_{f0+NFACE-3/2}; SEG threads, smem_raw of kFaceSmem
-// bytes.
+// x-face Gauss points (slice 0..2; lines are cell rows) or corner points (slice 3; lines are corner
+// rows, row r at y_{r-1/2}) of CTA b of the slice; SEG threads, smem_raw of face_smem<NC>() bytes.
 template <int NC, bool FLAGS, bool CHAR = false, bool Q = false>
 __device__ __forceinline__ void xface_item(const Params& P, const StepView& sv, const double* st,
                                            const double* __restrict__ ycoef,
                                            const uint8_t* __restrict__ flag, double* __restrict__ FX,
-                                           double* __restrict__ WX, double* __restrict__ WC, int f0,
-                                           int row, int slice, unsigned char* smem_raw) {
+                                           double* __restrict__ WX, double* __restrict__ WC, int b,
+                                           int slice, unsigned char* smem_raw) {
   double(*ev)[5][SPAN] = reinterpret_cast<double(*)[5][SPAN]>(smem_raw);
   const int NX4 = P.nx + 4, NY2 = P.ny + 2;
   using namespace shweno_tables;
-  // faces x_{f0-1/2} .. x_{f0+nf-3/2} exist; their stencils span columns 0 .. nf + 2
-  const int nf = min(NFACE, P.nx + 1 - f0), ncol = nf + 3;
+  const FaceRuns fr(P.nx + 1, slice < 3 ? P.ny : P.ny + 1, b);
+  // a run's faces x_{f0-1/2} .. x_{f0+nf-3/2} have stencils that span its columns 0 .. nf + 2
+  const int w = fr.nf + 3, ncol = fr.nrun * w;
   for (int it = threadIdx.x; it < 2 * NC * ncol; it += SEG) {
     const int col = it % ncol, rq = it / ncol;
-    const int tcol = f0 + col;
+    const int tcol = fr.f0 + col % w, row = fr.line + col / w;
     double e[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (tcol >= NX4) {
-    } else if constexpr (Q) {  // six coefficients per polynomial (reading R1')
+    if constexpr (Q) {  // six coefficients per polynomial (reading R1')
       if (slice < 3) {
         const double* src = ycoef + ((size_t)(rq * 6) * NY2 + (row + 1)) * NX4 + tcol;
 #pragma unroll
@@ -725,22 +746,20 @@ __device__ __forceinline__ void xface_item(const Params& P, const StepView& sv, 
     for (int k = 0; k < 5; ++k) ev[rq][k][col] = e[k];
   }
   __syncthreads();
-  // cell column c holds cell i = f0 + c - 2; a corner row uses the rows below and above
-  auto nl = [&](int c) {
-    const int i = f0 + c - 2;
+  // a run's column c holds cell i = f0 + c - 2; a corner row uses the rows below and above
+  auto nl = [&](int i, int row) {
     return slice < 3 ? cell_flag(P, flag, i, row)
                      : (cell_flag(P, flag, i, row - 1) | cell_flag(P, flag, i, row));
   };
-  const int fi = f0 + threadIdx.x;  // face x_{fi-1/2}
+  const int fi = fr.f0 + fr.ct, row = fr.line + fr.run;  // face x_{fi-1/2}
   double tc[NC][5];
   if constexpr (CHAR) {
-    FlagTable& ft = *reinterpret_cast<FlagTable*>(smem_raw + kEvBytes);
-    for (int c = 1 + threadIdx.x; c <= nf + 1; c += SEG) ft.lin[c] = !nl(c);
+    FlagTable& ft = *reinterpret_cast<FlagTable*>(smem_raw + ev_bytes<NC>());
+    for (int c = threadIdx.x; c < ncol; c += SEG) ft.lin[c] = !nl(fr.f0 + c % w - 2, fr.line + c / w);
     __syncthreads();
     double a[NC][25], Wref[NC];  // Wref: cells next to the face point (the four around a corner)
     CkLead lead;
-    const bool has_face = (int)threadIdx.x < nf;
-    if (has_face) {
+    if (fr.has_face) {
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
       if (slice < 3)
@@ -749,14 +768,14 @@ __device__ __forceinline__ void xface_item(const Params& P, const StepView& sv, 
         Wref[q] = 0.25 * (fetch(P, st, 0, q, fi - 1, row - 1, sv.t) + fetch(P, st, 0, q, fi, row - 1, sv.t) +
                           fetch(P, st, 0, q, fi - 1, row, sv.t) + fetch(P, st, 0, q, fi, row, sv.t));
     }
-    char_face_point<NC, FLAGS, Q>(P, ev, ft, threadIdx.x, 0, a, lead, Wref);
+    char_face_point<NC, FLAGS, Q>(P, ev, ft, fr.col - 1, 0, a, lead, Wref);
     }
     __syncthreads();  // the tables are read no more
-    ck_points<NC>(P, nf, has_face, a, lead, tc);
-    if (!has_face) return;
+    ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, a, lead, tc);
   } else {
-    if (!second_pass_cells<NC, FLAGS, Q>(P, smem_raw, nf, 0, nl, tc)) return;
+    second_pass_cells<NC, FLAGS, Q>(P, smem_raw, fr, 0, FLAGS && fr.has_cell && nl(fi - 1, row), tc);
   }
+  if (!fr.has_face) return;
   const double dt = sv.dt * P.ck.iL;  // in the coefficients' unit of time
   if (slice < 3) {
     double Fh[NC], We[NC];
@@ -773,23 +792,24 @@ __device__ __forceinline__ void xface_item(const Params& P, const StepView& sv, 
   }
 }
 
-// y-face Gauss points (slice 0..2) of column `col`, faces y_{f0-1/2} .. y_{f0+NFACE-3/2}.
+// y-face Gauss points (slice 0..2; lines are cell columns) of CTA b of the slice.
 template <int NC, bool FLAGS, bool CHAR = false, bool Q = false>
 __device__ __forceinline__ void yface_item(const Params& P, const StepView& sv, const double* st,
                                            const double* __restrict__ xcoef,
                                            const uint8_t* __restrict__ flag, double* __restrict__ FY,
-                                           double* __restrict__ WY, int f0, int col, int slice,
+                                           double* __restrict__ WY, int b, int slice,
                                            unsigned char* smem_raw) {
   double(*ev)[5][SPAN] = reinterpret_cast<double(*)[5][SPAN]>(smem_raw);
   const int NY4 = P.ny + 4;
   using namespace shweno_tables;
-  // faces y_{f0-1/2} .. y_{f0+nf-3/2} exist; their stencils span rows 0 .. nf + 2
-  const int nf = min(NFACE, P.ny + 1 - f0), nrow = nf + 3;
+  const FaceRuns fr(P.ny + 1, P.nx, b);
+  // a run's faces y_{f0-1/2} .. y_{f0+nf-3/2} have stencils that span its rows 0 .. nf + 2
+  const int w = fr.nf + 3, nrow = fr.nrun * w;
   for (int it = threadIdx.x; it < 2 * NC * nrow; it += SEG) {
     const int r = it % nrow, rq = it / nrow;
-    const int trow = f0 + r;
+    const int trow = fr.f0 + r % w, col = fr.line + r / w;
     double e[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (trow < NY4) {
+    {
       constexpr int KC = Q ? 6 : 5;
       const double* src = xcoef + ((size_t)(rq * KC) * P.nx + col) * NY4 + trow;
 #pragma unroll
@@ -804,28 +824,26 @@ __device__ __forceinline__ void yface_item(const Params& P, const StepView& sv, 
     for (int k = 0; k < 5; ++k) ev[rq][k][r] = e[k];
   }
   __syncthreads();
-  auto nl = [&](int c) { return cell_flag(P, flag, col, f0 + c - 2); };
-  const int fj = f0 + threadIdx.x;  // face y_{fj-1/2}
+  const int fj = fr.f0 + fr.ct, col = fr.line + fr.run;  // face y_{fj-1/2}
   double tc[NC][5];
   if constexpr (CHAR) {
-    FlagTable& ft = *reinterpret_cast<FlagTable*>(smem_raw + kEvBytes);
-    for (int c = 1 + threadIdx.x; c <= nf + 1; c += SEG) ft.lin[c] = !nl(c);
+    FlagTable& ft = *reinterpret_cast<FlagTable*>(smem_raw + ev_bytes<NC>());
+    for (int c = threadIdx.x; c < nrow; c += SEG) ft.lin[c] = !cell_flag(P, flag, fr.line + c / w, fr.f0 + c % w - 2);
     __syncthreads();
     double a[NC][25], Wref[NC];
     CkLead lead;
-    const bool has_face = (int)threadIdx.x < nf;
-    if (has_face) {
+    if (fr.has_face) {
 #pragma unroll
       for (int q = 0; q < NC; ++q)
         Wref[q] = 0.5 * (fetch(P, st, 0, q, col, fj - 1, sv.t) + fetch(P, st, 0, q, col, fj, sv.t));
-      char_face_point<NC, FLAGS, Q>(P, ev, ft, threadIdx.x, 1, a, lead, Wref);
+      char_face_point<NC, FLAGS, Q>(P, ev, ft, fr.col - 1, 1, a, lead, Wref);
     }
     __syncthreads();  // the tables are read no more
-    ck_points<NC>(P, nf, has_face, a, lead, tc);
-    if (!has_face) return;
+    ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, a, lead, tc);
   } else {
-    if (!second_pass_cells<NC, FLAGS, Q>(P, smem_raw, nf, 1, nl, tc)) return;
+    second_pass_cells<NC, FLAGS, Q>(P, smem_raw, fr, 1, FLAGS && fr.has_cell && cell_flag(P, flag, col, fj - 1), tc);
   }
+  if (!fr.has_face) return;
   double Gh[NC], We[NC];
   lobatto<NC>(tc, sv.dt * P.ck.iL, P.gamma, 1, Gh, We);
 #pragma unroll

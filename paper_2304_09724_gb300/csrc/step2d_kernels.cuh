@@ -36,14 +36,14 @@ __global__ void __launch_bounds__(TX * TY) coef2d_kernel(Params P, const Ctl* __
                                                          const uint8_t* __restrict__ flag,
                                                          double* __restrict__ ycoef,
                                                          double* __restrict__ xcoef) {
-  __shared__ double tile[16][TY + 2][TX + 2];
+  __shared__ double tile[2 * NC][TY + 2][TX + 2];
   if (!ctl->active) return;
-  coef2d_item<NC, TY, Q>(P, step_view(ctl), s0, s1, flag, ycoef, xcoef, blockIdx.x * TX - 2, blockIdx.y * TY - 2, tile,
+  coef2d_item<NC, TY, Q>(P, step_view(ctl), s0, s1, flag, ycoef, xcoef, blockIdx.z, blockIdx.x * TX - 2, blockIdx.y * TY - 2, tile,
                   threadIdx.x, threadIdx.y);
 }
 
 template <int NC, bool FLAGS, bool CHAR, bool Q>
-__global__ void __launch_bounds__(SEG) xface2d_kernel(Params P, const Ctl* __restrict__ ctl,
+__global__ void __launch_bounds__(SEG, NC == 1 ? 3 : 2) xface2d_kernel(Params P, const Ctl* __restrict__ ctl,
                                                       const double* s0, const double* s1,
                                                       const double* __restrict__ ycoef,
                                                       const uint8_t* __restrict__ flag,
@@ -52,16 +52,14 @@ __global__ void __launch_bounds__(SEG) xface2d_kernel(Params P, const Ctl* __res
                                                       double* __restrict__ WC) {
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   if (!ctl->active) return;
-  const int slice = blockIdx.z;  // 0..2: Gauss point of the rows; 3: corner rows
-  const int row = blockIdx.y;    // Gauss: cell row j; corner: corner row jc (y_{jc-1/2})
-  if (slice < 3 && row >= P.ny) return;
+  const int slice = blockIdx.y;  // 0..2: Gauss point of the rows; 3: corner rows
+  if (slice < 3 && (int)blockIdx.x >= FaceSplit(P.nx + 1).ctas(P.ny)) return;
   const StepView sv = step_view(ctl);
-  xface_item<NC, FLAGS, CHAR, Q>(P, sv, sv.odd ? s1 : s0, ycoef, flag, FX, WX, WC, blockIdx.x * NFACE, row, slice,
-                              dyn_smem);
+  xface_item<NC, FLAGS, CHAR, Q>(P, sv, sv.odd ? s1 : s0, ycoef, flag, FX, WX, WC, blockIdx.x, slice, dyn_smem);
 }
 
 template <int NC, bool FLAGS, bool CHAR, bool Q>
-__global__ void __launch_bounds__(SEG) yface2d_kernel(Params P, const Ctl* __restrict__ ctl,
+__global__ void __launch_bounds__(SEG, NC == 1 ? 3 : 2) yface2d_kernel(Params P, const Ctl* __restrict__ ctl,
                                                       const double* s0, const double* s1,
                                                       const double* __restrict__ xcoef,
                                                       const uint8_t* __restrict__ flag,
@@ -70,8 +68,7 @@ __global__ void __launch_bounds__(SEG) yface2d_kernel(Params P, const Ctl* __res
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   if (!ctl->active) return;
   const StepView sv = step_view(ctl);
-  yface_item<NC, FLAGS, CHAR, Q>(P, sv, sv.odd ? s1 : s0, xcoef, flag, FY, WY, blockIdx.x * NFACE, blockIdx.y,
-                              blockIdx.z, dyn_smem);
+  yface_item<NC, FLAGS, CHAR, Q>(P, sv, sv.odd ? s1 : s0, xcoef, flag, FY, WY, blockIdx.x, blockIdx.y, dyn_smem);
 }
 
 template <int NC>
@@ -123,24 +120,36 @@ static cudaError_t init_kernels2d_reading() {
 template <int NC, bool CHAR, bool Q>
 static void launch_faces2d(const Params& P, Ctl* ctl, const double* s0, const double* s1,
                            const uint8_t* flag, const Scratch2D& S, cudaStream_t st, cudaEvent_t* ev) {
-  dim3 xg((P.nx + 1 + NFACE - 1) / NFACE, P.ny + 1, 4);
+  dim3 xg(FaceSplit(P.nx + 1).ctas(P.ny + 1), 4), yg(FaceSplit(P.ny + 1).ctas(P.nx), 3);
+  // Both kernels read the first-pass tables and write arrays of their own.  Where one does not fill
+  // the GPU (304 CTA slots) the y-faces go beside the x-faces on the handle's second stream.
+  const bool beside = !ev && S.aux && 4 * xg.x < 304;
+  cudaStream_t sy = st;
+  if (beside) {
+    sy = S.aux;
+    cudaEventRecord(S.fork, st);
+    cudaStreamWaitEvent(sy, S.fork, 0);
+  }
   if (P.flag_mode == FLAG_ALL_NONLINEAR)
     xface2d_kernel<NC, false, CHAR, Q><<<xg, SEG, face_smem<NC>(), st>>>(P, ctl, s0, s1, S.ycoef, flag, S.FX, S.WX, S.WC);
   else
     xface2d_kernel<NC, true, CHAR, Q><<<xg, SEG, face_smem<NC>(), st>>>(P, ctl, s0, s1, S.ycoef, flag, S.FX, S.WX, S.WC);
   if (ev) cudaEventRecord(ev[2], st);
-  dim3 yg((P.ny + 1 + NFACE - 1) / NFACE, P.nx, 3);
   if (P.flag_mode == FLAG_ALL_NONLINEAR)
-    yface2d_kernel<NC, false, CHAR, Q><<<yg, SEG, face_smem<NC>(), st>>>(P, ctl, s0, s1, S.xcoef, flag, S.FY, S.WY);
+    yface2d_kernel<NC, false, CHAR, Q><<<yg, SEG, face_smem<NC>(), sy>>>(P, ctl, s0, s1, S.xcoef, flag, S.FY, S.WY);
   else
-    yface2d_kernel<NC, true, CHAR, Q><<<yg, SEG, face_smem<NC>(), st>>>(P, ctl, s0, s1, S.xcoef, flag, S.FY, S.WY);
+    yface2d_kernel<NC, true, CHAR, Q><<<yg, SEG, face_smem<NC>(), sy>>>(P, ctl, s0, s1, S.xcoef, flag, S.FY, S.WY);
+  if (beside) {
+    cudaEventRecord(S.join, sy);
+    cudaStreamWaitEvent(st, S.join, 0);
+  }
 }
 
 template <int NC, bool Q>
 static void launch_step2d_nc(const Params& P, Ctl* ctl, const double* s0, const double* s1,
                              double* o0, double* o1, const uint8_t* flag, const Scratch2D& S,
                              cudaStream_t st, cudaEvent_t* ev) {
-  dim3 cb(TX, TY), cg((P.nx + 4 + TX - 1) / TX, (P.ny + 4 + TY - 1) / TY);
+  dim3 cb(TX, TY), cg((P.nx + 4 + TX - 1) / TX, (P.ny + 4 + TY - 1) / TY, 4);
   if (ev) cudaEventRecord(ev[0], st);
   coef2d_kernel<NC, Q><<<cg, cb, 0, st>>>(P, ctl, s0, s1, flag, S.ycoef, S.xcoef);
   if (ev) cudaEventRecord(ev[1], st);
