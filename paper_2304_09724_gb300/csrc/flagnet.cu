@@ -109,16 +109,47 @@ __global__ void mlp_forward_kernel(const float* __restrict__ params, const float
 }
 
 // Gradient of mean BCE over n samples.  A CTA handles GB samples: each thread runs forward and
-// backward for one sample into shared memory, then the CTA reduces every parameter's gradient
-// over its samples and adds it to grad with one atomicAdd per parameter.
+// backward for one sample, keeping its activations and their gradients transposed in shared memory
+// ([unit][sample], rows padded by four words so that neither the threads' stores nor the 16-byte
+// reads of the sums collide), then the CTA sums every parameter's gradient over its samples, eight
+// parameters of a column to a thread, and adds it to grad with one atomicAdd per parameter.  The
+// weights are read 16 bytes at a time (the first layer's rows padded from 22 to 24).  Bound by the
+// chain of one warp per scheduler: about 2800 multiply-adds forward and backward, 2300 in the sums;
+// 16384 samples: 28 -> 9 us (rows of 32 floats put all 32 lanes' stores on one bank before, and
+// every multiply-add of the sums read both factors).
 constexpr int GB = 128;
-struct GradSmem {
-  float p[NPARAM];
-  float x[GB][NIN];
-  float h1[GB][NH], h2[GB][NH], d1[GB][NH], d2[GB][NH];
-  float d3[GB];
+constexpr int GROW = GB + 4;
+constexpr int NINP = 24;
+struct __align__(16) GradSmem {
+  float w1[NH][NINP], w2[NH][NH], b1[NH], b2[NH], w3[NH], b3;
+  float pad[3];
+  float x[NIN][GROW], h1[NH][GROW], h2[NH][GROW], d1[NH][GROW], d2[NH][GROW], d3[GROW];
   float red[GB / 32];
 };
+
+__global__ void mlp_zero_kernel(float* __restrict__ grad, float* __restrict__ loss) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < NPARAM) grad[k] = 0.f;
+  if (k == NPARAM) *loss = 0.f;
+}
+
+// s[0..7] = sum over the samples of d[i0 + u] * y
+__device__ __forceinline__ void grad_sums(const float (*d)[GROW], const float* y, int i0, float s[8]) {
+#pragma unroll
+  for (int u = 0; u < 8; ++u) s[u] = 0.f;
+#pragma unroll 4
+  for (int b = 0; b < GB; b += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(y + b);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const float4 w = *reinterpret_cast<const float4*>(&d[i0 + u][b]);
+      s[u] = fmaf(w.x, v.x, s[u]);
+      s[u] = fmaf(w.y, v.y, s[u]);
+      s[u] = fmaf(w.z, v.z, s[u]);
+      s[u] = fmaf(w.w, v.w, s[u]);
+    }
+  }
+}
 
 __global__ void __launch_bounds__(GB) mlp_grad_kernel(const float* __restrict__ params,
                                                       const float* __restrict__ X,
@@ -127,32 +158,61 @@ __global__ void __launch_bounds__(GB) mlp_grad_kernel(const float* __restrict__ 
                                                       float* __restrict__ loss) {
   extern __shared__ __align__(16) unsigned char raw[];
   GradSmem& S = *reinterpret_cast<GradSmem*>(raw);
-  for (int k = threadIdx.x; k < NPARAM; k += GB) S.p[k] = params[k];
-  __syncthreads();
   const int tid = threadIdx.x;
-  const int64_t b = (int64_t)blockIdx.x * GB + tid;
-  const float* p = S.p;
+  for (int k = tid; k < NPARAM; k += GB) {
+    const float v = params[k];
+    if (k < OFF_B1) S.w1[k / NIN][k % NIN] = v;
+    else if (k < OFF_W2) S.b1[k - OFF_B1] = v;
+    else if (k < OFF_B2) (&S.w2[0][0])[k - OFF_W2] = v;
+    else if (k < OFF_W3) S.b2[k - OFF_B2] = v;
+    else if (k < OFF_B3) S.w3[k - OFF_W3] = v;
+    else S.b3 = v;
+  }
+  if (tid < NH) S.w1[tid][NIN] = S.w1[tid][NIN + 1] = 0.f;
+  const int64_t b0 = (int64_t)blockIdx.x * GB;
+  const int64_t b = b0 + tid;
+  // the CTA's samples lie one after the other
+  const int cnt = (int)(n - b0 < GB ? n - b0 : GB);
+  for (int k = tid; k < GB * NIN; k += GB) S.x[k % NIN][k / NIN] = k < cnt * NIN ? X[b0 * NIN + k] : 0.f;
+  __syncthreads();
   float l = 0.f;
   if (b < n) {
-    float x[NIN], z1[NH], h1[NH], z2[NH];
+    float x[NINP], h1[NH];
 #pragma unroll
-    for (int j = 0; j < NIN; ++j) x[j] = S.x[tid][j] = X[b * NIN + j];
-#pragma unroll
+    for (int j = 0; j < NINP; ++j) x[j] = j < NIN ? S.x[j][tid] : 0.f;
+#pragma unroll 4
     for (int i = 0; i < NH; ++i) {
-      float z = p[OFF_B1 + i];
+      float z = S.b1[i];
 #pragma unroll
-      for (int j = 0; j < NIN; ++j) z = fmaf(p[OFF_W1 + i * NIN + j], x[j], z);
-      z1[i] = z;
-      h1[i] = S.h1[tid][i] = fmaxf(z, 0.f);
+      for (int j = 0; j < NINP; j += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(&S.w1[i][j]);
+        z = fmaf(w.x, x[j], z);
+        z = fmaf(w.y, x[j + 1], z);
+        if (j + 2 < NIN) {
+          z = fmaf(w.z, x[j + 2], z);
+          z = fmaf(w.w, x[j + 3], z);
+        }
+      }
+      S.h1[i][tid] = fmaxf(z, 0.f);
     }
-    float z3 = p[OFF_B3];
-    for (int i = 0; i < NH; ++i) {
-      float z = p[OFF_B2 + i];
 #pragma unroll
-      for (int j = 0; j < NH; ++j) z = fmaf(p[OFF_W2 + i * NH + j], h1[j], z);
-      z2[i] = z;
-      S.h2[tid][i] = fmaxf(z, 0.f);
-      z3 = fmaf(p[OFF_W3 + i], fmaxf(z, 0.f), z3);
+    for (int j = 0; j < NH; ++j) h1[j] = S.h1[j][tid];
+    float z3 = S.b3;
+    unsigned on2 = 0;  // units of the second layer that pass
+#pragma unroll 4
+    for (int i = 0; i < NH; ++i) {
+      float z = S.b2[i];
+#pragma unroll
+      for (int j = 0; j < NH; j += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(&S.w2[i][j]);
+        z = fmaf(w.x, h1[j], z);
+        z = fmaf(w.y, h1[j + 1], z);
+        z = fmaf(w.z, h1[j + 2], z);
+        z = fmaf(w.w, h1[j + 3], z);
+      }
+      on2 |= z > 0.f ? 1u << i : 0u;
+      S.h2[i][tid] = fmaxf(z, 0.f);
+      z3 = fmaf(S.w3[i], fmaxf(z, 0.f), z3);
     }
     const float yy = y[b];
     const float sg = 1.f / (1.f + expf(-z3));
@@ -162,18 +222,25 @@ __global__ void __launch_bounds__(GB) mlp_grad_kernel(const float* __restrict__ 
     l = pw * yy * sp_neg + (1.f - yy) * sp_pos;
     const float d3 = (-pw * yy * (1.f - sg) + (1.f - yy) * sg) / (float)n;
     S.d3[tid] = d3;
-    float d2[NH];
+    float s[NH];
 #pragma unroll
-    for (int i = 0; i < NH; ++i) d2[i] = S.d2[tid][i] = z2[i] > 0.f ? d3 * p[OFF_W3 + i] : 0.f;
-    for (int j = 0; j < NH; ++j) {
-      float s = 0.f;
+    for (int j = 0; j < NH; ++j) s[j] = 0.f;
+#pragma unroll 4
+    for (int i = 0; i < NH; ++i) {
+      const float d2 = S.d2[i][tid] = on2 >> i & 1u ? d3 * S.w3[i] : 0.f;
 #pragma unroll
-      for (int i = 0; i < NH; ++i) s = fmaf(p[OFF_W2 + i * NH + j], d2[i], s);
-      S.d1[tid][j] = z1[j] > 0.f ? s : 0.f;
+      for (int j = 0; j < NH; j += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(&S.w2[i][j]);
+        s[j] = fmaf(w.x, d2, s[j]);
+        s[j + 1] = fmaf(w.y, d2, s[j + 1]);
+        s[j + 2] = fmaf(w.z, d2, s[j + 2]);
+        s[j + 3] = fmaf(w.w, d2, s[j + 3]);
+      }
     }
+#pragma unroll
+    for (int j = 0; j < NH; ++j) S.d1[j][tid] = h1[j] > 0.f ? s[j] : 0.f;
   } else {
-    for (int j = 0; j < NIN; ++j) S.x[tid][j] = 0.f;
-    for (int i = 0; i < NH; ++i) S.h1[tid][i] = S.h2[tid][i] = S.d1[tid][i] = S.d2[tid][i] = 0.f;
+    for (int i = 0; i < NH; ++i) S.h1[i][tid] = S.h2[i][tid] = S.d1[i][tid] = S.d2[i][tid] = 0.f;
     S.d3[tid] = 0.f;
   }
   // loss: block sum, one atomic per CTA
@@ -185,28 +252,31 @@ __global__ void __launch_bounds__(GB) mlp_grad_kernel(const float* __restrict__ 
     for (int w = 0; w < GB / 32; ++w) s += S.red[w];
     atomicAdd(loss, s / (float)n);
   }
-  // parameter gradients: sums over the CTA's samples
-  for (int k = tid; k < NPARAM; k += GB) {
-    float s = 0.f;
-    if (k < OFF_B1) {
-      const int i = k / NIN, j = k % NIN;
-      for (int bb = 0; bb < GB; ++bb) s = fmaf(S.d1[bb][i], S.x[bb][j], s);
-    } else if (k < OFF_W2) {
-      const int i = k - OFF_B1;
-      for (int bb = 0; bb < GB; ++bb) s += S.d1[bb][i];
-    } else if (k < OFF_B2) {
-      const int i = (k - OFF_W2) / NH, j = (k - OFF_W2) % NH;
-      for (int bb = 0; bb < GB; ++bb) s = fmaf(S.d2[bb][i], S.h1[bb][j], s);
-    } else if (k < OFF_W3) {
-      const int i = k - OFF_B2;
-      for (int bb = 0; bb < GB; ++bb) s += S.d2[bb][i];
-    } else if (k < OFF_B3) {
-      const int i = k - OFF_W3;
-      for (int bb = 0; bb < GB; ++bb) s = fmaf(S.d3[bb], S.h2[bb][i], s);
-    } else {
-      for (int bb = 0; bb < GB; ++bb) s += S.d3[bb];
+  // parameter gradients: sums over the CTA's samples, warp w the rows 8 w .. 8 w + 7 of both layers
+  const int lane = tid & 31, i0 = (tid >> 5) * 8;
+  float s[8];
+  grad_sums(S.d2, S.h1[lane], i0, s);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) atomicAdd(&grad[OFF_W2 + (i0 + u) * NH + lane], s[u]);
+  if (lane < NIN) {
+    grad_sums(S.d1, S.x[lane], i0, s);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) atomicAdd(&grad[OFF_W1 + (i0 + u) * NIN + lane], s[u]);
+  } else if (lane < NIN + 8) {  // the biases of the warp's rows
+    float t1 = 0.f, t2 = 0.f, t3 = 0.f;
+    const int i = i0 + lane - NIN;
+    for (int bb = 0; bb < GB; ++bb) {
+      t1 += S.d1[i][bb];
+      t2 += S.d2[i][bb];
+      t3 = fmaf(S.d3[bb], S.h2[i][bb], t3);
     }
-    atomicAdd(&grad[k], s);
+    atomicAdd(&grad[OFF_B1 + i], t1);
+    atomicAdd(&grad[OFF_B2 + i], t2);
+    atomicAdd(&grad[OFF_W3 + i], t3);
+  } else if (tid == NIN + 8) {
+    float t = 0.f;
+    for (int bb = 0; bb < GB; ++bb) t += S.d3[bb];
+    atomicAdd(&grad[OFF_B3], t);
   }
 }
 
@@ -289,8 +359,7 @@ cudaError_t mlp_grad(const float* params, const float* X, const float* y, int64_
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  cudaMemsetAsync(grad, 0, NPARAM * sizeof(float), st);
-  cudaMemsetAsync(loss, 0, sizeof(float), st);
+  mlp_zero_kernel<<<(NPARAM + 256) / 256, 256, 0, st>>>(grad, loss);
   if (n > 0)
     mlp_grad_kernel<<<(unsigned)((n + GB - 1) / GB), GB, sizeof(GradSmem), st>>>(params, X, y, n, pw, grad, loss);
   return cudaGetLastError();
