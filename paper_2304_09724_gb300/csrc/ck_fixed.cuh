@@ -59,12 +59,40 @@ struct CkScale {
   FX_FN int of(int q, int s) const { return base[group(q)] + g * s; }
 };
 
+// Scale of an Euler point from its leading state Ws and the exponents top[group][degree >= 1] of its
+// other coefficients.
+template <int NC>
+FX_FN CkScale<NC> ck_scale_from(const double* Ws, const int (&top)[3][5], const CkLead& lead) {
+  CkScale<NC> S;
+  const int e0 = fx_max(fx_exp(fx_hi(Ws[0]) & 0x7fffffff), -300);  // an exact 0 then converts to 0 in every field
+  const int eE = fx_exp(fx_hi(Ws[NC - 1]) & 0x7fffffff);
+  int eh = fx_exp(lead.hH);
+  // a negative density or pressure (E0 + p0 then no longer bounds E0 and the kinetic energy)
+  const int ee = eE - e0 + 3;
+  if (ee > eh + 3) eh = ee;
+  S.eu = fx_max(fx_max(fx_exp(lead.hu), (eh + 1) >> 1), -300);
+  S.base[0] = e0;
+  S.base[1] = e0 + S.eu;
+  S.base[2] = e0 + 2 * S.eu;
+  S.finite = lead.hH < 0x7ff00000 && lead.hu < 0x7ff00000 && (fx_hi(lead.ir) & 0x7fffffff) < 0x7ff00000 &&
+             e0 <= 1024 && eE <= 1024;
+  S.g = 0;
+#pragma unroll
+  for (int s = 1; s < 5; ++s) {
+    int d = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) d = fx_max(d, top[i][s] - S.base[i]);
+    S.finite = S.finite && d < 3000;
+    S.g = fx_max(S.g, (d + s - 1) / s);
+  }
+  return S;
+}
+
 // a(q, m*5+n) (m + n <= 4; n = 0 only when DIM == 1): spatial Taylor coefficients in cell units.
 template <int NC, int DIM, typename Coef>
 FX_FN CkScale<NC> ck_scale(const Coef& a, const CkLead& lead) {
   using Scale = CkScale<NC>;
   constexpr int NG = Scale::NG;
-  Scale S;
   int top[NG][5];  // largest high word (magnitude bits) by group and degree
 #pragma unroll
   for (int i = 0; i < NG; ++i)
@@ -84,35 +112,28 @@ FX_FN CkScale<NC> ck_scale(const Coef& a, const CkLead& lead) {
 #pragma unroll
   for (int i = 0; i < NG; ++i)
 #pragma unroll
-    for (int s = 0; s < 5; ++s) all = fx_max(all, top[i][s]);
-  S.finite = all < 0x7ff00000;
+    for (int s = 0; s < 5; ++s) {
+      all = fx_max(all, top[i][s]);
+      top[i][s] = fx_exp(top[i][s]);
+    }
+  Scale S;
   if constexpr (NC == 1) {
     // u0 may vanish; 2^-40 of the steepest coefficient is as good a scale then
-    int e = fx_exp(top[0][0]);
+    int e = top[0][0];
 #pragma unroll
-    for (int s = 1; s < 5; ++s) e = fx_max(e, fx_exp(top[0][s]) - 40);
+    for (int s = 1; s < 5; ++s) e = fx_max(e, top[0][s] - 40);
     S.base[0] = S.eu = fx_max(e, -900);  // an exact 0 then converts to 0
+    S.g = 0;
+#pragma unroll
+    for (int s = 1; s < 5; ++s) S.g = fx_max(S.g, (fx_max(top[0][s] - S.base[0], 0) + s - 1) / s);
+    S.finite = true;
   } else {
-    const int e0 = fx_max(fx_exp(top[0][0]), -300);  // an exact 0 then converts to 0 in every field
-    int eh = fx_exp(lead.hH);
-    // a negative density or pressure (E0 + p0 then no longer bounds E0 and the kinetic energy)
-    const int ee = fx_exp(top[2][0]) - e0 + 3;
-    if (ee > eh + 3) eh = ee;
-    S.eu = fx_max(fx_max(fx_exp(lead.hu), (eh + 1) >> 1), -300);
-    S.base[0] = e0;
-    S.base[1] = e0 + S.eu;
-    S.base[2] = e0 + 2 * S.eu;
-    S.finite = S.finite && lead.hH < 0x7ff00000 && lead.hu < 0x7ff00000 && (fx_hi(lead.ir) & 0x7fffffff) < 0x7ff00000;
-  }
-  S.g = 0;
+    double Ws[NC];
 #pragma unroll
-  for (int s = 1; s < 5; ++s) {
-    int d = fx_exp(top[0][s]) - S.base[0];
-#pragma unroll
-    for (int i = 1; i < NG; ++i) d = fx_max(d, fx_exp(top[i][s]) - S.base[i]);
-    d = fx_max(d, 0);
-    S.g = fx_max(S.g, (d + s - 1) / s);
+    for (int q = 0; q < NC; ++q) Ws[q] = a(q, 0);
+    S = ck_scale_from<NC>(Ws, top, lead);
   }
+  S.finite = S.finite && all < 0x7ff00000;
   return S;
 }
 

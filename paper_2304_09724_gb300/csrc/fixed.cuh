@@ -30,6 +30,7 @@ namespace shweno {
 constexpr int FX_S = 31;  // bits of the low limb
 constexpr int FX_Q = 61;  // fraction bits of a coefficient
 constexpr int FX_C = 58;  // fraction bits of a constant
+constexpr int FX_D = 57;  // fraction bits of the second pass's data (room for end values of 8 times the data)
 
 struct Fx {
   int32_t h, l;
@@ -84,6 +85,13 @@ FX_FN Fx fx_split(int64_t z, FxRange& r) {
   v.h = (int32_t)(z >> FX_S);
   v.l = (int32_t)((uint32_t)z & 0x7fffffffu) - (int32_t)FX_HALF;
   r.h |= (uint32_t)(v.h + (1 << 28));
+  return v;
+}
+// The same for sums of at most four products with constants below 1 (second pass): |h| < 2^29.
+FX_FN Fx fx_split_wide(int64_t z, FxRange& r) {
+  FxRange in{0};
+  const Fx v = fx_split(z, in);
+  r.h |= (uint32_t)(v.h + (1 << 29)) >> 1;
   return v;
 }
 FX_FN int64_t fx_join(Fx a) { return (int64_t)((uint64_t)(int64_t)a.h << FX_S) + a.l; }

@@ -565,6 +565,36 @@ __device__ __forceinline__ void euler_eigvecs(const Prim& P, double g, int dir, 
   }
 }
 
+// Coefficients s_k of the waves from their speeds; returns whether the left side is the base.
+template <int NC>
+__device__ __forceinline__ int wave_coefficients(const double lam[NC], double tol, double s[NC]) {
+  int npos = 0, nneg = 0;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    if (lam[k] > tol) ++npos;
+    else if (lam[k] < -tol) ++nneg;
+  }
+  // waves with H != 0 measured from dR, or with H != 1 measured from dL
+  const int base_left = (NC - nneg) > (NC - npos) ? 1 : 0;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    const double H = lam[k] > tol ? 1.0 : (lam[k] < -tol ? 0.0 : 0.5);
+    s[k] = base_left ? H - 1.0 : H;
+  }
+  return base_left;
+}
+
+// Scales of a leading state for the Cauchy-Kovalevskaya recursion.
+template <int NC>
+__device__ __forceinline__ CkLead prim_lead(const Prim& P) {
+  CkLead l;
+  l.ir = P.ir;
+  l.hu = fx_hi(P.u) & 0x7fffffff;
+  if (NC == 4) l.hu = fx_max(l.hu, fx_hi(P.v) & 0x7fffffff);
+  l.hH = fx_hi(P.H) & 0x7fffffff;
+  return l;
+}
+
 template <int NC>
 struct Upwinder {
   double r[NC][NC];  // r[k] = k-th right eigenvector
@@ -583,22 +613,11 @@ struct Upwinder {
       const Prim P = euler_prim(Ws, NC, g);
       tol = 1e-12 * P.c;
       euler_eigvecs<NC>(P, g, dir, r, l, lam);
-      lead.ir = P.ir;
-      lead.hu = fx_hi(P.u) & 0x7fffffff;
-      if (NC == 4) lead.hu = fx_max(lead.hu, fx_hi(P.v) & 0x7fffffff);
-      lead.hH = fx_hi(P.H) & 0x7fffffff;
+      lead = prim_lead<NC>(P);
     }
-    int npos = 0, nneg = 0;
-    for (int k = 0; k < NC; ++k) {
-      if (lam[k] > tol) ++npos;
-      else if (lam[k] < -tol) ++nneg;
-    }
-    // waves with H != 0 measured from dR, or with H != 1 measured from dL
-    base_left = (NC - nneg) > (NC - npos) ? 1 : 0;
+    base_left = wave_coefficients<NC>(lam, tol, s);
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
-      const double H = lam[k] > tol ? 1.0 : (lam[k] < -tol ? 0.0 : 0.5);
-      s[k] = base_left ? H - 1.0 : H;
 #pragma unroll
       for (int q = 0; q < NC; ++q) l[k][q] *= s[k];  // apply() then needs no extra product
     }

@@ -367,70 +367,402 @@ static __device__ __noinline__ void ck_warp_euler2d(int half, int p0, int valid,
   }
 }
 
+// Both coordinates in units of L (dx != dy): factors of the spatial coefficients.
+template <int NC>
+__device__ __forceinline__ void ck_unit_lengths(const Params& P, double (&a)[NC][25]) {
+  if (P.ck.rx == P.ck.ry) return;
+  double fx = 1.0;
+#pragma unroll
+  for (int m = 0; m < 5; ++m, fx *= P.ck.rx) {
+    double f = fx;
+#pragma unroll
+    for (int n = 0; n + m < 5; ++n, f *= P.ck.ry)
+#pragma unroll
+      for (int q = 0; q < NC; ++q) a[q][m * 5 + n] *= f;
+  }
+}
+
 // Time-Taylor coefficients per unit L^k (P.ck.iL = 1 / L) of the CTA's points (threads 0 .. npt - 1, those
-// with has_face) from their spatial ones; called by every thread after the barrier that ends the use
-// of the tables.
+// with has_face) for 2D Euler; called by every thread after the barrier that ends the use of the
+// tables.  S: the point's scale, conv(q, m*5+n) its coefficients in that scale, Ws the leading state.
+template <typename Conv>
+__device__ __forceinline__ void ck_points4(const Params& P, int npt, bool has_face, CkScale<4> S, const Conv& conv,
+                                           const CkLead& lead, const double* Ws, double (&tc)[4][5]) {
+  const int tid = threadIdx.x;
+  const int col = kCkIn + (tid / CKP) * 60 * kCkRow + (tid % CKP) * 8;
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  if (has_face) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int s = 0; s < 5; ++s)
+#pragma unroll
+        for (int n = 0; n <= s; ++n) ck_st(col + (q * 15 + ck_pair(s - n, n)) * kCkRow, conv(q, (s - n) * 5 + n));
+    ck_st(kCkNinv + tid * 8, ck_ninv<4>(S, lead));
+    *reinterpret_cast<int*>(dyn_smem + kCkGrow + tid * 4) = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tc[q][0] = Ws[q];
+  } else if (tid < npt) {  // the last cell of a run: zeros stay zeros
+#pragma unroll 1
+    for (int k = 0; k < 60; ++k) ck_st(col + k * kCkRow, Fx{0, 0});
+    ck_st(kCkNinv + tid * 8, Fx{0, 0});
+  }
+  __syncthreads();
+  const int p0 = (tid >> 5) * 16;
+#pragma unroll 1
+  for (int half = 0; half * CKP < npt; ++half) {
+    const int valid = npt - half * CKP - p0;
+    if (valid > 0) ck_warp_euler2d(half, p0, valid, P.ck.K.third, P.ck.K.gm1, P.ck.K.gshift);
+    __syncwarp();
+  }
+  __syncthreads();
+  if (!has_face) return;
+  S.g += *reinterpret_cast<const int*>(dyn_smem + kCkGrow + tid * 4);
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int k = 1; k < 5; ++k) {
+      const int64_t t = ck_ld64(col + (q * 4 + k - 1) * kCkRow);
+      tc[q][k] = S.finite ? fx_to_double(t, S.of(q, 0) + k * (S.eu + S.g)) : fx_from_bits(0x7ff8000000000000ull);
+    }
+}
+
+// The same from FP64 coefficients a[q][m*5+n] in cell units, Burgers or Euler.
 template <int NC>
 __device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_face, double (&a)[NC][25],
                                           const CkLead& lead, double (&tc)[NC][5]) {
-  if (P.ck.rx != P.ck.ry) {  // dx != dy: both coordinates in units of L
-    double fx = 1.0;
-#pragma unroll
-    for (int m = 0; m < 5; ++m, fx *= P.ck.rx) {
-      double f = fx;
-#pragma unroll
-      for (int n = 0; n + m < 5; ++n, f *= P.ck.ry)
-#pragma unroll
-        for (int q = 0; q < NC; ++q) a[q][m * 5 + n] *= f;
-    }
-  }
+  ck_unit_lengths<NC>(P, a);
   if constexpr (NC == 1) {
     if (!has_face) return;
     ck_fixed<1, 2>(a, lead, P.ck.K, tc);
     tc[0][0] = a[0][0];
   } else {
-    extern __shared__ __align__(16) unsigned char dyn_smem[];
-    const int tid = threadIdx.x;
-    const int col = kCkIn + (tid / CKP) * 60 * kCkRow + (tid % CKP) * 8;
-    CkScale<NC> S{};
-    if (has_face) {
-      S = ck_scale<NC, 2>([&a](int q, int mn) { return a[q][mn]; }, lead);
-      FxRange none{0};  // the recursion checks its operands
-#pragma unroll
-      for (int q = 0; q < NC; ++q)
-#pragma unroll
-        for (int s = 0; s < 5; ++s)
-#pragma unroll
-          for (int n = 0; n <= s; ++n)
-            ck_st(col + (q * 15 + ck_pair(s - n, n)) * kCkRow, ck_convert<NC>(S, a[q][(s - n) * 5 + n], q, s, none));
-      ck_st(kCkNinv + tid * 8, ck_ninv<NC>(S, lead));
-      *reinterpret_cast<int*>(dyn_smem + kCkGrow + tid * 4) = 0;
-#pragma unroll
-      for (int q = 0; q < NC; ++q) tc[q][0] = a[q][0];
-    } else if (tid < npt) {  // the last cell of a run: zeros stay zeros
-#pragma unroll 1
-      for (int k = 0; k < 60; ++k) ck_st(col + k * kCkRow, Fx{0, 0});
-      ck_st(kCkNinv + tid * 8, Fx{0, 0});
-    }
-    __syncthreads();
-    const int p0 = (tid >> 5) * 16;
-#pragma unroll 1
-    for (int half = 0; half * CKP < npt; ++half) {
-      const int valid = npt - half * CKP - p0;
-      if (valid > 0) ck_warp_euler2d(half, p0, valid, P.ck.K.third, P.ck.K.gm1, P.ck.K.gshift);
-      __syncwarp();
-    }
-    __syncthreads();
-    if (!has_face) return;
-    S.g += *reinterpret_cast<const int*>(dyn_smem + kCkGrow + tid * 4);
-#pragma unroll
-    for (int q = 0; q < NC; ++q)
-#pragma unroll
-      for (int k = 1; k < 5; ++k) {
-        const int64_t t = ck_ld64(col + (q * 4 + k - 1) * kCkRow);
-        tc[q][k] = S.finite ? fx_to_double(t, S.of(q, 0) + k * (S.eu + S.g)) : fx_from_bits(0x7ff8000000000000ull);
-      }
+    CkScale<4> S{};
+    if (has_face) S = ck_scale<4, 2>([&a](int q, int mn) { return a[q][mn]; }, lead);
+    const double Ws[4] = {a[0][0], a[1][0], a[2][0], a[3][0]};
+    FxRange none{0};  // the recursion checks its operands
+    ck_points4(P, npt, has_face, S, [&](int q, int mn) { return ck_convert<4>(S, a[q][mn], q, mn / 5 + mn % 5, none); },
+               lead, Ws, tc);
   }
+}
+
+// ------------------------------------------------------------------ second pass in fixed point
+// 2D Euler, reading R1, componentwise: the end values, their differences and the upwinding in 64-bit
+// integers instead of FP64 (about 790 of a face point's 1680 remaining FP64 instructions).  A cell's
+// data (first-pass coefficients of its three columns) are converted in a scale of each component's
+// own, the largest of them in [1/2, 1), 57 fraction bits (its double has 53).  The
+// end values are sums of shifted data (their coefficients are eighths, but for the value's) times the
+// cell's weights; a face brings both sides to a scale that fits its units of density and velocity
+// and upwinds there with the FP64 eigenvectors, converted.  Whatever leaves the format is noticed
+// (FxRange) and the CTA takes the FP64 pass instead: data that are not finite, eigenvectors beyond
+// 2^40 in the face's units, end values above 8 times the data, weights of 4 and more.
+struct CellMixFx {
+  Fx A[4], B[4], C[4];
+  int h[4];  // exponents of the cell's data
+  bool lin;
+};
+
+// x 2^-58 c + ..., c a constant with FX_C fraction bits
+__device__ __forceinline__ int64_t fx_scaled(Fx x, Fx c) {
+  FxAcc s = fx_zero<FX_C>();
+  fx_mac(s, x, c);
+  return fx_sum<FX_C>(s);
+}
+
+// Exponents of the cell's data over all orders and its three columns; false if not finite.
+__device__ __forceinline__ bool cell_exponents(const double (*ev)[5][SPAN], int c, int h[4]) {
+  int all = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    int top = 0;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      top = max(top, max(fx_hi(ev[q][k][c - 1]) & 0x7fffffff, max(fx_hi(ev[q][k][c]) & 0x7fffffff, fx_hi(ev[q][k][c + 1]) & 0x7fffffff)));
+      top = max(top, max(fx_hi(ev[4 + q][k][c - 1]) & 0x7fffffff, fx_hi(ev[4 + q][k][c + 1]) & 0x7fffffff));
+    }
+    all = max(all, top);
+    h[q] = max(fx_exp(top), -300);  // an exact 0 then converts to 0
+  }
+  return all < 0x7ff00000;
+}
+
+// Order K of the thread's cell: its ends into the tables L and R (units of the cell's h).  The
+// components share one copy of the code: unrolled four times over, five orders, the pass alone
+// would overflow the instruction cache (128 KB), which the kernel then waits for.
+template <bool LIN, int K>
+__device__ __forceinline__ void cell_ends_fx(const double (*ev)[5][SPAN], int c, const CellMixFx& m,
+                                             int64_t (*L)[5][SEG], int64_t (*R)[5][SEG], FxRange& r) {
+  const Fx u0w{85004561, 143165568}, u0s{24606583, 1002159032}, u0d{-6710886, -858993460};  // 19/30, 11/60, -1/20
+#pragma unroll 1
+  for (int q = 0; q < 4; ++q) {
+    const int h = m.h[q];
+    const int64_t Wm = fx_from_double<FX_D>(ev[q][K][c - 1], h), W0 = fx_from_double<FX_D>(ev[q][K][c], h);
+    const int64_t Wp = fx_from_double<FX_D>(ev[q][K][c + 1], h);
+    const int64_t vm = fx_from_double<FX_D>(ev[4 + q][K][c - 1], h), vp = fx_from_double<FX_D>(ev[4 + q][K][c + 1], h);
+    const int64_t s = Wm + Wp, a = Wp - Wm, dv = vp - vm, sv = vm + vp;
+    FxRange in{0};  // the data themselves are in range by their scale
+    const Fx w0 = fx_split(W0 + FX_HALF, in);
+    int64_t g = 0, hh = 0;
+    if (!LIN) {
+      const Fx d2 = fx_split(W0 - Wm + FX_HALF, in), d3 = fx_split(Wp - W0 + FX_HALF, in);
+      FxAcc z = fx_zero<FX_C>();
+      fx_mac(z, d2, m.B[q]);
+      fx_mac(z, d3, m.C[q]);
+      g = fx_sum<FX_C>(z);
+      z = fx_zero<FX_C>();
+      fx_mac(z, w0, m.B[q]);
+      fx_mac(z, w0, m.C[q]);
+      hh = fx_sum<FX_C>(z);
+    }
+#pragma unroll
+    for (int p = 0; p + K <= 4; ++p) {
+      int64_t U, V = 0;
+      if (p == 0) {
+        FxAcc z = fx_zero<FX_C>();
+        fx_mac(z, w0, u0w);
+        fx_mac(z, fx_split(s + FX_HALF, in), u0s);
+        fx_mac(z, fx_split(dv + FX_HALF, in), u0d);
+        U = fx_sum<FX_C>(z);
+        V = (3 * a - sv + 4) >> 3;
+      } else if (p == 1) {
+        U = s - 2 * W0 - ((dv + 2) >> 2);
+        V = (5 * a - sv + 4) >> 3;
+      } else if (p == 2) {
+        U = ((s + 1) >> 1) - W0;
+        V = (3 * (sv - a) + 4) >> 3;
+      } else if (p == 3) {
+        U = 2 * W0 - s + ((dv + 1) >> 1);
+        V = (sv - a + 2) >> 2;
+      } else {
+        U = W0 - ((s + 1) >> 1) + ((dv + 2) >> 2);
+      }
+      if (!LIN) {
+        U = fx_scaled(fx_split_wide(U + FX_HALF, r), m.A[q]);
+        if (p < 4) V = fx_scaled(fx_split_wide(V + FX_HALF, r), m.A[q]);
+        if (p == 0) { U += hh; V += g >> 1; }
+        if (p == 1) U += g;
+      }
+      // odd p: the slope terms have one sign at both ends, so g is added after the mirror image
+      R[q][p][threadIdx.x] = U + V;
+      int64_t eL = (p & 1) ? V - U : U - V;
+      if (!LIN && p == 1) eL += 2 * g;
+      L[q][p][threadIdx.x] = eL;
+    }
+  }
+}
+
+// The face's upwinding in fixed point.  The linearised problem's solution (Upwinder) is
+// d* = base + sum_k s_k (l_k . d) r_k, d = dL - dR.  The entropy and shear waves share their speed, so
+// their s (call it c), and the four projections add up to the identity: d* = base + c d +
+// sum over the two acoustic waves of (s_k - c) (l_k . d) r_k.  A moving subsonic face needs one acoustic
+// wave and c = 0, a standing one (c = +-1/2) both; which one it is differs from lane to lane and is
+// chosen by the vectors, not by a branch.
+struct UpwindFx {
+  Fx l[2][4], r[2][4];  // (s_k - c) l_k times 2^-el, and r_k, in the face's units
+  int waves, c2;        // waves that contribute; 2 c
+  int el, base_left;
+  int f[4], sl[4], sr[4];  // the face's exponents; right shifts of the two sides' end values
+};
+
+// Order K of the thread's face: upwinded derivatives a[q][m*5+n] in units of f.
+template <int K>
+__device__ __forceinline__ void face_order_fx(const int64_t (*L)[5][SEG], const int64_t (*R)[5][SEG], int dir,
+                                              const UpwindFx& U, int64_t (&a)[4][25], FxRange& r) {
+#pragma unroll
+  for (int p = 0; p + K <= 4; ++p) {
+    if (p == 0 && K == 0) continue;
+    Fx d[4];
+    FxAcc out[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t x = R[q][p][threadIdx.x] >> U.sl[q], y = L[q][p][threadIdx.x + 1] >> U.sr[q];
+      d[q] = fx_split_wide(x - y + FX_HALF, r);
+      out[q] = fx_zero<FX_C>();
+      a[q][dir == 0 ? p * 5 + K : K * 5 + p] = (U.base_left ? x : y) + ((U.c2 * (x - y)) >> 1);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      if (U.waves <= k) continue;
+      FxAcc z = fx_zero<FX_C>();
+#pragma unroll
+      for (int q = 0; q < 4; ++q) fx_mac(z, d[q], U.l[k][q]);
+      const int64_t w = fx_sum<FX_C>(z);
+      if (((w ^ (w >> 63)) >> (59 - U.el)) != 0) r.h |= 0x80000000u;
+      const Fx al = fx_split((int64_t)((uint64_t)w << U.el) + FX_HALF, r);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) fx_mac(out[q], al, U.r[k][q]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q][dir == 0 ? p * 5 + K : K * 5 + p] += fx_sum<FX_C>(out[q]);
+  }
+}
+
+// Leading term and acoustic eigenvectors of the thread's face (FP64), its units, the converted waves.
+__device__ __forceinline__ void face_setup_fx(const Params& P, const int64_t (*L)[5][SEG], const int64_t (*R)[5][SEG],
+                                              const int hL[4], const int* hs, int dir, double Ws[4], CkLead& lead,
+                                              UpwindFx& X, FxRange& r) {
+  int hR[4];
+  double WL[4], WR[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    hR[q] = hs[q * SEG + threadIdx.x + 1];
+    WL[q] = fx_to_double(R[q][0][threadIdx.x], hL[q] + FX_Q - FX_D);
+    WR[q] = fx_to_double(L[q][0][threadIdx.x + 1], hR[q] + FX_Q - FX_D);
+  }
+  hllc_state<4>(WL, WR, P.gamma, dir, Ws);
+  const Prim S = euler_prim(Ws, 4, P.gamma);
+  lead = prim_lead<4>(S);
+  double rv[4][4], lv[4][4], lam[4], s[4];
+  euler_eigvecs<4>(S, P.gamma, dir, rv, lv, lam);
+  X.base_left = wave_coefficients<4>(lam, 1e-12 * S.c, s);
+  X.c2 = (int)(2.0 * s[1]);
+  const double b0 = s[0] - s[1], b3 = s[3] - s[1];
+  const bool low = b0 != 0.0;  // the first wave that contributes is u - c
+  X.waves = (low ? 1 : 0) + (b3 != 0.0 ? 1 : 0);
+  const int f0 = max(hL[0], hR[0]);
+  int F = max(max(max(hL[1], hR[1]), max(hL[2], hR[2])) - f0, (max(hL[3], hR[3]) - f0 + 1) >> 1);
+  F = max(F, max(fx_exp(lead.hu), (fx_exp(lead.hH) + 1) >> 1));
+  int top = 0, el = -2000;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int u = q == 0 ? 0 : q == 3 ? 2 * F : F;
+    X.f[q] = f0 + u;
+    X.sl[q] = min(X.f[q] - hL[q], 63);
+    X.sr[q] = min(X.f[q] - hR[q], 63);
+    const int hi = max(fx_hi(lv[0][q]) & 0x7fffffff, fx_hi(lv[3][q]) & 0x7fffffff);
+    top = max(top, hi);
+    el = max(el, fx_exp(hi) + u);
+  }
+  X.el = max(el, 0);
+  if (top >= 0x7ff00000 || X.el > 40 || lead.hH >= 0x7ff00000 || lead.hu >= 0x7ff00000) {
+    r.h |= 0x80000000u;
+    X.el = 0;
+  }
+  FxRange in{0};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int u = q == 0 ? 0 : q == 3 ? 2 * F : F;
+    X.l[0][q] = fx_split(fx_from_double<FX_C>(low ? b0 * lv[0][q] : b3 * lv[3][q], X.el - u) + FX_HALF, in);
+    X.l[1][q] = fx_split(fx_from_double<FX_C>(b3 * lv[3][q], X.el - u) + FX_HALF, in);
+    X.r[0][q] = fx_split(fx_from_double<FX_C>(low ? rv[0][q] : rv[3][q], u) + FX_HALF, in);
+    X.r[1][q] = fx_split(fx_from_double<FX_C>(rv[3][q], u) + FX_HALF, in);
+  }
+}
+
+template <bool FLAGS, int K>
+__device__ __forceinline__ void pass_order_fx(const Params& P, const double (*ev)[5][SPAN], unsigned char* tables,
+                                              const FaceRuns& fr, const CellMixFx& m, int dir, double Ws[4],
+                                              CkLead& lead, UpwindFx& X, int64_t (&a)[4][25], FxRange& r) {
+  auto L = reinterpret_cast<int64_t(*)[5][SEG]>(tables) + (K & 1) * 4;
+  int* hs = reinterpret_cast<int*>(tables + sizeof(EndTable<4>));
+  auto R = reinterpret_cast<int64_t(*)[5][SEG]>(tables + sizeof(EndTable<4>) + 4 * SEG * sizeof(int));  // each thread its own
+  if (fr.has_cell) {
+    if (FLAGS && m.lin) cell_ends_fx<true, K>(ev, fr.col, m, L, R, r);
+    else cell_ends_fx<false, K>(ev, fr.col, m, L, R, r);
+    if (K == 0)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) hs[q * SEG + threadIdx.x] = m.h[q];
+  }
+  __syncthreads();
+  if (fr.has_face) {
+    if (K == 0) face_setup_fx(P, L, R, m.h, hs, dir, Ws, lead, X, r);
+    face_order_fx<K>(L, R, dir, X, a, r);
+  }
+}
+
+static_assert(ev_bytes<4>() + sizeof(EndTable<4>) + 4 * SEG * sizeof(int) + 4 * 5 * SEG * 8 <= kCkBytes, "tables");
+// The whole pass of the CTA; false (for all threads) if something left the format.
+template <bool FLAGS>
+__device__ __forceinline__ bool second_pass_fx(const Params& P, unsigned char* smem_raw, const FaceRuns& fr, int dir,
+                                               bool nl, double (&tc)[4][5]) {
+  const double(*ev)[5][SPAN] = reinterpret_cast<const double(*)[5][SPAN]>(smem_raw);
+  unsigned char* tables = smem_raw + ev_bytes<4>();
+  FxRange r{0};
+  CellMixFx m;
+  if (fr.has_cell) {
+    CellMix<4> w;
+    cell_mix<4, false>(P, ev, fr.col, FLAGS && !nl, w);
+    m.lin = w.lin;
+    int top = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      top = max(top, max(fx_hi(w.A[q]) & 0x7fffffff, max(fx_hi(w.B[q]) & 0x7fffffff, fx_hi(w.C[q]) & 0x7fffffff)));
+    // weights are at most 1 / gam[0] unless they overflowed
+    if (!cell_exponents(ev, fr.col, m.h) || top >= 0x40100000) r.h = 0x80000000u;
+    FxRange in{0};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      m.A[q] = fx_split(fx_from_double<FX_C>(w.A[q], 0) + FX_HALF, in);
+      m.B[q] = fx_split(fx_from_double<FX_C>(w.B[q], 0) + FX_HALF, in);
+      m.C[q] = fx_split(fx_from_double<FX_C>(w.C[q], 0) + FX_HALF, in);
+    }
+  }
+  int64_t a[4][25];
+  double Ws[4];
+  CkLead lead{};
+  UpwindFx X;
+  pass_order_fx<FLAGS, 0>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
+  pass_order_fx<FLAGS, 1>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
+  pass_order_fx<FLAGS, 2>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
+  pass_order_fx<FLAGS, 3>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
+  pass_order_fx<FLAGS, 4>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
+  if (__syncthreads_or(r.bad() ? 1 : 0)) return false;
+  CkScale<4> S{};
+  if (fr.has_face) {
+    int top[3][5];  // exponents by group and degree
+    uint64_t bits[3][5];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int s = 0; s < 5; ++s) bits[i][s] = 0;
+    if (P.ck.rx != P.ck.ry) {  // dx != dy: both coordinates in units of L (one factor is 1)
+      const bool along_x = P.ck.rx != 1.0;
+      double f = 1.0;
+#pragma unroll
+      for (int i = 1; i < 5; ++i) {
+        f *= along_x ? P.ck.rx : P.ck.ry;
+        const Fx c = fx_const(f);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int j = 0; j + i < 5; ++j) {
+            FxRange in{0};
+            int64_t& z = a[q][along_x ? i * 5 + j : j * 5 + i];
+            z = fx_scaled(fx_split(z + FX_HALF, in), c);
+          }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int s = 1; s < 5; ++s)
+#pragma unroll
+        for (int n = 0; n <= s; ++n) {
+          const int64_t z = a[q][(s - n) * 5 + n];
+          bits[CkScale<4>::group(q)][s] |= (uint64_t)(z ^ (z >> 63));
+        }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int q = i == 0 ? 0 : i == 1 ? 1 : 3;
+      top[i][0] = 0;
+#pragma unroll
+      for (int s = 1; s < 5; ++s) top[i][s] = X.f[q] - FX_D + 64 - fx_clz(bits[i][s]);
+    }
+    S = ck_scale_from<4>(Ws, top, lead);
+  }
+  ck_points4(P, fr.nrun * (fr.nf + 1), fr.has_face, S,
+             [&](int q, int mn) {
+               FxRange none{0};
+               const int s = mn / 5 + mn % 5;
+               if (s == 0) return ck_convert<4>(S, Ws[q], q, 0, none);
+               const int n = FX_Q - FX_D + X.f[q] - S.of(q, s);  // left shift
+               const int64_t z = a[q][mn];
+               const int64_t x = n >= 0 ? (int64_t)((uint64_t)z << min(n, 63))
+                                        : ((z >> min(-n - 1, 62)) + 1) >> 1;
+               return fx_split(x + FX_HALF, none);
+             },
+             lead, Ws, tc);
+  return true;
 }
 
 // Second pass, leading term, upwinding and CK of the CTA's faces.  A thread with a face gets in
@@ -439,6 +771,11 @@ __device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_fac
 template <int NC, bool FLAGS, bool Q>
 __device__ __forceinline__ void second_pass_cells(const Params& P, unsigned char* smem_raw, const FaceRuns& fr, int dir,
                                                   bool nl, double (&tc)[NC][5]) {
+  // With per-cell flags the FP64 pass stays: linear cells spare it the weights and two thirds of the
+  // end values' operations (1024 x 256 double Mach reflection, learned: 10.2 ms a step, 10.6 in
+  // fixed point; 400^2 quadrants, all cells nonlinear: 6.1 ms, 4.6 in fixed point).
+  if constexpr (NC == 4 && !Q && !FLAGS)
+    if (second_pass_fx<FLAGS>(P, smem_raw, fr, dir, nl, tc)) return;
   const double(*ev)[5][SPAN] = reinterpret_cast<const double(*)[5][SPAN]>(smem_raw);
   EndTable<NC>& et = *reinterpret_cast<EndTable<NC>*>(smem_raw + ev_bytes<NC>());
   CellMix<NC> m;
