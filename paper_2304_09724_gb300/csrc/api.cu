@@ -319,9 +319,9 @@ shweno_status shweno_create(const shweno_grid* grid, double gamma, const shweno_
     h->scratch = (double*)dev_alloc(shweno::scratch2d_doubles(P) * sizeof(double));
     if (!h->scratch) return bail(SHWENO_E_NOMEM, "device allocation of the step scratch failed");
     h->S = shweno::carve_scratch2d(P, h->scratch);
-    if (cudaStreamCreateWithFlags(&h->S.aux, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&h->S.fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&h->S.join, cudaEventDisableTiming) != cudaSuccess)
+    if (shweno::faces_beside(P) && (cudaStreamCreateWithFlags(&h->S.aux, cudaStreamNonBlocking) != cudaSuccess ||
+                                    cudaEventCreateWithFlags(&h->S.fork, cudaEventDisableTiming) != cudaSuccess ||
+                                    cudaEventCreateWithFlags(&h->S.join, cudaEventDisableTiming) != cudaSuccess))
       return bail(SHWENO_E_CUDA, "creating the handle's second stream failed");
     const cudaError_t ea = shweno::init_kernels2d();
     if (ea != cudaSuccess) {
@@ -475,6 +475,7 @@ shweno_status shweno_run(shweno_handle* h, double t_final, double cfl, double* t
     return SHWENO_OK;
   }
   // steps per graph launch: enough to amortise launches, few enough to stop soon after t_final
+  // (8 steps a graph instead of 32 cost the Lax problem, N = 200, 5 %)
   const double work = (double)h->cells * (h->P.dim == 2 ? 64.0 : 1.0);
   const int chunk = work > 4e6 ? 2 : (work > 2.5e5 ? 8 : 32);
   s = build_graph(h, chunk);

@@ -664,16 +664,6 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   int64_t dmom210;
   int64_t dmom120;
   int64_t dmom030;
-  int64_t doth000;
-  int64_t doth100;
-  int64_t doth010;
-  int64_t doth200;
-  int64_t doth110;
-  int64_t doth020;
-  int64_t doth300;
-  int64_t doth210;
-  int64_t doth120;
-  int64_t doth030;
   int64_t dE000;
   int64_t dE100;
   int64_t dE010;
@@ -704,256 +694,158 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   dmom120 = 2 * f220;
   drho030 = 1 * fx_join(S.ldmom(0, 1, 3));
   dmom030 = 1 * f130;
-  {
-  const Fx oth000 = S.ldoth(0, 0, 0);
-  const Fx oth100 = S.ldoth(0, 1, 0);
-  const Fx oth200 = S.ldoth(0, 2, 0);
+  #pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+  const Fx ser000 = S.ldser(s, 0, 0, 0);
+  const Fx ser100 = S.ldser(s, 0, 1, 0);
+  const Fx ser200 = S.ldser(s, 0, 2, 0);
   int64_t z00;
   { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel100);
-    fx_mac(s, oth100, vel000);
-    z00 = fx_sum(s); }
-  doth000 = 1 * z00;
-  const Fx oth010 = S.ldoth(0, 0, 1);
-  const Fx oth110 = S.ldoth(0, 1, 1);
-  int64_t z10;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel200);
-    fx_mac(s, oth100, vel100);
-    fx_mac(s, oth200, vel000);
-    z10 = fx_sum(s); }
-  doth100 = 2 * z10;
-  const Fx oth300 = S.ldoth(0, 3, 0);
-  int64_t z01;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel110);
-    fx_mac(s, oth010, vel100);
-    fx_mac(s, oth100, vel010);
-    fx_mac(s, oth110, vel000);
-    z01 = fx_sum(s); }
-  doth010 = 1 * z01;
-  const Fx oth210 = S.ldoth(0, 2, 1);
-  int64_t z20;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel300);
-    fx_mac(s, oth100, vel200);
-    fx_mac(s, oth200, vel100);
-    fx_mac(s, oth300, vel000);
-    z20 = fx_sum(s); }
-  doth200 = 3 * z20;
-  const Fx oth020 = S.ldoth(0, 0, 2);
-  const Fx oth120 = S.ldoth(0, 1, 2);
-  int64_t z11;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel210);
-    fx_mac(s, oth010, vel200);
-    fx_mac(s, oth100, vel110);
-    fx_mac(s, oth110, vel100);
-    fx_mac(s, oth200, vel010);
-    fx_mac(s, oth210, vel000);
-    z11 = fx_sum(s); }
-  doth110 = 2 * z11;
-  const Fx oth400 = S.ldoth(0, 4, 0);
-  int64_t z02;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel120);
-    fx_mac(s, oth010, vel110);
-    fx_mac(s, oth020, vel100);
-    fx_mac(s, oth100, vel020);
-    fx_mac(s, oth110, vel010);
-    fx_mac(s, oth120, vel000);
-    z02 = fx_sum(s); }
-  doth020 = 1 * z02;
-  const Fx oth310 = S.ldoth(0, 3, 1);
-  int64_t z30;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel400);
-    fx_mac(s, oth100, vel300);
-    fx_mac(s, oth200, vel200);
-    fx_mac(s, oth300, vel100);
-    fx_mac(s, oth400, vel000);
-    z30 = fx_sum(s); }
-  doth300 = 4 * z30;
-  const Fx oth220 = S.ldoth(0, 2, 2);
-  int64_t z21;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel310);
-    fx_mac(s, oth010, vel300);
-    fx_mac(s, oth100, vel210);
-    fx_mac(s, oth110, vel200);
-    fx_mac(s, oth200, vel110);
-    fx_mac(s, oth210, vel100);
-    fx_mac(s, oth300, vel010);
-    fx_mac(s, oth310, vel000);
-    z21 = fx_sum(s); }
-  doth210 = 3 * z21;
-  const Fx oth030 = S.ldoth(0, 0, 3);
-  const Fx oth130 = S.ldoth(0, 1, 3);
-  int64_t z12;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel220);
-    fx_mac(s, oth010, vel210);
-    fx_mac(s, oth020, vel200);
-    fx_mac(s, oth100, vel120);
-    fx_mac(s, oth110, vel110);
-    fx_mac(s, oth120, vel100);
-    fx_mac(s, oth200, vel020);
-    fx_mac(s, oth210, vel010);
-    fx_mac(s, oth220, vel000);
-    z12 = fx_sum(s); }
-  doth120 = 2 * z12;
-  int64_t z03;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel130);
-    fx_mac(s, oth010, vel120);
-    fx_mac(s, oth020, vel110);
-    fx_mac(s, oth030, vel100);
-    fx_mac(s, oth100, vel030);
-    fx_mac(s, oth110, vel020);
-    fx_mac(s, oth120, vel010);
-    fx_mac(s, oth130, vel000);
-    z03 = fx_sum(s); }
-  doth030 = 1 * z03;
-  }
-  {
-  const Fx H000 = S.ldH(0, 0, 0);
-  const Fx H100 = S.ldH(0, 1, 0);
-  const Fx H200 = S.ldH(0, 2, 0);
-  int64_t z00;
-  { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel100);
-    fx_mac(s, H100, vel000);
+    fx_mac(s, ser000, vel100);
+    fx_mac(s, ser100, vel000);
     z00 = fx_sum(s); }
   dE000 = 1 * z00;
-  const Fx H010 = S.ldH(0, 0, 1);
-  const Fx H110 = S.ldH(0, 1, 1);
+  const Fx ser010 = S.ldser(s, 0, 0, 1);
+  const Fx ser110 = S.ldser(s, 0, 1, 1);
   int64_t z10;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel200);
-    fx_mac(s, H100, vel100);
-    fx_mac(s, H200, vel000);
+    fx_mac(s, ser000, vel200);
+    fx_mac(s, ser100, vel100);
+    fx_mac(s, ser200, vel000);
     z10 = fx_sum(s); }
   dE100 = 2 * z10;
-  const Fx H300 = S.ldH(0, 3, 0);
+  const Fx ser300 = S.ldser(s, 0, 3, 0);
   int64_t z01;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel110);
-    fx_mac(s, H010, vel100);
-    fx_mac(s, H100, vel010);
-    fx_mac(s, H110, vel000);
+    fx_mac(s, ser000, vel110);
+    fx_mac(s, ser010, vel100);
+    fx_mac(s, ser100, vel010);
+    fx_mac(s, ser110, vel000);
     z01 = fx_sum(s); }
   dE010 = 1 * z01;
-  const Fx H210 = S.ldH(0, 2, 1);
+  const Fx ser210 = S.ldser(s, 0, 2, 1);
   int64_t z20;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel300);
-    fx_mac(s, H100, vel200);
-    fx_mac(s, H200, vel100);
-    fx_mac(s, H300, vel000);
+    fx_mac(s, ser000, vel300);
+    fx_mac(s, ser100, vel200);
+    fx_mac(s, ser200, vel100);
+    fx_mac(s, ser300, vel000);
     z20 = fx_sum(s); }
   dE200 = 3 * z20;
-  const Fx H020 = S.ldH(0, 0, 2);
-  const Fx H120 = S.ldH(0, 1, 2);
+  const Fx ser020 = S.ldser(s, 0, 0, 2);
+  const Fx ser120 = S.ldser(s, 0, 1, 2);
   int64_t z11;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel210);
-    fx_mac(s, H010, vel200);
-    fx_mac(s, H100, vel110);
-    fx_mac(s, H110, vel100);
-    fx_mac(s, H200, vel010);
-    fx_mac(s, H210, vel000);
+    fx_mac(s, ser000, vel210);
+    fx_mac(s, ser010, vel200);
+    fx_mac(s, ser100, vel110);
+    fx_mac(s, ser110, vel100);
+    fx_mac(s, ser200, vel010);
+    fx_mac(s, ser210, vel000);
     z11 = fx_sum(s); }
   dE110 = 2 * z11;
-  const Fx H400 = S.ldH(0, 4, 0);
+  const Fx ser400 = S.ldser(s, 0, 4, 0);
   int64_t z02;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel120);
-    fx_mac(s, H010, vel110);
-    fx_mac(s, H020, vel100);
-    fx_mac(s, H100, vel020);
-    fx_mac(s, H110, vel010);
-    fx_mac(s, H120, vel000);
+    fx_mac(s, ser000, vel120);
+    fx_mac(s, ser010, vel110);
+    fx_mac(s, ser020, vel100);
+    fx_mac(s, ser100, vel020);
+    fx_mac(s, ser110, vel010);
+    fx_mac(s, ser120, vel000);
     z02 = fx_sum(s); }
   dE020 = 1 * z02;
-  const Fx H310 = S.ldH(0, 3, 1);
+  const Fx ser310 = S.ldser(s, 0, 3, 1);
   int64_t z30;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel400);
-    fx_mac(s, H100, vel300);
-    fx_mac(s, H200, vel200);
-    fx_mac(s, H300, vel100);
-    fx_mac(s, H400, vel000);
+    fx_mac(s, ser000, vel400);
+    fx_mac(s, ser100, vel300);
+    fx_mac(s, ser200, vel200);
+    fx_mac(s, ser300, vel100);
+    fx_mac(s, ser400, vel000);
     z30 = fx_sum(s); }
   dE300 = 4 * z30;
-  const Fx H220 = S.ldH(0, 2, 2);
+  const Fx ser220 = S.ldser(s, 0, 2, 2);
   int64_t z21;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel310);
-    fx_mac(s, H010, vel300);
-    fx_mac(s, H100, vel210);
-    fx_mac(s, H110, vel200);
-    fx_mac(s, H200, vel110);
-    fx_mac(s, H210, vel100);
-    fx_mac(s, H300, vel010);
-    fx_mac(s, H310, vel000);
+    fx_mac(s, ser000, vel310);
+    fx_mac(s, ser010, vel300);
+    fx_mac(s, ser100, vel210);
+    fx_mac(s, ser110, vel200);
+    fx_mac(s, ser200, vel110);
+    fx_mac(s, ser210, vel100);
+    fx_mac(s, ser300, vel010);
+    fx_mac(s, ser310, vel000);
     z21 = fx_sum(s); }
   dE210 = 3 * z21;
-  const Fx H030 = S.ldH(0, 0, 3);
-  const Fx H130 = S.ldH(0, 1, 3);
+  const Fx ser030 = S.ldser(s, 0, 0, 3);
+  const Fx ser130 = S.ldser(s, 0, 1, 3);
   int64_t z12;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel220);
-    fx_mac(s, H010, vel210);
-    fx_mac(s, H020, vel200);
-    fx_mac(s, H100, vel120);
-    fx_mac(s, H110, vel110);
-    fx_mac(s, H120, vel100);
-    fx_mac(s, H200, vel020);
-    fx_mac(s, H210, vel010);
-    fx_mac(s, H220, vel000);
+    fx_mac(s, ser000, vel220);
+    fx_mac(s, ser010, vel210);
+    fx_mac(s, ser020, vel200);
+    fx_mac(s, ser100, vel120);
+    fx_mac(s, ser110, vel110);
+    fx_mac(s, ser120, vel100);
+    fx_mac(s, ser200, vel020);
+    fx_mac(s, ser210, vel010);
+    fx_mac(s, ser220, vel000);
     z12 = fx_sum(s); }
   dE120 = 2 * z12;
   int64_t z03;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel130);
-    fx_mac(s, H010, vel120);
-    fx_mac(s, H020, vel110);
-    fx_mac(s, H030, vel100);
-    fx_mac(s, H100, vel030);
-    fx_mac(s, H110, vel020);
-    fx_mac(s, H120, vel010);
-    fx_mac(s, H130, vel000);
+    fx_mac(s, ser000, vel130);
+    fx_mac(s, ser010, vel120);
+    fx_mac(s, ser020, vel110);
+    fx_mac(s, ser030, vel100);
+    fx_mac(s, ser100, vel030);
+    fx_mac(s, ser110, vel020);
+    fx_mac(s, ser120, vel010);
+    fx_mac(s, ser130, vel000);
     z03 = fx_sum(s); }
   dE030 = 1 * z03;
-  }
-  { const int64_t own = dmom000 + S.swap(doth000);
+  if (s == 0) {
+    S.stoth(1, 0, 0, dE000);
+    S.stoth(1, 1, 0, dE100);
+    S.stoth(1, 0, 1, dE010);
+    S.stoth(1, 2, 0, dE200);
+    S.stoth(1, 1, 1, dE110);
+    S.stoth(1, 0, 2, dE020);
+    S.stoth(1, 3, 0, dE300);
+    S.stoth(1, 2, 1, dE210);
+    S.stoth(1, 1, 2, dE120);
+    S.stoth(1, 0, 3, dE030);
+  } }
+  S.sync();
+  { const int64_t own = dmom000 + S.ldown(1, 0, 0);
     const int64_t both = S.pick(drho000, dE000) + S.swap(S.pick(dE000, drho000));
     S.next(1, 0, 0, fx_time<1>(own, third), fx_time<1>(both, third), r); }
-  { const int64_t own = dmom100 + S.swap(doth010);
+  { const int64_t own = dmom100 + S.ldown(1, 1, 0);
     const int64_t both = S.pick(drho100, dE100) + S.swap(S.pick(dE010, drho010));
     S.next(1, 1, 0, fx_time<1>(own, third), fx_time<1>(both, third), r); }
-  { const int64_t own = dmom010 + S.swap(doth100);
+  { const int64_t own = dmom010 + S.ldown(1, 0, 1);
     const int64_t both = S.pick(drho010, dE010) + S.swap(S.pick(dE100, drho100));
     S.next(1, 0, 1, fx_time<1>(own, third), fx_time<1>(both, third), r); }
-  { const int64_t own = dmom200 + S.swap(doth020);
+  { const int64_t own = dmom200 + S.ldown(1, 2, 0);
     const int64_t both = S.pick(drho200, dE200) + S.swap(S.pick(dE020, drho020));
     S.next(1, 2, 0, fx_time<1>(own, third), fx_time<1>(both, third), r); }
-  { const int64_t own = dmom110 + S.swap(doth110);
+  { const int64_t own = dmom110 + S.ldown(1, 1, 1);
     const int64_t both = S.pick(drho110, dE110) + S.swap(S.pick(dE110, drho110));
     S.next(1, 1, 1, fx_time<1>(own, third), fx_time<1>(both, third), r); }
-  { const int64_t own = dmom020 + S.swap(doth200);
+  { const int64_t own = dmom020 + S.ldown(1, 0, 2);
     const int64_t both = S.pick(drho020, dE020) + S.swap(S.pick(dE200, drho200));
     S.next(1, 0, 2, fx_time<1>(own, third), fx_time<1>(both, third), r); }
-  { const int64_t own = dmom300 + S.swap(doth030);
+  { const int64_t own = dmom300 + S.ldown(1, 3, 0);
     const int64_t both = S.pick(drho300, dE300) + S.swap(S.pick(dE030, drho030));
     S.next(1, 3, 0, fx_time<1>(own, third), fx_time<1>(both, third), r); }
-  { const int64_t own = dmom210 + S.swap(doth120);
+  { const int64_t own = dmom210 + S.ldown(1, 2, 1);
     const int64_t both = S.pick(drho210, dE210) + S.swap(S.pick(dE120, drho120));
     S.next(1, 2, 1, fx_time<1>(own, third), fx_time<1>(both, third), r); }
-  { const int64_t own = dmom120 + S.swap(doth210);
+  { const int64_t own = dmom120 + S.ldown(1, 1, 2);
     const int64_t both = S.pick(drho120, dE120) + S.swap(S.pick(dE210, drho210));
     S.next(1, 1, 2, fx_time<1>(own, third), fx_time<1>(both, third), r); }
-  { const int64_t own = dmom030 + S.swap(doth300);
+  { const int64_t own = dmom030 + S.ldown(1, 0, 3);
     const int64_t both = S.pick(drho030, dE030) + S.swap(S.pick(dE300, drho300));
     S.next(1, 0, 3, fx_time<1>(own, third), fx_time<1>(both, third), r); }
   S.sync();
@@ -1285,12 +1177,6 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   int64_t dmom201;
   int64_t dmom111;
   int64_t dmom021;
-  int64_t doth001;
-  int64_t doth101;
-  int64_t doth011;
-  int64_t doth201;
-  int64_t doth111;
-  int64_t doth021;
   int64_t dE001;
   int64_t dE101;
   int64_t dE011;
@@ -1309,210 +1195,125 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   dmom111 = 2 * f211;
   drho021 = 1 * fx_join(S.ldmom(1, 1, 2));
   dmom021 = 1 * f121;
-  {
-  const Fx oth000 = S.ldoth(0, 0, 0);
-  const Fx oth001 = S.ldoth(1, 0, 0);
-  const Fx oth100 = S.ldoth(0, 1, 0);
-  const Fx oth101 = S.ldoth(1, 1, 0);
-  const Fx oth200 = S.ldoth(0, 2, 0);
-  const Fx oth201 = S.ldoth(1, 2, 0);
+  #pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+  const Fx ser000 = S.ldser(s, 0, 0, 0);
+  const Fx ser001 = S.ldser(s, 1, 0, 0);
+  const Fx ser100 = S.ldser(s, 0, 1, 0);
+  const Fx ser101 = S.ldser(s, 1, 1, 0);
+  const Fx ser200 = S.ldser(s, 0, 2, 0);
+  const Fx ser201 = S.ldser(s, 1, 2, 0);
   int64_t z00;
   { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel101);
-    fx_mac(s, oth001, vel100);
-    fx_mac(s, oth100, vel001);
-    fx_mac(s, oth101, vel000);
-    z00 = fx_sum(s); }
-  doth001 = 1 * z00;
-  const Fx oth010 = S.ldoth(0, 0, 1);
-  const Fx oth011 = S.ldoth(1, 0, 1);
-  const Fx oth110 = S.ldoth(0, 1, 1);
-  const Fx oth111 = S.ldoth(1, 1, 1);
-  int64_t z10;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel201);
-    fx_mac(s, oth001, vel200);
-    fx_mac(s, oth100, vel101);
-    fx_mac(s, oth101, vel100);
-    fx_mac(s, oth200, vel001);
-    fx_mac(s, oth201, vel000);
-    z10 = fx_sum(s); }
-  doth101 = 2 * z10;
-  const Fx oth300 = S.ldoth(0, 3, 0);
-  const Fx oth301 = S.ldoth(1, 3, 0);
-  int64_t z01;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel111);
-    fx_mac(s, oth001, vel110);
-    fx_mac(s, oth010, vel101);
-    fx_mac(s, oth011, vel100);
-    fx_mac(s, oth100, vel011);
-    fx_mac(s, oth101, vel010);
-    fx_mac(s, oth110, vel001);
-    fx_mac(s, oth111, vel000);
-    z01 = fx_sum(s); }
-  doth011 = 1 * z01;
-  const Fx oth210 = S.ldoth(0, 2, 1);
-  const Fx oth211 = S.ldoth(1, 2, 1);
-  int64_t z20;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel301);
-    fx_mac(s, oth001, vel300);
-    fx_mac(s, oth100, vel201);
-    fx_mac(s, oth101, vel200);
-    fx_mac(s, oth200, vel101);
-    fx_mac(s, oth201, vel100);
-    fx_mac(s, oth300, vel001);
-    fx_mac(s, oth301, vel000);
-    z20 = fx_sum(s); }
-  doth201 = 3 * z20;
-  const Fx oth020 = S.ldoth(0, 0, 2);
-  const Fx oth021 = S.ldoth(1, 0, 2);
-  const Fx oth120 = S.ldoth(0, 1, 2);
-  const Fx oth121 = S.ldoth(1, 1, 2);
-  int64_t z11;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel211);
-    fx_mac(s, oth001, vel210);
-    fx_mac(s, oth010, vel201);
-    fx_mac(s, oth011, vel200);
-    fx_mac(s, oth100, vel111);
-    fx_mac(s, oth101, vel110);
-    fx_mac(s, oth110, vel101);
-    fx_mac(s, oth111, vel100);
-    fx_mac(s, oth200, vel011);
-    fx_mac(s, oth201, vel010);
-    fx_mac(s, oth210, vel001);
-    fx_mac(s, oth211, vel000);
-    z11 = fx_sum(s); }
-  doth111 = 2 * z11;
-  int64_t z02;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel121);
-    fx_mac(s, oth001, vel120);
-    fx_mac(s, oth010, vel111);
-    fx_mac(s, oth011, vel110);
-    fx_mac(s, oth020, vel101);
-    fx_mac(s, oth021, vel100);
-    fx_mac(s, oth100, vel021);
-    fx_mac(s, oth101, vel020);
-    fx_mac(s, oth110, vel011);
-    fx_mac(s, oth111, vel010);
-    fx_mac(s, oth120, vel001);
-    fx_mac(s, oth121, vel000);
-    z02 = fx_sum(s); }
-  doth021 = 1 * z02;
-  }
-  {
-  const Fx H000 = S.ldH(0, 0, 0);
-  const Fx H001 = S.ldH(1, 0, 0);
-  const Fx H100 = S.ldH(0, 1, 0);
-  const Fx H101 = S.ldH(1, 1, 0);
-  const Fx H200 = S.ldH(0, 2, 0);
-  const Fx H201 = S.ldH(1, 2, 0);
-  int64_t z00;
-  { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel101);
-    fx_mac(s, H001, vel100);
-    fx_mac(s, H100, vel001);
-    fx_mac(s, H101, vel000);
+    fx_mac(s, ser000, vel101);
+    fx_mac(s, ser001, vel100);
+    fx_mac(s, ser100, vel001);
+    fx_mac(s, ser101, vel000);
     z00 = fx_sum(s); }
   dE001 = 1 * z00;
-  const Fx H010 = S.ldH(0, 0, 1);
-  const Fx H011 = S.ldH(1, 0, 1);
-  const Fx H110 = S.ldH(0, 1, 1);
-  const Fx H111 = S.ldH(1, 1, 1);
+  const Fx ser010 = S.ldser(s, 0, 0, 1);
+  const Fx ser011 = S.ldser(s, 1, 0, 1);
+  const Fx ser110 = S.ldser(s, 0, 1, 1);
+  const Fx ser111 = S.ldser(s, 1, 1, 1);
   int64_t z10;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel201);
-    fx_mac(s, H001, vel200);
-    fx_mac(s, H100, vel101);
-    fx_mac(s, H101, vel100);
-    fx_mac(s, H200, vel001);
-    fx_mac(s, H201, vel000);
+    fx_mac(s, ser000, vel201);
+    fx_mac(s, ser001, vel200);
+    fx_mac(s, ser100, vel101);
+    fx_mac(s, ser101, vel100);
+    fx_mac(s, ser200, vel001);
+    fx_mac(s, ser201, vel000);
     z10 = fx_sum(s); }
   dE101 = 2 * z10;
-  const Fx H300 = S.ldH(0, 3, 0);
-  const Fx H301 = S.ldH(1, 3, 0);
+  const Fx ser300 = S.ldser(s, 0, 3, 0);
+  const Fx ser301 = S.ldser(s, 1, 3, 0);
   int64_t z01;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel111);
-    fx_mac(s, H001, vel110);
-    fx_mac(s, H010, vel101);
-    fx_mac(s, H011, vel100);
-    fx_mac(s, H100, vel011);
-    fx_mac(s, H101, vel010);
-    fx_mac(s, H110, vel001);
-    fx_mac(s, H111, vel000);
+    fx_mac(s, ser000, vel111);
+    fx_mac(s, ser001, vel110);
+    fx_mac(s, ser010, vel101);
+    fx_mac(s, ser011, vel100);
+    fx_mac(s, ser100, vel011);
+    fx_mac(s, ser101, vel010);
+    fx_mac(s, ser110, vel001);
+    fx_mac(s, ser111, vel000);
     z01 = fx_sum(s); }
   dE011 = 1 * z01;
-  const Fx H210 = S.ldH(0, 2, 1);
-  const Fx H211 = S.ldH(1, 2, 1);
+  const Fx ser210 = S.ldser(s, 0, 2, 1);
+  const Fx ser211 = S.ldser(s, 1, 2, 1);
   int64_t z20;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel301);
-    fx_mac(s, H001, vel300);
-    fx_mac(s, H100, vel201);
-    fx_mac(s, H101, vel200);
-    fx_mac(s, H200, vel101);
-    fx_mac(s, H201, vel100);
-    fx_mac(s, H300, vel001);
-    fx_mac(s, H301, vel000);
+    fx_mac(s, ser000, vel301);
+    fx_mac(s, ser001, vel300);
+    fx_mac(s, ser100, vel201);
+    fx_mac(s, ser101, vel200);
+    fx_mac(s, ser200, vel101);
+    fx_mac(s, ser201, vel100);
+    fx_mac(s, ser300, vel001);
+    fx_mac(s, ser301, vel000);
     z20 = fx_sum(s); }
   dE201 = 3 * z20;
-  const Fx H020 = S.ldH(0, 0, 2);
-  const Fx H021 = S.ldH(1, 0, 2);
-  const Fx H120 = S.ldH(0, 1, 2);
-  const Fx H121 = S.ldH(1, 1, 2);
+  const Fx ser020 = S.ldser(s, 0, 0, 2);
+  const Fx ser021 = S.ldser(s, 1, 0, 2);
+  const Fx ser120 = S.ldser(s, 0, 1, 2);
+  const Fx ser121 = S.ldser(s, 1, 1, 2);
   int64_t z11;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel211);
-    fx_mac(s, H001, vel210);
-    fx_mac(s, H010, vel201);
-    fx_mac(s, H011, vel200);
-    fx_mac(s, H100, vel111);
-    fx_mac(s, H101, vel110);
-    fx_mac(s, H110, vel101);
-    fx_mac(s, H111, vel100);
-    fx_mac(s, H200, vel011);
-    fx_mac(s, H201, vel010);
-    fx_mac(s, H210, vel001);
-    fx_mac(s, H211, vel000);
+    fx_mac(s, ser000, vel211);
+    fx_mac(s, ser001, vel210);
+    fx_mac(s, ser010, vel201);
+    fx_mac(s, ser011, vel200);
+    fx_mac(s, ser100, vel111);
+    fx_mac(s, ser101, vel110);
+    fx_mac(s, ser110, vel101);
+    fx_mac(s, ser111, vel100);
+    fx_mac(s, ser200, vel011);
+    fx_mac(s, ser201, vel010);
+    fx_mac(s, ser210, vel001);
+    fx_mac(s, ser211, vel000);
     z11 = fx_sum(s); }
   dE111 = 2 * z11;
   int64_t z02;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel121);
-    fx_mac(s, H001, vel120);
-    fx_mac(s, H010, vel111);
-    fx_mac(s, H011, vel110);
-    fx_mac(s, H020, vel101);
-    fx_mac(s, H021, vel100);
-    fx_mac(s, H100, vel021);
-    fx_mac(s, H101, vel020);
-    fx_mac(s, H110, vel011);
-    fx_mac(s, H111, vel010);
-    fx_mac(s, H120, vel001);
-    fx_mac(s, H121, vel000);
+    fx_mac(s, ser000, vel121);
+    fx_mac(s, ser001, vel120);
+    fx_mac(s, ser010, vel111);
+    fx_mac(s, ser011, vel110);
+    fx_mac(s, ser020, vel101);
+    fx_mac(s, ser021, vel100);
+    fx_mac(s, ser100, vel021);
+    fx_mac(s, ser101, vel020);
+    fx_mac(s, ser110, vel011);
+    fx_mac(s, ser111, vel010);
+    fx_mac(s, ser120, vel001);
+    fx_mac(s, ser121, vel000);
     z02 = fx_sum(s); }
   dE021 = 1 * z02;
-  }
-  { const int64_t own = dmom001 + S.swap(doth001);
+  if (s == 0) {
+    S.stoth(2, 0, 0, dE001);
+    S.stoth(2, 1, 0, dE101);
+    S.stoth(2, 0, 1, dE011);
+    S.stoth(2, 2, 0, dE201);
+    S.stoth(2, 1, 1, dE111);
+    S.stoth(2, 0, 2, dE021);
+  } }
+  S.sync();
+  { const int64_t own = dmom001 + S.ldown(2, 0, 0);
     const int64_t both = S.pick(drho001, dE001) + S.swap(S.pick(dE001, drho001));
     S.next(2, 0, 0, fx_time<2>(own, third), fx_time<2>(both, third), r); }
-  { const int64_t own = dmom101 + S.swap(doth011);
+  { const int64_t own = dmom101 + S.ldown(2, 1, 0);
     const int64_t both = S.pick(drho101, dE101) + S.swap(S.pick(dE011, drho011));
     S.next(2, 1, 0, fx_time<2>(own, third), fx_time<2>(both, third), r); }
-  { const int64_t own = dmom011 + S.swap(doth101);
+  { const int64_t own = dmom011 + S.ldown(2, 0, 1);
     const int64_t both = S.pick(drho011, dE011) + S.swap(S.pick(dE101, drho101));
     S.next(2, 0, 1, fx_time<2>(own, third), fx_time<2>(both, third), r); }
-  { const int64_t own = dmom201 + S.swap(doth021);
+  { const int64_t own = dmom201 + S.ldown(2, 2, 0);
     const int64_t both = S.pick(drho201, dE201) + S.swap(S.pick(dE021, drho021));
     S.next(2, 2, 0, fx_time<2>(own, third), fx_time<2>(both, third), r); }
-  { const int64_t own = dmom111 + S.swap(doth111);
+  { const int64_t own = dmom111 + S.ldown(2, 1, 1);
     const int64_t both = S.pick(drho111, dE111) + S.swap(S.pick(dE111, drho111));
     S.next(2, 1, 1, fx_time<2>(own, third), fx_time<2>(both, third), r); }
-  { const int64_t own = dmom021 + S.swap(doth201);
+  { const int64_t own = dmom021 + S.ldown(2, 0, 2);
     const int64_t both = S.pick(drho021, dE021) + S.swap(S.pick(dE201, drho201));
     S.next(2, 0, 2, fx_time<2>(own, third), fx_time<2>(both, third), r); }
   S.sync();
@@ -1730,9 +1531,6 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   int64_t dmom002;
   int64_t dmom102;
   int64_t dmom012;
-  int64_t doth002;
-  int64_t doth102;
-  int64_t doth012;
   int64_t dE002;
   int64_t dE102;
   int64_t dE012;
@@ -1742,125 +1540,75 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   dmom102 = 2 * f202;
   drho012 = 1 * fx_join(S.ldmom(2, 1, 1));
   dmom012 = 1 * f112;
-  {
-  const Fx oth000 = S.ldoth(0, 0, 0);
-  const Fx oth001 = S.ldoth(1, 0, 0);
-  const Fx oth002 = S.ldoth(2, 0, 0);
-  const Fx oth100 = S.ldoth(0, 1, 0);
-  const Fx oth101 = S.ldoth(1, 1, 0);
-  const Fx oth102 = S.ldoth(2, 1, 0);
-  const Fx oth200 = S.ldoth(0, 2, 0);
-  const Fx oth201 = S.ldoth(1, 2, 0);
-  const Fx oth202 = S.ldoth(2, 2, 0);
+  #pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+  const Fx ser000 = S.ldser(s, 0, 0, 0);
+  const Fx ser001 = S.ldser(s, 1, 0, 0);
+  const Fx ser002 = S.ldser(s, 2, 0, 0);
+  const Fx ser100 = S.ldser(s, 0, 1, 0);
+  const Fx ser101 = S.ldser(s, 1, 1, 0);
+  const Fx ser102 = S.ldser(s, 2, 1, 0);
+  const Fx ser200 = S.ldser(s, 0, 2, 0);
+  const Fx ser201 = S.ldser(s, 1, 2, 0);
+  const Fx ser202 = S.ldser(s, 2, 2, 0);
   int64_t z00;
   { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel102);
-    fx_mac(s, oth001, vel101);
-    fx_mac(s, oth002, vel100);
-    fx_mac(s, oth100, vel002);
-    fx_mac(s, oth101, vel001);
-    fx_mac(s, oth102, vel000);
-    z00 = fx_sum(s); }
-  doth002 = 1 * z00;
-  const Fx oth010 = S.ldoth(0, 0, 1);
-  const Fx oth011 = S.ldoth(1, 0, 1);
-  const Fx oth012 = S.ldoth(2, 0, 1);
-  const Fx oth110 = S.ldoth(0, 1, 1);
-  const Fx oth111 = S.ldoth(1, 1, 1);
-  const Fx oth112 = S.ldoth(2, 1, 1);
-  int64_t z10;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel202);
-    fx_mac(s, oth001, vel201);
-    fx_mac(s, oth002, vel200);
-    fx_mac(s, oth100, vel102);
-    fx_mac(s, oth101, vel101);
-    fx_mac(s, oth102, vel100);
-    fx_mac(s, oth200, vel002);
-    fx_mac(s, oth201, vel001);
-    fx_mac(s, oth202, vel000);
-    z10 = fx_sum(s); }
-  doth102 = 2 * z10;
-  int64_t z01;
-  { FxAcc s = fx_zero();
-    fx_mac(s, oth000, vel112);
-    fx_mac(s, oth001, vel111);
-    fx_mac(s, oth002, vel110);
-    fx_mac(s, oth010, vel102);
-    fx_mac(s, oth011, vel101);
-    fx_mac(s, oth012, vel100);
-    fx_mac(s, oth100, vel012);
-    fx_mac(s, oth101, vel011);
-    fx_mac(s, oth102, vel010);
-    fx_mac(s, oth110, vel002);
-    fx_mac(s, oth111, vel001);
-    fx_mac(s, oth112, vel000);
-    z01 = fx_sum(s); }
-  doth012 = 1 * z01;
-  }
-  {
-  const Fx H000 = S.ldH(0, 0, 0);
-  const Fx H001 = S.ldH(1, 0, 0);
-  const Fx H002 = S.ldH(2, 0, 0);
-  const Fx H100 = S.ldH(0, 1, 0);
-  const Fx H101 = S.ldH(1, 1, 0);
-  const Fx H102 = S.ldH(2, 1, 0);
-  const Fx H200 = S.ldH(0, 2, 0);
-  const Fx H201 = S.ldH(1, 2, 0);
-  const Fx H202 = S.ldH(2, 2, 0);
-  int64_t z00;
-  { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel102);
-    fx_mac(s, H001, vel101);
-    fx_mac(s, H002, vel100);
-    fx_mac(s, H100, vel002);
-    fx_mac(s, H101, vel001);
-    fx_mac(s, H102, vel000);
+    fx_mac(s, ser000, vel102);
+    fx_mac(s, ser001, vel101);
+    fx_mac(s, ser002, vel100);
+    fx_mac(s, ser100, vel002);
+    fx_mac(s, ser101, vel001);
+    fx_mac(s, ser102, vel000);
     z00 = fx_sum(s); }
   dE002 = 1 * z00;
-  const Fx H010 = S.ldH(0, 0, 1);
-  const Fx H011 = S.ldH(1, 0, 1);
-  const Fx H012 = S.ldH(2, 0, 1);
-  const Fx H110 = S.ldH(0, 1, 1);
-  const Fx H111 = S.ldH(1, 1, 1);
-  const Fx H112 = S.ldH(2, 1, 1);
+  const Fx ser010 = S.ldser(s, 0, 0, 1);
+  const Fx ser011 = S.ldser(s, 1, 0, 1);
+  const Fx ser012 = S.ldser(s, 2, 0, 1);
+  const Fx ser110 = S.ldser(s, 0, 1, 1);
+  const Fx ser111 = S.ldser(s, 1, 1, 1);
+  const Fx ser112 = S.ldser(s, 2, 1, 1);
   int64_t z10;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel202);
-    fx_mac(s, H001, vel201);
-    fx_mac(s, H002, vel200);
-    fx_mac(s, H100, vel102);
-    fx_mac(s, H101, vel101);
-    fx_mac(s, H102, vel100);
-    fx_mac(s, H200, vel002);
-    fx_mac(s, H201, vel001);
-    fx_mac(s, H202, vel000);
+    fx_mac(s, ser000, vel202);
+    fx_mac(s, ser001, vel201);
+    fx_mac(s, ser002, vel200);
+    fx_mac(s, ser100, vel102);
+    fx_mac(s, ser101, vel101);
+    fx_mac(s, ser102, vel100);
+    fx_mac(s, ser200, vel002);
+    fx_mac(s, ser201, vel001);
+    fx_mac(s, ser202, vel000);
     z10 = fx_sum(s); }
   dE102 = 2 * z10;
   int64_t z01;
   { FxAcc s = fx_zero();
-    fx_mac(s, H000, vel112);
-    fx_mac(s, H001, vel111);
-    fx_mac(s, H002, vel110);
-    fx_mac(s, H010, vel102);
-    fx_mac(s, H011, vel101);
-    fx_mac(s, H012, vel100);
-    fx_mac(s, H100, vel012);
-    fx_mac(s, H101, vel011);
-    fx_mac(s, H102, vel010);
-    fx_mac(s, H110, vel002);
-    fx_mac(s, H111, vel001);
-    fx_mac(s, H112, vel000);
+    fx_mac(s, ser000, vel112);
+    fx_mac(s, ser001, vel111);
+    fx_mac(s, ser002, vel110);
+    fx_mac(s, ser010, vel102);
+    fx_mac(s, ser011, vel101);
+    fx_mac(s, ser012, vel100);
+    fx_mac(s, ser100, vel012);
+    fx_mac(s, ser101, vel011);
+    fx_mac(s, ser102, vel010);
+    fx_mac(s, ser110, vel002);
+    fx_mac(s, ser111, vel001);
+    fx_mac(s, ser112, vel000);
     z01 = fx_sum(s); }
   dE012 = 1 * z01;
-  }
-  { const int64_t own = dmom002 + S.swap(doth002);
+  if (s == 0) {
+    S.stoth(3, 0, 0, dE002);
+    S.stoth(3, 1, 0, dE102);
+    S.stoth(3, 0, 1, dE012);
+  } }
+  S.sync();
+  { const int64_t own = dmom002 + S.ldown(3, 0, 0);
     const int64_t both = S.pick(drho002, dE002) + S.swap(S.pick(dE002, drho002));
     S.next(3, 0, 0, fx_time<3>(own, third), fx_time<3>(both, third), r); }
-  { const int64_t own = dmom102 + S.swap(doth012);
+  { const int64_t own = dmom102 + S.ldown(3, 1, 0);
     const int64_t both = S.pick(drho102, dE102) + S.swap(S.pick(dE012, drho012));
     S.next(3, 1, 0, fx_time<3>(own, third), fx_time<3>(both, third), r); }
-  { const int64_t own = dmom012 + S.swap(doth102);
+  { const int64_t own = dmom012 + S.ldown(3, 0, 1);
     const int64_t both = S.pick(drho012, dE012) + S.swap(S.pick(dE102, drho102));
     S.next(3, 0, 1, fx_time<3>(own, third), fx_time<3>(both, third), r); }
   S.sync();
@@ -1972,8 +1720,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   }
   int64_t drho003;
   int64_t dmom003;
-  int64_t doth003;
   int64_t dE003;
+  int64_t doth003;
   drho003 = 1 * fx_join(S.ldmom(3, 1, 0));
   dmom003 = 1 * f103;
   {
@@ -1985,7 +1733,7 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   const Fx oth101 = S.ldoth(1, 1, 0);
   const Fx oth102 = S.ldoth(2, 1, 0);
   const Fx oth103 = S.ldoth(3, 1, 0);
-  int64_t z00;
+  int64_t z;
   { FxAcc s = fx_zero();
     fx_mac(s, oth000, vel103);
     fx_mac(s, oth001, vel102);
@@ -1995,8 +1743,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
     fx_mac(s, oth101, vel002);
     fx_mac(s, oth102, vel001);
     fx_mac(s, oth103, vel000);
-    z00 = fx_sum(s); }
-  doth003 = 1 * z00;
+    z = fx_sum(s); }
+  doth003 = 1 * z;
   }
   {
   const Fx H000 = S.ldH(0, 0, 0);
@@ -2007,7 +1755,7 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   const Fx H101 = S.ldH(1, 1, 0);
   const Fx H102 = S.ldH(2, 1, 0);
   const Fx H103 = S.ldH(3, 1, 0);
-  int64_t z00;
+  int64_t z;
   { FxAcc s = fx_zero();
     fx_mac(s, H000, vel103);
     fx_mac(s, H001, vel102);
@@ -2017,8 +1765,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
     fx_mac(s, H101, vel002);
     fx_mac(s, H102, vel001);
     fx_mac(s, H103, vel000);
-    z00 = fx_sum(s); }
-  dE003 = 1 * z00;
+    z = fx_sum(s); }
+  dE003 = 1 * z;
   }
   { const int64_t own = dmom003 + S.swap(doth003);
     const int64_t both = S.pick(drho003, dE003) + S.swap(S.pick(dE003, drho003));

@@ -145,6 +145,21 @@ class GenFixed:
         return "\n".join(head + self.lines + outs + ["}"])
 
 
+def flops_euler2d():
+    """Floating-point operations of the 2D Euler recursion in its minimal form (a fused multiply-add
+    counts 2): only the coefficients the outputs depend on, each product and quotient once."""
+    idx = [(m, n, k) for k in range(4) for m in range(5 - k) for n in range(5 - k - m)]
+    pairs = lambda s: sum((m + 1) * (n + 1) * (k + 1) for m, n, k in s)
+    inner = [i for i in idx if i[0] + i[1] > 0]
+    along = [i for i in idx if i[0] > 0]  # x-fluxes; as many y-fluxes
+    total = 2 * (2 * (pairs(idx) - len(idx)) + len(idx))      # u, v
+    total += 2 * (2 * pairs(idx) - len(idx))                  # mu, nv
+    total += 2 * pairs(inner) - len(inner)                    # mv
+    total += 2 * (2 * pairs(along) - len(along))              # uH, vH
+    total += 4 * len(idx) + 2 * len(along)                    # p, H; mu + p, nv + p
+    return total + 4 * 4 * sum((5 - k) * (4 - k) // 2 for k in range(4))  # time update of four fields
+
+
 class GenLane:
     """2D Euler in block fixed point with two lanes per point: lane "x" carries u and the x-fluxes,
     lane "y" (16 lanes up) v and the y-fluxes.  Both run the same code in their own coordinates:
@@ -176,7 +191,8 @@ class GenLane:
         v = f"{name}{i}{j}{t}"
         if v not in self.loaded:
             self.loaded.add(v)
-            self.out(f"const Fx {v} = S.ld{name}({t}, {i}, {j});")
+            arg = "s, " if name == "ser" else ""
+            self.out(f"const Fx {v} = S.ld{name}({arg}{t}, {i}, {j});")
         return v
 
     def uses(self, series, i, j, c):
@@ -229,27 +245,44 @@ class GenLane:
             self.out("}")
         # the time update: (i + 1) times the lane's fluxes, added to the other lane's
         nxt = self.pairs(D - 1)
-        for q in ("rho", "mom", "oth", "E"):
+        for q in ("rho", "mom", "E") + (("oth",) if c == 3 else ()):
             for i, j in nxt:
                 self.out(f"int64_t d{q}{i}{j}{c};")
         for i, j in nxt:
             self.out(f"drho{i}{j}{c} = {i + 1} * fx_join(S.ldmom({c}, {i + 1}, {j}));")
             self.out(f"dmom{i}{j}{c} = {i + 1} * f{i + 1}{j}{c};")
-        for q, series in (("oth", "oth"), ("E", "H")):
-            self.out("{")
+        # products with the other momentum and with H: one copy of the code for both (the recursion
+        # alone nearly fills the instruction cache); the first go to shared memory for the other lane
+        n = c + 1
+        if n < 4:
+            self.out("#pragma unroll 1")
+            self.out("for (int s = 0; s < 2; ++s) {")
             self.loaded = set()
             for x, (i, j) in enumerate(nxt):
                 for i2, j2 in nxt[x:x + 2]:
-                    self.uses(series, i2 + 1, j2, c)
-                z = f"z{i}{j}"
-                self.out(f"int64_t {z};")
-                self.product(series, z, i + 1, j, c)
-                self.out(f"d{q}{i}{j}{c} = {i + 1} * {z};")
-            self.out("}")
+                    self.uses("ser", i2 + 1, j2, c)
+                self.out(f"int64_t z{i}{j};")
+                self.product("ser", f"z{i}{j}", i + 1, j, c)
+                self.out(f"dE{i}{j}{c} = {i + 1} * z{i}{j};")
+            self.out("if (s == 0) {")
+            for i, j in nxt:
+                self.out(f"  S.stoth({n}, {i}, {j}, dE{i}{j}{c});")
+            self.out("} }")
+            self.out("S.sync();")
+        else:
+            for q, series in (("oth", "oth"), ("E", "H")):
+                self.out("{")
+                self.loaded = set()
+                for i, j in nxt:
+                    self.uses(series, i + 1, j, c)
+                    self.out("int64_t z;")
+                    self.product(series, "z", i + 1, j, c)
+                    self.out(f"d{q}{i}{j}{c} = {i + 1} * z;")
+                self.out("}")
         # each lane finishes its own momentum, lane x the density, lane y the energy
-        n = c + 1
         for i, j in nxt:
-            self.out(f"{{ const int64_t own = dmom{i}{j}{c} + S.swap(doth{j}{i}{c});")
+            other = f"S.ldown({n}, {i}, {j})" if n < 4 else f"S.swap(doth{j}{i}{c})"
+            self.out(f"{{ const int64_t own = dmom{i}{j}{c} + {other};")
             self.out(f"  const int64_t both = S.pick(drho{i}{j}{c}, dE{i}{j}{c}) + S.swap(S.pick(dE{j}{i}{c}, drho{j}{i}{c}));")
             self.out(f"  S.next({n}, {i}, {j}, fx_time<{n}>(own, third), fx_time<{n}>(both, third), {'r' if n < 4 else 'r0'}); }}")
         if n < 4:

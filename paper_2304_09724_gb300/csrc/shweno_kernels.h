@@ -40,6 +40,8 @@ void launch_step2d_quintic(const Params& P, Ctl* ctl, const double* s0, const do
                            double* o0, double* o1, const uint8_t* flag, const Scratch2D& S,
                            cudaStream_t st, cudaEvent_t* ev);
 Scratch2D carve_scratch2d(const Params& P, double* base);
+// Whether the mesh is small enough for its y-faces to run beside its x-faces (Scratch2D::aux).
+bool faces_beside(const Params& P);
 void launch_features2d(const Params& P, const Ctl* ctl, const double* s0, const double* s1,
                        float* out, cudaStream_t st);
 void launch_wdev2d(const Params& P, const Ctl* ctl, const double* s0, const double* s1,

@@ -302,6 +302,18 @@ struct CkLane {
   __device__ __forceinline__ Fx ldmom(int t, int i, int j) const { return ck_ld(at(mom0, momL, t, i, j)); }
   __device__ __forceinline__ Fx ldoth(int t, int i, int j) const { return ck_ld(at(oth0, othL, t, i, j)); }
   __device__ __forceinline__ Fx ldH(int t, int i, int j) const { return ck_ld(at(h0, lev + 57 * kCkRow, t, i, j)); }
+  // the other momentum (s = 0) or H (s = 1)
+  __device__ __forceinline__ Fx ldser(int s, int t, int i, int j) const {
+    return ck_ld(at(s ? h0 : oth0, s ? lev + 57 * kCkRow : othL, t, i, j));
+  }
+  // the lane's part of the other momentum's coefficient (i, j) of slice n, and the other lane's part
+  // of its own
+  __device__ __forceinline__ void stoth(int n, int i, int j, int64_t z) const {
+    ck_st64(othL + ck_level_row(n) * kCkRow + off[ck_pair(i, j)], z);
+  }
+  __device__ __forceinline__ int64_t ldown(int n, int i, int j) const {
+    return ck_ld64(momL + ck_level_row(n) * kCkRow + off[ck_pair(i, j)]);
+  }
   // both lanes of a point compute and write the same H
   __device__ __forceinline__ void stH(int t, int i, int j, Fx v) const { ck_st(at(h0, lev + 57 * kCkRow, t, i, j), v); }
   __device__ __forceinline__ int64_t ldE(int t, int i, int j) const {
@@ -487,10 +499,10 @@ __device__ __forceinline__ bool cell_exponents(const double (*ev)[5][SPAN], int 
 }
 
 // Order K of the thread's cell: its ends into the tables L and R (units of the cell's h).  The
-// components share one copy of the code: unrolled four times over, five orders, the pass alone
-// would overflow the instruction cache (128 KB), which the kernel then waits for.
-template <bool LIN, int K>
-__device__ __forceinline__ void cell_ends_fx(const double (*ev)[5][SPAN], int c, const CellMixFx& m,
+// components and the orders share one copy of the code: unrolled, the pass alone would overflow the
+// instruction cache (128 KB), which the kernel then waits for.
+template <bool LIN>
+__device__ __forceinline__ void cell_ends_fx(const double (*ev)[5][SPAN], int K, int c, const CellMixFx& m,
                                              int64_t (*L)[5][SEG], int64_t (*R)[5][SEG], FxRange& r) {
   const Fx u0w{85004561, 143165568}, u0s{24606583, 1002159032}, u0d{-6710886, -858993460};  // 19/30, 11/60, -1/20
 #pragma unroll 1
@@ -515,7 +527,8 @@ __device__ __forceinline__ void cell_ends_fx(const double (*ev)[5][SPAN], int c,
       hh = fx_sum<FX_C>(z);
     }
 #pragma unroll
-    for (int p = 0; p + K <= 4; ++p) {
+    for (int p = 0; p < 5; ++p) {
+      if (p + K > 4) break;
       int64_t U, V = 0;
       if (p == 0) {
         FxAcc z = fx_zero<FX_C>();
@@ -564,13 +577,16 @@ struct UpwindFx {
   int f[4], sl[4], sr[4];  // the face's exponents; right shifts of the two sides' end values
 };
 
-// Order K of the thread's face: upwinded derivatives a[q][m*5+n] in units of f.
-template <int K>
-__device__ __forceinline__ void face_order_fx(const int64_t (*L)[5][SEG], const int64_t (*R)[5][SEG], int dir,
+// Order K of the thread's face: upwinded derivatives a[q][m*5+n] in units of f (a in local memory: K is
+// a loop's).
+__device__ __forceinline__ void face_order_fx(const int64_t (*L)[5][SEG], const int64_t (*R)[5][SEG], int K, int dir,
                                               const UpwindFx& U, int64_t (&a)[4][25], FxRange& r) {
 #pragma unroll
-  for (int p = 0; p + K <= 4; ++p) {
+  for (int p = 0; p < 5; ++p) {
+    if (p + K > 4) break;
     if (p == 0 && K == 0) continue;
+    const int idx = dir == 0 ? p * 5 + K : K * 5 + p;
+    int64_t base[4];
     Fx d[4];
     FxAcc out[4];
 #pragma unroll
@@ -578,7 +594,7 @@ __device__ __forceinline__ void face_order_fx(const int64_t (*L)[5][SEG], const 
       const int64_t x = R[q][p][threadIdx.x] >> U.sl[q], y = L[q][p][threadIdx.x + 1] >> U.sr[q];
       d[q] = fx_split_wide(x - y + FX_HALF, r);
       out[q] = fx_zero<FX_C>();
-      a[q][dir == 0 ? p * 5 + K : K * 5 + p] = (U.base_left ? x : y) + ((U.c2 * (x - y)) >> 1);
+      base[q] = (U.base_left ? x : y) + ((U.c2 * (x - y)) >> 1);
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
@@ -593,7 +609,7 @@ __device__ __forceinline__ void face_order_fx(const int64_t (*L)[5][SEG], const 
       for (int q = 0; q < 4; ++q) fx_mac(out[q], al, U.r[k][q]);
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) a[q][dir == 0 ? p * 5 + K : K * 5 + p] += fx_sum<FX_C>(out[q]);
+    for (int q = 0; q < 4; ++q) a[q][idx] = base[q] + fx_sum<FX_C>(out[q]);
   }
 }
 
@@ -649,27 +665,6 @@ __device__ __forceinline__ void face_setup_fx(const Params& P, const int64_t (*L
   }
 }
 
-template <bool FLAGS, int K>
-__device__ __forceinline__ void pass_order_fx(const Params& P, const double (*ev)[5][SPAN], unsigned char* tables,
-                                              const FaceRuns& fr, const CellMixFx& m, int dir, double Ws[4],
-                                              CkLead& lead, UpwindFx& X, int64_t (&a)[4][25], FxRange& r) {
-  auto L = reinterpret_cast<int64_t(*)[5][SEG]>(tables) + (K & 1) * 4;
-  int* hs = reinterpret_cast<int*>(tables + sizeof(EndTable<4>));
-  auto R = reinterpret_cast<int64_t(*)[5][SEG]>(tables + sizeof(EndTable<4>) + 4 * SEG * sizeof(int));  // each thread its own
-  if (fr.has_cell) {
-    if (FLAGS && m.lin) cell_ends_fx<true, K>(ev, fr.col, m, L, R, r);
-    else cell_ends_fx<false, K>(ev, fr.col, m, L, R, r);
-    if (K == 0)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) hs[q * SEG + threadIdx.x] = m.h[q];
-  }
-  __syncthreads();
-  if (fr.has_face) {
-    if (K == 0) face_setup_fx(P, L, R, m.h, hs, dir, Ws, lead, X, r);
-    face_order_fx<K>(L, R, dir, X, a, r);
-  }
-}
-
 static_assert(ev_bytes<4>() + sizeof(EndTable<4>) + 4 * SEG * sizeof(int) + 4 * 5 * SEG * 8 <= kCkBytes, "tables");
 // The whole pass of the CTA; false (for all threads) if something left the format.
 template <bool FLAGS>
@@ -701,11 +696,24 @@ __device__ __forceinline__ bool second_pass_fx(const Params& P, unsigned char* s
   double Ws[4];
   CkLead lead{};
   UpwindFx X;
-  pass_order_fx<FLAGS, 0>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
-  pass_order_fx<FLAGS, 1>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
-  pass_order_fx<FLAGS, 2>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
-  pass_order_fx<FLAGS, 3>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
-  pass_order_fx<FLAGS, 4>(P, ev, tables, fr, m, dir, Ws, lead, X, a, r);
+  int* hs = reinterpret_cast<int*>(tables + sizeof(EndTable<4>));
+  auto R = reinterpret_cast<int64_t(*)[5][SEG]>(tables + sizeof(EndTable<4>) + 4 * SEG * sizeof(int));  // each thread its own
+#pragma unroll 1
+  for (int K = 0; K < 5; ++K) {  // one barrier per order, as in pass_order
+    auto L = reinterpret_cast<int64_t(*)[5][SEG]>(tables) + (K & 1) * 4;
+    if (fr.has_cell) {
+      if (FLAGS && m.lin) cell_ends_fx<true>(ev, K, fr.col, m, L, R, r);
+      else cell_ends_fx<false>(ev, K, fr.col, m, L, R, r);
+      if (K == 0)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) hs[q * SEG + threadIdx.x] = m.h[q];
+    }
+    __syncthreads();
+    if (fr.has_face) {
+      if (K == 0) face_setup_fx(P, L, R, m.h, hs, dir, Ws, lead, X, r);
+      face_order_fx(L, R, K, dir, X, a, r);
+    }
+  }
   if (__syncthreads_or(r.bad() ? 1 : 0)) return false;
   CkScale<4> S{};
   if (fr.has_face) {
@@ -771,10 +779,7 @@ __device__ __forceinline__ bool second_pass_fx(const Params& P, unsigned char* s
 template <int NC, bool FLAGS, bool Q>
 __device__ __forceinline__ void second_pass_cells(const Params& P, unsigned char* smem_raw, const FaceRuns& fr, int dir,
                                                   bool nl, double (&tc)[NC][5]) {
-  // With per-cell flags the FP64 pass stays: linear cells spare it the weights and two thirds of the
-  // end values' operations (1024 x 256 double Mach reflection, learned: 10.2 ms a step, 10.6 in
-  // fixed point; 400^2 quadrants, all cells nonlinear: 6.1 ms, 4.6 in fixed point).
-  if constexpr (NC == 4 && !Q && !FLAGS)
+  if constexpr (NC == 4 && !Q)
     if (second_pass_fx<FLAGS>(P, smem_raw, fr, dir, nl, tc)) return;
   const double(*ev)[5][SPAN] = reinterpret_cast<const double(*)[5][SPAN]>(smem_raw);
   EndTable<NC>& et = *reinterpret_cast<EndTable<NC>*>(smem_raw + ev_bytes<NC>());
@@ -1005,7 +1010,7 @@ __device__ __forceinline__ void coef2d_item(const Params& P, const StepView& sv,
   constexpr int NU = PAIR ? 2 : 1;
   const int nl = cell_flag(P, flag, ic, jr);
   const double h = ypass ? P.dy : P.dx;
-  const double sc = s == 0 ? 1.0 : (ypass ? P.dx : P.dy);  // derivative data of the pass across: h avg
+  const double sc = ypass ? P.dx : P.dy;  // set 1: derivative data of the pass across, h avg
   const size_t NX4 = P.nx + 4, NY2 = P.ny + 2, NY4 = P.ny + 4;
   double* out = ypass ? ycoef + (size_t)(jr + 1) * NX4 + (ic + 2) : xcoef + (size_t)ic * NY4 + (jr + 2);
   const size_t plane = ypass ? NY2 * NX4 : (size_t)P.nx * NY4;
@@ -1021,10 +1026,15 @@ __device__ __forceinline__ void coef2d_item(const Params& P, const StepView& sv,
       p1_coeffs_t<Q>(w[u][0], w[u][1], w[u][2], vm, v0, vp, c[u]);
     }
     first_pass_mix<Q, PAIR>(P, nl, w, c, C);
+    if (s == 1)
+#pragma unroll
+      for (int u = 0; u < NU; ++u)
+#pragma unroll
+        for (int k = 0; k < KC; ++k) C[u][k] *= sc;
 #pragma unroll
     for (int u = 0; u < NU; ++u)
 #pragma unroll
-      for (int k = 0; k < KC; ++k) out[((size_t)(s * NC + q0 + u) * KC + k) * plane] = sc * C[u][k];
+      for (int k = 0; k < KC; ++k) out[((size_t)(s * NC + q0 + u) * KC + k) * plane] = C[u][k];
   }
 }
 

@@ -28,17 +28,19 @@
 
 namespace shweno {
 
-constexpr int TY = 8;  // coef2d tile height of the one-mesh kernel
+constexpr int TY = 8;        // tile height of coef2d and update2d
+constexpr int TY_SMALL = 4;  // the same where the mesh has fewer tiles than the GPU has CTA slots: a
+                             // tile's warps then share fewer schedulers' FP64 units, or none at all
 
-template <int NC, bool Q>
-__global__ void __launch_bounds__(TX * TY) coef2d_kernel(Params P, const Ctl* __restrict__ ctl,
+template <int NC, bool Q, int TYK>
+__global__ void __launch_bounds__(TX * TYK) coef2d_kernel(Params P, const Ctl* __restrict__ ctl,
                                                          const double* s0, const double* s1,
                                                          const uint8_t* __restrict__ flag,
                                                          double* __restrict__ ycoef,
                                                          double* __restrict__ xcoef) {
-  __shared__ double tile[2 * NC][TY + 2][TX + 2];
+  __shared__ double tile[2 * NC][TYK + 2][TX + 2];
   if (!ctl->active) return;
-  coef2d_item<NC, TY, Q>(P, step_view(ctl), s0, s1, flag, ycoef, xcoef, blockIdx.z, blockIdx.x * TX - 2, blockIdx.y * TY - 2, tile,
+  coef2d_item<NC, TYK, Q>(P, step_view(ctl), s0, s1, flag, ycoef, xcoef, blockIdx.z, blockIdx.x * TX - 2, blockIdx.y * TYK - 2, tile,
                   threadIdx.x, threadIdx.y);
 }
 
@@ -82,7 +84,7 @@ __global__ void __launch_bounds__(256) update2d_kernel(Params P, Ctl* __restrict
                                                        const double* __restrict__ WC) {
   __shared__ double red[32];
   if (!ctl->active) return;
-  const int i = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * TY + threadIdx.y;
+  const int i = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   const StepView sv = step_view(ctl);
   double rate = 0.0;
   if (i < P.nx && j < P.ny) rate = update2d_cell<NC>(P, ctl, sv, sv.odd ? s1 : s0, sv.odd ? o0 : o1, FX, WX, FY, WY, WC, i, j);
@@ -122,8 +124,9 @@ static void launch_faces2d(const Params& P, Ctl* ctl, const double* s0, const do
                            const uint8_t* flag, const Scratch2D& S, cudaStream_t st, cudaEvent_t* ev) {
   dim3 xg(FaceSplit(P.nx + 1).ctas(P.ny + 1), 4), yg(FaceSplit(P.ny + 1).ctas(P.nx), 3);
   // Both kernels read the first-pass tables and write arrays of their own.  Where one does not fill
-  // the GPU (304 CTA slots) the y-faces go beside the x-faces on the handle's second stream.
-  const bool beside = !ev && S.aux && 4 * xg.x < 304;
+  // the GPU (the handle then has a second stream) the y-faces go beside the x-faces: 40^2 cells, 112
+  // and 101 us one after the other, about 115 together.
+  const bool beside = !ev && S.aux;
   cudaStream_t sy = st;
   if (beside) {
     sy = S.aux;
@@ -149,9 +152,13 @@ template <int NC, bool Q>
 static void launch_step2d_nc(const Params& P, Ctl* ctl, const double* s0, const double* s1,
                              double* o0, double* o1, const uint8_t* flag, const Scratch2D& S,
                              cudaStream_t st, cudaEvent_t* ev) {
-  dim3 cb(TX, TY), cg((P.nx + 4 + TX - 1) / TX, (P.ny + 4 + TY - 1) / TY, 4);
+  // 40^2 cells: coef2d 38 -> 29 us, update2d 27 -> 21 us with the low tiles
+  const bool small = ((P.nx + TX - 1) / TX) * ((P.ny + TY - 1) / TY) < 304;
+  const int th = small ? TY_SMALL : TY;
+  const dim3 cb(TX, th), cg((P.nx + 4 + TX - 1) / TX, (P.ny + 4 + th - 1) / th, 4);
   if (ev) cudaEventRecord(ev[0], st);
-  coef2d_kernel<NC, Q><<<cg, cb, 0, st>>>(P, ctl, s0, s1, flag, S.ycoef, S.xcoef);
+  if (small) coef2d_kernel<NC, Q, TY_SMALL><<<cg, cb, 0, st>>>(P, ctl, s0, s1, flag, S.ycoef, S.xcoef);
+  else coef2d_kernel<NC, Q, TY><<<cg, cb, 0, st>>>(P, ctl, s0, s1, flag, S.ycoef, S.xcoef);
   if (ev) cudaEventRecord(ev[1], st);
   if constexpr (NC == 4) {
     if (P.charwise) launch_faces2d<NC, true, Q>(P, ctl, s0, s1, flag, S, st, ev);
@@ -160,8 +167,9 @@ static void launch_step2d_nc(const Params& P, Ctl* ctl, const double* s0, const 
     launch_faces2d<NC, false, Q>(P, ctl, s0, s1, flag, S, st, ev);
   }
   if (ev) cudaEventRecord(ev[3], st);
-  dim3 ug((P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY);
-  update2d_kernel<NC><<<ug, cb, 0, st>>>(P, ctl, s0, s1, o0, o1, S.FX, S.WX, S.FY, S.WY, S.WC);
+  const int uh = small ? 2 : TY;
+  const dim3 ub(TX, uh), ug((P.nx + TX - 1) / TX, (P.ny + uh - 1) / uh);
+  update2d_kernel<NC><<<ug, ub, 0, st>>>(P, ctl, s0, s1, o0, o1, S.FX, S.WX, S.FY, S.WY, S.WC);
   if (ev) cudaEventRecord(ev[4], st);
 }
 
