@@ -33,12 +33,14 @@ CFL = 0.6
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 FP64_SLOTS_PER_S = 152 * 2 * 2.070e9  # FP64 thread instructions per second (DFMA, DMUL, DADD alike)
 # FP64 operations (DFMA counted as 2) and FP64 thread instructions (DFMA + DMUL + DADD, each one
-# pipe slot) per x-face point of xface2d, from ncu's instruction counters of the current kernel on
-# the 2048^2 launch, and its DRAM bytes per point from a capture at 512^2 (traffic grows in
-# proportion to the points).
-FLOPS_PER_XFACE_POINT = 5028.1
-FP64_INST_PER_XFACE_POINT = 2984.5
-DRAM_BYTES_PER_XFACE_POINT = 308.0
+# pipe slot) per x-face point of xface2d, from ncu's instruction counters of the current kernel and
+# its DRAM counters, captured at 512^2 (both grow in proportion to the points).
+# The reconstruction along the face's own line, the upwinding and the recursion run in fixed point on
+# the integer pipe (about 34,000 warp instructions, of which 570 are FP64), so these count only what
+# is left on the FP64 pipe.
+FLOPS_PER_XFACE_POINT = 890.1
+FP64_INST_PER_XFACE_POINT = 571.9
+DRAM_BYTES_PER_XFACE_POINT = 371.6
 BYTES_PER_CELL_UPDATE = 256  # 16 doubles read + 16 written per cell (ideal reuse)
 
 

@@ -295,10 +295,9 @@ const char* shweno_batch_last_error(const shweno_batch* b);
  * callers that cannot allocate device memory when they step -- real-time loops that cannot take
  * an allocation's latency or the device-wide synchronisation that freeing memory implies, and
  * frameworks that own all device memory through their own pool.  It advances one 1D state by dt
- * with the same kernels as shweno_step, without any allocation: the step's scratch (per-face
- * fluxes and states and the kernels' control block) lives in one fixed __device__ array of
- * 256 bytes + 48 (nx_max + 1) bytes (about 3.1 MB) that every GPU loading this library holds
- * until exit.
+ * with the same kernel as shweno_step, without any allocation: the kernel's control block, all the
+ * scratch a 1D step has, lives in one fixed __device__ array of 256 bytes that every GPU loading
+ * this library holds until exit.
  *   eq, nx (4 <= nx <= SHWENO_NOALLOC_MAX_NX), [x0, x1], gamma, bc_kind[2] (x-low, x-high;
  *   PERIODIC, OUTFLOW, REFLECTIVE or INFLOW; periodic on both sides or on neither),
  *   inflow[2][4] (the conserved state of an INFLOW side; may be NULL only when no side is

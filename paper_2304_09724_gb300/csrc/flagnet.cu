@@ -115,7 +115,7 @@ __global__ void mlp_forward_kernel(const float* __restrict__ params, const float
 // parameters of a column to a thread, and adds it to grad with one atomicAdd per parameter.  The
 // weights are read 16 bytes at a time (the first layer's rows padded from 22 to 24).  Bound by the
 // chain of one warp per scheduler: about 2800 multiply-adds forward and backward, 2300 in the sums;
-// 16384 samples: 28 -> 9 us (rows of 32 floats put all 32 lanes' stores on one bank before, and
+// one training step of 16384 samples: 40.5 -> 27.7 us (rows of 32 floats put all 32 lanes' stores on one bank before, and
 // every multiply-add of the sums read both factors).
 constexpr int GB = 128;
 constexpr int GROW = GB + 4;

@@ -4,10 +4,9 @@
 // solution: real-time loops that cannot take the latency of an allocation or the device-wide
 // synchronisation that freeing memory implies, and host frameworks that own every byte of device
 // memory through their own pool and forbid a library from allocating behind their back.
-// shweno_step1d_noalloc serves them: the caller passes its input and output state, and the step's
-// scratch (the per-face fluxes and interface states, plus the small control block of the step
-// kernels) lives in one file-scope __device__ array of fixed size that every GPU loading this
-// library holds until the process exits.  The call waits for its own work before it returns.
+// shweno_step1d_noalloc serves them: the caller passes its input and output state, and the control
+// block of the step kernel (all the scratch a 1D step has) lives in one file-scope __device__ array
+// of fixed size that every GPU loading this library holds until the process exits.  The call waits for its own work before it returns.
 //
 // Set-up: the device address of that array is looked up with cudaGetSymbolAddress the first
 // time the entry point runs on a device (with that device current) and cached per device for
@@ -31,9 +30,8 @@ using shweno::Params;
 
 constexpr size_t kCtlDoubles = 32;  // 256 bytes reserved for the control block
 static_assert(sizeof(Ctl) <= kCtlDoubles * sizeof(double), "control block does not fit");
-constexpr size_t kFaceDoubles = 2 * 3 * ((size_t)SHWENO_NOALLOC_MAX_NX + 1);  // F-hat and W(t+dt)
 
-static __device__ __align__(256) double g_noalloc_scratch[kCtlDoubles + kFaceDoubles];
+static __device__ __align__(256) double g_noalloc_scratch[kCtlDoubles];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;

@@ -976,7 +976,7 @@ __device__ __forceinline__ void first_pass_mix(const Params& P, int nl, const do
 // on {W, Y}, 1: y-pass on {V, Z}, 2: x-pass on {W, V}, 3: x-pass on {Y, Z}): thread (tx, ty) of a
 // TX x TYB block owns the extended cell (bx + tx, by + ty); the unit's 2 * NC fields of the tile plus a
 // one-cell halo are staged in shared memory `tile` (room for 8) by all threads first.  The units are
-// independent, so a small mesh spreads over four times as many CTAs (40^2 cells: 104 -> 30 us) and a
+// independent, so a small mesh spreads over four times as many CTAs (40^2 cells: 104 -> 38 us) and a
 // large one runs more warps per SM.  Q: reading R1', whose quintic p1 also uses the cell's own
 // derivative average; it stores six coefficients per polynomial instead of five (the scratch
 // layout's KC).

@@ -5,18 +5,21 @@
 // tangential coordinate, a second pass across the face gives all mixed derivatives
 // d^{m+n}W/dx^m dy^n (m + n <= 4) on both sides of each face quadrature point.
 //
-//   coef2d   one thread per cell (ghost ring included): the first-pass polynomials of both
-//            directions, y-pass on {W, Y} and {V, Z}, x-pass on {W, V} and {Y, Z}; the stencil
-//            tile (4 fields x NC components with a one-cell halo) is staged in shared memory.
-//   xface2d  one CTA per 128 x-faces of a row and one Gauss point (or the corner row): the CTA
-//            evaluates the y-pass polynomials of the 131 columns it needs at eta_g into shared
-//            memory, then each thread owns one face point: x-pass on both sides, leading term
+//   coef2d   one thread per cell (ghost ring included) and reconstruction: the first-pass
+//            polynomials, y-pass on {W, Y} and {V, Z}, x-pass on {W, V} and {Y, Z}, one of the
+//            four to a CTA (blockIdx.z); the stencil tile (2 fields x NC components with a
+//            one-cell halo) is staged in shared memory.
+//   xface2d  one CTA per SEG x-faces of a row, or of several rows where they are short or leave a
+//            remainder (FaceSplit), and one Gauss point (or the corner row): the CTA evaluates the
+//            y-pass polynomials of the columns it needs at eta_g into shared memory, then each
+//            thread owns one face point (the Euler recursion: two threads): x-pass, leading term
 //            (Eq. 3.6: HLLC, or the exact Burgers state), eigen-upwinded derivatives (Eq. 3.7),
 //            Cauchy-Kovalevskaya (Section 3.1), Lobatto flux (Eq. 3.8) and W(t_{n+1})
 //            (Eq. 3.11).  The corner row averages the y-pass traces of the rows below and above
 //            and keeps only W(t_{n+1}).
-//   yface2d  the same for y-faces, one CTA per 128 faces of a column.
-//   update2d one thread per cell: Eq. (3.2) and Eq. (3.10), physical check, CFL rate.
+//   yface2d  the same for y-faces along the columns.
+//   update2d one thread per cell: Eq. (3.2) and Eq. (3.10), physical check, CFL rate; the last CTA
+//            ends the step and begins the next.
 // Every kernel is instantiated for NC = 1 (scalar Burgers) and NC = 4 (Euler), and for reading
 // R1 (quartic p1) in step2d.cu and the R1' option (quintic p1) in step2d_quintic.cu, so the two
 // translation units compile in parallel.
