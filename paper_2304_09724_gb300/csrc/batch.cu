@@ -9,7 +9,7 @@
 // numbers; a CTA takes a ticket (atomicAdd on the head) and waits for that slot to be published.
 // The CTA that completes the last item of a phase pushes the next phase's items, or, after the
 // last phase, commits the step on the problem's own control block (t, step count, CFL rate --
-// exactly what end_step/begin_step do for one mesh) and pushes the next step.  Items of a
+// exactly what ctl_end and ctl_begin do for one mesh) and pushes the next step.  Items of a
 // problem are never in flight in two phases at once, so no CTA ever waits for another CTA's
 // item: the only wait is for an empty queue.  That wait is bounded (spin_limit iterations of
 // a short sleep); when it runs out the CTA raises the batch's timeout word and returns, and the
@@ -79,7 +79,7 @@ __device__ void push_items(BatchCtl* bc, long long* items, unsigned long long* s
   for (int k = 0; k < n; ++k) atomicExch(&seq[(j + k) & mask], j + k + 1);  // +1: 0 means empty
 }
 
-// Start of a step for problem p (begin_step of one mesh): returns false when the problem is done.
+// Start of a step for problem p (ctl_begin of one mesh): returns false when the problem is done.
 __device__ bool begin_problem_step(const BatchProblem& B) {
   volatile Ctl* c = B.ctl;
   if (c->err != ERR_NONE) { c->active = 0; return false; }
@@ -99,7 +99,7 @@ __device__ bool begin_problem_step(const BatchProblem& B) {
   return true;
 }
 
-// End of a step for problem p (end_step of one mesh): a step that raised an error is not
+// End of a step for problem p (ctl_end of one mesh): a step that raised an error is not
 // committed (the state stays the last good one); otherwise t, the step count and the CFL rate
 // advance and the next step begins.  Returns false when the problem is done.
 __device__ bool commit_problem_step(const BatchProblem& B) {
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(BT, HAS2D ? 1 : 3) batch_kernel(const BatchPro
         pstate[p] = 0;
         __threadfence();
         int next = ph + 1;
-        if (next == B.nphase) {  // end of the step: commit (end_step) and start the next one
+        if (next == B.nphase) {  // end of the step: commit (ctl_end) and start the next one
           const bool go = commit_problem_step(B);
           next = 0;
           if (!go) {
