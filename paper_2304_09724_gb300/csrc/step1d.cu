@@ -47,11 +47,12 @@ void launch_step1d(const Params& P, Ctl* ctl, const double* s0, const double* s1
                    double* o1, const uint8_t* flag, cudaStream_t st, cudaEvent_t* ev) {
   const int warps = (P.nx + W1D - 1) / W1D;
   if (ev) cudaEventRecord(ev[0], st);
-  if (P.ncomp == 3 && !P.charwise && warps <= 152) {
-    // one CTA of four warps per SM and W1D cells: the latency of one chain of FP64 instructions is
-    // all there is, so it is shortened.  Lax, 200 cells, whole run: 9.1 -> 5.6 ms against one warp
-    // per CTA.  The line is one CTA per SM (4560 cells): from there on a second CTA's warps share
-    // the schedulers and their FP64 units, and the one-warp form does the same work in fewer warps.
+  if (P.ncomp == 3 && !P.charwise && warps <= 304) {
+    // Four warps for W1D cells: the latency of one chain of FP64 instructions is all there is, so it
+    // is shortened.  Lax, 200 cells, whole run: 9.1 -> 5.6 ms against one warp per CTA.  The line is
+    // two CTAs per SM, as many as its registers hold, in one wave (9120 cells).  Per step, one warp per
+    // CTA / four: 4561 cells 40.3 / 33.9 us, 9120 cells 41.1 / 34.7, 18240 cells (a second wave)
+    // 43.3 / 64.7.
     if (P.quintic) step1d_small_kernel<true><<<warps, 128, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);
     else step1d_small_kernel<false><<<warps, 128, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);
   } else {

@@ -1,6 +1,6 @@
 """The 1D step kernel at the edges of its warps (30 cells each) and of its launch rules: one cell
-more or less than a warp, than two, than one CTA of four warps per SM (152 warps, 4560 cells: the
-Euler kernel changes there) and than 1216 warps (36480 cells: four warps per CTA from there on); both
+more or less than a warp, than two, than one CTA of four warps per SM (152 warps, 4560 cells), than
+two of them (304 warps, 9120 cells: the Euler kernel changes there) and than 1216 warps (36480 cells: four warps per CTA from there on); both
 equations, both readings of p1, both kinds of ends.  Against the oracle with the specification's
 tolerances (tests/gpu_util.py)."""
 import pytest
@@ -11,7 +11,7 @@ from tests import gpu_util as U
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [4, 29, 30, 31, 59, 60, 61, 119, 121, 4559, 4560, 4561, 36480, 36481])
+@pytest.mark.parametrize("n", [4, 29, 30, 31, 59, 60, 61, 119, 121, 4559, 4560, 4561, 9120, 9121, 36480, 36481])
 @pytest.mark.parametrize("eq", [WL.BURGERS, WL.EULER])
 def test_warp_and_launch_edges(n, eq):
     W, V = WL.random_smooth_1d(n, n, eq=eq)
