@@ -465,9 +465,16 @@ __device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_fac
 // own, the largest of them in [1/2, 1), 57 fraction bits (its double has 53).  The
 // end values are sums of shifted data (their coefficients are eighths, but for the value's) times the
 // cell's weights; a face brings both sides to a scale that fits its units of density and velocity
-// and upwinds there with the FP64 eigenvectors, converted.  Whatever leaves the format is noticed
-// (FxRange) and the CTA takes the FP64 pass instead: data that are not finite, eigenvectors beyond
-// 2^40 in the face's units, end values above 8 times the data, weights of 4 and more.
+// and upwinds there with the FP64 eigenvectors, converted.  What the format would hold worse than FP64
+// does is noticed and the CTA takes the FP64 pass instead: before any work, data that are not finite or
+// not of one size (cell_exponents); on the way (FxRange), face units far above the density or energy,
+// eigenvectors beyond 2^4 in them, end values above 8 times the data, weights of 4 and more.
+constexpr int FX_ABOVE = 2;       // most bits of a cell's data above the size its own state gives the component
+constexpr int FX_BELOW = 4;       // a momentum more bits than this below that size is a slow one,
+constexpr int FX_STILL = 48;      // and one more bits than this below it counts as none
+constexpr int FX_UNIT = 5;        // most bits of a face's density and energy below their units
+constexpr int FX_EL = FX_D - 53;  // most bits that the projections' scale takes off
+constexpr int FX_TINY = -300;     // least exponent of a scale
 struct CellMixFx {
   Fx A[4], B[4], C[4];
   int h[4];  // exponents of the cell's data
@@ -481,21 +488,47 @@ __device__ __forceinline__ int64_t fx_scaled(Fx x, Fx c) {
   return fx_sum<FX_C>(s);
 }
 
-// Exponents of the cell's data over all orders and its three columns; false if not finite.
-__device__ __forceinline__ bool cell_exponents(const double (*ev)[5][SPAN], int c, int h[4]) {
+// Exponents of the cell's data over all orders and its three columns; false if FP64 holds them better.
+// FP64 rounds every value by its own size, a block by its largest.
+//   A cold cell beside a hot one, which the weights cut off, would round at 2^-57 of the hot one, about
+// five times over (energy 2.5 beside 564: 1.4e-14 of the cold cell's end value, in FP64 3e-16; beside 1e12:
+// 5e-6).  So no value may be more than FX_ABOVE bits above the cell's own density, energy, or the momentum
+// sqrt(rho E) they allow: 5 * 2^-57 * 2^3 is FP64's 3e-16.
+//   A slow momentum rounds at 2^-57 of that one.  Where the energy varies along it, that is less than
+// what the rounding of the pressure, 2^-53 of rho c^2, does to it in every step; where the energy is the same in
+// all columns (the momentum across the face) or has no coefficients along the face (the other one),
+// the pressure moves nothing and FP64 would carry the momentum with all its bits.
+//   Share of the CTAs that go to FP64: vortex, smooth flows 0; quadrants 0 to 0.6 % (400^2, 300 steps); double Mach
+// reflection 10 to 12 % (1024 x 256, 400 steps), whose step takes 9.1 ms instead of 8.7 for it.  Sent there for
+// any slow momentum: quadrants 16 to 65 %.  Testing the cells: 0.3 % of the vortex step (2048^2).
+__device__ __forceinline__ bool cell_exponents(const double (*ev)[5][SPAN], int c, int dir, int h[4]) {
+  auto mag = [&](int f, int k, int col) { return fx_hi(ev[f][k][col]) & 0x7fffffff; };
+  const int n0 = fx_exp(mag(0, 0, c)), n3 = fx_exp(mag(3, 0, c)), nm = (n0 + n3 + 1) >> 1;
+  int along = 0;  // the energy's coefficients along the face
+#pragma unroll
+  for (int k = 1; k < 5; ++k) along = max(along, max(mag(3, k, c - 1), max(mag(3, k, c), mag(3, k, c + 1))));
+  const double Em = ev[3][0][c - 1], E0 = ev[3][0][c], Ep = ev[3][0][c + 1];
+  const bool even_along = fx_exp(along) < n3 - FX_STILL;
+  const bool even_across = fx_bits(Em) == fx_bits(E0) && fx_bits(Ep) == fx_bits(E0) &&
+                           fx_exp(max(mag(7, 0, c - 1), mag(7, 0, c + 1))) < n3 - FX_STILL;
   int all = 0;
+  bool ok = true;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     int top = 0;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      top = max(top, max(fx_hi(ev[q][k][c - 1]) & 0x7fffffff, max(fx_hi(ev[q][k][c]) & 0x7fffffff, fx_hi(ev[q][k][c + 1]) & 0x7fffffff)));
-      top = max(top, max(fx_hi(ev[4 + q][k][c - 1]) & 0x7fffffff, fx_hi(ev[4 + q][k][c + 1]) & 0x7fffffff));
-    }
+    for (int k = 0; k < 5; ++k)
+      top = max(top, max(max(mag(q, k, c - 1), max(mag(q, k, c), mag(q, k, c + 1))), max(mag(4 + q, k, c - 1), mag(4 + q, k, c + 1))));
     all = max(all, top);
-    h[q] = max(fx_exp(top), -300);  // an exact 0 then converts to 0
+    const int e = fx_exp(top);
+    const bool momentum = q == 1 || q == 2;
+    if (top > 0 && !(momentum && e < nm - FX_STILL)) {
+      ok = ok && e >= FX_TINY && e <= (q == 0 ? n0 : q == 3 ? n3 : nm) + FX_ABOVE;
+      if (momentum) ok = ok && !((q == 1 + dir ? even_across : even_along) && e < nm - FX_BELOW);
+    }
+    h[q] = max(e, FX_TINY);  // an exact 0 then converts to 0
   }
-  return all < 0x7ff00000;
+  return ok && all < 0x7ff00000;
 }
 
 // Order K of the thread's cell: its ends into the tables L and R (units of the cell's h).  The
@@ -639,18 +672,20 @@ __device__ __forceinline__ void face_setup_fx(const Params& P, const int64_t (*L
   int F = max(max(max(hL[1], hR[1]), max(hL[2], hR[2])) - f0, (max(hL[3], hR[3]) - f0 + 1) >> 1);
   F = max(F, max(fx_exp(lead.hu), (fx_exp(lead.hH) + 1) >> 1));
   int top = 0, el = -2000;
+  bool coarse = false;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int u = q == 0 ? 0 : q == 3 ? 2 * F : F;
     X.f[q] = f0 + u;
     X.sl[q] = min(X.f[q] - hL[q], 63);
     X.sr[q] = min(X.f[q] - hR[q], 63);
+    if (q == 0 || q == 3) coarse = coarse || X.f[q] - max(hL[q], hR[q]) > FX_UNIT;
     const int hi = max(fx_hi(lv[0][q]) & 0x7fffffff, fx_hi(lv[3][q]) & 0x7fffffff);
     top = max(top, hi);
     el = max(el, fx_exp(hi) + u);
   }
   X.el = max(el, 0);
-  if (top >= 0x7ff00000 || X.el > 40 || lead.hH >= 0x7ff00000 || lead.hu >= 0x7ff00000) {
+  if (coarse || top >= 0x7ff00000 || X.el > FX_EL || lead.hH >= 0x7ff00000 || lead.hu >= 0x7ff00000) {
     r.h |= 0x80000000u;
     X.el = 0;
   }
@@ -674,6 +709,8 @@ __device__ __forceinline__ bool second_pass_fx(const Params& P, unsigned char* s
   unsigned char* tables = smem_raw + ev_bytes<4>();
   FxRange r{0};
   CellMixFx m;
+  const bool ok = !fr.has_cell || cell_exponents(ev, fr.col, dir, m.h);
+  if (__syncthreads_or(ok ? 0 : 1)) return false;
   if (fr.has_cell) {
     CellMix<4> w;
     cell_mix<4, false>(P, ev, fr.col, FLAGS && !nl, w);
@@ -682,8 +719,7 @@ __device__ __forceinline__ bool second_pass_fx(const Params& P, unsigned char* s
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       top = max(top, max(fx_hi(w.A[q]) & 0x7fffffff, max(fx_hi(w.B[q]) & 0x7fffffff, fx_hi(w.C[q]) & 0x7fffffff)));
-    // weights are at most 1 / gam[0] unless they overflowed
-    if (!cell_exponents(ev, fr.col, m.h) || top >= 0x40100000) r.h = 0x80000000u;
+    if (top >= 0x40100000) r.h = 0x80000000u;  // weights are at most 1 / gam[0] unless they overflowed
     FxRange in{0};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
