@@ -1773,4 +1773,755 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
     S.next(4, 0, 0, fx_time<4>(own, third), fx_time<4>(both, third), r0); }
 }
 
+// ck_euler1d: 1D Euler in FP64; inputs a[q][m*5+n] and outputs tc[q][k], k = 1..4, in units of L.
+FX_FN void ck_euler1d(const double (&a)[3][25], double (&tc)[3][5], double gm1) {
+  const double inv_r0 = 1.0 / a[0][0];
+  const double w1_100 = a[1][5];
+  const double F0_100 = w1_100;
+  const double w0_001 = -(F0_100);
+  const double w1_000 = a[1][0];
+  const double w1_200 = a[1][10];
+  const double w0_100 = a[0][5];
+  const double u_000 = w1_000 * inv_r0;
+  const double u_100 = (w1_100 - w0_100 * u_000) * inv_r0;
+  const double w0_200 = a[0][10];
+  const double u_200 = (w1_200 - w0_100 * u_100 - w0_200 * u_000) * inv_r0;
+  const double mu_200 = w1_000 * u_200 + w1_100 * u_100 + w1_200 * u_000;
+  const double w2_200 = a[2][10];
+  const double p_200 = gm1 * (w2_200 - 0.5 * mu_200);
+  const double F1_200 = mu_200 + p_200;
+  const double w1_101 = -(2.0 * F1_200);
+  const double F0_101 = w1_101;
+  const double w0_002 = -((1.0 / 2.0) * F0_101);
+  const double w1_300 = a[1][15];
+  const double w0_300 = a[0][15];
+  const double u_300 = (w1_300 - w0_100 * u_200 - w0_200 * u_100 - w0_300 * u_000) * inv_r0;
+  const double mu_300 = w1_000 * u_300 + w1_100 * u_200 + w1_200 * u_100 + w1_300 * u_000;
+  const double w2_300 = a[2][15];
+  const double p_300 = gm1 * (w2_300 - 0.5 * mu_300);
+  const double F1_300 = mu_300 + p_300;
+  const double w1_201 = -(3.0 * F1_300);
+  const double mu_100 = w1_000 * u_100 + w1_100 * u_000;
+  const double w2_100 = a[2][5];
+  const double p_100 = gm1 * (w2_100 - 0.5 * mu_100);
+  const double F1_100 = mu_100 + p_100;
+  const double w1_001 = -(F1_100);
+  const double u_001 = (w1_001 - w0_001 * u_000) * inv_r0;
+  const double F0_200 = w1_200;
+  const double w0_101 = -(2.0 * F0_200);
+  const double u_101 = (w1_101 - w0_001 * u_100 - w0_100 * u_001 - w0_101 * u_000) * inv_r0;
+  const double F0_300 = w1_300;
+  const double w0_201 = -(3.0 * F0_300);
+  const double u_201 = (w1_201 - w0_001 * u_200 - w0_100 * u_101 - w0_101 * u_100 - w0_200 * u_001 - w0_201 * u_000) * inv_r0;
+  const double mu_201 = w1_000 * u_201 + w1_001 * u_200 + w1_100 * u_101 + w1_101 * u_100 + w1_200 * u_001 + w1_201 * u_000;
+  const double H_300 = w2_300 + p_300;
+  const double H_200 = w2_200 + p_200;
+  const double H_100 = w2_100 + p_100;
+  const double w2_000 = a[2][0];
+  const double mu_000 = w1_000 * u_000;
+  const double p_000 = gm1 * (w2_000 - 0.5 * mu_000);
+  const double H_000 = w2_000 + p_000;
+  const double uH_300 = u_000 * H_300 + u_100 * H_200 + u_200 * H_100 + u_300 * H_000;
+  const double F2_300 = uH_300;
+  const double w2_201 = -(3.0 * F2_300);
+  const double p_201 = gm1 * (w2_201 - 0.5 * mu_201);
+  const double F1_201 = mu_201 + p_201;
+  const double w1_102 = -(F1_201);
+  const double F0_102 = w1_102;
+  const double w0_003 = -((1.0 / 3.0) * F0_102);
+  const double w1_400 = a[1][20];
+  const double w0_400 = a[0][20];
+  const double u_400 = (w1_400 - w0_100 * u_300 - w0_200 * u_200 - w0_300 * u_100 - w0_400 * u_000) * inv_r0;
+  const double mu_400 = w1_000 * u_400 + w1_100 * u_300 + w1_200 * u_200 + w1_300 * u_100 + w1_400 * u_000;
+  const double w2_400 = a[2][20];
+  const double p_400 = gm1 * (w2_400 - 0.5 * mu_400);
+  const double F1_400 = mu_400 + p_400;
+  const double w1_301 = -(4.0 * F1_400);
+  const double F0_400 = w1_400;
+  const double w0_301 = -(4.0 * F0_400);
+  const double u_301 = (w1_301 - w0_001 * u_300 - w0_100 * u_201 - w0_101 * u_200 - w0_200 * u_101 - w0_201 * u_100 - w0_300 * u_001 - w0_301 * u_000) * inv_r0;
+  const double mu_301 = w1_000 * u_301 + w1_001 * u_300 + w1_100 * u_201 + w1_101 * u_200 + w1_200 * u_101 + w1_201 * u_100 + w1_300 * u_001 + w1_301 * u_000;
+  const double H_400 = w2_400 + p_400;
+  const double uH_400 = u_000 * H_400 + u_100 * H_300 + u_200 * H_200 + u_300 * H_100 + u_400 * H_000;
+  const double F2_400 = uH_400;
+  const double w2_301 = -(4.0 * F2_400);
+  const double p_301 = gm1 * (w2_301 - 0.5 * mu_301);
+  const double F1_301 = mu_301 + p_301;
+  const double w1_202 = -((3.0 / 2.0) * F1_301);
+  const double mu_101 = w1_000 * u_101 + w1_001 * u_100 + w1_100 * u_001 + w1_101 * u_000;
+  const double uH_200 = u_000 * H_200 + u_100 * H_100 + u_200 * H_000;
+  const double F2_200 = uH_200;
+  const double w2_101 = -(2.0 * F2_200);
+  const double p_101 = gm1 * (w2_101 - 0.5 * mu_101);
+  const double F1_101 = mu_101 + p_101;
+  const double w1_002 = -((1.0 / 2.0) * F1_101);
+  const double u_002 = (w1_002 - w0_001 * u_001 - w0_002 * u_000) * inv_r0;
+  const double F0_201 = w1_201;
+  const double w0_102 = -(F0_201);
+  const double u_102 = (w1_102 - w0_001 * u_101 - w0_002 * u_100 - w0_100 * u_002 - w0_101 * u_001 - w0_102 * u_000) * inv_r0;
+  const double F0_301 = w1_301;
+  const double w0_202 = -((3.0 / 2.0) * F0_301);
+  const double u_202 = (w1_202 - w0_001 * u_201 - w0_002 * u_200 - w0_100 * u_102 - w0_101 * u_101 - w0_102 * u_100 - w0_200 * u_002 - w0_201 * u_001 - w0_202 * u_000) * inv_r0;
+  const double mu_202 = w1_000 * u_202 + w1_001 * u_201 + w1_002 * u_200 + w1_100 * u_102 + w1_101 * u_101 + w1_102 * u_100 + w1_200 * u_002 + w1_201 * u_001 + w1_202 * u_000;
+  const double H_301 = w2_301 + p_301;
+  const double H_201 = w2_201 + p_201;
+  const double H_101 = w2_101 + p_101;
+  const double uH_100 = u_000 * H_100 + u_100 * H_000;
+  const double F2_100 = uH_100;
+  const double w2_001 = -(F2_100);
+  const double mu_001 = w1_000 * u_001 + w1_001 * u_000;
+  const double p_001 = gm1 * (w2_001 - 0.5 * mu_001);
+  const double H_001 = w2_001 + p_001;
+  const double uH_301 = u_000 * H_301 + u_001 * H_300 + u_100 * H_201 + u_101 * H_200 + u_200 * H_101 + u_201 * H_100 + u_300 * H_001 + u_301 * H_000;
+  const double F2_301 = uH_301;
+  const double w2_202 = -((3.0 / 2.0) * F2_301);
+  const double p_202 = gm1 * (w2_202 - 0.5 * mu_202);
+  const double F1_202 = mu_202 + p_202;
+  const double w1_103 = -((2.0 / 3.0) * F1_202);
+  const double F0_103 = w1_103;
+  const double w0_004 = -((1.0 / 4.0) * F0_103);
+  const double mu_102 = w1_000 * u_102 + w1_001 * u_101 + w1_002 * u_100 + w1_100 * u_002 + w1_101 * u_001 + w1_102 * u_000;
+  const double uH_201 = u_000 * H_201 + u_001 * H_200 + u_100 * H_101 + u_101 * H_100 + u_200 * H_001 + u_201 * H_000;
+  const double F2_201 = uH_201;
+  const double w2_102 = -(F2_201);
+  const double p_102 = gm1 * (w2_102 - 0.5 * mu_102);
+  const double F1_102 = mu_102 + p_102;
+  const double w1_003 = -((1.0 / 3.0) * F1_102);
+  const double u_003 = (w1_003 - w0_001 * u_002 - w0_002 * u_001 - w0_003 * u_000) * inv_r0;
+  const double F0_202 = w1_202;
+  const double w0_103 = -((2.0 / 3.0) * F0_202);
+  const double u_103 = (w1_103 - w0_001 * u_102 - w0_002 * u_101 - w0_003 * u_100 - w0_100 * u_003 - w0_101 * u_002 - w0_102 * u_001 - w0_103 * u_000) * inv_r0;
+  const double mu_103 = w1_000 * u_103 + w1_001 * u_102 + w1_002 * u_101 + w1_003 * u_100 + w1_100 * u_003 + w1_101 * u_002 + w1_102 * u_001 + w1_103 * u_000;
+  const double H_202 = w2_202 + p_202;
+  const double H_102 = w2_102 + p_102;
+  const double uH_101 = u_000 * H_101 + u_001 * H_100 + u_100 * H_001 + u_101 * H_000;
+  const double F2_101 = uH_101;
+  const double w2_002 = -((1.0 / 2.0) * F2_101);
+  const double mu_002 = w1_000 * u_002 + w1_001 * u_001 + w1_002 * u_000;
+  const double p_002 = gm1 * (w2_002 - 0.5 * mu_002);
+  const double H_002 = w2_002 + p_002;
+  const double uH_202 = u_000 * H_202 + u_001 * H_201 + u_002 * H_200 + u_100 * H_102 + u_101 * H_101 + u_102 * H_100 + u_200 * H_002 + u_201 * H_001 + u_202 * H_000;
+  const double F2_202 = uH_202;
+  const double w2_103 = -((2.0 / 3.0) * F2_202);
+  const double p_103 = gm1 * (w2_103 - 0.5 * mu_103);
+  const double F1_103 = mu_103 + p_103;
+  const double w1_004 = -((1.0 / 4.0) * F1_103);
+  const double uH_102 = u_000 * H_102 + u_001 * H_101 + u_002 * H_100 + u_100 * H_002 + u_101 * H_001 + u_102 * H_000;
+  const double F2_102 = uH_102;
+  const double w2_003 = -((1.0 / 3.0) * F2_102);
+  const double H_103 = w2_103 + p_103;
+  const double mu_003 = w1_000 * u_003 + w1_001 * u_002 + w1_002 * u_001 + w1_003 * u_000;
+  const double p_003 = gm1 * (w2_003 - 0.5 * mu_003);
+  const double H_003 = w2_003 + p_003;
+  const double uH_103 = u_000 * H_103 + u_001 * H_102 + u_002 * H_101 + u_003 * H_100 + u_100 * H_003 + u_101 * H_002 + u_102 * H_001 + u_103 * H_000;
+  const double F2_103 = uH_103;
+  const double w2_004 = -((1.0 / 4.0) * F2_103);
+  tc[0][1] = w0_001;
+  tc[0][2] = w0_002;
+  tc[0][3] = w0_003;
+  tc[0][4] = w0_004;
+  tc[1][1] = w1_001;
+  tc[1][2] = w1_002;
+  tc[1][3] = w1_003;
+  tc[1][4] = w1_004;
+  tc[2][1] = w2_001;
+  tc[2][2] = w2_002;
+  tc[2][3] = w2_003;
+  tc[2][4] = w2_004;
+}
+
+// ck_euler2d: 2D Euler in FP64; inputs a[q][m*5+n] and outputs tc[q][k], k = 1..4, in units of L.
+FX_FN void ck_euler2d(const double (&a)[4][25], double (&tc)[4][5], double gm1) {
+  const double inv_r0 = 1.0 / a[0][0];
+  const double w1_100 = a[1][5];
+  const double F0_100 = w1_100;
+  const double w2_010 = a[2][1];
+  const double G0_010 = w2_010;
+  const double w0_001 = -(F0_100 + G0_010);
+  const double w1_000 = a[1][0];
+  const double w1_200 = a[1][10];
+  const double w0_100 = a[0][5];
+  const double u_000 = w1_000 * inv_r0;
+  const double u_100 = (w1_100 - w0_100 * u_000) * inv_r0;
+  const double w0_200 = a[0][10];
+  const double u_200 = (w1_200 - w0_100 * u_100 - w0_200 * u_000) * inv_r0;
+  const double mu_200 = w1_000 * u_200 + w1_100 * u_100 + w1_200 * u_000;
+  const double w3_200 = a[3][10];
+  const double w2_000 = a[2][0];
+  const double w2_200 = a[2][10];
+  const double w2_100 = a[2][5];
+  const double v_000 = w2_000 * inv_r0;
+  const double v_100 = (w2_100 - w0_100 * v_000) * inv_r0;
+  const double v_200 = (w2_200 - w0_100 * v_100 - w0_200 * v_000) * inv_r0;
+  const double nv_200 = w2_000 * v_200 + w2_100 * v_100 + w2_200 * v_000;
+  const double p_200 = gm1 * (w3_200 - 0.5 * (mu_200 + nv_200));
+  const double F1_200 = mu_200 + p_200;
+  const double w2_110 = a[2][6];
+  const double w0_010 = a[0][1];
+  const double v_010 = (w2_010 - w0_010 * v_000) * inv_r0;
+  const double w0_110 = a[0][6];
+  const double v_110 = (w2_110 - w0_010 * v_100 - w0_100 * v_010 - w0_110 * v_000) * inv_r0;
+  const double w1_010 = a[1][1];
+  const double w1_110 = a[1][6];
+  const double mv_110 = w1_000 * v_110 + w1_010 * v_100 + w1_100 * v_010 + w1_110 * v_000;
+  const double G1_110 = mv_110;
+  const double w1_101 = -(2.0 * F1_200 + G1_110);
+  const double F0_101 = w1_101;
+  const double F2_110 = mv_110;
+  const double w2_020 = a[2][2];
+  const double w0_020 = a[0][2];
+  const double v_020 = (w2_020 - w0_010 * v_010 - w0_020 * v_000) * inv_r0;
+  const double nv_020 = w2_000 * v_020 + w2_010 * v_010 + w2_020 * v_000;
+  const double w3_020 = a[3][2];
+  const double w1_020 = a[1][2];
+  const double u_010 = (w1_010 - w0_010 * u_000) * inv_r0;
+  const double u_020 = (w1_020 - w0_010 * u_010 - w0_020 * u_000) * inv_r0;
+  const double mu_020 = w1_000 * u_020 + w1_010 * u_010 + w1_020 * u_000;
+  const double p_020 = gm1 * (w3_020 - 0.5 * (mu_020 + nv_020));
+  const double G2_020 = nv_020 + p_020;
+  const double w2_011 = -(F2_110 + 2.0 * G2_020);
+  const double G0_011 = w2_011;
+  const double w0_002 = -((1.0 / 2.0) * F0_101 + (1.0 / 2.0) * G0_011);
+  const double w1_300 = a[1][15];
+  const double w0_300 = a[0][15];
+  const double u_300 = (w1_300 - w0_100 * u_200 - w0_200 * u_100 - w0_300 * u_000) * inv_r0;
+  const double mu_300 = w1_000 * u_300 + w1_100 * u_200 + w1_200 * u_100 + w1_300 * u_000;
+  const double w3_300 = a[3][15];
+  const double w2_300 = a[2][15];
+  const double v_300 = (w2_300 - w0_100 * v_200 - w0_200 * v_100 - w0_300 * v_000) * inv_r0;
+  const double nv_300 = w2_000 * v_300 + w2_100 * v_200 + w2_200 * v_100 + w2_300 * v_000;
+  const double p_300 = gm1 * (w3_300 - 0.5 * (mu_300 + nv_300));
+  const double F1_300 = mu_300 + p_300;
+  const double w2_210 = a[2][11];
+  const double w0_210 = a[0][11];
+  const double v_210 = (w2_210 - w0_010 * v_200 - w0_100 * v_110 - w0_110 * v_100 - w0_200 * v_010 - w0_210 * v_000) * inv_r0;
+  const double w1_210 = a[1][11];
+  const double mv_210 = w1_000 * v_210 + w1_010 * v_200 + w1_100 * v_110 + w1_110 * v_100 + w1_200 * v_010 + w1_210 * v_000;
+  const double G1_210 = mv_210;
+  const double w1_201 = -(3.0 * F1_300 + G1_210);
+  const double mu_100 = w1_000 * u_100 + w1_100 * u_000;
+  const double w3_100 = a[3][5];
+  const double nv_100 = w2_000 * v_100 + w2_100 * v_000;
+  const double p_100 = gm1 * (w3_100 - 0.5 * (mu_100 + nv_100));
+  const double F1_100 = mu_100 + p_100;
+  const double mv_010 = w1_000 * v_010 + w1_010 * v_000;
+  const double G1_010 = mv_010;
+  const double w1_001 = -(F1_100 + G1_010);
+  const double u_001 = (w1_001 - w0_001 * u_000) * inv_r0;
+  const double F0_200 = w1_200;
+  const double G0_110 = w2_110;
+  const double w0_101 = -(2.0 * F0_200 + G0_110);
+  const double u_101 = (w1_101 - w0_001 * u_100 - w0_100 * u_001 - w0_101 * u_000) * inv_r0;
+  const double F0_300 = w1_300;
+  const double G0_210 = w2_210;
+  const double w0_201 = -(3.0 * F0_300 + G0_210);
+  const double u_201 = (w1_201 - w0_001 * u_200 - w0_100 * u_101 - w0_101 * u_100 - w0_200 * u_001 - w0_201 * u_000) * inv_r0;
+  const double mu_201 = w1_000 * u_201 + w1_001 * u_200 + w1_100 * u_101 + w1_101 * u_100 + w1_200 * u_001 + w1_201 * u_000;
+  const double H_300 = w3_300 + p_300;
+  const double H_200 = w3_200 + p_200;
+  const double H_100 = w3_100 + p_100;
+  const double w3_000 = a[3][0];
+  const double mu_000 = w1_000 * u_000;
+  const double nv_000 = w2_000 * v_000;
+  const double p_000 = gm1 * (w3_000 - 0.5 * (mu_000 + nv_000));
+  const double H_000 = w3_000 + p_000;
+  const double uH_300 = u_000 * H_300 + u_100 * H_200 + u_200 * H_100 + u_300 * H_000;
+  const double F3_300 = uH_300;
+  const double w3_210 = a[3][11];
+  const double u_110 = (w1_110 - w0_010 * u_100 - w0_100 * u_010 - w0_110 * u_000) * inv_r0;
+  const double u_210 = (w1_210 - w0_010 * u_200 - w0_100 * u_110 - w0_110 * u_100 - w0_200 * u_010 - w0_210 * u_000) * inv_r0;
+  const double mu_210 = w1_000 * u_210 + w1_010 * u_200 + w1_100 * u_110 + w1_110 * u_100 + w1_200 * u_010 + w1_210 * u_000;
+  const double nv_210 = w2_000 * v_210 + w2_010 * v_200 + w2_100 * v_110 + w2_110 * v_100 + w2_200 * v_010 + w2_210 * v_000;
+  const double p_210 = gm1 * (w3_210 - 0.5 * (mu_210 + nv_210));
+  const double H_210 = w3_210 + p_210;
+  const double w3_110 = a[3][6];
+  const double mu_110 = w1_000 * u_110 + w1_010 * u_100 + w1_100 * u_010 + w1_110 * u_000;
+  const double nv_110 = w2_000 * v_110 + w2_010 * v_100 + w2_100 * v_010 + w2_110 * v_000;
+  const double p_110 = gm1 * (w3_110 - 0.5 * (mu_110 + nv_110));
+  const double H_110 = w3_110 + p_110;
+  const double w3_010 = a[3][1];
+  const double mu_010 = w1_000 * u_010 + w1_010 * u_000;
+  const double nv_010 = w2_000 * v_010 + w2_010 * v_000;
+  const double p_010 = gm1 * (w3_010 - 0.5 * (mu_010 + nv_010));
+  const double H_010 = w3_010 + p_010;
+  const double vH_210 = v_000 * H_210 + v_010 * H_200 + v_100 * H_110 + v_110 * H_100 + v_200 * H_010 + v_210 * H_000;
+  const double G3_210 = vH_210;
+  const double w3_201 = -(3.0 * F3_300 + G3_210);
+  const double mv_300 = w1_000 * v_300 + w1_100 * v_200 + w1_200 * v_100 + w1_300 * v_000;
+  const double F2_300 = mv_300;
+  const double G2_210 = nv_210 + p_210;
+  const double w2_201 = -(3.0 * F2_300 + G2_210);
+  const double mv_200 = w1_000 * v_200 + w1_100 * v_100 + w1_200 * v_000;
+  const double F2_200 = mv_200;
+  const double G2_110 = nv_110 + p_110;
+  const double w2_101 = -(2.0 * F2_200 + G2_110);
+  const double mv_100 = w1_000 * v_100 + w1_100 * v_000;
+  const double F2_100 = mv_100;
+  const double G2_010 = nv_010 + p_010;
+  const double w2_001 = -(F2_100 + G2_010);
+  const double v_001 = (w2_001 - w0_001 * v_000) * inv_r0;
+  const double v_101 = (w2_101 - w0_001 * v_100 - w0_100 * v_001 - w0_101 * v_000) * inv_r0;
+  const double v_201 = (w2_201 - w0_001 * v_200 - w0_100 * v_101 - w0_101 * v_100 - w0_200 * v_001 - w0_201 * v_000) * inv_r0;
+  const double nv_201 = w2_000 * v_201 + w2_001 * v_200 + w2_100 * v_101 + w2_101 * v_100 + w2_200 * v_001 + w2_201 * v_000;
+  const double p_201 = gm1 * (w3_201 - 0.5 * (mu_201 + nv_201));
+  const double F1_201 = mu_201 + p_201;
+  const double F2_210 = mv_210;
+  const double w2_120 = a[2][7];
+  const double w0_120 = a[0][7];
+  const double v_120 = (w2_120 - w0_010 * v_110 - w0_020 * v_100 - w0_100 * v_020 - w0_110 * v_010 - w0_120 * v_000) * inv_r0;
+  const double nv_120 = w2_000 * v_120 + w2_010 * v_110 + w2_020 * v_100 + w2_100 * v_020 + w2_110 * v_010 + w2_120 * v_000;
+  const double w3_120 = a[3][7];
+  const double w1_120 = a[1][7];
+  const double u_120 = (w1_120 - w0_010 * u_110 - w0_020 * u_100 - w0_100 * u_020 - w0_110 * u_010 - w0_120 * u_000) * inv_r0;
+  const double mu_120 = w1_000 * u_120 + w1_010 * u_110 + w1_020 * u_100 + w1_100 * u_020 + w1_110 * u_010 + w1_120 * u_000;
+  const double p_120 = gm1 * (w3_120 - 0.5 * (mu_120 + nv_120));
+  const double G2_120 = nv_120 + p_120;
+  const double w2_111 = -(2.0 * F2_210 + 2.0 * G2_120);
+  const double F0_110 = w1_110;
+  const double G0_020 = w2_020;
+  const double w0_011 = -(F0_110 + 2.0 * G0_020);
+  const double v_011 = (w2_011 - w0_001 * v_010 - w0_010 * v_001 - w0_011 * v_000) * inv_r0;
+  const double F0_210 = w1_210;
+  const double G0_120 = w2_120;
+  const double w0_111 = -(2.0 * F0_210 + 2.0 * G0_120);
+  const double v_111 = (w2_111 - w0_001 * v_110 - w0_010 * v_101 - w0_011 * v_100 - w0_100 * v_011 - w0_101 * v_010 - w0_110 * v_001 - w0_111 * v_000) * inv_r0;
+  const double F1_110 = mu_110 + p_110;
+  const double mv_020 = w1_000 * v_020 + w1_010 * v_010 + w1_020 * v_000;
+  const double G1_020 = mv_020;
+  const double w1_011 = -(F1_110 + 2.0 * G1_020);
+  const double F1_210 = mu_210 + p_210;
+  const double mv_120 = w1_000 * v_120 + w1_010 * v_110 + w1_020 * v_100 + w1_100 * v_020 + w1_110 * v_010 + w1_120 * v_000;
+  const double G1_120 = mv_120;
+  const double w1_111 = -(2.0 * F1_210 + 2.0 * G1_120);
+  const double mv_111 = w1_000 * v_111 + w1_001 * v_110 + w1_010 * v_101 + w1_011 * v_100 + w1_100 * v_011 + w1_101 * v_010 + w1_110 * v_001 + w1_111 * v_000;
+  const double G1_111 = mv_111;
+  const double w1_102 = -(F1_201 + (1.0 / 2.0) * G1_111);
+  const double F0_102 = w1_102;
+  const double F2_111 = mv_111;
+  const double F2_120 = mv_120;
+  const double w2_030 = a[2][3];
+  const double w0_030 = a[0][3];
+  const double v_030 = (w2_030 - w0_010 * v_020 - w0_020 * v_010 - w0_030 * v_000) * inv_r0;
+  const double nv_030 = w2_000 * v_030 + w2_010 * v_020 + w2_020 * v_010 + w2_030 * v_000;
+  const double w3_030 = a[3][3];
+  const double w1_030 = a[1][3];
+  const double u_030 = (w1_030 - w0_010 * u_020 - w0_020 * u_010 - w0_030 * u_000) * inv_r0;
+  const double mu_030 = w1_000 * u_030 + w1_010 * u_020 + w1_020 * u_010 + w1_030 * u_000;
+  const double p_030 = gm1 * (w3_030 - 0.5 * (mu_030 + nv_030));
+  const double G2_030 = nv_030 + p_030;
+  const double w2_021 = -(F2_120 + 3.0 * G2_030);
+  const double F0_120 = w1_120;
+  const double G0_030 = w2_030;
+  const double w0_021 = -(F0_120 + 3.0 * G0_030);
+  const double v_021 = (w2_021 - w0_001 * v_020 - w0_010 * v_011 - w0_011 * v_010 - w0_020 * v_001 - w0_021 * v_000) * inv_r0;
+  const double nv_021 = w2_000 * v_021 + w2_001 * v_020 + w2_010 * v_011 + w2_011 * v_010 + w2_020 * v_001 + w2_021 * v_000;
+  const double H_120 = w3_120 + p_120;
+  const double H_020 = w3_020 + p_020;
+  const double uH_120 = u_000 * H_120 + u_010 * H_110 + u_020 * H_100 + u_100 * H_020 + u_110 * H_010 + u_120 * H_000;
+  const double F3_120 = uH_120;
+  const double H_030 = w3_030 + p_030;
+  const double vH_030 = v_000 * H_030 + v_010 * H_020 + v_020 * H_010 + v_030 * H_000;
+  const double G3_030 = vH_030;
+  const double w3_021 = -(F3_120 + 3.0 * G3_030);
+  const double F1_120 = mu_120 + p_120;
+  const double mv_030 = w1_000 * v_030 + w1_010 * v_020 + w1_020 * v_010 + w1_030 * v_000;
+  const double G1_030 = mv_030;
+  const double w1_021 = -(F1_120 + 3.0 * G1_030);
+  const double u_011 = (w1_011 - w0_001 * u_010 - w0_010 * u_001 - w0_011 * u_000) * inv_r0;
+  const double u_021 = (w1_021 - w0_001 * u_020 - w0_010 * u_011 - w0_011 * u_010 - w0_020 * u_001 - w0_021 * u_000) * inv_r0;
+  const double mu_021 = w1_000 * u_021 + w1_001 * u_020 + w1_010 * u_011 + w1_011 * u_010 + w1_020 * u_001 + w1_021 * u_000;
+  const double p_021 = gm1 * (w3_021 - 0.5 * (mu_021 + nv_021));
+  const double G2_021 = nv_021 + p_021;
+  const double w2_012 = -((1.0 / 2.0) * F2_111 + G2_021);
+  const double G0_012 = w2_012;
+  const double w0_003 = -((1.0 / 3.0) * F0_102 + (1.0 / 3.0) * G0_012);
+  const double w1_400 = a[1][20];
+  const double w0_400 = a[0][20];
+  const double u_400 = (w1_400 - w0_100 * u_300 - w0_200 * u_200 - w0_300 * u_100 - w0_400 * u_000) * inv_r0;
+  const double mu_400 = w1_000 * u_400 + w1_100 * u_300 + w1_200 * u_200 + w1_300 * u_100 + w1_400 * u_000;
+  const double w3_400 = a[3][20];
+  const double w2_400 = a[2][20];
+  const double v_400 = (w2_400 - w0_100 * v_300 - w0_200 * v_200 - w0_300 * v_100 - w0_400 * v_000) * inv_r0;
+  const double nv_400 = w2_000 * v_400 + w2_100 * v_300 + w2_200 * v_200 + w2_300 * v_100 + w2_400 * v_000;
+  const double p_400 = gm1 * (w3_400 - 0.5 * (mu_400 + nv_400));
+  const double F1_400 = mu_400 + p_400;
+  const double w2_310 = a[2][16];
+  const double w0_310 = a[0][16];
+  const double v_310 = (w2_310 - w0_010 * v_300 - w0_100 * v_210 - w0_110 * v_200 - w0_200 * v_110 - w0_210 * v_100 - w0_300 * v_010 - w0_310 * v_000) * inv_r0;
+  const double w1_310 = a[1][16];
+  const double mv_310 = w1_000 * v_310 + w1_010 * v_300 + w1_100 * v_210 + w1_110 * v_200 + w1_200 * v_110 + w1_210 * v_100 + w1_300 * v_010 + w1_310 * v_000;
+  const double G1_310 = mv_310;
+  const double w1_301 = -(4.0 * F1_400 + G1_310);
+  const double F0_400 = w1_400;
+  const double G0_310 = w2_310;
+  const double w0_301 = -(4.0 * F0_400 + G0_310);
+  const double u_301 = (w1_301 - w0_001 * u_300 - w0_100 * u_201 - w0_101 * u_200 - w0_200 * u_101 - w0_201 * u_100 - w0_300 * u_001 - w0_301 * u_000) * inv_r0;
+  const double mu_301 = w1_000 * u_301 + w1_001 * u_300 + w1_100 * u_201 + w1_101 * u_200 + w1_200 * u_101 + w1_201 * u_100 + w1_300 * u_001 + w1_301 * u_000;
+  const double H_400 = w3_400 + p_400;
+  const double uH_400 = u_000 * H_400 + u_100 * H_300 + u_200 * H_200 + u_300 * H_100 + u_400 * H_000;
+  const double F3_400 = uH_400;
+  const double w3_310 = a[3][16];
+  const double u_310 = (w1_310 - w0_010 * u_300 - w0_100 * u_210 - w0_110 * u_200 - w0_200 * u_110 - w0_210 * u_100 - w0_300 * u_010 - w0_310 * u_000) * inv_r0;
+  const double mu_310 = w1_000 * u_310 + w1_010 * u_300 + w1_100 * u_210 + w1_110 * u_200 + w1_200 * u_110 + w1_210 * u_100 + w1_300 * u_010 + w1_310 * u_000;
+  const double nv_310 = w2_000 * v_310 + w2_010 * v_300 + w2_100 * v_210 + w2_110 * v_200 + w2_200 * v_110 + w2_210 * v_100 + w2_300 * v_010 + w2_310 * v_000;
+  const double p_310 = gm1 * (w3_310 - 0.5 * (mu_310 + nv_310));
+  const double H_310 = w3_310 + p_310;
+  const double vH_310 = v_000 * H_310 + v_010 * H_300 + v_100 * H_210 + v_110 * H_200 + v_200 * H_110 + v_210 * H_100 + v_300 * H_010 + v_310 * H_000;
+  const double G3_310 = vH_310;
+  const double w3_301 = -(4.0 * F3_400 + G3_310);
+  const double mv_400 = w1_000 * v_400 + w1_100 * v_300 + w1_200 * v_200 + w1_300 * v_100 + w1_400 * v_000;
+  const double F2_400 = mv_400;
+  const double G2_310 = nv_310 + p_310;
+  const double w2_301 = -(4.0 * F2_400 + G2_310);
+  const double v_301 = (w2_301 - w0_001 * v_300 - w0_100 * v_201 - w0_101 * v_200 - w0_200 * v_101 - w0_201 * v_100 - w0_300 * v_001 - w0_301 * v_000) * inv_r0;
+  const double nv_301 = w2_000 * v_301 + w2_001 * v_300 + w2_100 * v_201 + w2_101 * v_200 + w2_200 * v_101 + w2_201 * v_100 + w2_300 * v_001 + w2_301 * v_000;
+  const double p_301 = gm1 * (w3_301 - 0.5 * (mu_301 + nv_301));
+  const double F1_301 = mu_301 + p_301;
+  const double F2_310 = mv_310;
+  const double w2_220 = a[2][12];
+  const double w0_220 = a[0][12];
+  const double v_220 = (w2_220 - w0_010 * v_210 - w0_020 * v_200 - w0_100 * v_120 - w0_110 * v_110 - w0_120 * v_100 - w0_200 * v_020 - w0_210 * v_010 - w0_220 * v_000) * inv_r0;
+  const double nv_220 = w2_000 * v_220 + w2_010 * v_210 + w2_020 * v_200 + w2_100 * v_120 + w2_110 * v_110 + w2_120 * v_100 + w2_200 * v_020 + w2_210 * v_010 + w2_220 * v_000;
+  const double w3_220 = a[3][12];
+  const double w1_220 = a[1][12];
+  const double u_220 = (w1_220 - w0_010 * u_210 - w0_020 * u_200 - w0_100 * u_120 - w0_110 * u_110 - w0_120 * u_100 - w0_200 * u_020 - w0_210 * u_010 - w0_220 * u_000) * inv_r0;
+  const double mu_220 = w1_000 * u_220 + w1_010 * u_210 + w1_020 * u_200 + w1_100 * u_120 + w1_110 * u_110 + w1_120 * u_100 + w1_200 * u_020 + w1_210 * u_010 + w1_220 * u_000;
+  const double p_220 = gm1 * (w3_220 - 0.5 * (mu_220 + nv_220));
+  const double G2_220 = nv_220 + p_220;
+  const double w2_211 = -(3.0 * F2_310 + 2.0 * G2_220);
+  const double F0_310 = w1_310;
+  const double G0_220 = w2_220;
+  const double w0_211 = -(3.0 * F0_310 + 2.0 * G0_220);
+  const double v_211 = (w2_211 - w0_001 * v_210 - w0_010 * v_201 - w0_011 * v_200 - w0_100 * v_111 - w0_101 * v_110 - w0_110 * v_101 - w0_111 * v_100 - w0_200 * v_011 - w0_201 * v_010 - w0_210 * v_001 - w0_211 * v_000) * inv_r0;
+  const double F1_310 = mu_310 + p_310;
+  const double mv_220 = w1_000 * v_220 + w1_010 * v_210 + w1_020 * v_200 + w1_100 * v_120 + w1_110 * v_110 + w1_120 * v_100 + w1_200 * v_020 + w1_210 * v_010 + w1_220 * v_000;
+  const double G1_220 = mv_220;
+  const double w1_211 = -(3.0 * F1_310 + 2.0 * G1_220);
+  const double mv_211 = w1_000 * v_211 + w1_001 * v_210 + w1_010 * v_201 + w1_011 * v_200 + w1_100 * v_111 + w1_101 * v_110 + w1_110 * v_101 + w1_111 * v_100 + w1_200 * v_011 + w1_201 * v_010 + w1_210 * v_001 + w1_211 * v_000;
+  const double G1_211 = mv_211;
+  const double w1_202 = -((3.0 / 2.0) * F1_301 + (1.0 / 2.0) * G1_211);
+  const double mu_101 = w1_000 * u_101 + w1_001 * u_100 + w1_100 * u_001 + w1_101 * u_000;
+  const double uH_200 = u_000 * H_200 + u_100 * H_100 + u_200 * H_000;
+  const double F3_200 = uH_200;
+  const double vH_110 = v_000 * H_110 + v_010 * H_100 + v_100 * H_010 + v_110 * H_000;
+  const double G3_110 = vH_110;
+  const double w3_101 = -(2.0 * F3_200 + G3_110);
+  const double nv_101 = w2_000 * v_101 + w2_001 * v_100 + w2_100 * v_001 + w2_101 * v_000;
+  const double p_101 = gm1 * (w3_101 - 0.5 * (mu_101 + nv_101));
+  const double F1_101 = mu_101 + p_101;
+  const double mv_011 = w1_000 * v_011 + w1_001 * v_010 + w1_010 * v_001 + w1_011 * v_000;
+  const double G1_011 = mv_011;
+  const double w1_002 = -((1.0 / 2.0) * F1_101 + (1.0 / 2.0) * G1_011);
+  const double u_002 = (w1_002 - w0_001 * u_001 - w0_002 * u_000) * inv_r0;
+  const double F0_201 = w1_201;
+  const double G0_111 = w2_111;
+  const double w0_102 = -(F0_201 + (1.0 / 2.0) * G0_111);
+  const double u_102 = (w1_102 - w0_001 * u_101 - w0_002 * u_100 - w0_100 * u_002 - w0_101 * u_001 - w0_102 * u_000) * inv_r0;
+  const double F0_301 = w1_301;
+  const double G0_211 = w2_211;
+  const double w0_202 = -((3.0 / 2.0) * F0_301 + (1.0 / 2.0) * G0_211);
+  const double u_202 = (w1_202 - w0_001 * u_201 - w0_002 * u_200 - w0_100 * u_102 - w0_101 * u_101 - w0_102 * u_100 - w0_200 * u_002 - w0_201 * u_001 - w0_202 * u_000) * inv_r0;
+  const double mu_202 = w1_000 * u_202 + w1_001 * u_201 + w1_002 * u_200 + w1_100 * u_102 + w1_101 * u_101 + w1_102 * u_100 + w1_200 * u_002 + w1_201 * u_001 + w1_202 * u_000;
+  const double H_301 = w3_301 + p_301;
+  const double H_201 = w3_201 + p_201;
+  const double H_101 = w3_101 + p_101;
+  const double uH_100 = u_000 * H_100 + u_100 * H_000;
+  const double F3_100 = uH_100;
+  const double vH_010 = v_000 * H_010 + v_010 * H_000;
+  const double G3_010 = vH_010;
+  const double w3_001 = -(F3_100 + G3_010);
+  const double mu_001 = w1_000 * u_001 + w1_001 * u_000;
+  const double nv_001 = w2_000 * v_001 + w2_001 * v_000;
+  const double p_001 = gm1 * (w3_001 - 0.5 * (mu_001 + nv_001));
+  const double H_001 = w3_001 + p_001;
+  const double uH_301 = u_000 * H_301 + u_001 * H_300 + u_100 * H_201 + u_101 * H_200 + u_200 * H_101 + u_201 * H_100 + u_300 * H_001 + u_301 * H_000;
+  const double F3_301 = uH_301;
+  const double uH_310 = u_000 * H_310 + u_010 * H_300 + u_100 * H_210 + u_110 * H_200 + u_200 * H_110 + u_210 * H_100 + u_300 * H_010 + u_310 * H_000;
+  const double F3_310 = uH_310;
+  const double H_220 = w3_220 + p_220;
+  const double vH_220 = v_000 * H_220 + v_010 * H_210 + v_020 * H_200 + v_100 * H_120 + v_110 * H_110 + v_120 * H_100 + v_200 * H_020 + v_210 * H_010 + v_220 * H_000;
+  const double G3_220 = vH_220;
+  const double w3_211 = -(3.0 * F3_310 + 2.0 * G3_220);
+  const double u_111 = (w1_111 - w0_001 * u_110 - w0_010 * u_101 - w0_011 * u_100 - w0_100 * u_011 - w0_101 * u_010 - w0_110 * u_001 - w0_111 * u_000) * inv_r0;
+  const double u_211 = (w1_211 - w0_001 * u_210 - w0_010 * u_201 - w0_011 * u_200 - w0_100 * u_111 - w0_101 * u_110 - w0_110 * u_101 - w0_111 * u_100 - w0_200 * u_011 - w0_201 * u_010 - w0_210 * u_001 - w0_211 * u_000) * inv_r0;
+  const double mu_211 = w1_000 * u_211 + w1_001 * u_210 + w1_010 * u_201 + w1_011 * u_200 + w1_100 * u_111 + w1_101 * u_110 + w1_110 * u_101 + w1_111 * u_100 + w1_200 * u_011 + w1_201 * u_010 + w1_210 * u_001 + w1_211 * u_000;
+  const double nv_211 = w2_000 * v_211 + w2_001 * v_210 + w2_010 * v_201 + w2_011 * v_200 + w2_100 * v_111 + w2_101 * v_110 + w2_110 * v_101 + w2_111 * v_100 + w2_200 * v_011 + w2_201 * v_010 + w2_210 * v_001 + w2_211 * v_000;
+  const double p_211 = gm1 * (w3_211 - 0.5 * (mu_211 + nv_211));
+  const double H_211 = w3_211 + p_211;
+  const double uH_210 = u_000 * H_210 + u_010 * H_200 + u_100 * H_110 + u_110 * H_100 + u_200 * H_010 + u_210 * H_000;
+  const double F3_210 = uH_210;
+  const double vH_120 = v_000 * H_120 + v_010 * H_110 + v_020 * H_100 + v_100 * H_020 + v_110 * H_010 + v_120 * H_000;
+  const double G3_120 = vH_120;
+  const double w3_111 = -(2.0 * F3_210 + 2.0 * G3_120);
+  const double mu_111 = w1_000 * u_111 + w1_001 * u_110 + w1_010 * u_101 + w1_011 * u_100 + w1_100 * u_011 + w1_101 * u_010 + w1_110 * u_001 + w1_111 * u_000;
+  const double nv_111 = w2_000 * v_111 + w2_001 * v_110 + w2_010 * v_101 + w2_011 * v_100 + w2_100 * v_011 + w2_101 * v_010 + w2_110 * v_001 + w2_111 * v_000;
+  const double p_111 = gm1 * (w3_111 - 0.5 * (mu_111 + nv_111));
+  const double H_111 = w3_111 + p_111;
+  const double uH_110 = u_000 * H_110 + u_010 * H_100 + u_100 * H_010 + u_110 * H_000;
+  const double F3_110 = uH_110;
+  const double vH_020 = v_000 * H_020 + v_010 * H_010 + v_020 * H_000;
+  const double G3_020 = vH_020;
+  const double w3_011 = -(F3_110 + 2.0 * G3_020);
+  const double mu_011 = w1_000 * u_011 + w1_001 * u_010 + w1_010 * u_001 + w1_011 * u_000;
+  const double nv_011 = w2_000 * v_011 + w2_001 * v_010 + w2_010 * v_001 + w2_011 * v_000;
+  const double p_011 = gm1 * (w3_011 - 0.5 * (mu_011 + nv_011));
+  const double H_011 = w3_011 + p_011;
+  const double vH_211 = v_000 * H_211 + v_001 * H_210 + v_010 * H_201 + v_011 * H_200 + v_100 * H_111 + v_101 * H_110 + v_110 * H_101 + v_111 * H_100 + v_200 * H_011 + v_201 * H_010 + v_210 * H_001 + v_211 * H_000;
+  const double G3_211 = vH_211;
+  const double w3_202 = -((3.0 / 2.0) * F3_301 + (1.0 / 2.0) * G3_211);
+  const double mv_301 = w1_000 * v_301 + w1_001 * v_300 + w1_100 * v_201 + w1_101 * v_200 + w1_200 * v_101 + w1_201 * v_100 + w1_300 * v_001 + w1_301 * v_000;
+  const double F2_301 = mv_301;
+  const double G2_211 = nv_211 + p_211;
+  const double w2_202 = -((3.0 / 2.0) * F2_301 + (1.0 / 2.0) * G2_211);
+  const double mv_201 = w1_000 * v_201 + w1_001 * v_200 + w1_100 * v_101 + w1_101 * v_100 + w1_200 * v_001 + w1_201 * v_000;
+  const double F2_201 = mv_201;
+  const double G2_111 = nv_111 + p_111;
+  const double w2_102 = -(F2_201 + (1.0 / 2.0) * G2_111);
+  const double mv_101 = w1_000 * v_101 + w1_001 * v_100 + w1_100 * v_001 + w1_101 * v_000;
+  const double F2_101 = mv_101;
+  const double G2_011 = nv_011 + p_011;
+  const double w2_002 = -((1.0 / 2.0) * F2_101 + (1.0 / 2.0) * G2_011);
+  const double v_002 = (w2_002 - w0_001 * v_001 - w0_002 * v_000) * inv_r0;
+  const double v_102 = (w2_102 - w0_001 * v_101 - w0_002 * v_100 - w0_100 * v_002 - w0_101 * v_001 - w0_102 * v_000) * inv_r0;
+  const double v_202 = (w2_202 - w0_001 * v_201 - w0_002 * v_200 - w0_100 * v_102 - w0_101 * v_101 - w0_102 * v_100 - w0_200 * v_002 - w0_201 * v_001 - w0_202 * v_000) * inv_r0;
+  const double nv_202 = w2_000 * v_202 + w2_001 * v_201 + w2_002 * v_200 + w2_100 * v_102 + w2_101 * v_101 + w2_102 * v_100 + w2_200 * v_002 + w2_201 * v_001 + w2_202 * v_000;
+  const double p_202 = gm1 * (w3_202 - 0.5 * (mu_202 + nv_202));
+  const double F1_202 = mu_202 + p_202;
+  const double F2_211 = mv_211;
+  const double F2_220 = mv_220;
+  const double w2_130 = a[2][8];
+  const double w0_130 = a[0][8];
+  const double v_130 = (w2_130 - w0_010 * v_120 - w0_020 * v_110 - w0_030 * v_100 - w0_100 * v_030 - w0_110 * v_020 - w0_120 * v_010 - w0_130 * v_000) * inv_r0;
+  const double nv_130 = w2_000 * v_130 + w2_010 * v_120 + w2_020 * v_110 + w2_030 * v_100 + w2_100 * v_030 + w2_110 * v_020 + w2_120 * v_010 + w2_130 * v_000;
+  const double w3_130 = a[3][8];
+  const double w1_130 = a[1][8];
+  const double u_130 = (w1_130 - w0_010 * u_120 - w0_020 * u_110 - w0_030 * u_100 - w0_100 * u_030 - w0_110 * u_020 - w0_120 * u_010 - w0_130 * u_000) * inv_r0;
+  const double mu_130 = w1_000 * u_130 + w1_010 * u_120 + w1_020 * u_110 + w1_030 * u_100 + w1_100 * u_030 + w1_110 * u_020 + w1_120 * u_010 + w1_130 * u_000;
+  const double p_130 = gm1 * (w3_130 - 0.5 * (mu_130 + nv_130));
+  const double G2_130 = nv_130 + p_130;
+  const double w2_121 = -(2.0 * F2_220 + 3.0 * G2_130);
+  const double F0_220 = w1_220;
+  const double G0_130 = w2_130;
+  const double w0_121 = -(2.0 * F0_220 + 3.0 * G0_130);
+  const double v_121 = (w2_121 - w0_001 * v_120 - w0_010 * v_111 - w0_011 * v_110 - w0_020 * v_101 - w0_021 * v_100 - w0_100 * v_021 - w0_101 * v_020 - w0_110 * v_011 - w0_111 * v_010 - w0_120 * v_001 - w0_121 * v_000) * inv_r0;
+  const double nv_121 = w2_000 * v_121 + w2_001 * v_120 + w2_010 * v_111 + w2_011 * v_110 + w2_020 * v_101 + w2_021 * v_100 + w2_100 * v_021 + w2_101 * v_020 + w2_110 * v_011 + w2_111 * v_010 + w2_120 * v_001 + w2_121 * v_000;
+  const double uH_220 = u_000 * H_220 + u_010 * H_210 + u_020 * H_200 + u_100 * H_120 + u_110 * H_110 + u_120 * H_100 + u_200 * H_020 + u_210 * H_010 + u_220 * H_000;
+  const double F3_220 = uH_220;
+  const double H_130 = w3_130 + p_130;
+  const double vH_130 = v_000 * H_130 + v_010 * H_120 + v_020 * H_110 + v_030 * H_100 + v_100 * H_030 + v_110 * H_020 + v_120 * H_010 + v_130 * H_000;
+  const double G3_130 = vH_130;
+  const double w3_121 = -(2.0 * F3_220 + 3.0 * G3_130);
+  const double F1_220 = mu_220 + p_220;
+  const double mv_130 = w1_000 * v_130 + w1_010 * v_120 + w1_020 * v_110 + w1_030 * v_100 + w1_100 * v_030 + w1_110 * v_020 + w1_120 * v_010 + w1_130 * v_000;
+  const double G1_130 = mv_130;
+  const double w1_121 = -(2.0 * F1_220 + 3.0 * G1_130);
+  const double u_121 = (w1_121 - w0_001 * u_120 - w0_010 * u_111 - w0_011 * u_110 - w0_020 * u_101 - w0_021 * u_100 - w0_100 * u_021 - w0_101 * u_020 - w0_110 * u_011 - w0_111 * u_010 - w0_120 * u_001 - w0_121 * u_000) * inv_r0;
+  const double mu_121 = w1_000 * u_121 + w1_001 * u_120 + w1_010 * u_111 + w1_011 * u_110 + w1_020 * u_101 + w1_021 * u_100 + w1_100 * u_021 + w1_101 * u_020 + w1_110 * u_011 + w1_111 * u_010 + w1_120 * u_001 + w1_121 * u_000;
+  const double p_121 = gm1 * (w3_121 - 0.5 * (mu_121 + nv_121));
+  const double G2_121 = nv_121 + p_121;
+  const double w2_112 = -(F2_211 + G2_121);
+  const double F0_111 = w1_111;
+  const double G0_021 = w2_021;
+  const double w0_012 = -((1.0 / 2.0) * F0_111 + G0_021);
+  const double v_012 = (w2_012 - w0_001 * v_011 - w0_002 * v_010 - w0_010 * v_002 - w0_011 * v_001 - w0_012 * v_000) * inv_r0;
+  const double F0_211 = w1_211;
+  const double G0_121 = w2_121;
+  const double w0_112 = -(F0_211 + G0_121);
+  const double v_112 = (w2_112 - w0_001 * v_111 - w0_002 * v_110 - w0_010 * v_102 - w0_011 * v_101 - w0_012 * v_100 - w0_100 * v_012 - w0_101 * v_011 - w0_102 * v_010 - w0_110 * v_002 - w0_111 * v_001 - w0_112 * v_000) * inv_r0;
+  const double F1_111 = mu_111 + p_111;
+  const double mv_021 = w1_000 * v_021 + w1_001 * v_020 + w1_010 * v_011 + w1_011 * v_010 + w1_020 * v_001 + w1_021 * v_000;
+  const double G1_021 = mv_021;
+  const double w1_012 = -((1.0 / 2.0) * F1_111 + G1_021);
+  const double F1_211 = mu_211 + p_211;
+  const double mv_121 = w1_000 * v_121 + w1_001 * v_120 + w1_010 * v_111 + w1_011 * v_110 + w1_020 * v_101 + w1_021 * v_100 + w1_100 * v_021 + w1_101 * v_020 + w1_110 * v_011 + w1_111 * v_010 + w1_120 * v_001 + w1_121 * v_000;
+  const double G1_121 = mv_121;
+  const double w1_112 = -(F1_211 + G1_121);
+  const double mv_112 = w1_000 * v_112 + w1_001 * v_111 + w1_002 * v_110 + w1_010 * v_102 + w1_011 * v_101 + w1_012 * v_100 + w1_100 * v_012 + w1_101 * v_011 + w1_102 * v_010 + w1_110 * v_002 + w1_111 * v_001 + w1_112 * v_000;
+  const double G1_112 = mv_112;
+  const double w1_103 = -((2.0 / 3.0) * F1_202 + (1.0 / 3.0) * G1_112);
+  const double F0_103 = w1_103;
+  const double F2_112 = mv_112;
+  const double F2_121 = mv_121;
+  const double F2_130 = mv_130;
+  const double w2_040 = a[2][4];
+  const double w0_040 = a[0][4];
+  const double v_040 = (w2_040 - w0_010 * v_030 - w0_020 * v_020 - w0_030 * v_010 - w0_040 * v_000) * inv_r0;
+  const double nv_040 = w2_000 * v_040 + w2_010 * v_030 + w2_020 * v_020 + w2_030 * v_010 + w2_040 * v_000;
+  const double w3_040 = a[3][4];
+  const double w1_040 = a[1][4];
+  const double u_040 = (w1_040 - w0_010 * u_030 - w0_020 * u_020 - w0_030 * u_010 - w0_040 * u_000) * inv_r0;
+  const double mu_040 = w1_000 * u_040 + w1_010 * u_030 + w1_020 * u_020 + w1_030 * u_010 + w1_040 * u_000;
+  const double p_040 = gm1 * (w3_040 - 0.5 * (mu_040 + nv_040));
+  const double G2_040 = nv_040 + p_040;
+  const double w2_031 = -(F2_130 + 4.0 * G2_040);
+  const double F0_130 = w1_130;
+  const double G0_040 = w2_040;
+  const double w0_031 = -(F0_130 + 4.0 * G0_040);
+  const double v_031 = (w2_031 - w0_001 * v_030 - w0_010 * v_021 - w0_011 * v_020 - w0_020 * v_011 - w0_021 * v_010 - w0_030 * v_001 - w0_031 * v_000) * inv_r0;
+  const double nv_031 = w2_000 * v_031 + w2_001 * v_030 + w2_010 * v_021 + w2_011 * v_020 + w2_020 * v_011 + w2_021 * v_010 + w2_030 * v_001 + w2_031 * v_000;
+  const double uH_130 = u_000 * H_130 + u_010 * H_120 + u_020 * H_110 + u_030 * H_100 + u_100 * H_030 + u_110 * H_020 + u_120 * H_010 + u_130 * H_000;
+  const double F3_130 = uH_130;
+  const double H_040 = w3_040 + p_040;
+  const double vH_040 = v_000 * H_040 + v_010 * H_030 + v_020 * H_020 + v_030 * H_010 + v_040 * H_000;
+  const double G3_040 = vH_040;
+  const double w3_031 = -(F3_130 + 4.0 * G3_040);
+  const double F1_130 = mu_130 + p_130;
+  const double mv_040 = w1_000 * v_040 + w1_010 * v_030 + w1_020 * v_020 + w1_030 * v_010 + w1_040 * v_000;
+  const double G1_040 = mv_040;
+  const double w1_031 = -(F1_130 + 4.0 * G1_040);
+  const double u_031 = (w1_031 - w0_001 * u_030 - w0_010 * u_021 - w0_011 * u_020 - w0_020 * u_011 - w0_021 * u_010 - w0_030 * u_001 - w0_031 * u_000) * inv_r0;
+  const double mu_031 = w1_000 * u_031 + w1_001 * u_030 + w1_010 * u_021 + w1_011 * u_020 + w1_020 * u_011 + w1_021 * u_010 + w1_030 * u_001 + w1_031 * u_000;
+  const double p_031 = gm1 * (w3_031 - 0.5 * (mu_031 + nv_031));
+  const double G2_031 = nv_031 + p_031;
+  const double w2_022 = -((1.0 / 2.0) * F2_121 + (3.0 / 2.0) * G2_031);
+  const double F0_121 = w1_121;
+  const double G0_031 = w2_031;
+  const double w0_022 = -((1.0 / 2.0) * F0_121 + (3.0 / 2.0) * G0_031);
+  const double v_022 = (w2_022 - w0_001 * v_021 - w0_002 * v_020 - w0_010 * v_012 - w0_011 * v_011 - w0_012 * v_010 - w0_020 * v_002 - w0_021 * v_001 - w0_022 * v_000) * inv_r0;
+  const double nv_022 = w2_000 * v_022 + w2_001 * v_021 + w2_002 * v_020 + w2_010 * v_012 + w2_011 * v_011 + w2_012 * v_010 + w2_020 * v_002 + w2_021 * v_001 + w2_022 * v_000;
+  const double H_121 = w3_121 + p_121;
+  const double H_021 = w3_021 + p_021;
+  const double uH_121 = u_000 * H_121 + u_001 * H_120 + u_010 * H_111 + u_011 * H_110 + u_020 * H_101 + u_021 * H_100 + u_100 * H_021 + u_101 * H_020 + u_110 * H_011 + u_111 * H_010 + u_120 * H_001 + u_121 * H_000;
+  const double F3_121 = uH_121;
+  const double H_031 = w3_031 + p_031;
+  const double vH_031 = v_000 * H_031 + v_001 * H_030 + v_010 * H_021 + v_011 * H_020 + v_020 * H_011 + v_021 * H_010 + v_030 * H_001 + v_031 * H_000;
+  const double G3_031 = vH_031;
+  const double w3_022 = -((1.0 / 2.0) * F3_121 + (3.0 / 2.0) * G3_031);
+  const double F1_121 = mu_121 + p_121;
+  const double mv_031 = w1_000 * v_031 + w1_001 * v_030 + w1_010 * v_021 + w1_011 * v_020 + w1_020 * v_011 + w1_021 * v_010 + w1_030 * v_001 + w1_031 * v_000;
+  const double G1_031 = mv_031;
+  const double w1_022 = -((1.0 / 2.0) * F1_121 + (3.0 / 2.0) * G1_031);
+  const double u_012 = (w1_012 - w0_001 * u_011 - w0_002 * u_010 - w0_010 * u_002 - w0_011 * u_001 - w0_012 * u_000) * inv_r0;
+  const double u_022 = (w1_022 - w0_001 * u_021 - w0_002 * u_020 - w0_010 * u_012 - w0_011 * u_011 - w0_012 * u_010 - w0_020 * u_002 - w0_021 * u_001 - w0_022 * u_000) * inv_r0;
+  const double mu_022 = w1_000 * u_022 + w1_001 * u_021 + w1_002 * u_020 + w1_010 * u_012 + w1_011 * u_011 + w1_012 * u_010 + w1_020 * u_002 + w1_021 * u_001 + w1_022 * u_000;
+  const double p_022 = gm1 * (w3_022 - 0.5 * (mu_022 + nv_022));
+  const double G2_022 = nv_022 + p_022;
+  const double w2_013 = -((1.0 / 3.0) * F2_112 + (2.0 / 3.0) * G2_022);
+  const double G0_013 = w2_013;
+  const double w0_004 = -((1.0 / 4.0) * F0_103 + (1.0 / 4.0) * G0_013);
+  const double mu_102 = w1_000 * u_102 + w1_001 * u_101 + w1_002 * u_100 + w1_100 * u_002 + w1_101 * u_001 + w1_102 * u_000;
+  const double uH_201 = u_000 * H_201 + u_001 * H_200 + u_100 * H_101 + u_101 * H_100 + u_200 * H_001 + u_201 * H_000;
+  const double F3_201 = uH_201;
+  const double vH_111 = v_000 * H_111 + v_001 * H_110 + v_010 * H_101 + v_011 * H_100 + v_100 * H_011 + v_101 * H_010 + v_110 * H_001 + v_111 * H_000;
+  const double G3_111 = vH_111;
+  const double w3_102 = -(F3_201 + (1.0 / 2.0) * G3_111);
+  const double nv_102 = w2_000 * v_102 + w2_001 * v_101 + w2_002 * v_100 + w2_100 * v_002 + w2_101 * v_001 + w2_102 * v_000;
+  const double p_102 = gm1 * (w3_102 - 0.5 * (mu_102 + nv_102));
+  const double F1_102 = mu_102 + p_102;
+  const double mv_012 = w1_000 * v_012 + w1_001 * v_011 + w1_002 * v_010 + w1_010 * v_002 + w1_011 * v_001 + w1_012 * v_000;
+  const double G1_012 = mv_012;
+  const double w1_003 = -((1.0 / 3.0) * F1_102 + (1.0 / 3.0) * G1_012);
+  const double u_003 = (w1_003 - w0_001 * u_002 - w0_002 * u_001 - w0_003 * u_000) * inv_r0;
+  const double F0_202 = w1_202;
+  const double G0_112 = w2_112;
+  const double w0_103 = -((2.0 / 3.0) * F0_202 + (1.0 / 3.0) * G0_112);
+  const double u_103 = (w1_103 - w0_001 * u_102 - w0_002 * u_101 - w0_003 * u_100 - w0_100 * u_003 - w0_101 * u_002 - w0_102 * u_001 - w0_103 * u_000) * inv_r0;
+  const double mu_103 = w1_000 * u_103 + w1_001 * u_102 + w1_002 * u_101 + w1_003 * u_100 + w1_100 * u_003 + w1_101 * u_002 + w1_102 * u_001 + w1_103 * u_000;
+  const double H_202 = w3_202 + p_202;
+  const double H_102 = w3_102 + p_102;
+  const double uH_101 = u_000 * H_101 + u_001 * H_100 + u_100 * H_001 + u_101 * H_000;
+  const double F3_101 = uH_101;
+  const double vH_011 = v_000 * H_011 + v_001 * H_010 + v_010 * H_001 + v_011 * H_000;
+  const double G3_011 = vH_011;
+  const double w3_002 = -((1.0 / 2.0) * F3_101 + (1.0 / 2.0) * G3_011);
+  const double mu_002 = w1_000 * u_002 + w1_001 * u_001 + w1_002 * u_000;
+  const double nv_002 = w2_000 * v_002 + w2_001 * v_001 + w2_002 * v_000;
+  const double p_002 = gm1 * (w3_002 - 0.5 * (mu_002 + nv_002));
+  const double H_002 = w3_002 + p_002;
+  const double uH_202 = u_000 * H_202 + u_001 * H_201 + u_002 * H_200 + u_100 * H_102 + u_101 * H_101 + u_102 * H_100 + u_200 * H_002 + u_201 * H_001 + u_202 * H_000;
+  const double F3_202 = uH_202;
+  const double uH_211 = u_000 * H_211 + u_001 * H_210 + u_010 * H_201 + u_011 * H_200 + u_100 * H_111 + u_101 * H_110 + u_110 * H_101 + u_111 * H_100 + u_200 * H_011 + u_201 * H_010 + u_210 * H_001 + u_211 * H_000;
+  const double F3_211 = uH_211;
+  const double vH_121 = v_000 * H_121 + v_001 * H_120 + v_010 * H_111 + v_011 * H_110 + v_020 * H_101 + v_021 * H_100 + v_100 * H_021 + v_101 * H_020 + v_110 * H_011 + v_111 * H_010 + v_120 * H_001 + v_121 * H_000;
+  const double G3_121 = vH_121;
+  const double w3_112 = -(F3_211 + G3_121);
+  const double u_112 = (w1_112 - w0_001 * u_111 - w0_002 * u_110 - w0_010 * u_102 - w0_011 * u_101 - w0_012 * u_100 - w0_100 * u_012 - w0_101 * u_011 - w0_102 * u_010 - w0_110 * u_002 - w0_111 * u_001 - w0_112 * u_000) * inv_r0;
+  const double mu_112 = w1_000 * u_112 + w1_001 * u_111 + w1_002 * u_110 + w1_010 * u_102 + w1_011 * u_101 + w1_012 * u_100 + w1_100 * u_012 + w1_101 * u_011 + w1_102 * u_010 + w1_110 * u_002 + w1_111 * u_001 + w1_112 * u_000;
+  const double nv_112 = w2_000 * v_112 + w2_001 * v_111 + w2_002 * v_110 + w2_010 * v_102 + w2_011 * v_101 + w2_012 * v_100 + w2_100 * v_012 + w2_101 * v_011 + w2_102 * v_010 + w2_110 * v_002 + w2_111 * v_001 + w2_112 * v_000;
+  const double p_112 = gm1 * (w3_112 - 0.5 * (mu_112 + nv_112));
+  const double H_112 = w3_112 + p_112;
+  const double uH_111 = u_000 * H_111 + u_001 * H_110 + u_010 * H_101 + u_011 * H_100 + u_100 * H_011 + u_101 * H_010 + u_110 * H_001 + u_111 * H_000;
+  const double F3_111 = uH_111;
+  const double vH_021 = v_000 * H_021 + v_001 * H_020 + v_010 * H_011 + v_011 * H_010 + v_020 * H_001 + v_021 * H_000;
+  const double G3_021 = vH_021;
+  const double w3_012 = -((1.0 / 2.0) * F3_111 + G3_021);
+  const double mu_012 = w1_000 * u_012 + w1_001 * u_011 + w1_002 * u_010 + w1_010 * u_002 + w1_011 * u_001 + w1_012 * u_000;
+  const double nv_012 = w2_000 * v_012 + w2_001 * v_011 + w2_002 * v_010 + w2_010 * v_002 + w2_011 * v_001 + w2_012 * v_000;
+  const double p_012 = gm1 * (w3_012 - 0.5 * (mu_012 + nv_012));
+  const double H_012 = w3_012 + p_012;
+  const double vH_112 = v_000 * H_112 + v_001 * H_111 + v_002 * H_110 + v_010 * H_102 + v_011 * H_101 + v_012 * H_100 + v_100 * H_012 + v_101 * H_011 + v_102 * H_010 + v_110 * H_002 + v_111 * H_001 + v_112 * H_000;
+  const double G3_112 = vH_112;
+  const double w3_103 = -((2.0 / 3.0) * F3_202 + (1.0 / 3.0) * G3_112);
+  const double mv_202 = w1_000 * v_202 + w1_001 * v_201 + w1_002 * v_200 + w1_100 * v_102 + w1_101 * v_101 + w1_102 * v_100 + w1_200 * v_002 + w1_201 * v_001 + w1_202 * v_000;
+  const double F2_202 = mv_202;
+  const double G2_112 = nv_112 + p_112;
+  const double w2_103 = -((2.0 / 3.0) * F2_202 + (1.0 / 3.0) * G2_112);
+  const double mv_102 = w1_000 * v_102 + w1_001 * v_101 + w1_002 * v_100 + w1_100 * v_002 + w1_101 * v_001 + w1_102 * v_000;
+  const double F2_102 = mv_102;
+  const double G2_012 = nv_012 + p_012;
+  const double w2_003 = -((1.0 / 3.0) * F2_102 + (1.0 / 3.0) * G2_012);
+  const double v_003 = (w2_003 - w0_001 * v_002 - w0_002 * v_001 - w0_003 * v_000) * inv_r0;
+  const double v_103 = (w2_103 - w0_001 * v_102 - w0_002 * v_101 - w0_003 * v_100 - w0_100 * v_003 - w0_101 * v_002 - w0_102 * v_001 - w0_103 * v_000) * inv_r0;
+  const double nv_103 = w2_000 * v_103 + w2_001 * v_102 + w2_002 * v_101 + w2_003 * v_100 + w2_100 * v_003 + w2_101 * v_002 + w2_102 * v_001 + w2_103 * v_000;
+  const double p_103 = gm1 * (w3_103 - 0.5 * (mu_103 + nv_103));
+  const double F1_103 = mu_103 + p_103;
+  const double F0_112 = w1_112;
+  const double G0_022 = w2_022;
+  const double w0_013 = -((1.0 / 3.0) * F0_112 + (2.0 / 3.0) * G0_022);
+  const double v_013 = (w2_013 - w0_001 * v_012 - w0_002 * v_011 - w0_003 * v_010 - w0_010 * v_003 - w0_011 * v_002 - w0_012 * v_001 - w0_013 * v_000) * inv_r0;
+  const double F1_112 = mu_112 + p_112;
+  const double mv_022 = w1_000 * v_022 + w1_001 * v_021 + w1_002 * v_020 + w1_010 * v_012 + w1_011 * v_011 + w1_012 * v_010 + w1_020 * v_002 + w1_021 * v_001 + w1_022 * v_000;
+  const double G1_022 = mv_022;
+  const double w1_013 = -((1.0 / 3.0) * F1_112 + (2.0 / 3.0) * G1_022);
+  const double mv_013 = w1_000 * v_013 + w1_001 * v_012 + w1_002 * v_011 + w1_003 * v_010 + w1_010 * v_003 + w1_011 * v_002 + w1_012 * v_001 + w1_013 * v_000;
+  const double G1_013 = mv_013;
+  const double w1_004 = -((1.0 / 4.0) * F1_103 + (1.0 / 4.0) * G1_013);
+  const double mv_103 = w1_000 * v_103 + w1_001 * v_102 + w1_002 * v_101 + w1_003 * v_100 + w1_100 * v_003 + w1_101 * v_002 + w1_102 * v_001 + w1_103 * v_000;
+  const double F2_103 = mv_103;
+  const double nv_013 = w2_000 * v_013 + w2_001 * v_012 + w2_002 * v_011 + w2_003 * v_010 + w2_010 * v_003 + w2_011 * v_002 + w2_012 * v_001 + w2_013 * v_000;
+  const double uH_112 = u_000 * H_112 + u_001 * H_111 + u_002 * H_110 + u_010 * H_102 + u_011 * H_101 + u_012 * H_100 + u_100 * H_012 + u_101 * H_011 + u_102 * H_010 + u_110 * H_002 + u_111 * H_001 + u_112 * H_000;
+  const double F3_112 = uH_112;
+  const double H_022 = w3_022 + p_022;
+  const double vH_022 = v_000 * H_022 + v_001 * H_021 + v_002 * H_020 + v_010 * H_012 + v_011 * H_011 + v_012 * H_010 + v_020 * H_002 + v_021 * H_001 + v_022 * H_000;
+  const double G3_022 = vH_022;
+  const double w3_013 = -((1.0 / 3.0) * F3_112 + (2.0 / 3.0) * G3_022);
+  const double u_013 = (w1_013 - w0_001 * u_012 - w0_002 * u_011 - w0_003 * u_010 - w0_010 * u_003 - w0_011 * u_002 - w0_012 * u_001 - w0_013 * u_000) * inv_r0;
+  const double mu_013 = w1_000 * u_013 + w1_001 * u_012 + w1_002 * u_011 + w1_003 * u_010 + w1_010 * u_003 + w1_011 * u_002 + w1_012 * u_001 + w1_013 * u_000;
+  const double p_013 = gm1 * (w3_013 - 0.5 * (mu_013 + nv_013));
+  const double G2_013 = nv_013 + p_013;
+  const double w2_004 = -((1.0 / 4.0) * F2_103 + (1.0 / 4.0) * G2_013);
+  const double uH_102 = u_000 * H_102 + u_001 * H_101 + u_002 * H_100 + u_100 * H_002 + u_101 * H_001 + u_102 * H_000;
+  const double F3_102 = uH_102;
+  const double vH_012 = v_000 * H_012 + v_001 * H_011 + v_002 * H_010 + v_010 * H_002 + v_011 * H_001 + v_012 * H_000;
+  const double G3_012 = vH_012;
+  const double w3_003 = -((1.0 / 3.0) * F3_102 + (1.0 / 3.0) * G3_012);
+  const double H_103 = w3_103 + p_103;
+  const double mu_003 = w1_000 * u_003 + w1_001 * u_002 + w1_002 * u_001 + w1_003 * u_000;
+  const double nv_003 = w2_000 * v_003 + w2_001 * v_002 + w2_002 * v_001 + w2_003 * v_000;
+  const double p_003 = gm1 * (w3_003 - 0.5 * (mu_003 + nv_003));
+  const double H_003 = w3_003 + p_003;
+  const double uH_103 = u_000 * H_103 + u_001 * H_102 + u_002 * H_101 + u_003 * H_100 + u_100 * H_003 + u_101 * H_002 + u_102 * H_001 + u_103 * H_000;
+  const double F3_103 = uH_103;
+  const double H_013 = w3_013 + p_013;
+  const double vH_013 = v_000 * H_013 + v_001 * H_012 + v_002 * H_011 + v_003 * H_010 + v_010 * H_003 + v_011 * H_002 + v_012 * H_001 + v_013 * H_000;
+  const double G3_013 = vH_013;
+  const double w3_004 = -((1.0 / 4.0) * F3_103 + (1.0 / 4.0) * G3_013);
+  tc[0][1] = w0_001;
+  tc[0][2] = w0_002;
+  tc[0][3] = w0_003;
+  tc[0][4] = w0_004;
+  tc[1][1] = w1_001;
+  tc[1][2] = w1_002;
+  tc[1][3] = w1_003;
+  tc[1][4] = w1_004;
+  tc[2][1] = w2_001;
+  tc[2][2] = w2_002;
+  tc[2][3] = w2_003;
+  tc[2][4] = w2_004;
+  tc[3][1] = w3_001;
+  tc[3][2] = w3_002;
+  tc[3][3] = w3_003;
+  tc[3][4] = w3_004;
+}
+
 }  // namespace shweno

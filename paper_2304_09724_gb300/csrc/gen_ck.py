@@ -1,6 +1,6 @@
 """Writes the Cauchy-Kovalevskaya (Lax-Wendroff) procedure of Eq. (2.6) and Section 3.1 as
 straight-line CUDA in block fixed point (see fixed.cuh): 1D and 2D Burgers and 1D Euler for one
-thread, 2D Euler for two lanes.
+thread, 2D Euler for two lanes; and 1D and 2D Euler in FP64.
 
 Method.  At an interface quadrature point the solution is a truncated power series in
 (X, Y, t), X = (x - x_p)/dx and Y = (y - y_p)/dy, with normalised coefficients
@@ -142,6 +142,168 @@ class GenFixed:
         ]
         if any(", r0)" in x for x in self.lines):
             head.append("  FxRange r0{0};  // leading coefficients are in range by their scales")
+        return "\n".join(head + self.lines + outs + ["}"])
+
+
+class Gen:
+    """The Euler recursion in FP64, for the points whose coefficients block fixed point would hold worse: the
+    same walk as GenFixed, every coefficient a double."""
+
+    def __init__(self, dim, eq):
+        self.dim, self.eq = dim, eq
+        self.lines = []
+        self.done = {}
+        self.ncomp = 3 if dim == 1 else 4
+
+    def idx_ok(self, m, n, k):
+        return m >= 0 and n >= 0 and k >= 0 and m + n + k <= 4 and (self.dim == 2 or n == 0)
+
+    def var(self, name, m, n, k):
+        """C expression for coefficient (m,n,k) of series `name`; emits code on first use."""
+        if not self.idx_ok(m, n, k):
+            return None
+        key = (name, m, n, k)
+        if key in self.done:
+            return self.done[key]
+        expr = self.build(name, m, n, k)
+        if expr is None:
+            self.done[key] = None
+            return None
+        v = f"{name}_{m}{n}{k}"
+        self.lines.append(f"  const double {v} = {expr};")
+        self.done[key] = v
+        return v
+
+    @staticmethod
+    def times(i, k, v):
+        """(i / k) v"""
+        return v if i == k else f"{i // k}.0 * {v}" if i % k == 0 else f"({i}.0 / {k}.0) * {v}"
+
+    # ---- series definitions ----
+    def state_names(self):
+        return ["w0", "w1", "w2"] if self.dim == 1 else ["w0", "w1", "w2", "w3"]
+
+    def build(self, name, m, n, k):
+        W = self.state_names()
+        if name in W:
+            q = W.index(name)
+            if k == 0:
+                return f"a[{q}][{m * 5 + n}]"
+            F = self.var(f"F{q}", m + 1, n, k - 1)
+            G = self.var(f"G{q}", m, n + 1, k - 1) if self.dim == 2 else None
+            terms = []
+            if F is not None:
+                terms.append(self.times(m + 1, k, F))
+            if G is not None:
+                terms.append(self.times(n + 1, k, G))
+            if not terms:
+                return None
+            return "-(" + " + ".join(terms) + ")"
+        if self.dim == 1:
+            r, mx, E = W
+            if name == "u":
+                return self.quotient(mx, r, "u", m, n, k)
+            if name == "mu":
+                return self.product(mx, "u", m, n, k)
+            if name == "p":
+                e = self.var(E, m, n, k)
+                mu = self.var("mu", m, n, k)
+                return f"gm1 * ({e} - 0.5 * {mu})"
+            if name == "H":
+                return f"{self.var(E, m, n, k)} + {self.var('p', m, n, k)}"
+            if name == "uH":
+                return self.product("u", "H", m, n, k)
+            if name == "F0":
+                return self.var(mx, m, n, k)
+            if name == "F1":
+                return f"{self.var('mu', m, n, k)} + {self.var('p', m, n, k)}"
+            if name == "F2":
+                return self.var("uH", m, n, k)
+            raise KeyError(name)
+        r, mx, my, E = W
+        if name == "u":
+            return self.quotient(mx, r, "u", m, n, k)
+        if name == "v":
+            return self.quotient(my, r, "v", m, n, k)
+        if name == "mu":
+            return self.product(mx, "u", m, n, k)
+        if name == "mv":
+            return self.product(mx, "v", m, n, k)
+        if name == "nv":
+            return self.product(my, "v", m, n, k)
+        if name == "p":
+            return f"gm1 * ({self.var(E, m, n, k)} - 0.5 * ({self.var('mu', m, n, k)} + {self.var('nv', m, n, k)}))"
+        if name == "H":
+            return f"{self.var(E, m, n, k)} + {self.var('p', m, n, k)}"
+        if name == "uH":
+            return self.product("u", "H", m, n, k)
+        if name == "vH":
+            return self.product("v", "H", m, n, k)
+        if name == "F0":
+            return self.var(mx, m, n, k)
+        if name == "F1":
+            return f"{self.var('mu', m, n, k)} + {self.var('p', m, n, k)}"
+        if name == "F2":
+            return self.var("mv", m, n, k)
+        if name == "F3":
+            return self.var("uH", m, n, k)
+        if name == "G0":
+            return self.var(my, m, n, k)
+        if name == "G1":
+            return self.var("mv", m, n, k)
+        if name == "G2":
+            return f"{self.var('nv', m, n, k)} + {self.var('p', m, n, k)}"
+        if name == "G3":
+            return self.var("vH", m, n, k)
+        raise KeyError(name)
+
+    def sub_indices(self, m, n, k):
+        for p in range(m + 1):
+            for q in range(n + 1):
+                for t in range(k + 1):
+                    yield p, q, t
+
+    def product(self, A, B, m, n, k):
+        terms = []
+        for p, q, t in self.sub_indices(m, n, k):
+            a = self.var(A, p, q, t)
+            b = self.var(B, m - p, n - q, k - t)
+            if a is not None and b is not None:
+                terms.append(f"{a} * {b}")
+        if not terms:
+            return None
+        return " + ".join(terms)
+
+    def quotient(self, A, B, name, m, n, k):
+        """name = A / B; name[g] = (A[g] - sum_{0 < b <= g} B[b] name[g - b]) / B[0], the sum
+        subtracted term by term."""
+        a = self.var(A, m, n, k)
+        terms = []
+        for p, q, t in self.sub_indices(m, n, k):
+            if (p, q, t) == (0, 0, 0):
+                continue
+            b = self.var(B, p, q, t)
+            c = self.var(name, m - p, n - q, k - t)
+            if b is not None and c is not None:
+                terms.append(f"{b} * {c}")
+        num = a if a is not None else "0.0"
+        if terms:
+            # a - t1 - t2 - ... left to right: every step contracts to one fused multiply-add
+            num = "(" + num + "".join(f" - {t}" for t in terms) + ")"
+        return f"{num} * inv_r0"
+
+    def emit(self, fname):
+        W = self.state_names()
+        outs = []
+        for q in range(self.ncomp):
+            for k in range(1, 5):
+                outs.append(f"  tc[{q}][{k}] = {self.var(W[q], 0, 0, k)};")
+        nc = self.ncomp
+        head = [
+            f"// {fname}: {self.dim}D Euler in FP64; inputs a[q][m*5+n] and outputs tc[q][k], k = 1..4, in units of L.",
+            f"FX_FN void {fname}(const double (&a)[{nc}][25], double (&tc)[{nc}][5], double gm1) {{",
+            "  const double inv_r0 = 1.0 / a[0][0];",
+        ]
         return "\n".join(head + self.lines + outs + ["}"])
 
 
@@ -321,6 +483,8 @@ def main():
               "FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxRange& r) {",
               "  FxRange r0{0};  // leading coefficients are in range by their scales",
               GenLane().run(), "}", ""]
+    for dim in (1, 2):
+        parts += [Gen(dim, "euler").emit(f"ck_euler{dim}d"), ""]
     parts.append("}  // namespace shweno")
     out = os.path.join(os.path.dirname(os.path.abspath(__file__)), "ck_fixed_generated.cuh")
     with open(out, "w") as f:

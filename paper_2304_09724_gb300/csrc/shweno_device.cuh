@@ -592,6 +592,7 @@ __device__ __forceinline__ CkLead prim_lead(const Prim& P) {
   l.hu = fx_hi(P.u) & 0x7fffffff;
   if (NC == 4) l.hu = fx_max(l.hu, fx_hi(P.v) & 0x7fffffff);
   l.hH = fx_hi(P.H) & 0x7fffffff;
+  l.hc = fx_hi(P.c) & 0x7fffffff;
   return l;
 }
 

@@ -139,7 +139,7 @@ __device__ __forceinline__ void face1d(const Params& P, const double l[NC][5], c
   double tc[NC][5];
 #pragma unroll
   for (int q = 0; q < NC; ++q) a[q][0] = tc[q][0] = Ws[q];
-  ck_fixed<NC, 1>(a, U.lead, P.ck.K, tc);
+  ck_fixed<NC, 1>(a, U.lead, P.ck, tc);
 #pragma unroll
   for (int q = 0; q < NC; ++q) Fh[q] = 0.0;
 #pragma unroll
@@ -278,7 +278,7 @@ __device__ __forceinline__ double step1d_cta(const Params& P, Ctl* ctl, const do
 #pragma unroll
       for (int m = 1; m < 5; ++m) a[q][m * 5] = S.a[q][m - 1][lane];
     }
-    ck_fixed<NC, 1>(a, U.lead, P.ck.K, tc);
+    ck_fixed<NC, 1>(a, U.lead, P.ck, tc);
     lobatto_node<NC>(tc, dt * P.ck.iL, P.gamma, w, W, F);
 #pragma unroll
     for (int q = 0; q < NC; ++q) {

@@ -439,18 +439,45 @@ __device__ __forceinline__ void ck_points4(const Params& P, int npt, bool has_fa
     }
 }
 
-// The same from FP64 coefficients a[q][m*5+n] in cell units, Burgers or Euler.
+// The same in FP64, one thread a point, from the coefficients a[q][m*5+n] in units of L.
+__device__ __forceinline__ void ck_points64(const Params& P, bool has_face, const double (&a)[4][25], double (&tc)[4][5]) {
+  if (!has_face) return;
+  ck_euler2d(a, tc, P.ck.gm1);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) tc[q][0] = a[q][0];
+}
+
+// Whether a point of a face across direction dir has a slow momentum along the face that FP64 holds better (see
+// cell_exponents).
+__device__ __forceinline__ bool ck_coarse2d(const double (&a)[4][25], int dir) {
+  auto mag = [&a](int q, int mn) { return fx_hi(a[q][mn]) & 0x7fffffff; };
+  const int n0 = fx_exp(mag(0, 0)), n3 = fx_exp(mag(3, 0)), nm = (n0 + n3 + 1) >> 1;
+  int E = 0, mom = 0;  // the energy's coefficients along the face, the momentum
+#pragma unroll
+  for (int m = 0; m < 5; ++m)
+#pragma unroll
+    for (int n = 0; n + m < 5; ++n) {
+      if ((dir ? m : n) > 0) E = max(E, mag(3, m * 5 + n));
+      mom = max(mom, mag(2 - dir, m * 5 + n));
+    }
+  const int below = nm - fx_exp(mom);
+  return mom > 0 && below > CK_BELOW && below <= FX_STILL && fx_exp(E) < n3 - FX_STILL;
+}
+
+// The same from FP64 coefficients a[q][m*5+n] in cell units, Burgers or Euler; called while the tables may still
+// be in use.
 template <int NC>
-__device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_face, double (&a)[NC][25],
+__device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_face, int dir, double (&a)[NC][25],
                                           const CkLead& lead, double (&tc)[NC][5]) {
   ck_unit_lengths<NC>(P, a);
   if constexpr (NC == 1) {
     if (!has_face) return;
-    ck_fixed<1, 2>(a, lead, P.ck.K, tc);
+    ck_fixed<1, 2>(a, lead, P.ck, tc);
     tc[0][0] = a[0][0];
   } else {
     CkScale<4> S{};
     if (has_face) S = ck_scale<4, 2>([&a](int q, int mn) { return a[q][mn]; }, lead);
+    if (__syncthreads_or(has_face && (ck_fast_unit(S.eu, lead) || ck_coarse2d(a, dir)) ? 1 : 0)) return ck_points64(P, has_face, a, tc);
     const double Ws[4] = {a[0][0], a[1][0], a[2][0], a[3][0]};
     FxRange none{0};  // the recursion checks its operands
     ck_points4(P, npt, has_face, S, [&](int q, int mn) { return ck_convert<4>(S, a[q][mn], q, mn / 5 + mn % 5, none); },
@@ -471,7 +498,7 @@ __device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_fac
 // eigenvectors beyond 2^4 in them, end values above 8 times the data, weights of 4 and more.
 constexpr int FX_ABOVE = 2;       // most bits of a cell's data above the size its own state gives the component
 constexpr int FX_BELOW = 4;       // a momentum more bits than this below that size is a slow one,
-constexpr int FX_STILL = 48;      // and one more bits than this below it counts as none
+                                  // and one more than FX_STILL counts as none
 constexpr int FX_UNIT = 5;        // most bits of a face's density and energy below their units
 constexpr int FX_EL = FX_D - 53;  // most bits that the projections' scale takes off
 constexpr int FX_TINY = -300;     // least exponent of a scale
@@ -494,23 +521,22 @@ __device__ __forceinline__ int64_t fx_scaled(Fx x, Fx c) {
 // five times over (energy 2.5 beside 564: 1.4e-14 of the cold cell's end value, in FP64 3e-16; beside 1e12:
 // 5e-6).  So no value may be more than FX_ABOVE bits above the cell's own density, energy, or the momentum
 // sqrt(rho E) they allow: 5 * 2^-57 * 2^3 is FP64's 3e-16.
-//   A slow momentum rounds at 2^-57 of that one.  Where the energy varies along it, that is less than
-// what the rounding of the pressure, 2^-53 of rho c^2, does to it in every step; where the energy is the same in
-// all columns (the momentum across the face) or has no coefficients along the face (the other one),
-// the pressure moves nothing and FP64 would carry the momentum with all its bits.
+//   A slow momentum rounds at 2^-57 of that one: less than what the rounding of the pressure, 2^-53 of
+// rho c^2, does in every step to the momentum across the face, and to the one along the face where the energy
+// varies along it.  Where it does not (a shear layer), the pressure moves nothing and FP64 carries
+// the momentum with all its bits.
 //   Share of the CTAs that go to FP64: vortex, smooth flows 0; quadrants 0 to 0.6 % (400^2, 300 steps); double Mach
-// reflection 10 to 12 % (1024 x 256, 400 steps), whose step takes 9.1 ms instead of 8.7 for it.  Sent there for
-// any slow momentum: quadrants 16 to 65 %.  Testing the cells: 0.3 % of the vortex step (2048^2).
+// reflection about 10 % (1024 x 256, 400 steps), whose step takes 8.5 ms (8.7 with every CTA in fixed
+// point).  If any slow momentum went there: quadrants 16 to 65 %.  Testing the cells: 0.2 % of the vortex step
+// (2048^2).  Drift of a shear flow at 1e-6 of the sound speed, three steps, error against 64-bit mantissas:
+// 2.0e-13 -> 7.5e-17.
 __device__ __forceinline__ bool cell_exponents(const double (*ev)[5][SPAN], int c, int dir, int h[4]) {
   auto mag = [&](int f, int k, int col) { return fx_hi(ev[f][k][col]) & 0x7fffffff; };
   const int n0 = fx_exp(mag(0, 0, c)), n3 = fx_exp(mag(3, 0, c)), nm = (n0 + n3 + 1) >> 1;
   int along = 0;  // the energy's coefficients along the face
 #pragma unroll
   for (int k = 1; k < 5; ++k) along = max(along, max(mag(3, k, c - 1), max(mag(3, k, c), mag(3, k, c + 1))));
-  const double Em = ev[3][0][c - 1], E0 = ev[3][0][c], Ep = ev[3][0][c + 1];
-  const bool even_along = fx_exp(along) < n3 - FX_STILL;
-  const bool even_across = fx_bits(Em) == fx_bits(E0) && fx_bits(Ep) == fx_bits(E0) &&
-                           fx_exp(max(mag(7, 0, c - 1), mag(7, 0, c + 1))) < n3 - FX_STILL;
+  const bool even = fx_exp(along) < n3 - FX_STILL;
   int all = 0;
   bool ok = true;
 #pragma unroll
@@ -524,7 +550,7 @@ __device__ __forceinline__ bool cell_exponents(const double (*ev)[5][SPAN], int 
     const bool momentum = q == 1 || q == 2;
     if (top > 0 && !(momentum && e < nm - FX_STILL)) {
       ok = ok && e >= FX_TINY && e <= (q == 0 ? n0 : q == 3 ? n3 : nm) + FX_ABOVE;
-      if (momentum) ok = ok && !((q == 1 + dir ? even_across : even_along) && e < nm - FX_BELOW);
+      if (q == 2 - dir) ok = ok && !(even && e < nm - FX_BELOW);
     }
     h[q] = max(e, FX_TINY);  // an exact 0 then converts to 0
   }
@@ -672,7 +698,7 @@ __device__ __forceinline__ void face_setup_fx(const Params& P, const int64_t (*L
   int F = max(max(max(hL[1], hR[1]), max(hL[2], hR[2])) - f0, (max(hL[3], hR[3]) - f0 + 1) >> 1);
   F = max(F, max(fx_exp(lead.hu), (fx_exp(lead.hH) + 1) >> 1));
   int top = 0, el = -2000;
-  bool coarse = false;
+  bool coarse = ck_fast_unit(F, lead);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int u = q == 0 ? 0 : q == 3 ? 2 * F : F;
@@ -828,11 +854,15 @@ __device__ __forceinline__ void second_pass_cells(const Params& P, unsigned char
   pass_order<NC, FLAGS, Q, 2>(P, ev, et, fr, m, dir, Ws, U, a);
   pass_order<NC, FLAGS, Q, 3>(P, ev, et, fr, m, dir, Ws, U, a);
   pass_order<NC, FLAGS, Q, 4>(P, ev, et, fr, m, dir, Ws, U, a);
-  __syncthreads();  // the tables are read no more
   if (fr.has_face)
 #pragma unroll
     for (int q = 0; q < NC; ++q) a[q][0] = Ws[q];
-  ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, a, U.lead, tc);
+  if constexpr (NC == 4 && !Q) {
+    ck_unit_lengths<NC>(P, a);
+    ck_points64(P, fr.has_face, a, tc);
+  } else {
+    ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, dir, a, U.lead, tc);
+  }
 }
 
 // ------------------------------------------------------------------ characteristic-wise face point
@@ -1153,8 +1183,7 @@ __device__ __forceinline__ void xface_item(const Params& P, const StepView& sv, 
     }
     char_face_point<NC, FLAGS, Q>(P, ev, ft, fr.col - 1, 0, a, lead, Wref);
     }
-    __syncthreads();  // the tables are read no more
-    ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, a, lead, tc);
+    ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, 0, a, lead, tc);
   } else {
     second_pass_cells<NC, FLAGS, Q>(P, smem_raw, fr, 0, FLAGS && fr.has_cell && nl(fi - 1, row), tc);
   }
@@ -1221,8 +1250,7 @@ __device__ __forceinline__ void yface_item(const Params& P, const StepView& sv, 
         Wref[q] = 0.5 * (fetch(P, st, 0, q, col, fj - 1, sv.t) + fetch(P, st, 0, q, col, fj, sv.t));
       char_face_point<NC, FLAGS, Q>(P, ev, ft, fr.col - 1, 1, a, lead, Wref);
     }
-    __syncthreads();  // the tables are read no more
-    ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, a, lead, tc);
+    ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, 1, a, lead, tc);
   } else {
     second_pass_cells<NC, FLAGS, Q>(P, smem_raw, fr, 1, FLAGS && fr.has_cell && cell_flag(P, flag, col, fj - 1), tc);
   }

@@ -1,0 +1,77 @@
+// Host program of tests/test_ck_host.py: one step of the 1D Euler recursion at random points, the
+// library's form (ck_fixed.cuh) and FP64 throughout against long double.  Prints, per gamma, the largest
+// error of each component of the state after the step, relative to rho, rho c and E: library, FP64.
+#include <cmath>
+#include <cstdio>
+#include <random>
+
+#include "ck_fixed.cuh"
+
+using namespace shweno;
+typedef long double T;
+
+static void recursion(const double (&a)[3][25], T g, T (&tc)[3][5]) {
+  T S[3][5][5], u[5][5], mu[5][5], p[5][5], H[5][5], F[3][5];
+  for (int q = 0; q < 3; ++q)
+    for (int m = 0; m < 5; ++m) S[q][m][0] = a[q][m * 5];
+  for (int k = 0; k < 4; ++k) {
+    for (int m = 0; m + k < 5; ++m) {
+      T s = S[1][m][k];
+      for (int i = 0; i <= m; ++i)
+        for (int t = 0; t <= k; ++t)
+          if (i + t) s -= S[0][i][t] * u[m - i][k - t];
+      u[m][k] = s / S[0][0][0];
+      mu[m][k] = 0;
+      for (int i = 0; i <= m; ++i)
+        for (int t = 0; t <= k; ++t) mu[m][k] += S[1][i][t] * u[m - i][k - t];
+      p[m][k] = (g - 1) * (S[2][m][k] - mu[m][k] / 2);
+      H[m][k] = S[2][m][k] + p[m][k];
+      F[0][m] = S[1][m][k];
+      F[1][m] = mu[m][k] + p[m][k];
+      F[2][m] = 0;
+      for (int i = 0; i <= m; ++i)
+        for (int t = 0; t <= k; ++t) F[2][m] += u[i][t] * H[m - i][k - t];
+    }
+    for (int q = 0; q < 3; ++q)
+      for (int m = 0; m + k < 4; ++m) S[q][m][k + 1] = -(m + 1) * F[q][m + 1] / (k + 1);
+  }
+  for (int q = 0; q < 3; ++q)
+    for (int k = 0; k < 5; ++k) tc[q][k] = S[q][0][k];
+}
+
+int main() {
+  std::mt19937_64 rng(1);
+  std::uniform_real_distribution<double> U(-1.0, 1.0);
+  for (double g : {1.001, 1.02, 1.1, 1.2, 1.4, 5.0 / 3.0, 3.0, 7.0, 30.0, 1e3, 1e6}) {
+    CkFixed C;
+    finalize_ck_fixed(C, 1, 1.0, 1.0, g);
+    double lib[3] = {}, fp[3] = {};
+    // a density wave of any shape at uniform pressure and Mach 0.05 of c = sqrt(gamma)
+    const double vel = 0.05 * std::sqrt(g);
+    for (int it = 0; it < 2000; ++it) {
+      double a[3][25] = {}, f = 1.0;
+      a[0][0] = 1.0 + 0.3 * U(rng);
+      for (int s = 1; s < 5; ++s) a[0][s * 5] = (f *= 0.1) * U(rng);
+      for (int s = 0; s < 5; ++s) {
+        a[1][s * 5] = a[0][s * 5] * vel;
+        a[2][s * 5] = 0.5 * a[0][s * 5] * vel * vel + (s == 0 ? 1.0 / (g - 1.0) : 0.0);
+      }
+      const double ir = 1.0 / a[0][0], u = a[1][0] * ir, p = (g - 1.0) * (a[2][0] - 0.5 * a[1][0] * u);
+      const CkLead lead{ir, fx_hi(u) & 0x7fffffff, fx_hi((a[2][0] + p) * ir) & 0x7fffffff, fx_hi(std::sqrt(g * p * ir)) & 0x7fffffff};
+      double tl[3][5], td[3][5];
+      T tt[3][5];
+      ck_fixed<3, 1>(a, lead, C, tl);
+      ck_euler1d(a, td, C.gm1);
+      recursion(a, g, tt);
+      const T tau = 0.5 / std::sqrt(g);
+      for (int q = 0; q < 3; ++q) {
+        T sl = 0, sd = 0, st = 0;
+        for (int k = 4; k > 0; --k) sl = (sl + tl[q][k]) * tau, sd = (sd + td[q][k]) * tau, st = (st + tt[q][k]) * tau;
+        const T w = q == 1 ? a[0][0] * std::sqrt(g * p * ir) : a[q][0];
+        lib[q] = std::fmax(lib[q], (double)(std::fabs(sl - st) / w));
+        fp[q] = std::fmax(fp[q], (double)(std::fabs(sd - st) / w));
+      }
+    }
+    std::printf("%g %.3e %.3e %.3e %.3e %.3e %.3e\n", g, lib[0], lib[1], lib[2], fp[0], fp[1], fp[2]);
+  }
+}
