@@ -11,6 +11,9 @@
 // field's scale times (2^g)^s, the size its coefficients of that degree have themselves; FP64
 // rounds the leading coefficients at 2^-54.  A field whose values lie far below its scale keeps fewer bits
 // than a double's.  Where that shows in a step, the recursion runs in FP64 (ck_euler1d, ck_euler2d):
+//   - gamma above 3: p = (gamma - 1)(E - rho u^2 / 2) magnifies its rounding, and the growth that holds the
+//     derivatives of p coarsens all others (steep random points: gamma 3 as FP64, 5 five times, 30 1e4 times
+//     FP64's error);
 //   - gamma near 1: sqrt(H0) is far above |u| + c then, and order k in time rounds at (sqrt(H0) / (|u| + c))^k
 //     times what it should (gamma 1.02, half a cell per step: 1.6e-15 of the density, FP64 1e-20);
 //   - a slow momentum along a 2D face where the energy does not vary (step2d_items.cuh).
@@ -31,6 +34,8 @@ struct CkFixed {
   double iL;      // 1 / L: the time coefficients come in units of L
   double rx, ry;  // L / dx, L / dy: coordinates in units of L
   double gm1;     // gamma - 1, for the recursion in FP64
+  // whether block fixed point is for this gas (Burgers: yes); below 1.0625 every point at rest has too fast a unit
+  int32_t fixed;
 };
 
 constexpr int CK_BELOW = 5;   // most bits of a momentum along the face below its scale; a slower one is FP64's,
@@ -47,9 +52,8 @@ inline void finalize_ck_fixed(CkFixed& C, int dim, double dx, double dy, double 
   C.ry = dim == 2 ? L / dy : 1.0;
   C.iL = 1.0 / L;
   C.K.third = fx_const(1.0 / 3.0);
-  C.K.gshift = 0;
-  for (double h = gamma - 1.0; h >= 4.0 && C.K.gshift < 60; h *= 0.5) ++C.K.gshift;
-  C.K.gm1 = fx_const(std::ldexp(gamma - 1.0, -C.K.gshift));
+  C.fixed = gamma >= 1.0625 && gamma <= 3.0;
+  C.K.gm1 = fx_const(C.fixed ? gamma - 1.0 : 0.0);
   C.gm1 = gamma - 1.0;
 }
 
@@ -167,7 +171,9 @@ FX_FN Fx ck_ninv(const CkScale<NC>& S, const CkLead& lead) {
   return fx_split(fx_from_double<FX_C>(-lead.ir, -S.base[0]) + FX_HALF, r);
 }
 
-constexpr int kCkTries = 8;  // growths tried at most; inputs below 2^-5s cannot leave the range
+// Growths tried.  With inputs of degree s below 2^-11s, that is at the last one, no coefficient of any slice can
+// leave the range: a majorant of the recursion (all signs equal, 1/rho0 = 2, gamma = 3) stays below 0.12.
+constexpr int kCkTries = 12;
 
 // Burgers and 1D Euler: the whole recursion in one thread's registers (2D Euler: step2d_items.cuh).  Writes tc[q][k],
 // k = 1..4, per L^k (tc[q][0] is left to the caller); NaN where the input is not finite.
@@ -177,7 +183,7 @@ FX_FN void ck_fixed(const double (&a)[NC][25], const CkLead& lead, const CkFixed
   auto coef = [&a](int q, int mn) { return a[q][mn]; };
   CkScale<NC> S = ck_scale<NC, DIM>(coef, lead);
   if constexpr (NC == 3)
-    if (ck_fast_unit(S.eu, lead)) return ck_euler1d(a, tc, C.gm1);
+    if (!C.fixed || ck_fast_unit(S.eu, lead)) return ck_euler1d(a, tc, C.gm1);
   Fx w[NC][25], ninv{0, 0};
   int64_t t[NC][5];
   if constexpr (NC > 1) ninv = ck_ninv<NC>(S, lead);
@@ -195,6 +201,7 @@ FX_FN void ck_fixed(const double (&a)[NC][25], const CkLead& lead, const CkFixed
     else if constexpr (NC == 1) ck_burgers2d_fx(w, ninv, K, t, r);
     else ck_euler1d_fx(w, ninv, K, t, r);
     if (!r.bad()) break;
+    if (tries == kCkTries - 1) S.finite = false;
   }
 #pragma unroll
   for (int q = 0; q < NC; ++q)

@@ -5,10 +5,9 @@
 
 namespace shweno {
 
-// Constants of the recursion: 1/3 and (gamma - 1) 2^-gshift.
+// Constants of the recursion: 1/3 and gamma - 1.
 struct CkFixedConst {
   Fx third, gm1;
-  int32_t gshift;
 };
 
 // Minus z / k: from the flux derivatives of slice k - 1 to slice k.
@@ -128,7 +127,7 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   Fx u_200; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_200n, ninv); u_200 = fx_split(fx_sum<FX_C>(s), r); }
   int64_t z_mu_200; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_200); fx_mac(s, w[1][5], u_100); fx_mac(s, w[1][10], u_000); z_mu_200 = fx_sum(s); }
   const int64_t z_w2_200 = fx_join(w[2][10]);
-  const Fx e_200 = fx_split(((z_w2_200 - ((z_mu_200) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_200 = fx_split(z_w2_200 - ((z_mu_200) >> 1) + FX_HALF, r);
   int64_t z_p_200; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_200, K.gm1); z_p_200 = fx_sum<FX_C>(s); }
   const Fx w1_101 = fx_split(fx_time<1>(2 * (z_mu_200 + z_p_200), K.third) + FX_HALF, r);
   const int64_t z_w1_101 = fx_join(w1_101);
@@ -137,12 +136,12 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   Fx u_300; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_300n, ninv); u_300 = fx_split(fx_sum<FX_C>(s), r); }
   int64_t z_mu_300; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_300); fx_mac(s, w[1][5], u_200); fx_mac(s, w[1][10], u_100); fx_mac(s, w[1][15], u_000); z_mu_300 = fx_sum(s); }
   const int64_t z_w2_300 = fx_join(w[2][15]);
-  const Fx e_300 = fx_split(((z_w2_300 - ((z_mu_300) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_300 = fx_split(z_w2_300 - ((z_mu_300) >> 1) + FX_HALF, r);
   int64_t z_p_300; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_300, K.gm1); z_p_300 = fx_sum<FX_C>(s); }
   const Fx w1_201 = fx_split(fx_time<1>(3 * (z_mu_300 + z_p_300), K.third) + FX_HALF, r);
   int64_t z_mu_100; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_100); fx_mac(s, w[1][5], u_000); z_mu_100 = fx_sum(s); }
   const int64_t z_w2_100 = fx_join(w[2][5]);
-  const Fx e_100 = fx_split(((z_w2_100 - ((z_mu_100) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_100 = fx_split(z_w2_100 - ((z_mu_100) >> 1) + FX_HALF, r);
   int64_t z_p_100; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_100, K.gm1); z_p_100 = fx_sum<FX_C>(s); }
   const Fx w1_001 = fx_split(fx_time<1>(1 * (z_mu_100 + z_p_100), K.third) + FX_HALF, r);
   Fx u_001n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_001, -(1 << 30)); fx_mac(s, w0_001, u_000); u_001n = fx_split(fx_sum(s), r); }
@@ -161,13 +160,13 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   const Fx H_100 = fx_split(z_w2_100 + z_p_100 + FX_HALF, r);
   const int64_t z_w2_000 = fx_join(w[2][0]);
   int64_t z_mu_000; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_000); z_mu_000 = fx_sum(s); }
-  const Fx e_000 = fx_split(((z_w2_000 - ((z_mu_000) >> 1)) << K.gshift) + FX_HALF, r0);
+  const Fx e_000 = fx_split(z_w2_000 - ((z_mu_000) >> 1) + FX_HALF, r0);
   int64_t z_p_000; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_000, K.gm1); z_p_000 = fx_sum<FX_C>(s); }
   const Fx H_000 = fx_split(z_w2_000 + z_p_000 + FX_HALF, r0);
   int64_t z_uH_300; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_300); fx_mac(s, u_100, H_200); fx_mac(s, u_200, H_100); fx_mac(s, u_300, H_000); z_uH_300 = fx_sum(s); }
   const Fx w2_201 = fx_split(fx_time<1>(3 * (z_uH_300), K.third) + FX_HALF, r);
   const int64_t z_w2_201 = fx_join(w2_201);
-  const Fx e_201 = fx_split(((z_w2_201 - ((z_mu_201) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_201 = fx_split(z_w2_201 - ((z_mu_201) >> 1) + FX_HALF, r);
   int64_t z_p_201; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_201, K.gm1); z_p_201 = fx_sum<FX_C>(s); }
   const Fx w1_102 = fx_split(fx_time<2>(2 * (z_mu_201 + z_p_201), K.third) + FX_HALF, r);
   const int64_t z_w1_102 = fx_join(w1_102);
@@ -176,7 +175,7 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   Fx u_400; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_400n, ninv); u_400 = fx_split(fx_sum<FX_C>(s), r); }
   int64_t z_mu_400; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_400); fx_mac(s, w[1][5], u_300); fx_mac(s, w[1][10], u_200); fx_mac(s, w[1][15], u_100); fx_mac(s, w[1][20], u_000); z_mu_400 = fx_sum(s); }
   const int64_t z_w2_400 = fx_join(w[2][20]);
-  const Fx e_400 = fx_split(((z_w2_400 - ((z_mu_400) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_400 = fx_split(z_w2_400 - ((z_mu_400) >> 1) + FX_HALF, r);
   int64_t z_p_400; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_400, K.gm1); z_p_400 = fx_sum<FX_C>(s); }
   const Fx w1_301 = fx_split(fx_time<1>(4 * (z_mu_400 + z_p_400), K.third) + FX_HALF, r);
   const int64_t z_w1_400 = fx_join(w[1][20]);
@@ -188,14 +187,14 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   int64_t z_uH_400; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_400); fx_mac(s, u_100, H_300); fx_mac(s, u_200, H_200); fx_mac(s, u_300, H_100); fx_mac(s, u_400, H_000); z_uH_400 = fx_sum(s); }
   const Fx w2_301 = fx_split(fx_time<1>(4 * (z_uH_400), K.third) + FX_HALF, r);
   const int64_t z_w2_301 = fx_join(w2_301);
-  const Fx e_301 = fx_split(((z_w2_301 - ((z_mu_301) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_301 = fx_split(z_w2_301 - ((z_mu_301) >> 1) + FX_HALF, r);
   int64_t z_p_301; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_301, K.gm1); z_p_301 = fx_sum<FX_C>(s); }
   const Fx w1_202 = fx_split(fx_time<2>(3 * (z_mu_301 + z_p_301), K.third) + FX_HALF, r);
   int64_t z_mu_101; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_101); fx_mac(s, w1_001, u_100); fx_mac(s, w[1][5], u_001); fx_mac(s, w1_101, u_000); z_mu_101 = fx_sum(s); }
   int64_t z_uH_200; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_200); fx_mac(s, u_100, H_100); fx_mac(s, u_200, H_000); z_uH_200 = fx_sum(s); }
   const Fx w2_101 = fx_split(fx_time<1>(2 * (z_uH_200), K.third) + FX_HALF, r);
   const int64_t z_w2_101 = fx_join(w2_101);
-  const Fx e_101 = fx_split(((z_w2_101 - ((z_mu_101) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_101 = fx_split(z_w2_101 - ((z_mu_101) >> 1) + FX_HALF, r);
   int64_t z_p_101; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_101, K.gm1); z_p_101 = fx_sum<FX_C>(s); }
   const Fx w1_002 = fx_split(fx_time<2>(1 * (z_mu_101 + z_p_101), K.third) + FX_HALF, r);
   Fx u_002n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_002, -(1 << 30)); fx_mac(s, w0_001, u_001); fx_mac(s, w0_002, u_000); u_002n = fx_split(fx_sum(s), r); }
@@ -216,13 +215,13 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   const Fx w2_001 = fx_split(fx_time<1>(1 * (z_uH_100), K.third) + FX_HALF, r);
   const int64_t z_w2_001 = fx_join(w2_001);
   int64_t z_mu_001; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_001); fx_mac(s, w1_001, u_000); z_mu_001 = fx_sum(s); }
-  const Fx e_001 = fx_split(((z_w2_001 - ((z_mu_001) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_001 = fx_split(z_w2_001 - ((z_mu_001) >> 1) + FX_HALF, r);
   int64_t z_p_001; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_001, K.gm1); z_p_001 = fx_sum<FX_C>(s); }
   const Fx H_001 = fx_split(z_w2_001 + z_p_001 + FX_HALF, r);
   int64_t z_uH_301; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_301); fx_mac(s, u_001, H_300); fx_mac(s, u_100, H_201); fx_mac(s, u_101, H_200); fx_mac(s, u_200, H_101); fx_mac(s, u_201, H_100); fx_mac(s, u_300, H_001); fx_mac(s, u_301, H_000); z_uH_301 = fx_sum(s); }
   const Fx w2_202 = fx_split(fx_time<2>(3 * (z_uH_301), K.third) + FX_HALF, r);
   const int64_t z_w2_202 = fx_join(w2_202);
-  const Fx e_202 = fx_split(((z_w2_202 - ((z_mu_202) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_202 = fx_split(z_w2_202 - ((z_mu_202) >> 1) + FX_HALF, r);
   int64_t z_p_202; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_202, K.gm1); z_p_202 = fx_sum<FX_C>(s); }
   const Fx w1_103 = fx_split(fx_time<3>(2 * (z_mu_202 + z_p_202), K.third) + FX_HALF, r);
   const int64_t z_w1_103 = fx_join(w1_103);
@@ -231,7 +230,7 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   int64_t z_uH_201; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_201); fx_mac(s, u_001, H_200); fx_mac(s, u_100, H_101); fx_mac(s, u_101, H_100); fx_mac(s, u_200, H_001); fx_mac(s, u_201, H_000); z_uH_201 = fx_sum(s); }
   const Fx w2_102 = fx_split(fx_time<2>(2 * (z_uH_201), K.third) + FX_HALF, r);
   const int64_t z_w2_102 = fx_join(w2_102);
-  const Fx e_102 = fx_split(((z_w2_102 - ((z_mu_102) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_102 = fx_split(z_w2_102 - ((z_mu_102) >> 1) + FX_HALF, r);
   int64_t z_p_102; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_102, K.gm1); z_p_102 = fx_sum<FX_C>(s); }
   const Fx w1_003 = fx_split(fx_time<3>(1 * (z_mu_102 + z_p_102), K.third) + FX_HALF, r);
   Fx u_003n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_003, -(1 << 30)); fx_mac(s, w0_001, u_002); fx_mac(s, w0_002, u_001); fx_mac(s, w0_003, u_000); u_003n = fx_split(fx_sum(s), r); }
@@ -247,13 +246,13 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   const Fx w2_002 = fx_split(fx_time<2>(1 * (z_uH_101), K.third) + FX_HALF, r);
   const int64_t z_w2_002 = fx_join(w2_002);
   int64_t z_mu_002; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_002); fx_mac(s, w1_001, u_001); fx_mac(s, w1_002, u_000); z_mu_002 = fx_sum(s); }
-  const Fx e_002 = fx_split(((z_w2_002 - ((z_mu_002) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_002 = fx_split(z_w2_002 - ((z_mu_002) >> 1) + FX_HALF, r);
   int64_t z_p_002; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_002, K.gm1); z_p_002 = fx_sum<FX_C>(s); }
   const Fx H_002 = fx_split(z_w2_002 + z_p_002 + FX_HALF, r);
   int64_t z_uH_202; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_202); fx_mac(s, u_001, H_201); fx_mac(s, u_002, H_200); fx_mac(s, u_100, H_102); fx_mac(s, u_101, H_101); fx_mac(s, u_102, H_100); fx_mac(s, u_200, H_002); fx_mac(s, u_201, H_001); fx_mac(s, u_202, H_000); z_uH_202 = fx_sum(s); }
   const Fx w2_103 = fx_split(fx_time<3>(2 * (z_uH_202), K.third) + FX_HALF, r);
   const int64_t z_w2_103 = fx_join(w2_103);
-  const Fx e_103 = fx_split(((z_w2_103 - ((z_mu_103) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_103 = fx_split(z_w2_103 - ((z_mu_103) >> 1) + FX_HALF, r);
   int64_t z_p_103; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_103, K.gm1); z_p_103 = fx_sum<FX_C>(s); }
   const Fx w1_004 = fx_split(fx_time<4>(1 * (z_mu_103 + z_p_103), K.third) + FX_HALF, r);
   int64_t z_uH_102; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_102); fx_mac(s, u_001, H_101); fx_mac(s, u_002, H_100); fx_mac(s, u_100, H_002); fx_mac(s, u_101, H_001); fx_mac(s, u_102, H_000); z_uH_102 = fx_sum(s); }
@@ -261,7 +260,7 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   const Fx H_103 = fx_split(z_w2_103 + z_p_103 + FX_HALF, r);
   const int64_t z_w2_003 = fx_join(w2_003);
   int64_t z_mu_003; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_003); fx_mac(s, w1_001, u_002); fx_mac(s, w1_002, u_001); fx_mac(s, w1_003, u_000); z_mu_003 = fx_sum(s); }
-  const Fx e_003 = fx_split(((z_w2_003 - ((z_mu_003) >> 1)) << K.gshift) + FX_HALF, r);
+  const Fx e_003 = fx_split(z_w2_003 - ((z_mu_003) >> 1) + FX_HALF, r);
   int64_t z_p_003; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_003, K.gm1); z_p_003 = fx_sum<FX_C>(s); }
   const Fx H_003 = fx_split(z_w2_003 + z_p_003 + FX_HALF, r);
   int64_t z_uH_103; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_103); fx_mac(s, u_001, H_102); fx_mac(s, u_002, H_101); fx_mac(s, u_003, H_100); fx_mac(s, u_100, H_003); fx_mac(s, u_101, H_002); fx_mac(s, u_102, H_001); fx_mac(s, u_103, H_000); z_uH_103 = fx_sum(s); }
@@ -283,7 +282,7 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
 // 2D Euler, two lanes per point: S gives the shared series and constants, ninv = -1/rho0;
 // S.next() takes the coefficients of the next slice.
 template <typename Store>
-FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxRange& r) {
+FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
   FxRange r0{0};  // leading coefficients are in range by their scales
   // ---- slice 0
   Fx vel000;
@@ -560,87 +559,87 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   int64_t f220;
   int64_t f130;
   { const int64_t E = S.ldE(0, 0, 0);
-    const Fx e = fx_split(((E - ((k000 + S.swap(k000)) >> 1)) << gshift) + FX_HALF, r0);
+    const Fx e = fx_split(E - ((k000 + S.swap(k000)) >> 1) + FX_HALF, r0);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 0, 0, fx_split(E + p + FX_HALF, r0));
   }
   { const int64_t E = S.ldE(0, 1, 0);
-    const Fx e = fx_split(((E - ((k100 + S.swap(k010)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k100 + S.swap(k010)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 1, 0, fx_split(E + p + FX_HALF, r));
     f100 = k100 + p;
   }
   { const int64_t E = S.ldE(0, 0, 1);
-    const Fx e = fx_split(((E - ((k010 + S.swap(k100)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k010 + S.swap(k100)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 0, 1, fx_split(E + p + FX_HALF, r));
   }
   { const int64_t E = S.ldE(0, 2, 0);
-    const Fx e = fx_split(((E - ((k200 + S.swap(k020)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k200 + S.swap(k020)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 2, 0, fx_split(E + p + FX_HALF, r));
     f200 = k200 + p;
   }
   { const int64_t E = S.ldE(0, 1, 1);
-    const Fx e = fx_split(((E - ((k110 + S.swap(k110)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k110 + S.swap(k110)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 1, 1, fx_split(E + p + FX_HALF, r));
     f110 = k110 + p;
   }
   { const int64_t E = S.ldE(0, 0, 2);
-    const Fx e = fx_split(((E - ((k020 + S.swap(k200)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k020 + S.swap(k200)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 0, 2, fx_split(E + p + FX_HALF, r));
   }
   { const int64_t E = S.ldE(0, 3, 0);
-    const Fx e = fx_split(((E - ((k300 + S.swap(k030)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k300 + S.swap(k030)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 3, 0, fx_split(E + p + FX_HALF, r));
     f300 = k300 + p;
   }
   { const int64_t E = S.ldE(0, 2, 1);
-    const Fx e = fx_split(((E - ((k210 + S.swap(k120)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k210 + S.swap(k120)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 2, 1, fx_split(E + p + FX_HALF, r));
     f210 = k210 + p;
   }
   { const int64_t E = S.ldE(0, 1, 2);
-    const Fx e = fx_split(((E - ((k120 + S.swap(k210)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k120 + S.swap(k210)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 1, 2, fx_split(E + p + FX_HALF, r));
     f120 = k120 + p;
   }
   { const int64_t E = S.ldE(0, 0, 3);
-    const Fx e = fx_split(((E - ((k030 + S.swap(k300)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k030 + S.swap(k300)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 0, 3, fx_split(E + p + FX_HALF, r));
   }
   { const int64_t E = S.ldE(0, 4, 0);
-    const Fx e = fx_split(((E - ((k400 + S.swap(k040)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k400 + S.swap(k040)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 4, 0, fx_split(E + p + FX_HALF, r));
     f400 = k400 + p;
   }
   { const int64_t E = S.ldE(0, 3, 1);
-    const Fx e = fx_split(((E - ((k310 + S.swap(k130)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k310 + S.swap(k130)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 3, 1, fx_split(E + p + FX_HALF, r));
     f310 = k310 + p;
   }
   { const int64_t E = S.ldE(0, 2, 2);
-    const Fx e = fx_split(((E - ((k220 + S.swap(k220)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k220 + S.swap(k220)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 2, 2, fx_split(E + p + FX_HALF, r));
     f220 = k220 + p;
   }
   { const int64_t E = S.ldE(0, 1, 3);
-    const Fx e = fx_split(((E - ((k130 + S.swap(k310)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k130 + S.swap(k310)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 1, 3, fx_split(E + p + FX_HALF, r));
     f130 = k130 + p;
   }
   { const int64_t E = S.ldE(0, 0, 4);
-    const Fx e = fx_split(((E - ((k040 + S.swap(k400)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k040 + S.swap(k400)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(0, 0, 4, fx_split(E + p + FX_HALF, r));
   }
@@ -1110,58 +1109,58 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   int64_t f211;
   int64_t f121;
   { const int64_t E = E001;
-    const Fx e = fx_split(((E - ((k001 + S.swap(k001)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k001 + S.swap(k001)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 0, 0, fx_split(E + p + FX_HALF, r));
   }
   { const int64_t E = E101;
-    const Fx e = fx_split(((E - ((k101 + S.swap(k011)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k101 + S.swap(k011)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 1, 0, fx_split(E + p + FX_HALF, r));
     f101 = k101 + p;
   }
   { const int64_t E = E011;
-    const Fx e = fx_split(((E - ((k011 + S.swap(k101)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k011 + S.swap(k101)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 0, 1, fx_split(E + p + FX_HALF, r));
   }
   { const int64_t E = E201;
-    const Fx e = fx_split(((E - ((k201 + S.swap(k021)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k201 + S.swap(k021)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 2, 0, fx_split(E + p + FX_HALF, r));
     f201 = k201 + p;
   }
   { const int64_t E = E111;
-    const Fx e = fx_split(((E - ((k111 + S.swap(k111)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k111 + S.swap(k111)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 1, 1, fx_split(E + p + FX_HALF, r));
     f111 = k111 + p;
   }
   { const int64_t E = E021;
-    const Fx e = fx_split(((E - ((k021 + S.swap(k201)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k021 + S.swap(k201)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 0, 2, fx_split(E + p + FX_HALF, r));
   }
   { const int64_t E = E301;
-    const Fx e = fx_split(((E - ((k301 + S.swap(k031)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k301 + S.swap(k031)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 3, 0, fx_split(E + p + FX_HALF, r));
     f301 = k301 + p;
   }
   { const int64_t E = E211;
-    const Fx e = fx_split(((E - ((k211 + S.swap(k121)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k211 + S.swap(k121)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 2, 1, fx_split(E + p + FX_HALF, r));
     f211 = k211 + p;
   }
   { const int64_t E = E121;
-    const Fx e = fx_split(((E - ((k121 + S.swap(k211)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k121 + S.swap(k211)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 1, 2, fx_split(E + p + FX_HALF, r));
     f121 = k121 + p;
   }
   { const int64_t E = E031;
-    const Fx e = fx_split(((E - ((k031 + S.swap(k301)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k031 + S.swap(k301)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(1, 0, 3, fx_split(E + p + FX_HALF, r));
   }
@@ -1493,35 +1492,35 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   int64_t f202;
   int64_t f112;
   { const int64_t E = E002;
-    const Fx e = fx_split(((E - ((k002 + S.swap(k002)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k002 + S.swap(k002)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(2, 0, 0, fx_split(E + p + FX_HALF, r));
   }
   { const int64_t E = E102;
-    const Fx e = fx_split(((E - ((k102 + S.swap(k012)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k102 + S.swap(k012)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(2, 1, 0, fx_split(E + p + FX_HALF, r));
     f102 = k102 + p;
   }
   { const int64_t E = E012;
-    const Fx e = fx_split(((E - ((k012 + S.swap(k102)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k012 + S.swap(k102)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(2, 0, 1, fx_split(E + p + FX_HALF, r));
   }
   { const int64_t E = E202;
-    const Fx e = fx_split(((E - ((k202 + S.swap(k022)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k202 + S.swap(k022)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(2, 2, 0, fx_split(E + p + FX_HALF, r));
     f202 = k202 + p;
   }
   { const int64_t E = E112;
-    const Fx e = fx_split(((E - ((k112 + S.swap(k112)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k112 + S.swap(k112)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(2, 1, 1, fx_split(E + p + FX_HALF, r));
     f112 = k112 + p;
   }
   { const int64_t E = E022;
-    const Fx e = fx_split(((E - ((k022 + S.swap(k202)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k022 + S.swap(k202)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(2, 0, 2, fx_split(E + p + FX_HALF, r));
   }
@@ -1703,18 +1702,18 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxR
   }
   int64_t f103;
   { const int64_t E = E003;
-    const Fx e = fx_split(((E - ((k003 + S.swap(k003)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k003 + S.swap(k003)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(3, 0, 0, fx_split(E + p + FX_HALF, r));
   }
   { const int64_t E = E103;
-    const Fx e = fx_split(((E - ((k103 + S.swap(k013)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k103 + S.swap(k013)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(3, 1, 0, fx_split(E + p + FX_HALF, r));
     f103 = k103 + p;
   }
   { const int64_t E = E013;
-    const Fx e = fx_split(((E - ((k013 + S.swap(k103)) >> 1)) << gshift) + FX_HALF, r);
+    const Fx e = fx_split(E - ((k013 + S.swap(k103)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
     S.stH(3, 0, 1, fx_split(E + p + FX_HALF, r));
   }

@@ -118,7 +118,7 @@ class GenFixed:
             self.lines.append(f"  const int64_t {v} = fx_join({self.fx(name, m, n, k)});")
         elif name == "p":
             kin = self.z("mu", m, n, k) + (f" + {self.z('nv', m, n, k)}" if self.dim == 2 else "")
-            self.lines.append(f"  const Fx e_{m}{n}{k} = fx_split((({self.z(W[-1], m, n, k)} - (({kin}) >> 1)) << K.gshift) + FX_HALF, {self.rng(m, n, k)});")
+            self.lines.append(f"  const Fx e_{m}{n}{k} = fx_split({self.z(W[-1], m, n, k)} - (({kin}) >> 1) + FX_HALF, {self.rng(m, n, k)});")
             self.lines.append(f"  int64_t {v}; {{ FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_{m}{n}{k}, K.gm1); {v} = fx_sum<FX_C>(s); }}")
         else:
             A, B = {"mu": (W[1], "u"), "mv": (W[1], "v"), "nv": (W[-2], "v"), "uH": ("u", "H"), "vH": ("v", "H")}[name]
@@ -399,7 +399,7 @@ class GenLane:
         for i, j in self.pairs(D):
             E = f"S.ldE(0, {i}, {j})" if c == 0 else f"E{i}{j}{c}"
             self.out(f"{{ const int64_t E = {E};")
-            self.out(f"  const Fx e = fx_split(((E - ((k{i}{j}{c} + S.swap(k{j}{i}{c})) >> 1)) << gshift) + FX_HALF, {rng(i, j)});")
+            self.out(f"  const Fx e = fx_split(E - ((k{i}{j}{c} + S.swap(k{j}{i}{c})) >> 1) + FX_HALF, {rng(i, j)});")
             self.out(f"  FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);")
             self.out(f"  S.stH({c}, {i}, {j}, fx_split(E + p + FX_HALF, {rng(i, j)}));")
             if i >= 1:
@@ -463,8 +463,8 @@ def main():
     parts = ["// Generated by gen_ck.py -- do not edit.  The Cauchy-Kovalevskaya recursions",
              "// in block fixed point (see fixed.cuh, ck_fixed.cuh and gen_ck.py for the method).",
              "#pragma once", '#include "fixed.cuh"', "", "namespace shweno {", "",
-             "// Constants of the recursion: 1/3 and (gamma - 1) 2^-gshift.",
-             "struct CkFixedConst {", "  Fx third, gm1;", "  int32_t gshift;", "};", "",
+             "// Constants of the recursion: 1/3 and gamma - 1.",
+             "struct CkFixedConst {", "  Fx third, gm1;", "};", "",
              "// Minus z / k: from the flux derivatives of slice k - 1 to slice k.",
              "template <int K>",
              "FX_FN int64_t fx_time(int64_t z, Fx third) {",
@@ -480,7 +480,7 @@ def main():
     parts += ["// 2D Euler, two lanes per point: S gives the shared series and constants, ninv = -1/rho0;",
               "// S.next() takes the coefficients of the next slice.",
               "template <typename Store>",
-              "FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, int gshift, FxRange& r) {",
+              "FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {",
               "  FxRange r0{0};  // leading coefficients are in range by their scales",
               GenLane().run(), "}", ""]
     for dim in (1, 2):

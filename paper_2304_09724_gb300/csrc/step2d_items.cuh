@@ -247,6 +247,7 @@ constexpr int kCkE = kCkH0 + 15 * kCkRow;        // [10] E of the level in work,
 constexpr int kCkNinv = kCkE + 10 * kCkRow;      // [SEG] -1/rho0
 constexpr int kCkGrow = kCkNinv + SEG * 8;       // [SEG] growth added on the way
 constexpr size_t kCkBytes = kCkGrow + SEG * 4;
+constexpr int kCkLost = 1 << 20;                 // growth of a point whose values never fitted: its result is NaN
 
 template <int NC>
 constexpr size_t face_smem() {
@@ -343,7 +344,7 @@ struct CkLane {
 // The recursion of the 16 points p0.. of a half (valid: points that exist), by one whole warp.
 // Results: t[q][k] (64-bit, k = 1..4) in row q * 4 + k - 1 of the point's column of the half's input.
 // Out of line: one copy of the recursion for all kernels of a translation unit.
-static __device__ __noinline__ void ck_warp_euler2d(int half, int p0, int valid, Fx third, Fx gm1, int gshift) {
+static __device__ __noinline__ void ck_warp_euler2d(int half, int p0, int valid, Fx third, Fx gm1) {
   const int lane = threadIdx.x & 31, dir = lane >> 4, pt = p0 + (lane & 15);
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   CkLane S(half, pt, dir);
@@ -351,10 +352,14 @@ static __device__ __noinline__ void ck_warp_euler2d(int half, int p0, int valid,
 #pragma unroll 1
   for (int tries = 1;; ++tries) {
     FxRange r{0};
-    ck_euler2d_lane(S, ninv, gm1, third, gshift, r);
+    ck_euler2d_lane(S, ninv, gm1, third, r);
     int bad = (lane & 15) < valid && r.bad() ? 1 : 0;
     bad |= __shfl_xor_sync(0xffffffffu, bad, 16);
-    if (!__any_sync(0xffffffffu, bad) || tries == kCkTries) break;
+    if (!__any_sync(0xffffffffu, bad)) break;
+    if (tries == kCkTries) {
+      if (bad && dir == 0) *reinterpret_cast<int*>(dyn_smem + kCkGrow + (half * CKP + pt) * 4) = kCkLost;
+      break;
+    }
     __syncwarp();
     if (bad) {  // divide the coefficients of degree s by 2^s: each lane half of the components
       FxRange none{0};
@@ -424,12 +429,14 @@ __device__ __forceinline__ void ck_points4(const Params& P, int npt, bool has_fa
 #pragma unroll 1
   for (int half = 0; half * CKP < npt; ++half) {
     const int valid = npt - half * CKP - p0;
-    if (valid > 0) ck_warp_euler2d(half, p0, valid, P.ck.K.third, P.ck.K.gm1, P.ck.K.gshift);
+    if (valid > 0) ck_warp_euler2d(half, p0, valid, P.ck.K.third, P.ck.K.gm1);
     __syncwarp();
   }
   __syncthreads();
   if (!has_face) return;
-  S.g += *reinterpret_cast<const int*>(dyn_smem + kCkGrow + tid * 4);
+  const int grown = *reinterpret_cast<const int*>(dyn_smem + kCkGrow + tid * 4);
+  S.g += grown;
+  S.finite = S.finite && grown != kCkLost;
 #pragma unroll
   for (int q = 0; q < 4; ++q)
 #pragma unroll
@@ -477,7 +484,7 @@ __device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_fac
   } else {
     CkScale<4> S{};
     if (has_face) S = ck_scale<4, 2>([&a](int q, int mn) { return a[q][mn]; }, lead);
-    if (__syncthreads_or(has_face && (ck_fast_unit(S.eu, lead) || ck_coarse2d(a, dir)) ? 1 : 0)) return ck_points64(P, has_face, a, tc);
+    if (__syncthreads_or(!P.ck.fixed || (has_face && (ck_fast_unit(S.eu, lead) || ck_coarse2d(a, dir))) ? 1 : 0)) return ck_points64(P, has_face, a, tc);
     const double Ws[4] = {a[0][0], a[1][0], a[2][0], a[3][0]};
     FxRange none{0};  // the recursion checks its operands
     ck_points4(P, npt, has_face, S, [&](int q, int mn) { return ck_convert<4>(S, a[q][mn], q, mn / 5 + mn % 5, none); },
@@ -735,6 +742,7 @@ __device__ __forceinline__ bool second_pass_fx(const Params& P, unsigned char* s
   unsigned char* tables = smem_raw + ev_bytes<4>();
   FxRange r{0};
   CellMixFx m;
+  if (!P.ck.fixed) return false;
   const bool ok = !fr.has_cell || cell_exponents(ev, fr.col, dir, m.h);
   if (__syncthreads_or(ok ? 0 : 1)) return false;
   if (fr.has_cell) {

@@ -1,6 +1,8 @@
 // Host program of tests/test_ck_host.py: one step of the 1D Euler recursion at random points, the
 // library's form (ck_fixed.cuh) and FP64 throughout against long double.  Prints, per gamma, the largest
-// error of each component of the state after the step, relative to rho, rho c and E: library, FP64.
+// error of each component of the state after the step, relative to rho, rho c and E: library, FP64; and the
+// same for steep points (every coefficient as large as the state) of any velocity up to Mach 0.7, root mean
+// square, relative to the sum of the time series' terms.
 #include <cmath>
 #include <cstdio>
 #include <random>
@@ -42,7 +44,7 @@ static void recursion(const double (&a)[3][25], T g, T (&tc)[3][5]) {
 int main() {
   std::mt19937_64 rng(1);
   std::uniform_real_distribution<double> U(-1.0, 1.0);
-  for (double g : {1.001, 1.02, 1.1, 1.2, 1.4, 5.0 / 3.0, 3.0, 7.0, 30.0, 1e3, 1e6}) {
+  for (double g : {1.001, 1.02, 1.1, 1.2, 1.4, 5.0 / 3.0, 3.0, 4.0, 7.0, 30.0, 1e3, 1e6}) {
     CkFixed C;
     finalize_ck_fixed(C, 1, 1.0, 1.0, g);
     double lib[3] = {}, fp[3] = {};
@@ -72,6 +74,34 @@ int main() {
         fp[q] = std::fmax(fp[q], (double)(std::fabs(sd - st) / w));
       }
     }
-    std::printf("%g %.3e %.3e %.3e %.3e %.3e %.3e\n", g, lib[0], lib[1], lib[2], fp[0], fp[1], fp[2]);
+    double sl2[3] = {}, sf2[3] = {};
+    for (int it = 0; it < 2000; ++it) {
+      double a[3][25] = {};
+      const double rho = 1.0 + 0.3 * U(rng), p = 1.0 + 0.3 * U(rng), u = 0.7 * std::sqrt(g) * U(rng);
+      const double W[3] = {rho, rho * u, p / (g - 1.0) + 0.5 * rho * u * u};
+      for (int q = 0; q < 3; ++q)
+        for (int s = 0; s < 5; ++s) a[q][s * 5] = s == 0 ? W[q] : U(rng) * (q == 0 ? 1.0 : q == 1 ? std::sqrt(g) : W[2]);
+      const double ir = 1.0 / rho, v = W[1] * ir, pp = (g - 1.0) * (W[2] - 0.5 * W[1] * v), c = std::sqrt(g * pp * ir);
+      const CkLead lead{ir, fx_hi(v) & 0x7fffffff, fx_hi((W[2] + pp) * ir) & 0x7fffffff, fx_hi(c) & 0x7fffffff};
+      double tl[3][5], td[3][5];
+      T tt[3][5];
+      ck_fixed<3, 1>(a, lead, C, tl);
+      ck_euler1d(a, td, C.gm1);
+      recursion(a, g, tt);
+      const T tau = 0.3 / std::sqrt(g);
+      for (int q = 0; q < 3; ++q) {
+        T el = 0, ef = 0, sum = 0;
+        for (int k = 4; k > 0; --k) {
+          el = (el + tl[q][k] - tt[q][k]) * tau;
+          ef = (ef + td[q][k] - tt[q][k]) * tau;
+          sum = (sum + std::fabs(tt[q][k])) * tau;
+        }
+        const T w = (q == 1 ? rho * c : std::fabs(W[q])) + sum;
+        sl2[q] += (double)(el / w * el / w);
+        sf2[q] += (double)(ef / w * ef / w);
+      }
+    }
+    std::printf("%g %.3e %.3e %.3e %.3e %.3e %.3e ", g, lib[0], lib[1], lib[2], fp[0], fp[1], fp[2]);
+    for (int q = 0; q < 3; ++q) std::printf("%.3e %.3e%s", std::sqrt(sl2[q] / 2000), std::sqrt(sf2[q] / 2000), q < 2 ? " " : "\n");
   }
 }
