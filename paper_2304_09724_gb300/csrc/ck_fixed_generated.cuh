@@ -27,25 +27,25 @@ FX_FN int64_t fx_time(int64_t z, Fx third) {
 FX_FN void ck_burgers1d_fx(const Fx (&w)[1][25], Fx ninv, const CkFixedConst& K, int64_t (&t)[1][5], FxRange& r) {
   (void)ninv;
   int64_t f_100; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][5]); f_100 = fx_sum(s); }
-  const Fx w0_001 = fx_split(fx_time<1>(1 * f_100, K.third) + FX_HALF, r);
+  const Fx w0_001 = fx_split_any(fx_time<1>(1 * f_100, K.third) + FX_HALF, r);
   int64_t f_200; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][10]); f_200 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w[0][5], w[0][5]); f_200 += fx_sum(s) >> 1; }
-  const Fx w0_101 = fx_split(fx_time<1>(2 * f_200, K.third) + FX_HALF, r);
+  const Fx w0_101 = fx_split_any(fx_time<1>(2 * f_200, K.third) + FX_HALF, r);
   int64_t f_101; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_101); fx_mac(s, w0_001, w[0][5]); f_101 = fx_sum(s); }
-  const Fx w0_002 = fx_split(fx_time<2>(1 * f_101, K.third) + FX_HALF, r);
+  const Fx w0_002 = fx_split_any(fx_time<2>(1 * f_101, K.third) + FX_HALF, r);
   int64_t f_300; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][15]); fx_mac(s, w[0][5], w[0][10]); f_300 = fx_sum(s); }
-  const Fx w0_201 = fx_split(fx_time<1>(3 * f_300, K.third) + FX_HALF, r);
+  const Fx w0_201 = fx_split_any(fx_time<1>(3 * f_300, K.third) + FX_HALF, r);
   int64_t f_201; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_201); fx_mac(s, w0_001, w[0][10]); fx_mac(s, w[0][5], w0_101); f_201 = fx_sum(s); }
-  const Fx w0_102 = fx_split(fx_time<2>(2 * f_201, K.third) + FX_HALF, r);
+  const Fx w0_102 = fx_split_any(fx_time<2>(2 * f_201, K.third) + FX_HALF, r);
   int64_t f_102; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_102); fx_mac(s, w0_001, w0_101); fx_mac(s, w0_002, w[0][5]); f_102 = fx_sum(s); }
-  const Fx w0_003 = fx_split(fx_time<3>(1 * f_102, K.third) + FX_HALF, r);
+  const Fx w0_003 = fx_split_any(fx_time<3>(1 * f_102, K.third) + FX_HALF, r);
   int64_t f_400; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][20]); fx_mac(s, w[0][5], w[0][15]); f_400 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w[0][10], w[0][10]); f_400 += fx_sum(s) >> 1; }
-  const Fx w0_301 = fx_split(fx_time<1>(4 * f_400, K.third) + FX_HALF, r);
+  const Fx w0_301 = fx_split_any(fx_time<1>(4 * f_400, K.third) + FX_HALF, r);
   int64_t f_301; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_301); fx_mac(s, w0_001, w[0][15]); fx_mac(s, w[0][5], w0_201); fx_mac(s, w0_101, w[0][10]); f_301 = fx_sum(s); }
-  const Fx w0_202 = fx_split(fx_time<2>(3 * f_301, K.third) + FX_HALF, r);
+  const Fx w0_202 = fx_split_any(fx_time<2>(3 * f_301, K.third) + FX_HALF, r);
   int64_t f_202; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_202); fx_mac(s, w0_001, w0_201); fx_mac(s, w0_002, w[0][10]); fx_mac(s, w[0][5], w0_102); f_202 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w0_101, w0_101); f_202 += fx_sum(s) >> 1; }
-  const Fx w0_103 = fx_split(fx_time<3>(2 * f_202, K.third) + FX_HALF, r);
+  const Fx w0_103 = fx_split_any(fx_time<3>(2 * f_202, K.third) + FX_HALF, r);
   int64_t f_103; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_103); fx_mac(s, w0_001, w0_102); fx_mac(s, w0_002, w0_101); fx_mac(s, w0_003, w[0][5]); f_103 = fx_sum(s); }
-  const Fx w0_004 = fx_split(fx_time<4>(1 * f_103, K.third) + FX_HALF, r);
+  const Fx w0_004 = fx_split_any(fx_time<4>(1 * f_103, K.third) + FX_HALF, r);
   t[0][1] = fx_join(w0_001);
   t[0][2] = fx_join(w0_002);
   t[0][3] = fx_join(w0_003);
@@ -58,54 +58,54 @@ FX_FN void ck_burgers2d_fx(const Fx (&w)[1][25], Fx ninv, const CkFixedConst& K,
   (void)ninv;
   int64_t f_100; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][5]); f_100 = fx_sum(s); }
   int64_t f_010; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][1]); f_010 = fx_sum(s); }
-  const Fx w0_001 = fx_split(fx_time<1>(1 * f_100 + 1 * f_010, K.third) + FX_HALF, r);
+  const Fx w0_001 = fx_split_any(fx_time<1>(1 * f_100 + 1 * f_010, K.third) + FX_HALF, r);
   int64_t f_200; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][10]); f_200 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w[0][5], w[0][5]); f_200 += fx_sum(s) >> 1; }
   int64_t f_110; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][6]); fx_mac(s, w[0][1], w[0][5]); f_110 = fx_sum(s); }
-  const Fx w0_101 = fx_split(fx_time<1>(2 * f_200 + 1 * f_110, K.third) + FX_HALF, r);
+  const Fx w0_101 = fx_split_any(fx_time<1>(2 * f_200 + 1 * f_110, K.third) + FX_HALF, r);
   int64_t f_101; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_101); fx_mac(s, w0_001, w[0][5]); f_101 = fx_sum(s); }
   int64_t f_020; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][2]); f_020 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w[0][1], w[0][1]); f_020 += fx_sum(s) >> 1; }
-  const Fx w0_011 = fx_split(fx_time<1>(1 * f_110 + 2 * f_020, K.third) + FX_HALF, r);
+  const Fx w0_011 = fx_split_any(fx_time<1>(1 * f_110 + 2 * f_020, K.third) + FX_HALF, r);
   int64_t f_011; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_011); fx_mac(s, w0_001, w[0][1]); f_011 = fx_sum(s); }
-  const Fx w0_002 = fx_split(fx_time<2>(1 * f_101 + 1 * f_011, K.third) + FX_HALF, r);
+  const Fx w0_002 = fx_split_any(fx_time<2>(1 * f_101 + 1 * f_011, K.third) + FX_HALF, r);
   int64_t f_300; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][15]); fx_mac(s, w[0][5], w[0][10]); f_300 = fx_sum(s); }
   int64_t f_210; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][11]); fx_mac(s, w[0][1], w[0][10]); fx_mac(s, w[0][5], w[0][6]); f_210 = fx_sum(s); }
-  const Fx w0_201 = fx_split(fx_time<1>(3 * f_300 + 1 * f_210, K.third) + FX_HALF, r);
+  const Fx w0_201 = fx_split_any(fx_time<1>(3 * f_300 + 1 * f_210, K.third) + FX_HALF, r);
   int64_t f_201; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_201); fx_mac(s, w0_001, w[0][10]); fx_mac(s, w[0][5], w0_101); f_201 = fx_sum(s); }
   int64_t f_120; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][7]); fx_mac(s, w[0][1], w[0][6]); fx_mac(s, w[0][2], w[0][5]); f_120 = fx_sum(s); }
-  const Fx w0_111 = fx_split(fx_time<1>(2 * f_210 + 2 * f_120, K.third) + FX_HALF, r);
+  const Fx w0_111 = fx_split_any(fx_time<1>(2 * f_210 + 2 * f_120, K.third) + FX_HALF, r);
   int64_t f_111; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_111); fx_mac(s, w0_001, w[0][6]); fx_mac(s, w[0][1], w0_101); fx_mac(s, w0_011, w[0][5]); f_111 = fx_sum(s); }
-  const Fx w0_102 = fx_split(fx_time<2>(2 * f_201 + 1 * f_111, K.third) + FX_HALF, r);
+  const Fx w0_102 = fx_split_any(fx_time<2>(2 * f_201 + 1 * f_111, K.third) + FX_HALF, r);
   int64_t f_102; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_102); fx_mac(s, w0_001, w0_101); fx_mac(s, w0_002, w[0][5]); f_102 = fx_sum(s); }
   int64_t f_030; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][3]); fx_mac(s, w[0][1], w[0][2]); f_030 = fx_sum(s); }
-  const Fx w0_021 = fx_split(fx_time<1>(1 * f_120 + 3 * f_030, K.third) + FX_HALF, r);
+  const Fx w0_021 = fx_split_any(fx_time<1>(1 * f_120 + 3 * f_030, K.third) + FX_HALF, r);
   int64_t f_021; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_021); fx_mac(s, w0_001, w[0][2]); fx_mac(s, w[0][1], w0_011); f_021 = fx_sum(s); }
-  const Fx w0_012 = fx_split(fx_time<2>(1 * f_111 + 2 * f_021, K.third) + FX_HALF, r);
+  const Fx w0_012 = fx_split_any(fx_time<2>(1 * f_111 + 2 * f_021, K.third) + FX_HALF, r);
   int64_t f_012; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_012); fx_mac(s, w0_001, w0_011); fx_mac(s, w0_002, w[0][1]); f_012 = fx_sum(s); }
-  const Fx w0_003 = fx_split(fx_time<3>(1 * f_102 + 1 * f_012, K.third) + FX_HALF, r);
+  const Fx w0_003 = fx_split_any(fx_time<3>(1 * f_102 + 1 * f_012, K.third) + FX_HALF, r);
   int64_t f_400; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][20]); fx_mac(s, w[0][5], w[0][15]); f_400 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w[0][10], w[0][10]); f_400 += fx_sum(s) >> 1; }
   int64_t f_310; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][16]); fx_mac(s, w[0][1], w[0][15]); fx_mac(s, w[0][5], w[0][11]); fx_mac(s, w[0][6], w[0][10]); f_310 = fx_sum(s); }
-  const Fx w0_301 = fx_split(fx_time<1>(4 * f_400 + 1 * f_310, K.third) + FX_HALF, r);
+  const Fx w0_301 = fx_split_any(fx_time<1>(4 * f_400 + 1 * f_310, K.third) + FX_HALF, r);
   int64_t f_301; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_301); fx_mac(s, w0_001, w[0][15]); fx_mac(s, w[0][5], w0_201); fx_mac(s, w0_101, w[0][10]); f_301 = fx_sum(s); }
   int64_t f_220; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][12]); fx_mac(s, w[0][1], w[0][11]); fx_mac(s, w[0][2], w[0][10]); fx_mac(s, w[0][5], w[0][7]); f_220 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w[0][6], w[0][6]); f_220 += fx_sum(s) >> 1; }
-  const Fx w0_211 = fx_split(fx_time<1>(3 * f_310 + 2 * f_220, K.third) + FX_HALF, r);
+  const Fx w0_211 = fx_split_any(fx_time<1>(3 * f_310 + 2 * f_220, K.third) + FX_HALF, r);
   int64_t f_211; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_211); fx_mac(s, w0_001, w[0][11]); fx_mac(s, w[0][1], w0_201); fx_mac(s, w0_011, w[0][10]); fx_mac(s, w[0][5], w0_111); fx_mac(s, w0_101, w[0][6]); f_211 = fx_sum(s); }
-  const Fx w0_202 = fx_split(fx_time<2>(3 * f_301 + 1 * f_211, K.third) + FX_HALF, r);
+  const Fx w0_202 = fx_split_any(fx_time<2>(3 * f_301 + 1 * f_211, K.third) + FX_HALF, r);
   int64_t f_202; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_202); fx_mac(s, w0_001, w0_201); fx_mac(s, w0_002, w[0][10]); fx_mac(s, w[0][5], w0_102); f_202 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w0_101, w0_101); f_202 += fx_sum(s) >> 1; }
   int64_t f_130; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][8]); fx_mac(s, w[0][1], w[0][7]); fx_mac(s, w[0][2], w[0][6]); fx_mac(s, w[0][3], w[0][5]); f_130 = fx_sum(s); }
-  const Fx w0_121 = fx_split(fx_time<1>(2 * f_220 + 3 * f_130, K.third) + FX_HALF, r);
+  const Fx w0_121 = fx_split_any(fx_time<1>(2 * f_220 + 3 * f_130, K.third) + FX_HALF, r);
   int64_t f_121; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_121); fx_mac(s, w0_001, w[0][7]); fx_mac(s, w[0][1], w0_111); fx_mac(s, w0_011, w[0][6]); fx_mac(s, w[0][2], w0_101); fx_mac(s, w0_021, w[0][5]); f_121 = fx_sum(s); }
-  const Fx w0_112 = fx_split(fx_time<2>(2 * f_211 + 2 * f_121, K.third) + FX_HALF, r);
+  const Fx w0_112 = fx_split_any(fx_time<2>(2 * f_211 + 2 * f_121, K.third) + FX_HALF, r);
   int64_t f_112; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_112); fx_mac(s, w0_001, w0_111); fx_mac(s, w0_002, w[0][6]); fx_mac(s, w[0][1], w0_102); fx_mac(s, w0_011, w0_101); fx_mac(s, w0_012, w[0][5]); f_112 = fx_sum(s); }
-  const Fx w0_103 = fx_split(fx_time<3>(2 * f_202 + 1 * f_112, K.third) + FX_HALF, r);
+  const Fx w0_103 = fx_split_any(fx_time<3>(2 * f_202 + 1 * f_112, K.third) + FX_HALF, r);
   int64_t f_103; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_103); fx_mac(s, w0_001, w0_102); fx_mac(s, w0_002, w0_101); fx_mac(s, w0_003, w[0][5]); f_103 = fx_sum(s); }
   int64_t f_040; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w[0][4]); fx_mac(s, w[0][1], w[0][3]); f_040 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w[0][2], w[0][2]); f_040 += fx_sum(s) >> 1; }
-  const Fx w0_031 = fx_split(fx_time<1>(1 * f_130 + 4 * f_040, K.third) + FX_HALF, r);
+  const Fx w0_031 = fx_split_any(fx_time<1>(1 * f_130 + 4 * f_040, K.third) + FX_HALF, r);
   int64_t f_031; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_031); fx_mac(s, w0_001, w[0][3]); fx_mac(s, w[0][1], w0_021); fx_mac(s, w0_011, w[0][2]); f_031 = fx_sum(s); }
-  const Fx w0_022 = fx_split(fx_time<2>(1 * f_121 + 3 * f_031, K.third) + FX_HALF, r);
+  const Fx w0_022 = fx_split_any(fx_time<2>(1 * f_121 + 3 * f_031, K.third) + FX_HALF, r);
   int64_t f_022; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_022); fx_mac(s, w0_001, w0_021); fx_mac(s, w0_002, w[0][2]); fx_mac(s, w[0][1], w0_012); f_022 = fx_sum(s); }{ FxAcc s = fx_zero(); fx_mac(s, w0_011, w0_011); f_022 += fx_sum(s) >> 1; }
-  const Fx w0_013 = fx_split(fx_time<3>(1 * f_112 + 2 * f_022, K.third) + FX_HALF, r);
+  const Fx w0_013 = fx_split_any(fx_time<3>(1 * f_112 + 2 * f_022, K.third) + FX_HALF, r);
   int64_t f_013; { FxAcc s = fx_zero(); fx_mac(s, w[0][0], w0_013); fx_mac(s, w0_001, w0_012); fx_mac(s, w0_002, w0_011); fx_mac(s, w0_003, w[0][1]); f_013 = fx_sum(s); }
-  const Fx w0_004 = fx_split(fx_time<4>(1 * f_103 + 1 * f_013, K.third) + FX_HALF, r);
+  const Fx w0_004 = fx_split_any(fx_time<4>(1 * f_103 + 1 * f_013, K.third) + FX_HALF, r);
   t[0][1] = fx_join(w0_001);
   t[0][2] = fx_join(w0_002);
   t[0][3] = fx_join(w0_003);
@@ -118,7 +118,7 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   (void)ninv;
   FxRange r0{0};  // leading coefficients are in range by their scales
   const int64_t z_w1_100 = fx_join(w[1][5]);
-  const Fx w0_001 = fx_split(fx_time<1>(1 * (z_w1_100), K.third) + FX_HALF, r);
+  const Fx w0_001 = fx_split_any(fx_time<1>(1 * (z_w1_100), K.third) + FX_HALF, r);
   Fx u_000n; { FxAcc s = fx_zero(true); fx_mac_int(s, w[1][0], -(1 << 30)); u_000n = fx_split(fx_sum(s), r0); }
   Fx u_000; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_000n, ninv); u_000 = fx_split(fx_sum<FX_C>(s), r0); }
   Fx u_100n; { FxAcc s = fx_zero(true); fx_mac_int(s, w[1][5], -(1 << 30)); fx_mac(s, w[0][5], u_000); u_100n = fx_split(fx_sum(s), r); }
@@ -129,29 +129,29 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   const int64_t z_w2_200 = fx_join(w[2][10]);
   const Fx e_200 = fx_split(z_w2_200 - ((z_mu_200) >> 1) + FX_HALF, r);
   int64_t z_p_200; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_200, K.gm1); z_p_200 = fx_sum<FX_C>(s); }
-  const Fx w1_101 = fx_split(fx_time<1>(2 * (z_mu_200 + z_p_200), K.third) + FX_HALF, r);
+  const Fx w1_101 = fx_split_any(fx_time<1>(2 * (z_mu_200 + z_p_200), K.third) + FX_HALF, r);
   const int64_t z_w1_101 = fx_join(w1_101);
-  const Fx w0_002 = fx_split(fx_time<2>(1 * (z_w1_101), K.third) + FX_HALF, r);
+  const Fx w0_002 = fx_split_any(fx_time<2>(1 * (z_w1_101), K.third) + FX_HALF, r);
   Fx u_300n; { FxAcc s = fx_zero(true); fx_mac_int(s, w[1][15], -(1 << 30)); fx_mac(s, w[0][5], u_200); fx_mac(s, w[0][10], u_100); fx_mac(s, w[0][15], u_000); u_300n = fx_split(fx_sum(s), r); }
   Fx u_300; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_300n, ninv); u_300 = fx_split(fx_sum<FX_C>(s), r); }
   int64_t z_mu_300; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_300); fx_mac(s, w[1][5], u_200); fx_mac(s, w[1][10], u_100); fx_mac(s, w[1][15], u_000); z_mu_300 = fx_sum(s); }
   const int64_t z_w2_300 = fx_join(w[2][15]);
   const Fx e_300 = fx_split(z_w2_300 - ((z_mu_300) >> 1) + FX_HALF, r);
   int64_t z_p_300; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_300, K.gm1); z_p_300 = fx_sum<FX_C>(s); }
-  const Fx w1_201 = fx_split(fx_time<1>(3 * (z_mu_300 + z_p_300), K.third) + FX_HALF, r);
+  const Fx w1_201 = fx_split_any(fx_time<1>(3 * (z_mu_300 + z_p_300), K.third) + FX_HALF, r);
   int64_t z_mu_100; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_100); fx_mac(s, w[1][5], u_000); z_mu_100 = fx_sum(s); }
   const int64_t z_w2_100 = fx_join(w[2][5]);
   const Fx e_100 = fx_split(z_w2_100 - ((z_mu_100) >> 1) + FX_HALF, r);
   int64_t z_p_100; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_100, K.gm1); z_p_100 = fx_sum<FX_C>(s); }
-  const Fx w1_001 = fx_split(fx_time<1>(1 * (z_mu_100 + z_p_100), K.third) + FX_HALF, r);
+  const Fx w1_001 = fx_split_any(fx_time<1>(1 * (z_mu_100 + z_p_100), K.third) + FX_HALF, r);
   Fx u_001n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_001, -(1 << 30)); fx_mac(s, w0_001, u_000); u_001n = fx_split(fx_sum(s), r); }
   Fx u_001; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_001n, ninv); u_001 = fx_split(fx_sum<FX_C>(s), r); }
   const int64_t z_w1_200 = fx_join(w[1][10]);
-  const Fx w0_101 = fx_split(fx_time<1>(2 * (z_w1_200), K.third) + FX_HALF, r);
+  const Fx w0_101 = fx_split_any(fx_time<1>(2 * (z_w1_200), K.third) + FX_HALF, r);
   Fx u_101n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_101, -(1 << 30)); fx_mac(s, w0_001, u_100); fx_mac(s, w[0][5], u_001); fx_mac(s, w0_101, u_000); u_101n = fx_split(fx_sum(s), r); }
   Fx u_101; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_101n, ninv); u_101 = fx_split(fx_sum<FX_C>(s), r); }
   const int64_t z_w1_300 = fx_join(w[1][15]);
-  const Fx w0_201 = fx_split(fx_time<1>(3 * (z_w1_300), K.third) + FX_HALF, r);
+  const Fx w0_201 = fx_split_any(fx_time<1>(3 * (z_w1_300), K.third) + FX_HALF, r);
   Fx u_201n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_201, -(1 << 30)); fx_mac(s, w0_001, u_200); fx_mac(s, w[0][5], u_101); fx_mac(s, w0_101, u_100); fx_mac(s, w[0][10], u_001); fx_mac(s, w0_201, u_000); u_201n = fx_split(fx_sum(s), r); }
   Fx u_201; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_201n, ninv); u_201 = fx_split(fx_sum<FX_C>(s), r); }
   int64_t z_mu_201; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_201); fx_mac(s, w1_001, u_200); fx_mac(s, w[1][5], u_101); fx_mac(s, w1_101, u_100); fx_mac(s, w[1][10], u_001); fx_mac(s, w1_201, u_000); z_mu_201 = fx_sum(s); }
@@ -164,47 +164,47 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   int64_t z_p_000; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_000, K.gm1); z_p_000 = fx_sum<FX_C>(s); }
   const Fx H_000 = fx_split(z_w2_000 + z_p_000 + FX_HALF, r0);
   int64_t z_uH_300; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_300); fx_mac(s, u_100, H_200); fx_mac(s, u_200, H_100); fx_mac(s, u_300, H_000); z_uH_300 = fx_sum(s); }
-  const Fx w2_201 = fx_split(fx_time<1>(3 * (z_uH_300), K.third) + FX_HALF, r);
+  const Fx w2_201 = fx_split_any(fx_time<1>(3 * (z_uH_300), K.third) + FX_HALF, r);
   const int64_t z_w2_201 = fx_join(w2_201);
   const Fx e_201 = fx_split(z_w2_201 - ((z_mu_201) >> 1) + FX_HALF, r);
   int64_t z_p_201; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_201, K.gm1); z_p_201 = fx_sum<FX_C>(s); }
-  const Fx w1_102 = fx_split(fx_time<2>(2 * (z_mu_201 + z_p_201), K.third) + FX_HALF, r);
+  const Fx w1_102 = fx_split_any(fx_time<2>(2 * (z_mu_201 + z_p_201), K.third) + FX_HALF, r);
   const int64_t z_w1_102 = fx_join(w1_102);
-  const Fx w0_003 = fx_split(fx_time<3>(1 * (z_w1_102), K.third) + FX_HALF, r);
+  const Fx w0_003 = fx_split_any(fx_time<3>(1 * (z_w1_102), K.third) + FX_HALF, r);
   Fx u_400n; { FxAcc s = fx_zero(true); fx_mac_int(s, w[1][20], -(1 << 30)); fx_mac(s, w[0][5], u_300); fx_mac(s, w[0][10], u_200); fx_mac(s, w[0][15], u_100); fx_mac(s, w[0][20], u_000); u_400n = fx_split(fx_sum(s), r); }
   Fx u_400; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_400n, ninv); u_400 = fx_split(fx_sum<FX_C>(s), r); }
   int64_t z_mu_400; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_400); fx_mac(s, w[1][5], u_300); fx_mac(s, w[1][10], u_200); fx_mac(s, w[1][15], u_100); fx_mac(s, w[1][20], u_000); z_mu_400 = fx_sum(s); }
   const int64_t z_w2_400 = fx_join(w[2][20]);
   const Fx e_400 = fx_split(z_w2_400 - ((z_mu_400) >> 1) + FX_HALF, r);
   int64_t z_p_400; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_400, K.gm1); z_p_400 = fx_sum<FX_C>(s); }
-  const Fx w1_301 = fx_split(fx_time<1>(4 * (z_mu_400 + z_p_400), K.third) + FX_HALF, r);
+  const Fx w1_301 = fx_split_any(fx_time<1>(4 * (z_mu_400 + z_p_400), K.third) + FX_HALF, r);
   const int64_t z_w1_400 = fx_join(w[1][20]);
-  const Fx w0_301 = fx_split(fx_time<1>(4 * (z_w1_400), K.third) + FX_HALF, r);
+  const Fx w0_301 = fx_split_any(fx_time<1>(4 * (z_w1_400), K.third) + FX_HALF, r);
   Fx u_301n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_301, -(1 << 30)); fx_mac(s, w0_001, u_300); fx_mac(s, w[0][5], u_201); fx_mac(s, w0_101, u_200); fx_mac(s, w[0][10], u_101); fx_mac(s, w0_201, u_100); fx_mac(s, w[0][15], u_001); fx_mac(s, w0_301, u_000); u_301n = fx_split(fx_sum(s), r); }
   Fx u_301; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_301n, ninv); u_301 = fx_split(fx_sum<FX_C>(s), r); }
   int64_t z_mu_301; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_301); fx_mac(s, w1_001, u_300); fx_mac(s, w[1][5], u_201); fx_mac(s, w1_101, u_200); fx_mac(s, w[1][10], u_101); fx_mac(s, w1_201, u_100); fx_mac(s, w[1][15], u_001); fx_mac(s, w1_301, u_000); z_mu_301 = fx_sum(s); }
   const Fx H_400 = fx_split(z_w2_400 + z_p_400 + FX_HALF, r);
   int64_t z_uH_400; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_400); fx_mac(s, u_100, H_300); fx_mac(s, u_200, H_200); fx_mac(s, u_300, H_100); fx_mac(s, u_400, H_000); z_uH_400 = fx_sum(s); }
-  const Fx w2_301 = fx_split(fx_time<1>(4 * (z_uH_400), K.third) + FX_HALF, r);
+  const Fx w2_301 = fx_split_any(fx_time<1>(4 * (z_uH_400), K.third) + FX_HALF, r);
   const int64_t z_w2_301 = fx_join(w2_301);
   const Fx e_301 = fx_split(z_w2_301 - ((z_mu_301) >> 1) + FX_HALF, r);
   int64_t z_p_301; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_301, K.gm1); z_p_301 = fx_sum<FX_C>(s); }
-  const Fx w1_202 = fx_split(fx_time<2>(3 * (z_mu_301 + z_p_301), K.third) + FX_HALF, r);
+  const Fx w1_202 = fx_split_any(fx_time<2>(3 * (z_mu_301 + z_p_301), K.third) + FX_HALF, r);
   int64_t z_mu_101; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_101); fx_mac(s, w1_001, u_100); fx_mac(s, w[1][5], u_001); fx_mac(s, w1_101, u_000); z_mu_101 = fx_sum(s); }
   int64_t z_uH_200; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_200); fx_mac(s, u_100, H_100); fx_mac(s, u_200, H_000); z_uH_200 = fx_sum(s); }
-  const Fx w2_101 = fx_split(fx_time<1>(2 * (z_uH_200), K.third) + FX_HALF, r);
+  const Fx w2_101 = fx_split_any(fx_time<1>(2 * (z_uH_200), K.third) + FX_HALF, r);
   const int64_t z_w2_101 = fx_join(w2_101);
   const Fx e_101 = fx_split(z_w2_101 - ((z_mu_101) >> 1) + FX_HALF, r);
   int64_t z_p_101; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_101, K.gm1); z_p_101 = fx_sum<FX_C>(s); }
-  const Fx w1_002 = fx_split(fx_time<2>(1 * (z_mu_101 + z_p_101), K.third) + FX_HALF, r);
+  const Fx w1_002 = fx_split_any(fx_time<2>(1 * (z_mu_101 + z_p_101), K.third) + FX_HALF, r);
   Fx u_002n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_002, -(1 << 30)); fx_mac(s, w0_001, u_001); fx_mac(s, w0_002, u_000); u_002n = fx_split(fx_sum(s), r); }
   Fx u_002; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_002n, ninv); u_002 = fx_split(fx_sum<FX_C>(s), r); }
   const int64_t z_w1_201 = fx_join(w1_201);
-  const Fx w0_102 = fx_split(fx_time<2>(2 * (z_w1_201), K.third) + FX_HALF, r);
+  const Fx w0_102 = fx_split_any(fx_time<2>(2 * (z_w1_201), K.third) + FX_HALF, r);
   Fx u_102n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_102, -(1 << 30)); fx_mac(s, w0_001, u_101); fx_mac(s, w0_002, u_100); fx_mac(s, w[0][5], u_002); fx_mac(s, w0_101, u_001); fx_mac(s, w0_102, u_000); u_102n = fx_split(fx_sum(s), r); }
   Fx u_102; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_102n, ninv); u_102 = fx_split(fx_sum<FX_C>(s), r); }
   const int64_t z_w1_301 = fx_join(w1_301);
-  const Fx w0_202 = fx_split(fx_time<2>(3 * (z_w1_301), K.third) + FX_HALF, r);
+  const Fx w0_202 = fx_split_any(fx_time<2>(3 * (z_w1_301), K.third) + FX_HALF, r);
   Fx u_202n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_202, -(1 << 30)); fx_mac(s, w0_001, u_201); fx_mac(s, w0_002, u_200); fx_mac(s, w[0][5], u_102); fx_mac(s, w0_101, u_101); fx_mac(s, w0_102, u_100); fx_mac(s, w[0][10], u_002); fx_mac(s, w0_201, u_001); fx_mac(s, w0_202, u_000); u_202n = fx_split(fx_sum(s), r); }
   Fx u_202; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_202n, ninv); u_202 = fx_split(fx_sum<FX_C>(s), r); }
   int64_t z_mu_202; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_202); fx_mac(s, w1_001, u_201); fx_mac(s, w1_002, u_200); fx_mac(s, w[1][5], u_102); fx_mac(s, w1_101, u_101); fx_mac(s, w1_102, u_100); fx_mac(s, w[1][10], u_002); fx_mac(s, w1_201, u_001); fx_mac(s, w1_202, u_000); z_mu_202 = fx_sum(s); }
@@ -212,51 +212,51 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   const Fx H_201 = fx_split(z_w2_201 + z_p_201 + FX_HALF, r);
   const Fx H_101 = fx_split(z_w2_101 + z_p_101 + FX_HALF, r);
   int64_t z_uH_100; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_100); fx_mac(s, u_100, H_000); z_uH_100 = fx_sum(s); }
-  const Fx w2_001 = fx_split(fx_time<1>(1 * (z_uH_100), K.third) + FX_HALF, r);
+  const Fx w2_001 = fx_split_any(fx_time<1>(1 * (z_uH_100), K.third) + FX_HALF, r);
   const int64_t z_w2_001 = fx_join(w2_001);
   int64_t z_mu_001; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_001); fx_mac(s, w1_001, u_000); z_mu_001 = fx_sum(s); }
   const Fx e_001 = fx_split(z_w2_001 - ((z_mu_001) >> 1) + FX_HALF, r);
   int64_t z_p_001; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_001, K.gm1); z_p_001 = fx_sum<FX_C>(s); }
   const Fx H_001 = fx_split(z_w2_001 + z_p_001 + FX_HALF, r);
   int64_t z_uH_301; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_301); fx_mac(s, u_001, H_300); fx_mac(s, u_100, H_201); fx_mac(s, u_101, H_200); fx_mac(s, u_200, H_101); fx_mac(s, u_201, H_100); fx_mac(s, u_300, H_001); fx_mac(s, u_301, H_000); z_uH_301 = fx_sum(s); }
-  const Fx w2_202 = fx_split(fx_time<2>(3 * (z_uH_301), K.third) + FX_HALF, r);
+  const Fx w2_202 = fx_split_any(fx_time<2>(3 * (z_uH_301), K.third) + FX_HALF, r);
   const int64_t z_w2_202 = fx_join(w2_202);
   const Fx e_202 = fx_split(z_w2_202 - ((z_mu_202) >> 1) + FX_HALF, r);
   int64_t z_p_202; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_202, K.gm1); z_p_202 = fx_sum<FX_C>(s); }
-  const Fx w1_103 = fx_split(fx_time<3>(2 * (z_mu_202 + z_p_202), K.third) + FX_HALF, r);
+  const Fx w1_103 = fx_split_any(fx_time<3>(2 * (z_mu_202 + z_p_202), K.third) + FX_HALF, r);
   const int64_t z_w1_103 = fx_join(w1_103);
-  const Fx w0_004 = fx_split(fx_time<4>(1 * (z_w1_103), K.third) + FX_HALF, r);
+  const Fx w0_004 = fx_split_any(fx_time<4>(1 * (z_w1_103), K.third) + FX_HALF, r);
   int64_t z_mu_102; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_102); fx_mac(s, w1_001, u_101); fx_mac(s, w1_002, u_100); fx_mac(s, w[1][5], u_002); fx_mac(s, w1_101, u_001); fx_mac(s, w1_102, u_000); z_mu_102 = fx_sum(s); }
   int64_t z_uH_201; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_201); fx_mac(s, u_001, H_200); fx_mac(s, u_100, H_101); fx_mac(s, u_101, H_100); fx_mac(s, u_200, H_001); fx_mac(s, u_201, H_000); z_uH_201 = fx_sum(s); }
-  const Fx w2_102 = fx_split(fx_time<2>(2 * (z_uH_201), K.third) + FX_HALF, r);
+  const Fx w2_102 = fx_split_any(fx_time<2>(2 * (z_uH_201), K.third) + FX_HALF, r);
   const int64_t z_w2_102 = fx_join(w2_102);
   const Fx e_102 = fx_split(z_w2_102 - ((z_mu_102) >> 1) + FX_HALF, r);
   int64_t z_p_102; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_102, K.gm1); z_p_102 = fx_sum<FX_C>(s); }
-  const Fx w1_003 = fx_split(fx_time<3>(1 * (z_mu_102 + z_p_102), K.third) + FX_HALF, r);
+  const Fx w1_003 = fx_split_any(fx_time<3>(1 * (z_mu_102 + z_p_102), K.third) + FX_HALF, r);
   Fx u_003n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_003, -(1 << 30)); fx_mac(s, w0_001, u_002); fx_mac(s, w0_002, u_001); fx_mac(s, w0_003, u_000); u_003n = fx_split(fx_sum(s), r); }
   Fx u_003; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_003n, ninv); u_003 = fx_split(fx_sum<FX_C>(s), r); }
   const int64_t z_w1_202 = fx_join(w1_202);
-  const Fx w0_103 = fx_split(fx_time<3>(2 * (z_w1_202), K.third) + FX_HALF, r);
+  const Fx w0_103 = fx_split_any(fx_time<3>(2 * (z_w1_202), K.third) + FX_HALF, r);
   Fx u_103n; { FxAcc s = fx_zero(true); fx_mac_int(s, w1_103, -(1 << 30)); fx_mac(s, w0_001, u_102); fx_mac(s, w0_002, u_101); fx_mac(s, w0_003, u_100); fx_mac(s, w[0][5], u_003); fx_mac(s, w0_101, u_002); fx_mac(s, w0_102, u_001); fx_mac(s, w0_103, u_000); u_103n = fx_split(fx_sum(s), r); }
   Fx u_103; { FxAcc s = fx_zero<FX_C>(true); fx_mac(s, u_103n, ninv); u_103 = fx_split(fx_sum<FX_C>(s), r); }
   int64_t z_mu_103; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_103); fx_mac(s, w1_001, u_102); fx_mac(s, w1_002, u_101); fx_mac(s, w1_003, u_100); fx_mac(s, w[1][5], u_003); fx_mac(s, w1_101, u_002); fx_mac(s, w1_102, u_001); fx_mac(s, w1_103, u_000); z_mu_103 = fx_sum(s); }
   const Fx H_202 = fx_split(z_w2_202 + z_p_202 + FX_HALF, r);
   const Fx H_102 = fx_split(z_w2_102 + z_p_102 + FX_HALF, r);
   int64_t z_uH_101; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_101); fx_mac(s, u_001, H_100); fx_mac(s, u_100, H_001); fx_mac(s, u_101, H_000); z_uH_101 = fx_sum(s); }
-  const Fx w2_002 = fx_split(fx_time<2>(1 * (z_uH_101), K.third) + FX_HALF, r);
+  const Fx w2_002 = fx_split_any(fx_time<2>(1 * (z_uH_101), K.third) + FX_HALF, r);
   const int64_t z_w2_002 = fx_join(w2_002);
   int64_t z_mu_002; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_002); fx_mac(s, w1_001, u_001); fx_mac(s, w1_002, u_000); z_mu_002 = fx_sum(s); }
   const Fx e_002 = fx_split(z_w2_002 - ((z_mu_002) >> 1) + FX_HALF, r);
   int64_t z_p_002; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_002, K.gm1); z_p_002 = fx_sum<FX_C>(s); }
   const Fx H_002 = fx_split(z_w2_002 + z_p_002 + FX_HALF, r);
   int64_t z_uH_202; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_202); fx_mac(s, u_001, H_201); fx_mac(s, u_002, H_200); fx_mac(s, u_100, H_102); fx_mac(s, u_101, H_101); fx_mac(s, u_102, H_100); fx_mac(s, u_200, H_002); fx_mac(s, u_201, H_001); fx_mac(s, u_202, H_000); z_uH_202 = fx_sum(s); }
-  const Fx w2_103 = fx_split(fx_time<3>(2 * (z_uH_202), K.third) + FX_HALF, r);
+  const Fx w2_103 = fx_split_any(fx_time<3>(2 * (z_uH_202), K.third) + FX_HALF, r);
   const int64_t z_w2_103 = fx_join(w2_103);
   const Fx e_103 = fx_split(z_w2_103 - ((z_mu_103) >> 1) + FX_HALF, r);
   int64_t z_p_103; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_103, K.gm1); z_p_103 = fx_sum<FX_C>(s); }
-  const Fx w1_004 = fx_split(fx_time<4>(1 * (z_mu_103 + z_p_103), K.third) + FX_HALF, r);
+  const Fx w1_004 = fx_split_any(fx_time<4>(1 * (z_mu_103 + z_p_103), K.third) + FX_HALF, r);
   int64_t z_uH_102; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_102); fx_mac(s, u_001, H_101); fx_mac(s, u_002, H_100); fx_mac(s, u_100, H_002); fx_mac(s, u_101, H_001); fx_mac(s, u_102, H_000); z_uH_102 = fx_sum(s); }
-  const Fx w2_003 = fx_split(fx_time<3>(1 * (z_uH_102), K.third) + FX_HALF, r);
+  const Fx w2_003 = fx_split_any(fx_time<3>(1 * (z_uH_102), K.third) + FX_HALF, r);
   const Fx H_103 = fx_split(z_w2_103 + z_p_103 + FX_HALF, r);
   const int64_t z_w2_003 = fx_join(w2_003);
   int64_t z_mu_003; { FxAcc s = fx_zero(); fx_mac(s, w[1][0], u_003); fx_mac(s, w1_001, u_002); fx_mac(s, w1_002, u_001); fx_mac(s, w1_003, u_000); z_mu_003 = fx_sum(s); }
@@ -264,7 +264,7 @@ FX_FN void ck_euler1d_fx(const Fx (&w)[3][25], Fx ninv, const CkFixedConst& K, i
   int64_t z_p_003; { FxAcc s = fx_zero<FX_C>(); fx_mac(s, e_003, K.gm1); z_p_003 = fx_sum<FX_C>(s); }
   const Fx H_003 = fx_split(z_w2_003 + z_p_003 + FX_HALF, r);
   int64_t z_uH_103; { FxAcc s = fx_zero(); fx_mac(s, u_000, H_103); fx_mac(s, u_001, H_102); fx_mac(s, u_002, H_101); fx_mac(s, u_003, H_100); fx_mac(s, u_100, H_003); fx_mac(s, u_101, H_002); fx_mac(s, u_102, H_001); fx_mac(s, u_103, H_000); z_uH_103 = fx_sum(s); }
-  const Fx w2_004 = fx_split(fx_time<4>(1 * (z_uH_103), K.third) + FX_HALF, r);
+  const Fx w2_004 = fx_split_any(fx_time<4>(1 * (z_uH_103), K.third) + FX_HALF, r);
   t[0][1] = fx_join(w0_001);
   t[0][2] = fx_join(w0_002);
   t[0][3] = fx_join(w0_003);
@@ -303,44 +303,44 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
   {
   const Fx rho100 = S.ldrho(0, 1, 0);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 0, 0), -(1 << 30));
-    const Fx n = fx_split(fx_sum(s), r0);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel000 = fx_split(fx_sum<FX_C>(z), r0); }
+    const Fx n = fx_split_any(fx_sum(s), r0);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel000 = fx_split_any(fx_sum<FX_C>(z), r0); }
   const Fx rho010 = S.ldrho(0, 0, 1);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 1, 0), -(1 << 30));
     fx_mac(s, rho100, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel100 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel100 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho200 = S.ldrho(0, 2, 0);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 0, 1), -(1 << 30));
     fx_mac(s, rho010, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel010 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel010 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho110 = S.ldrho(0, 1, 1);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 2, 0), -(1 << 30));
     fx_mac(s, rho100, vel100);
     fx_mac(s, rho200, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel200 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel200 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho020 = S.ldrho(0, 0, 2);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 1, 1), -(1 << 30));
     fx_mac(s, rho010, vel100);
     fx_mac(s, rho100, vel010);
     fx_mac(s, rho110, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel110 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel110 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho300 = S.ldrho(0, 3, 0);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 0, 2), -(1 << 30));
     fx_mac(s, rho010, vel010);
     fx_mac(s, rho020, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel020 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel020 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho210 = S.ldrho(0, 2, 1);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 3, 0), -(1 << 30));
     fx_mac(s, rho100, vel200);
     fx_mac(s, rho200, vel100);
     fx_mac(s, rho300, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel300 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel300 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho120 = S.ldrho(0, 1, 2);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 2, 1), -(1 << 30));
     fx_mac(s, rho010, vel200);
@@ -348,8 +348,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho110, vel100);
     fx_mac(s, rho200, vel010);
     fx_mac(s, rho210, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel210 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel210 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho030 = S.ldrho(0, 0, 3);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 1, 2), -(1 << 30));
     fx_mac(s, rho010, vel110);
@@ -357,23 +357,23 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho100, vel020);
     fx_mac(s, rho110, vel010);
     fx_mac(s, rho120, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel120 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel120 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho400 = S.ldrho(0, 4, 0);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 0, 3), -(1 << 30));
     fx_mac(s, rho010, vel020);
     fx_mac(s, rho020, vel010);
     fx_mac(s, rho030, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel030 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel030 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho310 = S.ldrho(0, 3, 1);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 4, 0), -(1 << 30));
     fx_mac(s, rho100, vel300);
     fx_mac(s, rho200, vel200);
     fx_mac(s, rho300, vel100);
     fx_mac(s, rho400, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel400 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel400 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho220 = S.ldrho(0, 2, 2);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 3, 1), -(1 << 30));
     fx_mac(s, rho010, vel300);
@@ -383,8 +383,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho210, vel100);
     fx_mac(s, rho300, vel010);
     fx_mac(s, rho310, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel310 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel310 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho130 = S.ldrho(0, 1, 3);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 2, 2), -(1 << 30));
     fx_mac(s, rho010, vel210);
@@ -395,8 +395,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho200, vel020);
     fx_mac(s, rho210, vel010);
     fx_mac(s, rho220, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel220 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel220 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho040 = S.ldrho(0, 0, 4);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 1, 3), -(1 << 30));
     fx_mac(s, rho010, vel120);
@@ -406,15 +406,15 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho110, vel020);
     fx_mac(s, rho120, vel010);
     fx_mac(s, rho130, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel130 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel130 = fx_split_any(fx_sum<FX_C>(z), r); }
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(0, 0, 4), -(1 << 30));
     fx_mac(s, rho010, vel030);
     fx_mac(s, rho020, vel020);
     fx_mac(s, rho030, vel010);
     fx_mac(s, rho040, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel040 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel040 = fx_split_any(fx_sum<FX_C>(z), r); }
   }
   int64_t k000;
   int64_t k100;
@@ -559,89 +559,89 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
   int64_t f220;
   int64_t f130;
   { const int64_t E = S.ldE(0, 0, 0);
-    const Fx e = fx_split(E - ((k000 + S.swap(k000)) >> 1) + FX_HALF, r0);
+    const Fx e = fx_split_any(E - ((k000 + S.swap(k000)) >> 1) + FX_HALF, r0);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 0, 0, fx_split(E + p + FX_HALF, r0));
+    S.stH(0, 0, 0, fx_split_any(E + p + FX_HALF, r0));
   }
   { const int64_t E = S.ldE(0, 1, 0);
-    const Fx e = fx_split(E - ((k100 + S.swap(k010)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k100 + S.swap(k010)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 1, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 1, 0, fx_split_any(E + p + FX_HALF, r));
     f100 = k100 + p;
   }
   { const int64_t E = S.ldE(0, 0, 1);
-    const Fx e = fx_split(E - ((k010 + S.swap(k100)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k010 + S.swap(k100)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 0, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 0, 1, fx_split_any(E + p + FX_HALF, r));
   }
   { const int64_t E = S.ldE(0, 2, 0);
-    const Fx e = fx_split(E - ((k200 + S.swap(k020)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k200 + S.swap(k020)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 2, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 2, 0, fx_split_any(E + p + FX_HALF, r));
     f200 = k200 + p;
   }
   { const int64_t E = S.ldE(0, 1, 1);
-    const Fx e = fx_split(E - ((k110 + S.swap(k110)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k110 + S.swap(k110)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 1, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 1, 1, fx_split_any(E + p + FX_HALF, r));
     f110 = k110 + p;
   }
   { const int64_t E = S.ldE(0, 0, 2);
-    const Fx e = fx_split(E - ((k020 + S.swap(k200)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k020 + S.swap(k200)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 0, 2, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 0, 2, fx_split_any(E + p + FX_HALF, r));
   }
   { const int64_t E = S.ldE(0, 3, 0);
-    const Fx e = fx_split(E - ((k300 + S.swap(k030)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k300 + S.swap(k030)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 3, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 3, 0, fx_split_any(E + p + FX_HALF, r));
     f300 = k300 + p;
   }
   { const int64_t E = S.ldE(0, 2, 1);
-    const Fx e = fx_split(E - ((k210 + S.swap(k120)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k210 + S.swap(k120)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 2, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 2, 1, fx_split_any(E + p + FX_HALF, r));
     f210 = k210 + p;
   }
   { const int64_t E = S.ldE(0, 1, 2);
-    const Fx e = fx_split(E - ((k120 + S.swap(k210)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k120 + S.swap(k210)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 1, 2, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 1, 2, fx_split_any(E + p + FX_HALF, r));
     f120 = k120 + p;
   }
   { const int64_t E = S.ldE(0, 0, 3);
-    const Fx e = fx_split(E - ((k030 + S.swap(k300)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k030 + S.swap(k300)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 0, 3, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 0, 3, fx_split_any(E + p + FX_HALF, r));
   }
   { const int64_t E = S.ldE(0, 4, 0);
-    const Fx e = fx_split(E - ((k400 + S.swap(k040)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k400 + S.swap(k040)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 4, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 4, 0, fx_split_any(E + p + FX_HALF, r));
     f400 = k400 + p;
   }
   { const int64_t E = S.ldE(0, 3, 1);
-    const Fx e = fx_split(E - ((k310 + S.swap(k130)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k310 + S.swap(k130)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 3, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 3, 1, fx_split_any(E + p + FX_HALF, r));
     f310 = k310 + p;
   }
   { const int64_t E = S.ldE(0, 2, 2);
-    const Fx e = fx_split(E - ((k220 + S.swap(k220)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k220 + S.swap(k220)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 2, 2, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 2, 2, fx_split_any(E + p + FX_HALF, r));
     f220 = k220 + p;
   }
   { const int64_t E = S.ldE(0, 1, 3);
-    const Fx e = fx_split(E - ((k130 + S.swap(k310)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k130 + S.swap(k310)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 1, 3, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 1, 3, fx_split_any(E + p + FX_HALF, r));
     f130 = k130 + p;
   }
   { const int64_t E = S.ldE(0, 0, 4);
-    const Fx e = fx_split(E - ((k040 + S.swap(k400)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k040 + S.swap(k400)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(0, 0, 4, fx_split(E + p + FX_HALF, r));
+    S.stH(0, 0, 4, fx_split_any(E + p + FX_HALF, r));
   }
   int64_t drho000;
   int64_t drho100;
@@ -875,24 +875,24 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
   const Fx rho101 = S.ldrho(1, 1, 0);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 0, 0), -(1 << 30));
     fx_mac(s, rho001, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel001 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel001 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho010 = S.ldrho(0, 0, 1);
   const Fx rho011 = S.ldrho(1, 0, 1);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 1, 0), -(1 << 30));
     fx_mac(s, rho001, vel100);
     fx_mac(s, rho100, vel001);
     fx_mac(s, rho101, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel101 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel101 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho200 = S.ldrho(0, 2, 0);
   const Fx rho201 = S.ldrho(1, 2, 0);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 0, 1), -(1 << 30));
     fx_mac(s, rho001, vel010);
     fx_mac(s, rho010, vel001);
     fx_mac(s, rho011, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel011 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel011 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho110 = S.ldrho(0, 1, 1);
   const Fx rho111 = S.ldrho(1, 1, 1);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 2, 0), -(1 << 30));
@@ -901,8 +901,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho101, vel100);
     fx_mac(s, rho200, vel001);
     fx_mac(s, rho201, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel201 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel201 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho020 = S.ldrho(0, 0, 2);
   const Fx rho021 = S.ldrho(1, 0, 2);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 1, 1), -(1 << 30));
@@ -913,8 +913,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho101, vel010);
     fx_mac(s, rho110, vel001);
     fx_mac(s, rho111, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel111 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel111 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho300 = S.ldrho(0, 3, 0);
   const Fx rho301 = S.ldrho(1, 3, 0);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 0, 2), -(1 << 30));
@@ -923,8 +923,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho011, vel010);
     fx_mac(s, rho020, vel001);
     fx_mac(s, rho021, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel021 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel021 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho210 = S.ldrho(0, 2, 1);
   const Fx rho211 = S.ldrho(1, 2, 1);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 3, 0), -(1 << 30));
@@ -935,8 +935,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho201, vel100);
     fx_mac(s, rho300, vel001);
     fx_mac(s, rho301, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel301 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel301 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho120 = S.ldrho(0, 1, 2);
   const Fx rho121 = S.ldrho(1, 1, 2);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 2, 1), -(1 << 30));
@@ -951,8 +951,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho201, vel010);
     fx_mac(s, rho210, vel001);
     fx_mac(s, rho211, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel211 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel211 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho030 = S.ldrho(0, 0, 3);
   const Fx rho031 = S.ldrho(1, 0, 3);
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 1, 2), -(1 << 30));
@@ -967,8 +967,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho111, vel010);
     fx_mac(s, rho120, vel001);
     fx_mac(s, rho121, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel121 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel121 = fx_split_any(fx_sum<FX_C>(z), r); }
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(1, 0, 3), -(1 << 30));
     fx_mac(s, rho001, vel030);
     fx_mac(s, rho010, vel021);
@@ -977,8 +977,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho021, vel010);
     fx_mac(s, rho030, vel001);
     fx_mac(s, rho031, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel031 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel031 = fx_split_any(fx_sum<FX_C>(z), r); }
   }
   int64_t k001;
   int64_t k101;
@@ -1109,60 +1109,60 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
   int64_t f211;
   int64_t f121;
   { const int64_t E = E001;
-    const Fx e = fx_split(E - ((k001 + S.swap(k001)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k001 + S.swap(k001)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 0, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 0, 0, fx_split_any(E + p + FX_HALF, r));
   }
   { const int64_t E = E101;
-    const Fx e = fx_split(E - ((k101 + S.swap(k011)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k101 + S.swap(k011)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 1, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 1, 0, fx_split_any(E + p + FX_HALF, r));
     f101 = k101 + p;
   }
   { const int64_t E = E011;
-    const Fx e = fx_split(E - ((k011 + S.swap(k101)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k011 + S.swap(k101)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 0, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 0, 1, fx_split_any(E + p + FX_HALF, r));
   }
   { const int64_t E = E201;
-    const Fx e = fx_split(E - ((k201 + S.swap(k021)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k201 + S.swap(k021)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 2, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 2, 0, fx_split_any(E + p + FX_HALF, r));
     f201 = k201 + p;
   }
   { const int64_t E = E111;
-    const Fx e = fx_split(E - ((k111 + S.swap(k111)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k111 + S.swap(k111)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 1, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 1, 1, fx_split_any(E + p + FX_HALF, r));
     f111 = k111 + p;
   }
   { const int64_t E = E021;
-    const Fx e = fx_split(E - ((k021 + S.swap(k201)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k021 + S.swap(k201)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 0, 2, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 0, 2, fx_split_any(E + p + FX_HALF, r));
   }
   { const int64_t E = E301;
-    const Fx e = fx_split(E - ((k301 + S.swap(k031)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k301 + S.swap(k031)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 3, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 3, 0, fx_split_any(E + p + FX_HALF, r));
     f301 = k301 + p;
   }
   { const int64_t E = E211;
-    const Fx e = fx_split(E - ((k211 + S.swap(k121)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k211 + S.swap(k121)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 2, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 2, 1, fx_split_any(E + p + FX_HALF, r));
     f211 = k211 + p;
   }
   { const int64_t E = E121;
-    const Fx e = fx_split(E - ((k121 + S.swap(k211)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k121 + S.swap(k211)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 1, 2, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 1, 2, fx_split_any(E + p + FX_HALF, r));
     f121 = k121 + p;
   }
   { const int64_t E = E031;
-    const Fx e = fx_split(E - ((k031 + S.swap(k301)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k031 + S.swap(k301)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(1, 0, 3, fx_split(E + p + FX_HALF, r));
+    S.stH(1, 0, 3, fx_split_any(E + p + FX_HALF, r));
   }
   int64_t drho001;
   int64_t drho101;
@@ -1338,8 +1338,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(2, 0, 0), -(1 << 30));
     fx_mac(s, rho001, vel001);
     fx_mac(s, rho002, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel002 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel002 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho010 = S.ldrho(0, 0, 1);
   const Fx rho011 = S.ldrho(1, 0, 1);
   const Fx rho012 = S.ldrho(2, 0, 1);
@@ -1349,8 +1349,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho100, vel002);
     fx_mac(s, rho101, vel001);
     fx_mac(s, rho102, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel102 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel102 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho200 = S.ldrho(0, 2, 0);
   const Fx rho201 = S.ldrho(1, 2, 0);
   const Fx rho202 = S.ldrho(2, 2, 0);
@@ -1360,8 +1360,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho010, vel002);
     fx_mac(s, rho011, vel001);
     fx_mac(s, rho012, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel012 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel012 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho110 = S.ldrho(0, 1, 1);
   const Fx rho111 = S.ldrho(1, 1, 1);
   const Fx rho112 = S.ldrho(2, 1, 1);
@@ -1374,8 +1374,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho200, vel002);
     fx_mac(s, rho201, vel001);
     fx_mac(s, rho202, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel202 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel202 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho020 = S.ldrho(0, 0, 2);
   const Fx rho021 = S.ldrho(1, 0, 2);
   const Fx rho022 = S.ldrho(2, 0, 2);
@@ -1391,8 +1391,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho110, vel002);
     fx_mac(s, rho111, vel001);
     fx_mac(s, rho112, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel112 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel112 = fx_split_any(fx_sum<FX_C>(z), r); }
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(2, 0, 2), -(1 << 30));
     fx_mac(s, rho001, vel021);
     fx_mac(s, rho002, vel020);
@@ -1402,8 +1402,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho020, vel002);
     fx_mac(s, rho021, vel001);
     fx_mac(s, rho022, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel022 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel022 = fx_split_any(fx_sum<FX_C>(z), r); }
   }
   int64_t k002;
   int64_t k102;
@@ -1492,37 +1492,37 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
   int64_t f202;
   int64_t f112;
   { const int64_t E = E002;
-    const Fx e = fx_split(E - ((k002 + S.swap(k002)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k002 + S.swap(k002)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(2, 0, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(2, 0, 0, fx_split_any(E + p + FX_HALF, r));
   }
   { const int64_t E = E102;
-    const Fx e = fx_split(E - ((k102 + S.swap(k012)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k102 + S.swap(k012)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(2, 1, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(2, 1, 0, fx_split_any(E + p + FX_HALF, r));
     f102 = k102 + p;
   }
   { const int64_t E = E012;
-    const Fx e = fx_split(E - ((k012 + S.swap(k102)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k012 + S.swap(k102)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(2, 0, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(2, 0, 1, fx_split_any(E + p + FX_HALF, r));
   }
   { const int64_t E = E202;
-    const Fx e = fx_split(E - ((k202 + S.swap(k022)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k202 + S.swap(k022)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(2, 2, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(2, 2, 0, fx_split_any(E + p + FX_HALF, r));
     f202 = k202 + p;
   }
   { const int64_t E = E112;
-    const Fx e = fx_split(E - ((k112 + S.swap(k112)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k112 + S.swap(k112)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(2, 1, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(2, 1, 1, fx_split_any(E + p + FX_HALF, r));
     f112 = k112 + p;
   }
   { const int64_t E = E022;
-    const Fx e = fx_split(E - ((k022 + S.swap(k202)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k022 + S.swap(k202)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(2, 0, 2, fx_split(E + p + FX_HALF, r));
+    S.stH(2, 0, 2, fx_split_any(E + p + FX_HALF, r));
   }
   int64_t drho002;
   int64_t drho102;
@@ -1630,8 +1630,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho001, vel002);
     fx_mac(s, rho002, vel001);
     fx_mac(s, rho003, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel003 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel003 = fx_split_any(fx_sum<FX_C>(z), r); }
   const Fx rho010 = S.ldrho(0, 0, 1);
   const Fx rho011 = S.ldrho(1, 0, 1);
   const Fx rho012 = S.ldrho(2, 0, 1);
@@ -1644,8 +1644,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho101, vel002);
     fx_mac(s, rho102, vel001);
     fx_mac(s, rho103, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel103 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel103 = fx_split_any(fx_sum<FX_C>(z), r); }
   { FxAcc s = fx_zero(true); fx_mac_int(s, S.ldmom(3, 0, 1), -(1 << 30));
     fx_mac(s, rho001, vel012);
     fx_mac(s, rho002, vel011);
@@ -1654,8 +1654,8 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
     fx_mac(s, rho011, vel002);
     fx_mac(s, rho012, vel001);
     fx_mac(s, rho013, vel000);
-    const Fx n = fx_split(fx_sum(s), r);
-    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel013 = fx_split(fx_sum<FX_C>(z), r); }
+    const Fx n = fx_split_any(fx_sum(s), r);
+    FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel013 = fx_split_any(fx_sum<FX_C>(z), r); }
   }
   int64_t k003;
   int64_t k103;
@@ -1702,20 +1702,20 @@ FX_DEV void ck_euler2d_lane(Store& S, Fx ninv, Fx gm1, Fx third, FxRange& r) {
   }
   int64_t f103;
   { const int64_t E = E003;
-    const Fx e = fx_split(E - ((k003 + S.swap(k003)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k003 + S.swap(k003)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(3, 0, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(3, 0, 0, fx_split_any(E + p + FX_HALF, r));
   }
   { const int64_t E = E103;
-    const Fx e = fx_split(E - ((k103 + S.swap(k013)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k103 + S.swap(k013)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(3, 1, 0, fx_split(E + p + FX_HALF, r));
+    S.stH(3, 1, 0, fx_split_any(E + p + FX_HALF, r));
     f103 = k103 + p;
   }
   { const int64_t E = E013;
-    const Fx e = fx_split(E - ((k013 + S.swap(k103)) >> 1) + FX_HALF, r);
+    const Fx e = fx_split_any(E - ((k013 + S.swap(k103)) >> 1) + FX_HALF, r);
     FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);
-    S.stH(3, 0, 1, fx_split(E + p + FX_HALF, r));
+    S.stH(3, 0, 1, fx_split_any(E + p + FX_HALF, r));
   }
   int64_t drho003;
   int64_t dmom003;

@@ -57,7 +57,7 @@ class GenFixed:
             z = f"{m + 1} * {self.zf(f'F{q}', m + 1, n, k - 1)}"
             if self.dim == 2:
                 z += f" + {n + 1} * {self.zf(f'G{q}', m, n + 1, k - 1)}"
-            self.lines.append(f"  const Fx {v} = fx_split(fx_time<{k}>({z}, K.third) + FX_HALF, r);")
+            self.lines.append(f"  const Fx {v} = fx_split_any(fx_time<{k}>({z}, K.third) + FX_HALF, r);")
         elif name in ("u", "v"):
             num, den = W[1 if name == "u" else 2], W[0]
             acc = [f"fx_mac_int(s, {self.fx(num, m, n, k)}, -(1 << 30));"]
@@ -380,8 +380,8 @@ class GenLane:
             for p, q, t in self.subs(i, j, c):
                 if p + q + t:
                     self.out(f"  fx_mac(s, rho{p}{q}{t}, vel{i - p}{j - q}{c - t});")
-            self.out(f"  const Fx n = fx_split(fx_sum(s), {rng(i, j)});")
-            self.out(f"  FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel{i}{j}{c} = fx_split(fx_sum<FX_C>(z), {rng(i, j)}); }}")
+            self.out(f"  const Fx n = fx_split_any(fx_sum(s), {rng(i, j)});")
+            self.out(f"  FxAcc z = fx_zero<FX_C>(true); fx_mac(z, n, ninv); vel{i}{j}{c} = fx_split_any(fx_sum<FX_C>(z), {rng(i, j)}); }}")
         self.out("}")
         # mom vel, then the pressure and H
         for i, j in self.pairs(D):
@@ -399,9 +399,9 @@ class GenLane:
         for i, j in self.pairs(D):
             E = f"S.ldE(0, {i}, {j})" if c == 0 else f"E{i}{j}{c}"
             self.out(f"{{ const int64_t E = {E};")
-            self.out(f"  const Fx e = fx_split(E - ((k{i}{j}{c} + S.swap(k{j}{i}{c})) >> 1) + FX_HALF, {rng(i, j)});")
+            self.out(f"  const Fx e = fx_split_any(E - ((k{i}{j}{c} + S.swap(k{j}{i}{c})) >> 1) + FX_HALF, {rng(i, j)});")
             self.out(f"  FxAcc s = fx_zero<FX_C>(); fx_mac(s, e, gm1); const int64_t p = fx_sum<FX_C>(s);")
-            self.out(f"  S.stH({c}, {i}, {j}, fx_split(E + p + FX_HALF, {rng(i, j)}));")
+            self.out(f"  S.stH({c}, {i}, {j}, fx_split_any(E + p + FX_HALF, {rng(i, j)}));")
             if i >= 1:
                 self.out(f"  f{i}{j}{c} = k{i}{j}{c} + p;")
             self.out("}")

@@ -332,10 +332,10 @@ struct CkLane {
       both_out[n - 1] = both;
     }
     if (n == 4) return;
-    ck_st(momL + ck_level_row(n) * kCkRow + off[ck_pair(i, j)], fx_split(own + FX_HALF, r));
+    ck_st(momL + ck_level_row(n) * kCkRow + off[ck_pair(i, j)], fx_split_any(own + FX_HALF, r));
     FxRange rb{0};
-    const Fx v = fx_split(both + FX_HALF, rb);
-    r.h |= dir ? 0u : rb.h;
+    const Fx v = fx_split_any(both + FX_HALF, rb);
+    r.t |= dir ? 0u : rb.t;
     const Fx e = Fx{(int32_t)((uint64_t)both & 0xffffffffu), (int32_t)(both >> 32)};  // low word first
     ck_st((dir ? e0 : lev + ck_level_row(n) * kCkRow) + off[ck_pair(i, j)], dir ? e : v);
   }

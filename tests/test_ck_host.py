@@ -15,10 +15,19 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "..", "paper_2304_09724_gb300", "csrc")
 
 
+def build(tmp_path, name):
+    exe = str(tmp_path / name)
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wno-return-type", "-I", CSRC, os.path.join(HERE, name + ".cpp"), "-o", exe])
+    return [list(map(float, line.split())) for line in subprocess.check_output([exe], text=True).splitlines()]
+
+
+def test_range_check_sees_every_value(tmp_path):
+    """The operand checks over all of 64 bits: nothing in range refused, nothing out of range let through."""
+    assert build(tmp_path, "fx_host") == [[0, 0, 0], [0, 0, 0]]
+
+
 def test_recursion_over_gas_constants(tmp_path):
-    exe = str(tmp_path / "ck_host")
-    subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wno-return-type", "-I", CSRC, os.path.join(HERE, "ck_host.cpp"), "-o", exe])
-    rows = [list(map(float, line.split())) for line in subprocess.check_output([exe], text=True).splitlines()]
+    rows = build(tmp_path, "ck_host")
     assert len(rows) == 12
     for gamma, *err in rows:
         for q in range(3):
