@@ -415,6 +415,7 @@ struct shweno_batch {
   long long spin_limit = 4000000;  // x ~256 ns sleeps: about a second
   std::string err;
   cudaGraphExec_t graph = nullptr;
+  double graph_cfl = 0.0;  // the CFL number that its launches carry
   std::vector<double> tuned;  // autotuner timings (ms) per candidate
   int mode = SHWENO_BATCH_AUTO;  // SHWENO_BATCH_AUTO / _PERSISTENT / _LOCKSTEP
   int* lstart = nullptr;         // lockstep block tables: [kind][problem + 1] prefix sums
@@ -640,6 +641,7 @@ shweno_status run_once(shweno_batch* b, const double* t_final, double cfl, int64
       cudaError_t e = cudaGraphInstantiate(&b->graph, g, 0);
       cudaGraphDestroy(g);
       if (e != cudaSuccess) return bfail(b, SHWENO_E_CUDA, "graph instantiation failed");
+      b->graph_cfl = cfl;
     }
     if (cudaGraphLaunch(b->graph, b->stream) != cudaSuccess) return bfail(b, SHWENO_E_CUDA, "graph launch failed");
   } else {
@@ -750,10 +752,7 @@ shweno_status shweno_batch_run(shweno_batch* b, const double* t_final, double cf
   using namespace shweno;
   if (!b || !t_final || !(cfl > 0.0)) return bfail(b, SHWENO_E_INVALID, "invalid argument");
   const int n = (int)b->views.size();
-  // the cached graph bakes in the cfl; rebuild when it changes
-  static thread_local double last_cfl = -1.0;
-  if (b->graph && cfl != last_cfl) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
-  last_cfl = cfl;
+  if (b->graph && cfl != b->graph_cfl) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
   shweno_status s = use_lockstep(b) ? run_lockstep(b, t_final, cfl, max_steps)
                                     : run_once(b, t_final, cfl, max_steps, max_steps <= 0);
   if (per_problem) {
