@@ -244,8 +244,9 @@ shweno_status shweno_get_flags(shweno_handle* h, uint8_t* out, int on_device);
  * Both modes run the same items and the same step commit: the same step counts and times, states
  * equal to round-off (the compiler may fuse a product into a multiply-add differently in the two
  * kernels).  Each step is committed on the problem's own control block, so every handle stays
- * usable on its own afterwards.  The handles must outlive the batch and must not be used on their own
- * while a batch run is in flight. */
+ * usable on its own afterwards.  A run (or the autotuner) starts after everything that the handles
+ * have in flight on their own streams.  The handles must outlive the batch and must not be used on
+ * their own while a batch run is in flight. */
 typedef struct shweno_batch shweno_batch;
 
 /* Run modes (shweno_batch_set_mode).  AUTO: lockstep when every problem is 2D (their items are

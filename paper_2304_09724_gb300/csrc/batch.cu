@@ -407,6 +407,7 @@ struct shweno_batch {
   int nchunks = 0;
   double* t_final = nullptr;
   cudaStream_t stream = nullptr;
+  cudaEvent_t joined = nullptr;  // orders the batch's stream after its handles'
   bool own_stream = false;
   int tile1d = 512;
   int ctas_per_sm = 2;
@@ -513,6 +514,11 @@ shweno_status shweno_batch_create(shweno_handle* const* hs, int n, void* cuda_st
     }
     b->own_stream = true;
   }
+  if (cudaEventCreateWithFlags(&b->joined, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    shweno_batch_destroy(b);
+    return SHWENO_E_CUDA;
+  }
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -568,6 +574,7 @@ shweno_status shweno_batch_destroy(shweno_batch* b) {
   if (!b) return SHWENO_OK;
   if (b->stream) cudaStreamSynchronize(b->stream);
   if (b->graph) cudaGraphExecDestroy(b->graph);
+  if (b->joined) cudaEventDestroy(b->joined);
   cudaFree(b->probs);
   cudaFree(b->pstate);
   cudaFree(b->bc);
@@ -605,10 +612,22 @@ void enqueue_batch(shweno_batch* b, double cfl) {
                                                                   cap - 1, b->spin_limit);
 }
 
+// Orders b->stream after everything its handles have in flight on their own streams (shweno_set_state and
+// shweno_advance return before their work is done).  One event serves all: a wait keeps the record it saw.
+shweno_status join_handles(shweno_batch* b) {
+  for (const auto& v : b->views)
+    if (v.stream != b->stream &&
+        (cudaEventRecord(b->joined, v.stream) != cudaSuccess || cudaStreamWaitEvent(b->stream, b->joined, 0) != cudaSuccess))
+      return bfail(b, SHWENO_E_CUDA, "waiting for a handle's stream failed");
+  return SHWENO_OK;
+}
+
 // Problem table, start step counts and end times of one run, uploaded on b->stream.
 shweno_status prepare_run(shweno_batch* b, const double* t_final, int64_t max_steps) {
   using namespace shweno;
   const int n = (int)b->views.size();
+  const shweno_status js = join_handles(b);
+  if (js != SHWENO_OK) return js;
   for (int p = 0; p < n; ++p) {
     fill_problem(b, p);
     b->host_probs[p].max_steps = max_steps > 0 ? max_steps : INT64_MAX;
@@ -784,6 +803,8 @@ shweno_status shweno_batch_autotune(shweno_batch* b, const double* t_final, doub
     if (ctas_per_sm_out) *ctas_per_sm_out = b->ctas_per_sm;
     return SHWENO_OK;
   }
+  const shweno_status js = join_handles(b);
+  if (js != SHWENO_OK) return js;
   // backups of the states and control blocks
   std::vector<double*> bk(n, nullptr);
   std::vector<Ctl> cbk(n);
