@@ -19,6 +19,7 @@
 //                then dilated by one cell (3x3 OR), imposed-state ghost cells count as troubled.
 #include <cuda_runtime.h>
 
+#include "device_once.h"
 #include "flagnet_items.cuh"
 #include "shweno_kernels.h"
 
@@ -352,12 +353,14 @@ void mlp_forward(const float* params, const float* X, int64_t n, float* prob, cu
 }
 cudaError_t mlp_grad(const float* params, const float* X, const float* y, int64_t n, float pw,
                      float* grad, float* loss, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(GradSmem));
+  static DeviceOnce limit;  // the kernel's shared-memory limit belongs to the device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (limit.needed(dev)) {
+    e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem));
     if (e != cudaSuccess) return e;
-    attr = true;
+    limit.done(dev);
   }
   mlp_zero_kernel<<<(NPARAM + 256) / 256, 256, 0, st>>>(grad, loss);
   if (n > 0)
