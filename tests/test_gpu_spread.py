@@ -92,3 +92,22 @@ def test_quiet_side_in_a_batch(mode):
     b.close()
     for sol in sols:
         sol.close()
+
+
+@pytest.mark.parametrize("gam", [(0.1, 0.45, 0.45), (0.2, 0.5, 0.3), (0.26, 0.37, 0.37), (0.6, 0.2, 0.2)])
+def test_linear_weights_of_any_size(gam):
+    """A cell's p1 carries up to 1 / gam[0]: 10 and 5 are out of the fixed-point format, 3.8 and 1.7 in it."""
+    st, _, dt, _ = blocked("energy", 3.0)
+    h = S.shweno_create(S.make_grid(2, S.EULER, NX, NY), 1.4, S.make_bc((0, 0, 0, 0)), S.make_opts(gam=gam))
+    S.shweno_set_state(h, *(np.ascontiguousarray(st[k]) for k in "WVYZ"))
+    P = O.make_problem(2, S.EULER, NX, NY, 0.0, 1.0, 0.0, 1.0, gam=gam)
+    o = st
+    for _ in range(2):
+        S.shweno_step(h, 300.0 * dt)
+        o = O.step(P, o, 300.0 * dt)
+    g = {k: np.empty_like(st[k]) for k in "WVYZ"}
+    S.shweno_get_state(h, *(g[k] for k in "WVYZ"))
+    S.shweno_destroy(h)
+    wl = WL.vortex(8)
+    wl.nx, wl.ny, wl.domain = NX, NY, (0.0, 1.0, 0.0, 1.0)
+    U.check(g, o, "WVYZ", shocked=True, what=f"gam {gam}", wl=wl)
