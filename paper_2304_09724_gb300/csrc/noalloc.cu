@@ -6,7 +6,8 @@
 // memory through their own pool and forbid a library from allocating behind their back.
 // shweno_step1d_noalloc serves them: the caller passes its input and output state, and the control
 // block of the step kernel (all the scratch a 1D step has) lives in one file-scope __device__ array
-// of fixed size that every GPU loading this library holds until the process exits.  The call waits for its own work before it returns.
+// of fixed size that every GPU loading this library holds until the process exits.  The call waits
+// for its own work before it returns.
 //
 // Set-up: the device address of that array is looked up with cudaGetSymbolAddress the first
 // time the entry point runs on a device (with that device current) and cached per device for

@@ -8,6 +8,8 @@
 
 namespace shweno {
 
+constexpr int kSMs = 152;  // of a GB300: the launch rules below count CTAs by it
+
 // Scratch buffers of one 2D step (all device memory owned by the handle).
 struct Scratch2D {
   double* ycoef;  // [2 sets][ncomp][KC coefs][ny+2][nx+4], KC = 5 (R1) or 6 (R1')

@@ -47,7 +47,7 @@ void launch_step1d(const Params& P, Ctl* ctl, const double* s0, const double* s1
                    double* o1, const uint8_t* flag, cudaStream_t st, cudaEvent_t* ev) {
   const int warps = (P.nx + W1D - 1) / W1D;
   if (ev) cudaEventRecord(ev[0], st);
-  if (P.ncomp == 3 && !P.charwise && warps <= 304) {
+  if (P.ncomp == 3 && !P.charwise && warps <= 2 * kSMs) {
     // Four warps for W1D cells: the latency of one chain of FP64 instructions is all there is, so it
     // is shortened.  Lax, 200 cells, whole run: 9.1 -> 5.6 ms against one warp per CTA.  The line is
     // two CTAs per SM, as many as its registers hold, in one wave (9120 cells).  Per step, one warp per
@@ -57,9 +57,9 @@ void launch_step1d(const Params& P, Ctl* ctl, const double* s0, const double* s1
     else step1d_small_kernel<false><<<warps, 128, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);
   } else {
     // One warp per CTA while the mesh does not fill the GPU: the CTAs then go to different SMs, each
-    // warp has a scheduler's FP64 unit to itself.  From 152 SMs x 4 schedulers x 2 warps on, four:
+    // warp has a scheduler's FP64 unit to itself.  From two warps per scheduler on, four:
     // three such CTAs per SM (4M cells: 13.9 ms with two, 12.0 with three).
-    const int per = warps < 1216 ? 1 : 4;
+    const int per = warps < 8 * kSMs ? 1 : 4;
     const dim3 g((warps + per - 1) / per), b(32 * per);
     if (P.ncomp == 1) {
       if (P.quintic) step1d_kernel<1, true><<<g, b, 0, st>>>(P, ctl, s0, s1, o0, o1, flag);

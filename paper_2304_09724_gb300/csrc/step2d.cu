@@ -26,8 +26,8 @@ Scratch2D carve_scratch2d(const Params& P, double* base) {
   return S;
 }
 
-// One of the face kernels alone does not fill the 304 CTA slots.
-bool faces_beside(const Params& P) { return 4 * (long long)FaceSplit(P.nx + 1).ctas(P.ny + 1) < 304; }
+// One of the face kernels alone does not fill two CTAs per SM.
+bool faces_beside(const Params& P) { return 4 * (long long)FaceSplit(P.nx + 1).ctas(P.ny + 1) < 2 * kSMs; }
 
 cudaError_t init_kernels2d() {
   const cudaError_t e = init_kernels2d_reading<false>();

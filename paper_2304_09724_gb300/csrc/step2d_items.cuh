@@ -238,6 +238,7 @@ __device__ __forceinline__ void pass_order(const Params& P, const double (*ev)[5
 // half-warp reads 128 consecutive bytes), and the owner converts the results back.  One thread
 // cannot hold the recursion's series in registers beside its accumulators (10 KB of spills);
 // split over two lanes and shared memory it needs about 5500 instructions a lane and no spills.
+// In FP64 (ck_points64) one thread does hold it.
 constexpr int CKP = 64;               // points in work at a time
 constexpr int kCkRow = CKP * 8;       // bytes of one coefficient of them
 constexpr int kCkIn = 0;              // [2 halves][4 comps][15] level 0 (in the end: the results)
@@ -1182,14 +1183,14 @@ __device__ __forceinline__ void xface_item(const Params& P, const StepView& sv, 
     CkLead lead;
     if (fr.has_face) {
 #pragma unroll
-    for (int q = 0; q < NC; ++q) {
-      if (slice < 3)
-        Wref[q] = 0.5 * (fetch(P, st, 0, q, fi - 1, row, sv.t) + fetch(P, st, 0, q, fi, row, sv.t));
-      else
-        Wref[q] = 0.25 * (fetch(P, st, 0, q, fi - 1, row - 1, sv.t) + fetch(P, st, 0, q, fi, row - 1, sv.t) +
-                          fetch(P, st, 0, q, fi - 1, row, sv.t) + fetch(P, st, 0, q, fi, row, sv.t));
-    }
-    char_face_point<NC, FLAGS, Q>(P, ev, ft, fr.col - 1, 0, a, lead, Wref);
+      for (int q = 0; q < NC; ++q) {
+        if (slice < 3)
+          Wref[q] = 0.5 * (fetch(P, st, 0, q, fi - 1, row, sv.t) + fetch(P, st, 0, q, fi, row, sv.t));
+        else
+          Wref[q] = 0.25 * (fetch(P, st, 0, q, fi - 1, row - 1, sv.t) + fetch(P, st, 0, q, fi, row - 1, sv.t) +
+                            fetch(P, st, 0, q, fi - 1, row, sv.t) + fetch(P, st, 0, q, fi, row, sv.t));
+      }
+      char_face_point<NC, FLAGS, Q>(P, ev, ft, fr.col - 1, 0, a, lead, Wref);
     }
     ck_points<NC>(P, fr.nrun * (fr.nf + 1), fr.has_face, 0, a, lead, tc);
   } else {

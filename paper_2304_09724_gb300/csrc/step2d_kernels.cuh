@@ -156,7 +156,7 @@ static void launch_step2d_nc(const Params& P, Ctl* ctl, const double* s0, const 
                              double* o0, double* o1, const uint8_t* flag, const Scratch2D& S,
                              cudaStream_t st, cudaEvent_t* ev) {
   // 40^2 cells: coef2d 38 -> 29 us, update2d 27 -> 21 us with the low tiles
-  const bool small = ((P.nx + TX - 1) / TX) * ((P.ny + TY - 1) / TY) < 304;
+  const bool small = ((P.nx + TX - 1) / TX) * ((P.ny + TY - 1) / TY) < 2 * kSMs;
   const int th = small ? TY_SMALL : TY;
   const dim3 cb(TX, th), cg((P.nx + 4 + TX - 1) / TX, (P.ny + 4 + th - 1) / th, 4);
   if (ev) cudaEventRecord(ev[0], st);
