@@ -504,8 +504,8 @@ __device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_fac
 // does is noticed and the CTA takes the FP64 pass instead: before any work, data that are not finite or
 // not of one size (cell_exponents); on the way (FxRange), face units far above the density or energy,
 // eigenvectors beyond 2^4 in them, end values above 8 times the data, weights of 4 and more.
-constexpr int FX_ABOVE = 2;       // most bits of a cell's data above the size its own state gives the component
-constexpr int FX_BELOW = 4;       // a momentum more bits than this below that size is a slow one,
+constexpr int FX_ABOVE = 4;       // most bits of a cell's data above the size its own state gives the component
+constexpr int FX_BELOW = 6;       // a momentum more bits than this below that size is a slow one,
                                   // and one more than FX_STILL counts as none
 constexpr int FX_UNIT = 5;        // most bits of a face's density and energy below their units
 constexpr int FX_EL = FX_D - 53;  // most bits that the projections' scale takes off
@@ -524,20 +524,23 @@ __device__ __forceinline__ int64_t fx_scaled(Fx x, Fx c) {
 }
 
 // Exponents of the cell's data over all orders and its three columns; false if FP64 holds them better.
-// FP64 rounds every value by its own size, a block by its largest.
-//   A cold cell beside a hot one, which the weights cut off, would round at 2^-57 of the hot one, about
-// five times over (energy 2.5 beside 564: 1.4e-14 of the cold cell's end value, in FP64 3e-16; beside 1e12:
-// 5e-6).  So no value may be more than FX_ABOVE bits above the cell's own density, energy, or the momentum
-// sqrt(rho E) they allow: 5 * 2^-57 * 2^3 is FP64's 3e-16.
+// FP64 rounds every value by its own size, a block by its largest.  The lines below lie where the error of a whole
+// step against 64-bit mantissas begins to exceed that of the FP64 pass.
+//   A cold cell beside a hot one, which the weights cut off, rounds at 2^-57 of the hot one (energy 2.5
+// beside 564: 1.4e-14 of the cold cell's end value, in FP64 3e-16; beside 1e12: 5e-6).  So no value may be
+// more than FX_ABOVE bits above the cell's own density, energy, or the momentum sqrt(rho E) they allow.  Cells beside
+// a block of 2^k times their density and energy, error of their slopes relative to the FP64 pass, mean of
+// three flows: 1.0 at k = 3, 1.1 at 4, 1.6 at 5, 2.7 at 6, 3.8 at 7, 13 at 10.
 //   A slow momentum rounds at 2^-57 of that one: less than what the rounding of the pressure, 2^-53 of
 // rho c^2, does in every step to the momentum across the face, and to the one along the face where the energy
 // varies along it.  Where it does not (a shear layer), the pressure moves nothing and FP64 carries
-// the momentum with all its bits.
-//   Share of the CTAs that go to FP64: vortex, smooth flows 0; quadrants 0 to 0.6 % (400^2, 300 steps); double Mach
-// reflection about 10 % (1024 x 256, 400 steps), whose step takes 8.5 ms (8.7 with every CTA in fixed
-// point).  If any slow momentum went there: quadrants 16 to 65 %.  Testing the cells: 0.2 % of the vortex step
-// (2048^2).  Drift of a shear flow at 1e-6 of the sound speed, three steps, error against 64-bit mantissas:
-// 2.0e-13 -> 7.5e-17.
+// the momentum with all its bits.  Shear flow, three steps, error of the drift's slope relative to the FP64
+// pass: 0.9 at 6 bits below, 1.2 at 7, 1.4 at 8, 2.5 at 9, 6 at 10, 10 at 11.
+//   Share of the CTAs that go to FP64: vortex, smooth flows 0; quadrants 0 to 0.6 % (400^2, 300 steps), random ones
+// (rho, p in [0.1, 2]) 0 to 13 %; double Mach reflection 11 % (1024 x 256, 400 steps), whose step takes 8.5 ms (8.7
+// with every CTA in fixed point).  If any slow momentum went there: quadrants 16 to 65 %.  Testing the cells:
+// 0.2 % of the vortex step (2048^2).  Drift of a shear flow at 1e-6 of the sound speed, three steps, error
+// against 64-bit mantissas: 2.0e-13 -> 7.5e-17.
 __device__ __forceinline__ bool cell_exponents(const double (*ev)[5][SPAN], int c, int dir, int h[4]) {
   auto mag = [&](int f, int k, int col) { return fx_hi(ev[f][k][col]) & 0x7fffffff; };
   const int n0 = fx_exp(mag(0, 0, c)), n3 = fx_exp(mag(3, 0, c)), nm = (n0 + n3 + 1) >> 1;
