@@ -40,7 +40,7 @@ FP64_SLOTS_PER_S = 152 * 2 * 2.070e9  # FP64 thread instructions per second (DFM
 # is left on the FP64 pipe.
 FLOPS_PER_XFACE_POINT = 890.1
 FP64_INST_PER_XFACE_POINT = 571.9
-DRAM_BYTES_PER_XFACE_POINT = 371.6
+DRAM_BYTES_PER_XFACE_POINT = 366.4
 BYTES_PER_CELL_UPDATE = 256  # 16 doubles read + 16 written per cell (ideal reuse)
 
 

@@ -1,7 +1,7 @@
 // Device building blocks of the ADER-SHWENO step (arXiv 2304.09724), shared by the 1D and 2D
 // kernels: boundary-condition lookup, the SHWENO reconstruction pieces, the leading-term
 // Riemann solvers, the eigen-upwinded linearised Riemann problem and the physical fluxes.
-// Everything is FP64; the FP64 pipe (2 DFMA/clk/SM on sm_103) bounds the step, so each
+// Everything here is FP64; the FP64 pipe (2 DFMA/clk/SM on sm_103) bounds most of the kernels, so each
 // routine is arranged to spend as few FP64 instructions as the mathematics allows.
 #pragma once
 #include <cstdint>
