@@ -16,7 +16,8 @@
 //     FP64's error);
 //   - gamma near 1: sqrt(H0) is far above |u| + c then, and order k in time rounds at (sqrt(H0) / (|u| + c))^k
 //     times what it should (gamma 1.02, half a cell per step: 1.6e-15 of the density, FP64 1e-20);
-//   - a slow momentum along a 2D face where the energy does not vary (step2d_items.cuh).
+//   - a slow momentum along a 2D face where the energy does not vary (step2d_items.cuh);
+//   - a density or velocity below 2^-300, where the exponents end.
 // It does not show in a slow momentum across the face: the star state's energy is rounded there, in FP64
 // too.  1D contacts, 100 cells, 8 steps, velocity 1e-2 / 1e-4 / 1e-8, error of the momentum against 64-bit
 // mantissas: 1.18e-14 / 1.05e-12 / 6.3e-9, with the FP64 recursion 1.17e-14 / 1.05e-12 / 6.4e-9.  156 random shock
@@ -42,6 +43,7 @@ struct CkFixed {
 // fixed point, error of the drift's slope relative to FP64: 1.0 at 8 bits below, 1.1 at 9, 2 at 10, 3 at 11.
 constexpr int CK_BELOW = 8;
 constexpr int FX_STILL = 48;  // a momentum more bits than this below its scale counts as none
+constexpr int CK_TINY = -300;  // least exponent of the units of density and velocity
 
 FX_FN Fx fx_const(double x) {
   FxRange r{0};
@@ -68,8 +70,11 @@ struct CkLead {
   int32_t hu, hH, hc;
 };
 // Whether the unit of velocity 2^eu is more than 4 times the larger of velocity and sound speed (never for gamma
-// of 1.4 and more); order 4 in time of half a cell per step then rounds at more than 16 quanta.
-FX_FN bool ck_fast_unit(int eu, const CkLead& lead) { return eu > fx_max(fx_exp(lead.hu), fx_exp(lead.hc)) + 1; }
+// of 1.4 and more); order 4 in time of half a cell per step then rounds at more than 16 quanta.  Or it is the
+// least one: a state may lie anywhere below it.
+FX_FN bool ck_off_unit(int eu, const CkLead& lead) {
+  return eu > fx_max(fx_exp(lead.hu), fx_exp(lead.hc)) + 1 || eu <= CK_TINY;
+}
 
 // Scales of one point: the exponents of its fields and the growth.
 template <int NC>
@@ -81,18 +86,24 @@ struct CkScale {
   FX_FN int of(int q, int s) const { return base[group(q)] + g * s; }
 };
 
+// Euler: whether the point's units of density and velocity do not fit it.
+template <int NC>
+FX_FN bool ck_off_units(const CkScale<NC>& S, const CkLead& lead) {
+  return ck_off_unit(S.eu, lead) || S.base[0] <= CK_TINY;
+}
+
 // Scale of an Euler point from its leading state Ws and the exponents top[group][degree >= 1] of its
 // other coefficients.
 template <int NC>
 FX_FN CkScale<NC> ck_scale_from(const double* Ws, const int (&top)[3][5], const CkLead& lead) {
   CkScale<NC> S;
-  const int e0 = fx_max(fx_exp(fx_hi(Ws[0]) & 0x7fffffff), -300);  // an exact 0 then converts to 0 in every field
+  const int e0 = fx_max(fx_exp(fx_hi(Ws[0]) & 0x7fffffff), CK_TINY);  // an exact 0 then converts to 0 in every field
   const int eE = fx_exp(fx_hi(Ws[NC - 1]) & 0x7fffffff);
   int eh = fx_exp(lead.hH);
   // a negative density or pressure (E0 + p0 then no longer bounds E0 and the kinetic energy)
   const int ee = eE - e0 + 3;
   if (ee > eh + 3) eh = ee;
-  S.eu = fx_max(fx_max(fx_exp(lead.hu), (eh + 1) >> 1), -300);
+  S.eu = fx_max(fx_max(fx_exp(lead.hu), (eh + 1) >> 1), CK_TINY);
   S.base[0] = e0;
   S.base[1] = e0 + S.eu;
   S.base[2] = e0 + 2 * S.eu;
@@ -185,7 +196,7 @@ FX_FN void ck_fixed(const double (&a)[NC][25], const CkLead& lead, const CkFixed
   auto coef = [&a](int q, int mn) { return a[q][mn]; };
   CkScale<NC> S = ck_scale<NC, DIM>(coef, lead);
   if constexpr (NC == 3)
-    if (!C.fixed || ck_fast_unit(S.eu, lead)) return ck_euler1d(a, tc, C.gm1);
+    if (!C.fixed || ck_off_units(S, lead)) return ck_euler1d(a, tc, C.gm1);
   Fx w[NC][25], ninv{0, 0};
   int64_t t[NC][5];
   if constexpr (NC > 1) ninv = ck_ninv<NC>(S, lead);

@@ -485,7 +485,7 @@ __device__ __forceinline__ void ck_points(const Params& P, int npt, bool has_fac
   } else {
     CkScale<4> S{};
     if (has_face) S = ck_scale<4, 2>([&a](int q, int mn) { return a[q][mn]; }, lead);
-    if (__syncthreads_or(!P.ck.fixed || (has_face && (ck_fast_unit(S.eu, lead) || ck_coarse2d(a, dir))) ? 1 : 0)) return ck_points64(P, has_face, a, tc);
+    if (__syncthreads_or(!P.ck.fixed || (has_face && (ck_off_units(S, lead) || ck_coarse2d(a, dir))) ? 1 : 0)) return ck_points64(P, has_face, a, tc);
     const double Ws[4] = {a[0][0], a[1][0], a[2][0], a[3][0]};
     FxRange none{0};  // the recursion checks its operands
     ck_points4(P, npt, has_face, S, [&](int q, int mn) { return ck_convert<4>(S, a[q][mn], q, mn / 5 + mn % 5, none); },
@@ -509,7 +509,7 @@ constexpr int FX_BELOW = 6;       // a momentum more bits than this below that s
                                   // and one more than FX_STILL counts as none
 constexpr int FX_UNIT = 5;        // most bits of a face's density and energy below their units
 constexpr int FX_EL = FX_D - 53;  // most bits that the projections' scale takes off
-constexpr int FX_TINY = -300;     // least exponent of a scale
+constexpr int FX_TINY = CK_TINY;  // least exponent of a scale
 struct CellMixFx {
   Fx A[4], B[4], C[4];
   int h[4];  // exponents of the cell's data
@@ -709,7 +709,7 @@ __device__ __forceinline__ void face_setup_fx(const Params& P, const int64_t (*L
   int F = max(max(max(hL[1], hR[1]), max(hL[2], hR[2])) - f0, (max(hL[3], hR[3]) - f0 + 1) >> 1);
   F = max(F, max(fx_exp(lead.hu), (fx_exp(lead.hH) + 1) >> 1));
   int top = 0, el = -2000;
-  bool coarse = ck_fast_unit(F, lead);
+  bool coarse = ck_off_unit(F, lead);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int u = q == 0 ? 0 : q == 3 ? 2 * F : F;

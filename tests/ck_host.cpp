@@ -41,7 +41,44 @@ static void recursion(const double (&a)[3][25], T g, T (&tc)[3][5]) {
     for (int k = 0; k < 5; ++k) tc[q][k] = S[q][0][k];
 }
 
-int main() {
+// Largest difference between the library's step at a state and at the same state in other units (powers of two,
+// which FP64 carries exactly), relative to the state: small or large density and velocity.
+static void units() {
+  std::mt19937_64 rng(3);
+  std::uniform_real_distribution<double> U(-1.0, 1.0);
+  CkFixed C;
+  finalize_ck_fixed(C, 1, 1.0, 1.0, 1.4);
+  for (int er : {0, -200, -299, -301, -330, -400, 300, 500})
+    for (int ev : {0, 20, -20, -100, -290, -305}) {
+      double worst = 0.0;
+      for (int it = 0; it < 200; ++it) {
+        double a[2][3][25] = {}, t[2][3][5];
+        const double W[3] = {1.0 + 0.3 * U(rng), 0.4 * U(rng), 2.5 + 0.3 * U(rng)};
+        for (int q = 0; q < 3; ++q)
+          for (int s = 0; s < 5; ++s) {
+            a[0][q][s * 5] = s == 0 ? W[q] : std::ldexp(U(rng), -3 * s);
+            a[1][q][s * 5] = std::ldexp(a[0][q][s * 5], er + q * ev);
+          }
+        for (int v = 0; v < 2; ++v) {
+          const double ir = 1.0 / a[v][0][0], u = a[v][1][0] * ir, p = 0.4 * (a[v][2][0] - 0.5 * a[v][1][0] * u);
+          const CkLead lead{ir, fx_hi(u) & 0x7fffffff, fx_hi((a[v][2][0] + p) * ir) & 0x7fffffff, fx_hi(std::sqrt(1.4 * p * ir)) & 0x7fffffff};
+          ck_fixed<3, 1>(a[v], lead, C, t[v]);
+        }
+        for (int q = 0; q < 3; ++q)
+          for (int k = 1; k < 5; ++k) {
+            const double unit = std::ldexp(1.0, er + (q + k) * ev);  // 0 or denormal: out of a double's range
+            if (unit > 1e-290 && unit < 1e290) worst = std::fmax(worst, std::fabs(t[1][q][k] / unit - t[0][q][k]));
+          }
+      }
+      std::printf("%d %d %.3e\n", er, ev, worst);
+    }
+}
+
+int main(int argc, char**) {
+  if (argc > 1) {
+    units();
+    return 0;
+  }
   std::mt19937_64 rng(1);
   std::uniform_real_distribution<double> U(-1.0, 1.0);
   for (double g : {1.001, 1.02, 1.1, 1.2, 1.4, 5.0 / 3.0, 3.0, 4.0, 7.0, 30.0, 1e3, 1e6}) {

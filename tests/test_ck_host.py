@@ -15,10 +15,10 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "..", "paper_2304_09724_gb300", "csrc")
 
 
-def build(tmp_path, name):
+def build(tmp_path, name, *args):
     exe = str(tmp_path / name)
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wno-return-type", "-I", CSRC, os.path.join(HERE, name + ".cpp"), "-o", exe])
-    return [list(map(float, line.split())) for line in subprocess.check_output([exe], text=True).splitlines()]
+    return [list(map(float, line.split())) for line in subprocess.check_output([exe, *args], text=True).splitlines()]
 
 
 def test_range_check_sees_every_value(tmp_path):
@@ -64,6 +64,14 @@ def majorant(eps, gm1):
                     S[q][m, n, k + 1] = ((m + 1) * f + (n + 1) * g) / (k + 1)
                     worst = max(worst, S[q][m, n, k + 1]) if k < 3 else worst
     return worst
+
+
+def test_any_units(tmp_path):
+    """The same states in units from 2^-400 to 2^500: a time series differs by its rounding only."""
+    rows = build(tmp_path, "ck_host", "units")
+    assert len(rows) == 48
+    for er, ev, worst in rows:
+        assert worst <= 1e-13, f"density 2^{er:g}, velocity 2^{ev:g}: {worst}"
 
 
 def test_growths_suffice():

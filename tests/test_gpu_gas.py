@@ -1,6 +1,7 @@
 """2D Euler over the gas constants, with cell data that jump from cell to cell: the fixed-point kernels hold gases of
-gamma near 1.4 to 3 (csrc/ck_fixed.cuh) and leave the others to FP64.  Against the oracle with the
-specification's tolerances (tests/gpu_util.py), in all four readings of the reconstruction."""
+gamma near 1.4 to 3 (csrc/ck_fixed.cuh) and leave the others to FP64; and over units of density and velocity far
+below their exponents' range.  Against the oracle with the specification's tolerances
+(tests/gpu_util.py), in all four readings of the reconstruction."""
 import numpy as np
 import pytest
 
@@ -40,3 +41,31 @@ def test_steep_cells(gamma, opt):
     wl = WL.vortex(8)
     wl.nx, wl.ny, wl.domain = nx, ny, (0.0, 1.0, 0.0, 1.0)
     U.check(g, o, "WVYZ", shocked=True, what=f"gamma {gamma:g} {opt}", wl=wl)
+
+
+@pytest.mark.parametrize("er,ev", [(-330, 20), (-305, 0), (-290, -5), (30, -20), (20, 15)])
+@pytest.mark.parametrize("opt", ["plain", "quintic", "charwise", "charwise quintic"])
+@pytest.mark.parametrize("dim", [1, 2])
+def test_units(er, ev, opt, dim):
+    """Density 2^er and velocity 2^ev times that of an ordinary smooth flow."""
+    kw = dict(charwise="charwise" in opt, quintic="quintic" in opt)
+    nx, ny = 40, (1 if dim == 1 else 18)
+    keys = "WV" if dim == 1 else "WVYZ"
+    st = dict(zip(keys, WL.random_smooth_1d(5, nx) if dim == 1 else WL.random_smooth_2d(5, nx, ny)))
+    power = [er] + [er + ev] * dim + [er + 2 * ev]
+    f = np.ldexp(1.0, power).reshape((-1,) + (1,) * dim)
+    st = {k: np.ascontiguousarray(v * f) for k, v in st.items()}
+    dt = float(np.ldexp(0.003, -ev))
+    args = (dim, S.EULER, nx, ny)
+    sol = S.Solver(*args, **kw)
+    sol.set_state(st)
+    P = O.make_problem(*args, 0.0, 1.0, 0.0, 1.0, **kw)
+    o = st
+    for _ in range(2):
+        sol.step(dt)
+        o = O.step(P, o, dt)
+    g = sol.get_state()
+    sol.close()
+    wl = WL.euler1d_sine(8) if dim == 1 else WL.vortex(8)
+    wl.nx, wl.ny, wl.domain = nx, ny, (0.0, 1.0, 0.0, 1.0)
+    U.check({k: v / f for k, v in g.items()}, {k: v / f for k, v in o.items()}, keys, shocked=False, what=f"2^{er} 2^{ev} {opt}", wl=wl)
